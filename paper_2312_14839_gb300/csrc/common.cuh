@@ -85,6 +85,13 @@ struct NewtonScalars {
   int pad_;
 };
 
+// The scalars a step reads back, in one block so that one copy brings them all.
+struct DeviceScalars {
+  PcgState pcg;
+  NewtonScalars ns;
+  int err;             // error bits
+};
+
 // ------------------------------------------------------------------------------------------
 // Shell: everything lives in device memory owned by the library.
 // ------------------------------------------------------------------------------------------
@@ -126,7 +133,16 @@ struct Shell {
   float* d_p32 = nullptr;           // FP32 PCG vectors of a mixed-precision shell
   float *d_x32 = nullptr, *d_r32 = nullptr, *d_z32 = nullptr, *d_Ap32 = nullptr;
   void* d_Dinv = nullptr;           // [n_nodes * 144] block-Jacobi inverses (FP32 or FP64)
+  DeviceScalars* d_scal = nullptr;  // d_pcg, d_ns and d_err point into it
+  DeviceScalars* h_scal = nullptr;  // pinned; h_pcg, h_ns and h_err point into it
   PcgState* d_pcg = nullptr;
+
+  // resident solve (resident.cu): rows per CTA (0: the shell does not use it), its exchange slots and
+  // vector, the next launch's first tag and the CTAs counted in so far; res_reset: clear them first
+  int res_per = 0;
+  bool res_reset = true;
+  unsigned res_tag = 1, res_stat_count = 0;
+  void* d_resident = nullptr;
 
   // Newton workspace
   double *d_qn = nullptr, *d_y = nullptr, *d_g = nullptr, *d_gin = nullptr, *d_d = nullptr;
@@ -278,6 +294,15 @@ shell_status launch_pcg_iteration(Shell& s, const unsigned char* mask, const dou
 // the whole mixed-precision solve as one graph: a conditional WHILE node around one iteration
 shell_status launch_pcg_loop_graph(Shell& s, const unsigned char* mask);
 shell_status launch_pcg_persistent(Shell& s, const unsigned char* mask);
+// the linear solve of one Newton iteration as one cooperative launch with the matrix resident in
+// shared memory (resident.cu); setup_resident leaves res_per 0 on shells it cannot hold.
+// rhs_sign * rhs is the right-hand side; stats: take the diagonal statistics (else those in d_ns);
+// fix: the regulariser's local part; dots: M d into d_Md and d.Md, d.gin, g.d into d_ns->dots (rhs =
+// g). *launched false: the device cannot run it now, nothing was enqueued.
+shell_status setup_resident(Shell& s);
+shell_status launch_solve_resident(Shell& s, const unsigned char* mask, const double* rhs, double rhs_sign, double tau,
+                                   double rtol, int fixed, int limit, bool stats, bool fix, bool dots, double* x,
+                                   bool* launched);
 // kernels per mixed-precision PCG iteration, and whether the p-update rides in the SpMV
 bool pcg_folds_pupdate(const Shell& s);
 int pcg_kernels_per_iteration(const Shell& s);

@@ -129,14 +129,12 @@ static void destroy_shell(shell_s* s) {
   void* ptrs[] = {s->d_patch_nodes, s->d_patch_blocks, s->d_row_ptr, s->d_col, s->d_diag_block, s->d_tpos,
                   s->d_color_list, s->d_rest, s->d_restgp, s->d_mass, s->d_fgrav, s->d_val,
                   s->d_x, s->d_r, s->d_z, s->d_p, s->d_Ap, s->d_p32, s->d_x32, s->d_r32, s->d_z32, s->d_Ap32, s->d_Dinv, s->d_phi64, s->d_phi32,
-                  s->d_pcg, s->d_qn, s->d_y, s->d_g, s->d_gin, s->d_d, s->d_Md, s->d_Ep,
-                  s->d_qwork, s->d_vwork, s->d_qfix, s->d_warm, s->d_mask, s->d_ns, s->d_err, s->d_qmy,
+                  s->d_scal, s->d_resident, s->d_qn, s->d_y, s->d_g, s->d_gin, s->d_d, s->d_Md, s->d_Ep,
+                  s->d_qwork, s->d_vwork, s->d_qfix, s->d_warm, s->d_mask, s->d_qmy,
                   s->d_energy_tmp, s->red.partials, s->red.ticket, s->red_aux.partials, s->red_aux.ticket, s->d_rhs, s->d_g2, s->d_Ep2,
                   s->d_search, s->d_ray_nets, s->d_ccd_nets, s->d_persist};
   for (void* p : ptrs) dfree(p);
-  if (s->h_ns) cudaFreeHost(s->h_ns);
-  if (s->h_pcg) cudaFreeHost(s->h_pcg);
-  if (s->h_err) cudaFreeHost(s->h_err);
+  if (s->h_scal) cudaFreeHost(s->h_scal);
   delete[] s->h_color_patches;
   delete s;
 }
@@ -165,11 +163,12 @@ static void trace_report(Shell& s) {
   s.trace_n = 0;
 }
 
-static shell_status sync_and_check(Shell& s) {
-  BHEM_CUDA(cudaMemcpyAsync(s.h_err, s.d_err, sizeof(int), cudaMemcpyDeviceToHost, s.stream));
+// Waits for the stream; reports the error bits that the caller's copy brought to h_err.
+static shell_status wait_and_check(Shell& s) {
   BHEM_CUDA(cudaStreamSynchronize(s.stream));
   const int bits = *s.h_err;
   if (bits) {
+    s.res_reset = true;   // a solve that gave up leaves counters behind
     BHEM_CUDA(cudaMemsetAsync(s.d_err, 0, sizeof(int), s.stream));
     BHEM_CUDA(cudaStreamSynchronize(s.stream));
   }
@@ -178,6 +177,17 @@ static shell_status sync_and_check(Shell& s) {
   if (bits & ERRBIT_TIMEOUT)
     return fail(SHELL_ERR_TIMEOUT, "a bounded device-side wait expired (bulk copy, grid barrier or tensor-core MMA)");
   return SHELL_OK;
+}
+
+static shell_status sync_and_check(Shell& s) {
+  BHEM_CUDA(cudaMemcpyAsync(s.h_err, s.d_err, sizeof(int), cudaMemcpyDeviceToHost, s.stream));
+  return wait_and_check(s);
+}
+
+// All scalars to the host (h_pcg, h_ns) with one copy, then as sync_and_check.
+static shell_status read_scalars(Shell& s) {
+  BHEM_CUDA(cudaMemcpyAsync(s.h_scal, s.d_scal, sizeof(DeviceScalars), cudaMemcpyDeviceToHost, s.stream));
+  return wait_and_check(s);
 }
 
 }  // namespace bhem
@@ -227,6 +237,7 @@ extern "C" shell_status shell_create(const shell_grid* grid, const shell_materia
   s->mu = material->young / (2.0 * (1.0 + material->poisson));
   s->val_fp64 = opt.precision == SHELL_PREC_FP64;
   s->pcg_host_loop = getenv("BHEM_PCG_HOST_LOOP") != nullptr;
+  bool resident = true;
   {
     const char* m = getenv("BHEM_PCG_LOOP");
     s->pcg_mode = s->pcg_host_loop ? 2 : 1;
@@ -235,14 +246,18 @@ extern "C" shell_status shell_create(const shell_grid* grid, const shell_materia
     if (m && std::strcmp(m, "graph") == 0) s->pcg_cluster_max_nodes = 0;
     if (m && std::strcmp(m, "cluster") == 0) s->pcg_cluster_max_nodes = 1 << 30;
     s->pcg_host_loop = s->pcg_mode == 2;
+    // a caller that names a form of the solve or of its SpMV gets that form
+    resident = !m && !s->pcg_host_loop && opt.solver == SHELL_SOLVER_PCG && opt.spmv == SHELL_SPMV_AUTO;
     const char* pu = getenv("BHEM_PCG_PUPDATE");
     s->pcg_fold_pupdate = !(pu && std::strcmp(pu, "1") == 0);
+    resident = resident && s->pcg_fold_pupdate;
     const char* f = getenv("BHEM_FUSE_FIRST_HESSIAN");
     s->fuse_first_hessian = !(f && std::strcmp(f, "0") == 0);
     const char* el = getenv("BHEM_ELEMENT");
     s->elem_tc = !(el && std::strcmp(el, "ffma") == 0);
     const char* sy = getenv("BHEM_SPMV_SYM");
     s->spmv_sym = sy && std::strcmp(sy, "1") == 0;
+    resident = resident && !s->spmv_sym;
     const char* pd = getenv("BHEM_PDL");
     s->pdl = !(pd && std::strcmp(pd, "0") == 0);
   }
@@ -287,11 +302,11 @@ extern "C" shell_status shell_create(const shell_grid* grid, const shell_materia
     }
   }
   A(s->d_x, m); A(s->d_r, m); A(s->d_z, m); A(s->d_p, m); A(s->d_Ap, m);
-  A(s->d_pcg, 1); A(s->d_p32, m); A(s->d_x32, m); A(s->d_r32, m); A(s->d_z32, m); A(s->d_Ap32, m);
+  A(s->d_scal, 1); A(s->d_p32, m); A(s->d_x32, m); A(s->d_r32, m); A(s->d_z32, m); A(s->d_Ap32, m);
   A(s->d_phi64, 1568); A(s->d_phi32, 1568);
   A(s->d_qn, m); A(s->d_y, m); A(s->d_g, m); A(s->d_gin, m); A(s->d_d, m); A(s->d_Md, m);
   A(s->d_rhs, m); A(s->d_Ep, np); A(s->d_qwork, m); A(s->d_vwork, m); A(s->d_qfix, m); A(s->d_qmy, m);
-  A(s->d_warm, m); A(s->d_mask, m); A(s->d_ns, 1); A(s->d_err, 1); A(s->d_energy_tmp, 1);
+  A(s->d_warm, m); A(s->d_mask, m); A(s->d_energy_tmp, 1);
   A(s->d_g2, m); A(s->d_Ep2, np);
   // partials: one per CTA of the largest reducing launch (8 patches, 4 FP64 block rows, 16 nodes or
   // 1024 vector CTAs per CTA) per reduced value
@@ -303,10 +318,17 @@ extern "C" shell_status shell_create(const shell_grid* grid, const shell_materia
   A(s->red_aux.ticket, 1);
 #undef A
   if (st == SHELL_OK) {
-    cudaError_t e1 = cudaMallocHost((void**)&s->h_ns, sizeof(NewtonScalars));
-    cudaError_t e2 = cudaMallocHost((void**)&s->h_pcg, sizeof(PcgState));
-    cudaError_t e3 = cudaMallocHost((void**)&s->h_err, sizeof(int));
-    if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess) st = fail(SHELL_ERR_OOM, "cudaMallocHost failed");
+    if (cudaMallocHost((void**)&s->h_scal, sizeof(DeviceScalars)) != cudaSuccess) {
+      s->h_scal = nullptr;
+      st = fail(SHELL_ERR_OOM, "cudaMallocHost failed");
+    } else {
+      s->d_pcg = &s->d_scal->pcg;
+      s->d_ns = &s->d_scal->ns;
+      s->d_err = &s->d_scal->err;
+      s->h_pcg = &s->h_scal->pcg;
+      s->h_ns = &s->h_scal->ns;
+      s->h_err = &s->h_scal->err;
+    }
   }
   if (st != SHELL_OK) {
     destroy_shell(s);
@@ -325,10 +347,9 @@ extern "C" shell_status shell_create(const shell_grid* grid, const shell_materia
   if (e == cudaSuccess) e = up(s->d_color_list, T.color_list.data(), sizeof(int) * np);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(s->d_rest, rest_dofs, sizeof(double) * m, cudaMemcpyDefault, s->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(s->d_err, 0, sizeof(int), s->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(s->d_scal, 0, sizeof(DeviceScalars), s->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(s->red.ticket, 0, sizeof(unsigned), s->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(s->red_aux.ticket, 0, sizeof(unsigned), s->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(s->d_pcg, 0, sizeof(PcgState), s->stream);
   if (e != cudaSuccess) {
     destroy_shell(s);
     return fail(SHELL_ERR_CUDA, std::string("upload: ") + cudaGetErrorString(e));
@@ -338,6 +359,7 @@ extern "C" shell_status shell_create(const shell_grid* grid, const shell_materia
     s->trace = (tv && tv[0] == '1') ? 1 : 0;
   }
   st = setup_spmv(*s);
+  if (st == SHELL_OK && resident) st = setup_resident(*s);
   if (st == SHELL_OK) st = launch_rest_setup(*s);
   if (st == SHELL_OK) st = sync_and_check(*s);
   if (st != SHELL_OK) {
@@ -530,6 +552,17 @@ extern "C" shell_status shell_pcg_solve(shell_t* shell, const unsigned char* fix
   if (!shell || !rhs || !x) return fail(SHELL_ERR_ARG, "NULL argument");
   if (max_iter < 0 || fixed_iters < 0 || !(tau >= 0.0)) return fail(SHELL_ERR_ARG, "invalid PCG limits");
   int it = 0, neg = 0;
+  if (shell->res_per > 0) {
+    bool launched = false;
+    BHEM_TRY(launch_solve_resident(*shell, fixed_mask, rhs, 1.0, tau, rtol, fixed_iters,
+                                   fixed_iters > 0 ? fixed_iters : max_iter, true, false, false, x, &launched));
+    if (launched) {
+      BHEM_TRY(read_scalars(*shell));
+      if (iters) *iters = shell->h_pcg->iters;
+      if (neg_curv) *neg_curv = shell->h_pcg->negcurv;
+      return SHELL_OK;
+    }
+  }
   KindStats K;
   BHEM_TRY(kind_stats(*shell, fixed_mask, K));
   const double td[4] = {tau * K.dbar[0], tau * K.dbar[1], tau * K.dbar[2], tau * K.dbar[3]};
@@ -551,8 +584,7 @@ static shell_status residual(Shell& s, const double* q, const shell_step_params&
   BHEM_TRY(launch_energy_grad64(s, q, nullptr, 0.0, s.d_Ep, nullptr, s.d_g, &s.d_ns->energy));
   BHEM_TRY(launch_grad_finish(s, q, s.d_y, P.dt, P.gravity, mask, s.d_g, s.d_gin, &s.d_ns->gnorm2));
   if (also_wait) BHEM_CUDA(cudaStreamWaitEvent(s.stream, also_wait, 0));
-  BHEM_CUDA(cudaMemcpyAsync(s.h_ns, s.d_ns, sizeof(NewtonScalars), cudaMemcpyDeviceToHost, s.stream));
-  BHEM_TRY(sync_and_check(s));
+  BHEM_TRY(read_scalars(s));
   *gnorm = std::sqrt(s.h_ns->gnorm2);
   return SHELL_OK;
 }
@@ -573,10 +605,9 @@ static shell_status residual_with_hessian(Shell& s, const double* q, const shell
   o.energy64 = s.d_Ep;
   o.grad64 = s.d_g;
   BHEM_TRY(launch_element_full(s, q, false, o));
-  BHEM_TRY(launch_diag_check(s, mask, s.d_ns->diag_stats, true));
+  if (s.res_per == 0) BHEM_TRY(launch_diag_check(s, mask, s.d_ns->diag_stats, true));   // else taken by the solve
   BHEM_TRY(launch_grad_finish(s, q, s.d_y, P.dt, P.gravity, mask, s.d_g, s.d_gin, &s.d_ns->gnorm2));
-  BHEM_CUDA(cudaMemcpyAsync(s.h_ns, s.d_ns, sizeof(NewtonScalars), cudaMemcpyDeviceToHost, s.stream));
-  BHEM_TRY(sync_and_check(s));
+  BHEM_TRY(read_scalars(s));
   *gnorm = std::sqrt(s.h_ns->gnorm2);
   return SHELL_OK;
 }
@@ -587,8 +618,7 @@ static shell_status residual_with_hessian(Shell& s, const double* q, const shell
 static shell_status residual_reuse(Shell& s, const shell_step_params& P, const unsigned char* mask,
                                    double* gnorm) {
   BHEM_TRY(launch_grad_linear(s, s.d_Md, 1.0, P.dt, mask, s.d_g, s.d_gin, &s.d_ns->gnorm2));
-  BHEM_CUDA(cudaMemcpyAsync(s.h_ns, s.d_ns, sizeof(NewtonScalars), cudaMemcpyDeviceToHost, s.stream));
-  BHEM_TRY(sync_and_check(s));
+  BHEM_TRY(read_scalars(s));
   *gnorm = std::sqrt(s.h_ns->gnorm2);
   return SHELL_OK;
 }
@@ -665,7 +695,7 @@ static shell_status newton_core(Shell& s, const shell_step_params& P, const unsi
     // iteration's tau; each negative curvature met by PCG multiplies tau by 10 (at least 1e-8),
     // beyond 1e4 the step gives up.
     KindStats K;
-    const bool from_pending = hess_pending || hess_ready;
+    bool stats_read = hess_pending || (hess_ready && s.res_per == 0);
     if (hess_pending) {   // assembled and its statistics read with the residual (joined there)
       BHEM_CUDA(cudaStreamWaitEvent(s.stream, s.ev_hess, 0));
       hess_pending = false;
@@ -675,36 +705,58 @@ static shell_status newton_core(Shell& s, const shell_step_params& P, const unsi
       BHEM_TRY(assemble_hessian(s, q, inv_dt2));
     }
     mark(s, "assemble_enqueued");
-    BHEM_TRY(launch_negate(s, s.d_g, s.d_rhs));
-    if (from_pending) kind_stats_from_host(s, K);
-    else BHEM_TRY(kind_stats(s, mask, K));
-    mark(s, "kind_stats");
-    BHEM_TRY(fix_diagonal(s, mask, K));
     double tau = tau_carry / 10.0;
     if (tau < 1e-8) tau = 0.0;
-    for (;;) {
-      if (tau > 1e4) { status = SHELL_ERR_INDEFINITE; break; }
-      int pit = 0, neg = 0;
-      const double td[4] = {tau * K.dbar[0], tau * K.dbar[1], tau * K.dbar[2], tau * K.dbar[3]};
-      if (s.opt.solver == SHELL_SOLVER_DIRECT)
-        BHEM_TRY(run_direct(s, mask, td, s.d_rhs, &neg));
-      else
-        BHEM_TRY(run_pcg(s, mask, td, s.d_rhs, P.pcg_rtol, P.pcg_max, P.pcg_fixed_iters, &pit, &neg));
-      st.pcg_iters_total += pit;
-      if (tau > 0.0) st.regularizations++;
-      if (!neg) break;
-      tau = std::max(10.0 * tau, 1e-8);
+    const bool search = gn > 1e-6 * gref;
+    bool solved = false;   // by the resident solve, with M d and the line search's dot products
+    if (s.res_per > 0) {
+      for (bool first = true;; first = false) {
+        if (tau > 1e4) { status = SHELL_ERR_INDEFINITE; break; }
+        BHEM_TRY(launch_solve_resident(s, mask, s.d_g, -1.0, tau, P.pcg_rtol, P.pcg_fixed_iters,
+                                       P.pcg_fixed_iters > 0 ? P.pcg_fixed_iters : P.pcg_max, first, first, search,
+                                       s.d_d, &solved));
+        if (!solved) break;
+        BHEM_TRY(read_scalars(s));
+        mark(s, "solve_resident");
+        st.pcg_iters_total += s.h_pcg->iters;
+        if (tau > 0.0) st.regularizations++;
+        if (!s.h_pcg->negcurv) break;
+        tau = std::max(10.0 * tau, 1e-8);
+      }
+      if (status != SHELL_OK) break;
     }
-    if (status != SHELL_OK) break;
+    if (!solved) {
+      BHEM_TRY(launch_negate(s, s.d_g, s.d_rhs));
+      if (stats_read) kind_stats_from_host(s, K);
+      else BHEM_TRY(kind_stats(s, mask, K));
+      mark(s, "kind_stats");
+      BHEM_TRY(fix_diagonal(s, mask, K));
+      for (;;) {
+        if (tau > 1e4) { status = SHELL_ERR_INDEFINITE; break; }
+        int pit = 0, neg = 0;
+        const double td[4] = {tau * K.dbar[0], tau * K.dbar[1], tau * K.dbar[2], tau * K.dbar[3]};
+        if (s.opt.solver == SHELL_SOLVER_DIRECT)
+          BHEM_TRY(run_direct(s, mask, td, s.d_rhs, &neg));
+        else
+          BHEM_TRY(run_pcg(s, mask, td, s.d_rhs, P.pcg_rtol, P.pcg_max, P.pcg_fixed_iters, &pit, &neg));
+        st.pcg_iters_total += pit;
+        if (tau > 0.0) st.regularizations++;
+        if (!neg) break;
+        tau = std::max(10.0 * tau, 1e-8);
+      }
+      if (status != SHELL_OK) break;
+      BHEM_CUDA(cudaMemcpyAsync(s.d_d, s.d_x, sizeof(double) * m, cudaMemcpyDeviceToDevice, s.stream));
+    }
     tau_carry = tau;
-    BHEM_CUDA(cudaMemcpyAsync(s.d_d, s.d_x, sizeof(double) * m, cudaMemcpyDeviceToDevice, s.stream));
     // line search on phi(a) = Pi(q + a d) - Pi(q) = dV(a) + a d.g_in + a^2/2 d^T M d / dt^2
     double alpha = 1.0;
-    if (gn > 1e-6 * gref) {
-      BHEM_TRY(launch_mass_mult(s, s.d_d, s.d_Md));
-      BHEM_TRY(launch_dots3(s, m, s.d_d, s.d_Md, s.d_d, s.d_gin, s.d_g, s.d_d, s.d_ns->dots));
-      BHEM_CUDA(cudaMemcpyAsync(s.h_ns, s.d_ns, sizeof(NewtonScalars), cudaMemcpyDeviceToHost, s.stream));
-      BHEM_CUDA(cudaStreamSynchronize(s.stream));
+    if (search) {
+      if (!solved) {
+        BHEM_TRY(launch_mass_mult(s, s.d_d, s.d_Md));
+        BHEM_TRY(launch_dots3(s, m, s.d_d, s.d_Md, s.d_d, s.d_gin, s.d_g, s.d_d, s.d_ns->dots));
+        BHEM_CUDA(cudaMemcpyAsync(s.h_ns, s.d_ns, sizeof(NewtonScalars), cudaMemcpyDeviceToHost, s.stream));
+        BHEM_CUDA(cudaStreamSynchronize(s.stream));
+      }
       mark(s, "ls_dots");
       const double dMd = s.h_ns->dots[0] * inv_dt2, dgin = s.h_ns->dots[1], gd = s.h_ns->dots[2];
       if (!(gd < 0.0)) { status = SHELL_ERR_LINESEARCH; break; }
