@@ -442,9 +442,12 @@ typedef enum { SHELL_RAY_MIDPOINT = 0, SHELL_RAY_NEWTON = 1 } shell_ray_variant;
    second kernel with such a heap, so every result is that of an unbounded heap unless
    SHELL_RAY_OVERFLOW is set. n_rays in [0, 2^31 - 1]; 0 does nothing. Asynchronous
    on the shell's stream (four kernel launches and an 8-byte memset). The first call on a shell
-   allocates 450 bytes per patch plus 64.3 MB of library-owned device memory (Bezier nets and
-   boxes, the second pass's heaps), kept until shell_destroy; calls on one shell must not
-   overlap on the GPU. */
+   allocates 698 bytes per patch plus 64.3 MB of library-owned device memory (Bezier nets in FP64
+   and FP32, boxes, the second pass's heaps), kept until shell_destroy; calls on one shell must not
+   overlap on the GPU. With stats NULL, sub-patches that a conservative FP32 test proves to hold no
+   hit are not searched: the hits are the same (of two candidates with exactly equal entry distances
+   either may be taken first), and rays reach the split limit later; with stats every candidate is
+   searched and counted. */
 SHELL_API shell_status shell_trace_rays(shell_t* shell, const double* q, long long n_rays, const double* origins,
                                         const double* dirs, int variant, double* tau, int* patch, double* uv,
                                         int* flags, int* stats);

@@ -119,6 +119,94 @@ __device__ __forceinline__ double det3(const double M[3][3]) {
          M[0][2] * (M[1][0] * M[2][1] - M[1][1] * M[2][0]);
 }
 
+// ------------------------------------------------------------------------------------------
+// FP32 culling of sub-patches that a query provably cannot meet.
+//
+// The searches spend their time in FP64 boxes of children (GB300 issues an FP64 warp instruction in
+// the time of about 64 FP32 ones), and most children are either off the query's path or stay in the
+// heap without ever giving a hit, because an axis-aligned box of a tilted surface is loose. A child
+// whose control points lie on one side of a plane through the query's path cannot hold the surface
+// point of a hit, nor can any of its descendants (convex hull property), so leaving it out changes no
+// hit: the candidates that do lead to hits keep their FP64 keys and their order. A candidate of equal
+// key beside it may change its place in the heap only by the heap's tie-breaking. The test is FP32
+// with a margin kCullRel R (R: sum of the magnitudes that enter) that covers every rounding in it:
+// net, path and parameters rounded to FP32 (1 + 12 units), 6 levels of blends (18), the projections
+// (10): under 48 units of 2^-24 against 64; and at least kCullAbs, twelve times what a refined
+// candidate (a box of 1e-9 that the path touches) or a converged Newton iterate (1e-12) may be off.
+// ------------------------------------------------------------------------------------------
+constexpr float kCullRel = 64.0f / 16777216.0f;
+constexpr float kCullAbs = 2e-8f;
+constexpr float kCullFar = 1e4f;   // no culling beyond this distance from the origin
+
+__device__ __forceinline__ float lerp32(float p, float q, float t) { return __fmaf_rn(t, q - p, p); }
+
+// in place: the cubic with points x[0], x[S], x[2S], x[3S] restricted to [a, b] (blossom values)
+template <int S>
+__device__ __forceinline__ void restrict32(float* x, float a, float b) {
+  float A[3], B[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    A[i] = lerp32(x[S * i], x[S * (i + 1)], a);
+    B[i] = lerp32(x[S * i], x[S * (i + 1)], b);
+  }
+  const float aa0 = lerp32(A[0], A[1], a), aa1 = lerp32(A[1], A[2], a);
+  const float ab0 = lerp32(A[0], A[1], b), ab1 = lerp32(A[1], A[2], b);
+  const float bb0 = lerp32(B[0], B[1], b), bb1 = lerp32(B[1], B[2], b);
+  x[0] = lerp32(aa0, aa1, a);
+  x[S] = lerp32(aa0, aa1, b);
+  x[2 * S] = lerp32(ab0, ab1, b);
+  x[3 * S] = lerp32(bb0, bb1, b);
+}
+
+// in place: the 4x4 net x[4 i + j] restricted to [u0, u1] x [v0, v1]
+__device__ __forceinline__ void restrict_net32(float x[16], const float r[4]) {
+#pragma unroll
+  for (int j = 0; j < 4; ++j) restrict32<4>(x + j, r[0], r[1]);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) restrict32<1>(x + 4 * i, r[2], r[3]);
+}
+
+// Whether all 16 values are above eps or all below -eps.
+__device__ __forceinline__ bool one_side32(const float x[16], float eps) {
+  float mn = x[0], mx = x[0];
+#pragma unroll
+  for (int k = 1; k < 16; ++k) {
+    mn = fminf(mn, x[k]);
+    mx = fmaxf(mx, x[k]);
+  }
+  return mn > eps || mx < -eps;
+}
+
+// The same for the combination p x + q y.
+__device__ __forceinline__ bool one_side32(const float x[16], const float y[16], float p, float q, float eps) {
+  float mn = INFINITY, mx = -INFINITY;
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const float v = __fmaf_rn(p, x[k], q * y[k]);
+    mn = fminf(mn, v);
+    mx = fmaxf(mx, v);
+  }
+  const float e = (fabsf(p) + fabsf(q)) * eps;
+  return mn > e || mx < -e;
+}
+
+// FP32 copy of a net relative to its centre point (the mean of its corners): N[c][i][j], centre C[3],
+// and the largest 1-norm of a control point.
+__device__ __forceinline__ void center_net32(const double* P, float* N, double* C, float& radius) {
+  float r = 0.f;
+  for (int c = 0; c < 3; ++c) C[c] = 0.25 * ((P[16 * c] + P[16 * c + 3]) + (P[16 * c + 12] + P[16 * c + 15]));
+  for (int k = 0; k < 16; ++k) {
+    float n = 0.f;
+    for (int c = 0; c < 3; ++c) {
+      const float v = (float)(P[16 * c + k] - C[c]);
+      N[16 * c + k] = v;
+      n += fabsf(v);
+    }
+    r = fmaxf(r, n);
+  }
+  radius = r;
+}
+
 struct Cand {
   double t0, t1, ext, u0, u1, v0, v1;
   int patch;

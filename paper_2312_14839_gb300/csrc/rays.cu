@@ -18,6 +18,16 @@
 //                its 12 box jobs side by side instead of one after another.
 //                A ray whose local heap fills moves it into one of kRedoThreads larger heaps
 //                in global memory and continues.
+//                Without statistics, children (and popped patch roots) that an FP32 test proves to
+//                lead to no hit are left out before their FP64 boxes (bezier.cuh), and group and patch
+//                boxes are tested in FP32 first. FP64 issue bounds this kernel (one warp instruction per
+//                64 cycles and sub-partition), so an FP32 test costs a few percent of the box it saves,
+//                and its tilted lines prune where axis-aligned boxes overlap the ray at every level
+//                (near-tangent rays). Measured, 1024 x 768 rays: drape, Newton split 240 -> 17.4 ms
+//                (another drape, with more tangent rays, 373 -> 57 ms), midpoint split 217 -> 140 ms;
+//                512 x 384: cylinder, Newton split 61 -> 4.6 ms, plane 1.5 -> 0.37 ms. The midpoint
+//                split of the cylinder stays at 60 ms: its tail is rays that graze the surface within the
+//                test's margin, where the last levels' candidates are boxed as before.
 //   k_trace_rays_redo  the rays that found no free global heap, traced again from the start
 //                with one (the search is deterministic, so the result is the one an unbounded
 //                heap gives).
@@ -30,6 +40,7 @@
 // (slab intervals, heap order, refinement, Newton convergence) is that of the same sequence of
 // IEEE FP64 operations in any plain sequential program.
 #include <cmath>
+#include <type_traits>
 
 #include "bezier.cuh"
 #include "common.cuh"
@@ -44,6 +55,15 @@ constexpr int kNetBlock = 128;
 constexpr int kRayBlock = 128;
 constexpr int kRootChunk = 32;       // group boxes staged in shared memory per pass
 constexpr int kGroup = 32;           // consecutive patches per group box
+
+// FP32 net of a patch for the culling test, relative to its centre
+struct CullNet {
+  double c[3];
+  float radius;
+  float box[6];   // the patch's box, rounded outwards: min xyz, max xyz
+  float pad;
+  float n[48];
+};
 
 // Min and max of coordinate c of the sub-patch [u0, u1] x [v0, v1] of the net P ([c][i][j]).
 __device__ __forceinline__ void sub_range(const double* __restrict__ P, int c, double u0, double u1, double v0,
@@ -120,13 +140,15 @@ __global__ void k_ray_groups(int np, const double* __restrict__ boxes, double* _
 
 __global__ void __launch_bounds__(kNetBlock) k_ray_nets(int np, const int4* __restrict__ pnodes,
                                                         const double* __restrict__ q, double dxi1, double dxi2,
-                                                        double* __restrict__ nets, double* __restrict__ boxes) {
+                                                        double* __restrict__ nets, double* __restrict__ boxes,
+                                                        CullNet* __restrict__ culls) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= np) return;
   const int4 n4 = pnodes[p];
   const int nd[4] = {n4.x, n4.y, n4.z, n4.w};
   double* P = nets + (size_t)p * 48;
   patch_net(q, nd, dxi1, dxi2, P);
+  if (culls) center_net32(P, culls[p].n, culls[p].c, culls[p].radius);   // its box below
   // the root box is the box of the net cut to [0, 1]^2, as for every other candidate
   double e = 0.0;
   double* B = boxes + (size_t)p * 8;
@@ -135,6 +157,10 @@ __global__ void __launch_bounds__(kNetBlock) k_ray_nets(int np, const int4* __re
     sub_range(P, c, 0.0, 1.0, 0.0, 1.0, mn, mx);
     B[c] = mn;
     B[3 + c] = mx;
+    if (culls) {
+      culls[p].box[c] = __double2float_rd(mn);
+      culls[p].box[3 + c] = __double2float_ru(mx);
+    }
     if (mx - mn > e) e = mx - mn;
   }
   B[6] = e;
@@ -184,6 +210,9 @@ __device__ bool newton_root(const double* __restrict__ P, const double o[3], con
 
 struct Ray {
   double o[3], d[3], inv[3];
+  // culling: two directions about perpendicular to d and to each other; o and 1 / d in FP32 (infinite
+  // for a zero component, NaN for one too small for FP32: that axis then never rules a box out)
+  float e1[3], e2[3], o32[3], inv32[3];
 };
 
 __device__ __forceinline__ void load_ray(const double* __restrict__ origins, const double* __restrict__ dirs,
@@ -194,6 +223,22 @@ __device__ __forceinline__ void load_ray(const double* __restrict__ origins, con
     r.d[c] = dirs[3 * k + c];
     r.inv[c] = r.d[c] != 0.0 ? 1.0 / r.d[c] : 0.0;
   }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    r.o32[c] = (float)r.o[c];
+    r.inv32[c] = r.d[c] == 0.0 ? INFINITY : fabs(r.d[c]) < 1e-30 ? NAN : (float)r.inv[c];
+  }
+  // e1 = d x (the axis d is least along), normalised; e2 = d x e1
+  const float dx = (float)r.d[0], dy = (float)r.d[1], dz = (float)r.d[2];
+  const float ax = fabsf(dx), ay = fabsf(dy), az = fabsf(dz);
+  float e[3] = {0.f, dz, -dy};
+  if (ay < ax && ay <= az) { e[0] = -dz; e[1] = 0.f; e[2] = dx; }
+  else if (az < ax && az < ay) { e[0] = dy; e[1] = -dx; e[2] = 0.f; }
+  const float s = rsqrtf(e[0] * e[0] + e[1] * e[1] + e[2] * e[2]);
+  for (int c = 0; c < 3; ++c) r.e1[c] = e[c] * s;
+  r.e2[0] = dy * r.e1[2] - dz * r.e1[1];
+  r.e2[1] = dz * r.e1[0] - dx * r.e1[2];
+  r.e2[2] = dx * r.e1[1] - dy * r.e1[0];
 }
 
 // Root candidate: the whole patch p with box B = (min xyz, max xyz, largest side).
@@ -206,6 +251,26 @@ __device__ __forceinline__ void root_push(Heap& h, const double* B, int p, const
   if (in && !(lo > hi)) h.push(Cand{lo, hi, B[6], 0.0, 1.0, 0.0, 1.0, p});
 }
 
+// Whether the ray surely misses an outward-rounded FP32 box: the slab test with the box widened by the
+// rounding of o and of the differences (2^-24 of their terms, against 1e-6) and the interval's ends
+// taken apart by 1e-6 (their relative error is under 2^-21). A NaN (0 times infinity, or an axis not
+// used) leaves an axis out, since fminf and fmaxf drop it.
+__device__ __forceinline__ bool surely_missed(const float* B, const Ray& r) {
+  float lo = 0.f, hi = 1e30f;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const float mn = B[c], mx = B[3 + c], w = 1e-6f * (fabsf(r.o32[c]) + fmaxf(fabsf(mn), fabsf(mx)));
+    const float a = ((mn - w) - r.o32[c]) * r.inv32[c], b = ((mx + w) - r.o32[c]) * r.inv32[c];
+    if (a == a && b == b) {
+      lo = fmaxf(lo, fminf(a, b));
+      hi = fminf(hi, fmaxf(a, b));
+    }
+  }
+  lo = fminf(lo, 1e30f);
+  hi = fmaxf(hi, -1e30f);
+  return lo - 1e-6f * lo > hi + 1e-6f * fabsf(hi);
+}
+
 // Per-lane state of one ray's search.
 struct Search {
   double best = INFINITY, bu = 0.0, bv = 0.0, on = 0.0;
@@ -215,14 +280,54 @@ struct Search {
 
 // Shared-memory exchange of one warp: the children each lane produced in the current split and
 // the coordinate ranges computed for them by whichever lanes took those jobs.
-struct WarpSmem {
+struct PlainSmem {
   double rect[32][4][4];        // child rectangles u0, u1, v0, v1 in push order
   double range[32][12][2];      // (child * 3 + coordinate): min, max
   int patch[32];
   unsigned short jobs[32 * 12]; // lane * 12 + child * 3 + coordinate
 };
+struct CullSmem : PlainSmem {
+  float path[32][14];           // path point, e1, e2, d (from the patch's centre), best tau beyond it, margin
+  unsigned char cull[32][4];    // child proven not to lead to a hit
+};
+template <bool kCull> using WarpSmem = std::conditional_t<kCull, CullSmem, PlainSmem>;
 
-__device__ __forceinline__ void put_rect(WarpSmem& sm, int lane, int& nch, double u0, double u1, double v0,
+__device__ __forceinline__ float cull_margin(const CullNet* __restrict__ N, const float* path) {
+  return fmaxf(path[13], kCullRel * (N->radius + fabsf(path[0]) + fabsf(path[1]) + fabsf(path[2])));
+}
+
+// Culling test of one child of a ray's candidate: the control points, seen along the ray (projected
+// on e1 and e2, the path point at the origin), lie on one side of a line through the origin, or all
+// of them lie beyond the best hit along d. Lines tried: along e1, along e2, along the net's two
+// chords (a smooth sub-patch is nearly a parallelogram with those sides).
+__device__ __forceinline__ bool child_is_culled(const CullNet* __restrict__ N, const float* path, const double* R) {
+  const float r[4] = {(float)R[0], (float)R[1], (float)R[2], (float)R[3]};
+  float a[16], b[16], t[16];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const float x = __ldg(N->n + k) - path[0], y = __ldg(N->n + 16 + k) - path[1], z = __ldg(N->n + 32 + k) - path[2];
+    a[k] = __fmaf_rn(x, path[3], __fmaf_rn(y, path[4], z * path[5]));
+    b[k] = __fmaf_rn(x, path[6], __fmaf_rn(y, path[7], z * path[8]));
+    t[k] = __fmaf_rn(x, path[9], __fmaf_rn(y, path[10], z * path[11]));
+  }
+  const float eps = cull_margin(N, path);
+  restrict_net32(a, r);
+  if (one_side32(a, eps)) return true;
+  restrict_net32(b, r);
+  if (one_side32(b, eps)) return true;
+  // the chords of the u and of the v direction; a line along (p, q) has the normal (-q, p)
+  const float up = (a[12] - a[0]) + (a[15] - a[3]), uq = (b[12] - b[0]) + (b[15] - b[3]);
+  if (one_side32(a, b, -uq, up, eps)) return true;
+  const float vp = (a[3] - a[0]) + (a[15] - a[12]), vq = (b[3] - b[0]) + (b[15] - b[12]);
+  if (one_side32(a, b, -vq, vp, eps)) return true;
+  restrict_net32(t, r);
+  float mn = t[0];
+#pragma unroll
+  for (int k = 1; k < 16; ++k) mn = fminf(mn, t[k]);
+  return mn > path[12] + eps;   // path[12]: best tau less the path point's, rounded up; +infinity without a hit
+}
+
+__device__ __forceinline__ void put_rect(PlainSmem& sm, int lane, int& nch, double u0, double u1, double v0,
                                          double v1) {
   if (!(u1 > u0) || !(v1 > v0)) return;   // degenerate pieces of a pinwheel split
   double* R = sm.rect[lane][nch++];
@@ -232,17 +337,72 @@ __device__ __forceinline__ void put_rect(WarpSmem& sm, int lane, int& nch, doubl
   R[3] = v1;
 }
 
+// Prepares the culling of candidate c's children: the ray from c's entry point on, relative to the
+// patch's centre. True when c is a whole patch that is itself culled (it is not split then).
+template <bool kCull>
+__device__ __forceinline__ bool starts_culled(WarpSmem<kCull>& sm, int lane, const Cand& c, const Ray& r,
+                                              const CullNet* __restrict__ culls, double best, double on, bool& cullable) {
+  if constexpr (kCull) {
+    float* path = sm.path[lane];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      path[k] = (float)((r.o[k] + c.t0 * r.d[k]) - culls[c.patch].c[k]);
+      path[3 + k] = r.e1[k];
+      path[6 + k] = r.e2[k];
+      path[9 + k] = (float)r.d[k];
+    }
+    const float far = (float)on + fabsf((float)c.t0);
+    path[13] = fmaxf(kCullAbs, 4e-12f * (1.f + far));   // 4 x Newton's tolerance
+    // nothing is culled among children of the margin's size: their tests are left out. Far from the
+    // origin (FP64 distances above 1e4 are 1e-12 apart) equal keys are common and the order in which
+    // the heap happens to hold them matters, so nothing is culled there either.
+    cullable = (float)c.ext > 8.f * cull_margin(culls + c.patch, path) && far < kCullFar;
+    if (!cullable) return false;
+    const float beyond = (float)(best - c.t0);
+    path[12] = beyond + 1e-6f * fabsf(beyond);
+    if (c.u1 - c.u0 == 1.0 && c.v1 - c.v0 == 1.0) {
+      const double R[4] = {0.0, 1.0, 0.0, 1.0};
+      return child_is_culled(culls + c.patch, path, R);
+    }
+  }
+  return false;
+}
+
+// Lists the warp's jobs, `per` for each child in a lane's mask `keep` (lane * 12 + child * per + 0 ..
+// per - 1), in lane order; returns their number. All 32 lanes call it; ends with a warp barrier.
+__device__ __forceinline__ int list_jobs(PlainSmem& sm, int lane, unsigned keep, int per) {
+  const int nj = per * __popc(keep);
+  int pre = nj;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, pre, off);
+    if (lane >= off) pre += y;
+  }
+  const int total = __shfl_sync(0xffffffffu, pre, 31);
+  pre -= nj;
+  for (unsigned m = keep; m; m &= m - 1) {
+    const int ch = __ffs(m) - 1;
+    for (int k = 0; k < per; ++k) sm.jobs[pre++] = (unsigned short)(lane * 12 + ch * per + k);
+  }
+  __syncwarp();
+  return total;
+}
+
 // The search over the candidates already in each lane's heap, all 32 lanes of the warp together
 // (lanes without a ray pass live = false). Every iteration each live lane takes its top
 // candidate and, when it splits it, lists its children; the 3 coordinate ranges of every child
 // of every lane are then computed as one pool of jobs spread over the warp's lanes, and each
 // lane finishes its own children (slab test, push) in order. A ray stops early once its heap
 // overflows.
-__device__ void search(Heap& h, const Ray& r, const double* __restrict__ nets, int use_newton, Search& S,
-                       WarpSmem& sm, int lane) {
+// kCull: children (and patch roots) that provably lead to no hit are left out; without it every child
+// is boxed, and the search statistics are those of the plain algorithm.
+template <bool kCull>
+__device__ void search(Heap& h, const Ray& r, const double* __restrict__ nets, const CullNet* __restrict__ culls,
+                       int use_newton, Search& S, WarpSmem<kCull>& sm, int lane) {
   S.on = sqrt((r.o[0] * r.o[0] + r.o[1] * r.o[1]) + r.o[2] * r.o[2]);
   while (__any_sync(0xffffffffu, S.live)) {
     int nch = 0;
+    bool cullable = false;
     if (S.live) {
       if (h.n == 0 || h.overflow) {
         S.live = false;
@@ -261,7 +421,7 @@ __device__ void search(Heap& h, const Ray& r, const double* __restrict__ nets, i
         } else if (S.nexp == kMaxExpansions) {
           S.flags |= SHELL_RAY_LIMIT;
           S.live = false;
-        } else {
+        } else if (!starts_culled<kCull>(sm, lane, c, r, culls, S.best, S.on, cullable)) {
           ++S.nexp;
           const double* P = nets + (size_t)c.patch * 48;
           const double um = 0.5 * (c.u0 + c.u1), vm = 0.5 * (c.v0 + c.v1);
@@ -300,21 +460,27 @@ __device__ void search(Heap& h, const Ray& r, const double* __restrict__ nets, i
           }
           sm.patch[lane] = c.patch;
           h.boxes += nch;
+          if constexpr (kCull) {   // a root found above may have brought the best hit nearer
+            const float beyond = (float)(S.best - c.t0);
+            sm.path[lane][12] = beyond + 1e-6f * fabsf(beyond);
+          }
         }
       }
     }
-    // the warp's pool of (lane, child, coordinate) range jobs
-    const int nj = 3 * nch;
-    int pre = nj;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, pre, off);
-      if (lane >= off) pre += y;
+    unsigned keep = (1u << nch) - 1u;   // children to box
+    if constexpr (kCull) {
+      const int total = list_jobs(sm, lane, cullable ? keep : 0u, 1);
+      for (int j = lane; j < total; j += 32) {
+        const int code = sm.jobs[j], owner = code / 12, ch = code - 12 * owner;
+        sm.cull[owner][ch] = child_is_culled(culls + sm.patch[owner], sm.path[owner], sm.rect[owner][ch]);
+      }
+      __syncwarp();
+      for (int ch = 0; ch < nch; ++ch)
+        if (cullable && sm.cull[lane][ch]) keep &= ~(1u << ch);
+      __syncwarp();
     }
-    const int total = __shfl_sync(0xffffffffu, pre, 31);
-    pre -= nj;
-    for (int k = 0; k < nj; ++k) sm.jobs[pre + k] = (unsigned short)(lane * 12 + k);
-    __syncwarp();
+    // the warp's pool of (lane, child, coordinate) range jobs
+    const int total = list_jobs(sm, lane, keep, 3);
     for (int j = lane; j < total; j += 32) {
       const int code = sm.jobs[j], owner = code / 12, k = code - 12 * owner;
       const double* R = sm.rect[owner][k / 3];
@@ -325,6 +491,7 @@ __device__ void search(Heap& h, const Ray& r, const double* __restrict__ nets, i
     }
     __syncwarp();
     for (int ch = 0; ch < nch; ++ch) {
+      if (!(keep >> ch & 1)) continue;
       double lo = 0.0, hi = INFINITY, e = 0.0;
       bool in = true;
       for (int cc = 0; cc < 3 && in; ++cc) {
@@ -372,15 +539,18 @@ __device__ __forceinline__ void write_hit(const RayOut& out, long long k, const 
 // First pass: one ray per thread, a kHeapCap-entry heap in local memory, the search shared by the
 // warp. A ray whose heap overflows stops and is appended to redo_list for the second pass (or,
 // when the list is full, reported with SHELL_RAY_OVERFLOW).
+template <bool kCull>
 __global__ void __launch_bounds__(kRayBlock, 4) k_trace_rays(long long n, const double* __restrict__ origins,
                                                           const double* __restrict__ dirs, int np,
                                                           const double* __restrict__ nets,
                                                           const double* __restrict__ boxes,
-                                                          const double* __restrict__ gboxes, int use_newton,
+                                                          const double* __restrict__ gboxes,
+                                                          const CullNet* __restrict__ culls, int use_newton,
                                                           RayOut out, int* __restrict__ redo_count,
                                                           int* __restrict__ redo_list, Cand* __restrict__ heaps) {
-  __shared__ double sbox[kRootChunk * 8];
-  __shared__ WarpSmem wsm[kRayBlock / 32];
+  using Box = std::conditional_t<kCull, float, double>;
+  __shared__ Box sbox[kRootChunk * 8];
+  __shared__ WarpSmem<kCull> wsm[kRayBlock / 32];
   const int lane = threadIdx.x & 31;
   const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const bool active = k < n;
@@ -396,25 +566,35 @@ __global__ void __launch_bounds__(kRayBlock, 4) k_trace_rays(long long n, const 
   for (int base = 0; base < ngroups; base += kRootChunk) {
     const int m = min(kRootChunk, ngroups - base);
     __syncthreads();
-    for (int i = threadIdx.x; i < m * 8; i += blockDim.x) sbox[i] = gboxes[(size_t)base * 8 + i];
+    for (int i = threadIdx.x; i < m * 8; i += blockDim.x) {
+      const double v = gboxes[(size_t)base * 8 + i];
+      if constexpr (kCull) sbox[i] = i % 8 < 3 ? __double2float_rd(v) : __double2float_ru(v);
+      else sbox[i] = v;
+    }
     __syncthreads();
     if (!active) continue;
     for (int j = 0; j < m; ++j) {
-      const double* G = sbox + 8 * j;
-      double lo = 0.0, hi = INFINITY;
-      bool in = true;
-#pragma unroll
-      for (int c = 0; c < 3; ++c)
-        if (in) in = slab(G[c], G[3 + c], r.o[c], r.d[c], r.inv[c], lo, hi);
-      if (!in || lo > hi) continue;
+      const Box* G = sbox + 8 * j;
       const int p0 = (base + j) * kGroup, p1 = min(np, p0 + kGroup);
-      for (int p = p0; p < p1; ++p) root_push(h, boxes + 8 * (size_t)p, p, r);
+      if constexpr (kCull) {
+        if (surely_missed(G, r)) continue;
+        for (int p = p0; p < p1; ++p)
+          if (!surely_missed(culls[p].box, r)) root_push(h, boxes + 8 * (size_t)p, p, r);
+      } else {
+        double lo = 0.0, hi = INFINITY;
+        bool in = true;
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+          if (in) in = slab(G[c], G[3 + c], r.o[c], r.d[c], r.inv[c], lo, hi);
+        if (!in || lo > hi) continue;
+        for (int p = p0; p < p1; ++p) root_push(h, boxes + 8 * (size_t)p, p, r);
+      }
     }
   }
   h.boxes = np;
   Search S;
   S.live = active;
-  search(h, r, nets, use_newton, S, wsm[threadIdx.x >> 5], lane);
+  search<kCull>(h, r, nets, culls, use_newton, S, wsm[threadIdx.x >> 5], lane);
   if (!active) return;
   if (h.overflow) {
     const int slot = atomicAdd(redo_count, 1);
@@ -428,14 +608,16 @@ __global__ void __launch_bounds__(kRayBlock, 4) k_trace_rays(long long n, const 
 
 // Second pass over the rays whose first-pass heap overflowed: the same search from the start
 // with a kRedoHeap-entry heap per thread in global memory (heaps: kRedoThreads x kRedoHeap).
+template <bool kCull>
 __global__ void __launch_bounds__(kRedoThreads) k_trace_rays_redo(const double* __restrict__ origins,
                                                                   const double* __restrict__ dirs, int np,
                                                                   const double* __restrict__ nets,
-                                                                  const double* __restrict__ boxes, int use_newton,
+                                                                  const double* __restrict__ boxes,
+                                                                  const CullNet* __restrict__ culls, int use_newton,
                                                                   RayOut out, const int* __restrict__ redo_count,
                                                                   const int* __restrict__ redo_list,
                                                                   Cand* __restrict__ heaps) {
-  __shared__ WarpSmem wsm[kRedoThreads / 32];
+  __shared__ WarpSmem<kCull> wsm[kRedoThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31;
   const int count = min(*redo_count, kRedoList);
   for (int base = 0; base < count; base += kRedoThreads) {   // uniform trip count: the warp stays whole
@@ -451,7 +633,7 @@ __global__ void __launch_bounds__(kRedoThreads) k_trace_rays_redo(const double* 
     h.boxes = np;
     Search S;
     S.live = active;
-    search(h, r, nets, use_newton, S, wsm[tid >> 5], lane);
+    search<kCull>(h, r, nets, culls, use_newton, S, wsm[tid >> 5], lane);
     if (active) write_hit(out, k, S, h);
   }
 }
@@ -495,7 +677,7 @@ extern "C" shell_status shell_trace_rays(shell_t* shell, const double* q, long l
   BHEM_TRY(search_scratch(s, &heaps_v, &redo_count, &redo_list));
   if (!s.d_ray_nets) {
     const size_t ngroups = ((size_t)np + kGroup - 1) / kGroup;
-    const cudaError_t e = cudaMalloc((void**)&s.d_ray_nets, sizeof(double) * (56 * (size_t)np + 8 * ngroups));
+    const cudaError_t e = cudaMalloc((void**)&s.d_ray_nets, sizeof(double) * (56 * (size_t)np + 8 * ngroups) + sizeof(CullNet) * np);
     if (e != cudaSuccess) {
       cudaGetLastError();
       s.d_ray_nets = nullptr;
@@ -507,16 +689,26 @@ extern "C" shell_status shell_trace_rays(shell_t* shell, const double* q, long l
   double* boxes = nets + 48 * (size_t)np;
   double* gboxes = boxes + 8 * (size_t)np;
   const int ngroups = (np + kGroup - 1) / kGroup;
+  // with statistics, which are those of the plain search, nothing is culled
+  CullNet* culls = stats ? nullptr : reinterpret_cast<CullNet*>(gboxes + 8 * (size_t)ngroups);
   RayOut out{tau, patch, uv, flags, stats};
   BHEM_CUDA(cudaMemsetAsync(redo_count, 0, 2 * sizeof(int), s.stream));
   k_ray_nets<<<grid_for(np, kNetBlock), kNetBlock, 0, s.stream>>>(np, s.d_patch_nodes, q, s.grid.dxi1,
-                                                                  s.grid.dxi2, nets, boxes);
+                                                                  s.grid.dxi2, nets, boxes, culls);
   k_ray_groups<<<grid_for(ngroups, kNetBlock), kNetBlock, 0, s.stream>>>(np, boxes, gboxes);
   const int use_newton = variant == SHELL_RAY_NEWTON;
-  k_trace_rays<<<(unsigned)((n_rays + kRayBlock - 1) / kRayBlock), kRayBlock, 0, s.stream>>>(
-      n_rays, origins, dirs, np, nets, boxes, gboxes, use_newton, out, redo_count, redo_list, heaps);
-  k_trace_rays_redo<<<1, kRedoThreads, 0, s.stream>>>(origins, dirs, np, nets, boxes, use_newton, out, redo_count,
-                                                      redo_list, heaps);
+  const unsigned ctas = (unsigned)((n_rays + kRayBlock - 1) / kRayBlock);
+  if (culls) {
+    k_trace_rays<true><<<ctas, kRayBlock, 0, s.stream>>>(n_rays, origins, dirs, np, nets, boxes, gboxes, culls,
+                                                         use_newton, out, redo_count, redo_list, heaps);
+    k_trace_rays_redo<true><<<1, kRedoThreads, 0, s.stream>>>(origins, dirs, np, nets, boxes, culls, use_newton, out,
+                                                              redo_count, redo_list, heaps);
+  } else {
+    k_trace_rays<false><<<ctas, kRayBlock, 0, s.stream>>>(n_rays, origins, dirs, np, nets, boxes, gboxes, culls,
+                                                          use_newton, out, redo_count, redo_list, heaps);
+    k_trace_rays_redo<false><<<1, kRedoThreads, 0, s.stream>>>(origins, dirs, np, nets, boxes, culls, use_newton, out,
+                                                               redo_count, redo_list, heaps);
+  }
   s.launches += 4;
   BHEM_CUDA(cudaGetLastError());
   return SHELL_OK;

@@ -116,3 +116,43 @@ def test_full_size_camera_sampled():
             ref = O.trace_rays(g, q, o[idx], d[idx], variant == "newton", want_stats=True)
             _assert_identical({k: v[idx] for k, v in gpu.items()}, ref, variant)
             assert 0.4 < (gpu["flags"] & 1).mean() < 0.8
+
+
+def _same_hits(sh, q, o, d, variant):
+    """The search without statistics, which culls sub-patches by an FP32 test, returns bit for bit the
+    hits of the search with statistics, which boxes every candidate."""
+    dq = torch.as_tensor(np.ascontiguousarray(q).reshape(-1), dtype=torch.float64, device="cuda")
+    do, dd = torch.as_tensor(o, device="cuda"), torch.as_tensor(d, device="cuda")
+    full = sh.trace_rays(dq, do, dd, variant=variant, want_stats=True)
+    culled = sh.trace_rays(dq, do, dd, variant=variant)
+    for k in culled:
+        np.testing.assert_array_equal(culled[k].cpu().numpy(), full[k].cpu().numpy(), err_msg=k)
+    return full["flags"].cpu().numpy()
+
+
+@pytest.mark.parametrize("variant", ["newton", "midpoint"])
+@pytest.mark.parametrize("scale,shift", [(1.0, 0.0), (1e-3, 0.0), (1e3, 0.0), (1.0, 1e5), (1e-3, 10.0)])
+def test_culled_search_gives_the_same_hits(variant, scale, shift):
+    """Camera rays on the three scenes at sizes from millimetres to kilometres and far from the
+    origin (where FP32 rounding of positions exceeds the patches), axis-parallel rays at node lines,
+    rays tangent to the cylinder, and rays lying in the flat sheet."""
+    for name, (g, q, eye, tgt) in S.ray_scenes().items():
+        off = np.array([shift, -shift, 0.5 * shift])
+        qs = q * scale
+        qs[:, :3] += off
+        o, d = S.camera_rays(90, 70, eye, tgt)
+        rng = np.random.default_rng(3)
+        ov = rng.uniform(-0.1, 1.1, size=(400, 3))
+        ov[:200, :2] = np.round(ov[:200, :2] * 10) / 10   # node lines
+        ov[:, 2] = 2.0
+        dv = np.tile([0.0, 0.0, -1.0], (400, 1))
+        ot = np.stack([np.full(64, 0.3) + np.linspace(-1e-6, 1e-6, 64), np.full(64, -1.0), rng.uniform(0, 1, 64)], 1)
+        dt = np.tile([0.0, 1.0, 0.0], (64, 1))
+        oi = np.stack([np.full(40, -0.05), rng.uniform(0, 1, 40), np.zeros(40)], 1)
+        di = rng.normal(size=(40, 3)) * [1.0, 1.0, 0.0]
+        di /= np.linalg.norm(di, axis=1, keepdims=True)
+        o = np.concatenate([o, ov, ot, oi]) * scale + off
+        d = np.concatenate([d, dv, dt, di])
+        with _shell(g, qs) as sh:
+            flags = _same_hits(sh, qs, o, d, variant)
+        assert (flags & 1).sum() > 300, name
