@@ -78,6 +78,40 @@ __device__ __forceinline__ void curve_restrict(const double in[4], double a, dou
   out[3] = lerp(BB[0], BB[1], b);
 }
 
+// 4x4 transpose over four neighbouring lanes (c = lane % 4): lane c's o[j] becomes lane j's o[c].
+// All 32 lanes of the warp call it.
+__device__ __forceinline__ void transpose4(double o[4], int c) {
+  {
+    const bool h = c & 2;
+    const double a = __shfl_xor_sync(0xffffffffu, h ? o[0] : o[2], 2);
+    const double b = __shfl_xor_sync(0xffffffffu, h ? o[1] : o[3], 2);
+    o[0] = h ? a : o[0];
+    o[1] = h ? b : o[1];
+    o[2] = h ? o[2] : a;
+    o[3] = h ? o[3] : b;
+  }
+  {
+    const bool h = c & 1;
+    const double a = __shfl_xor_sync(0xffffffffu, h ? o[0] : o[1], 1);
+    const double b = __shfl_xor_sync(0xffffffffu, h ? o[2] : o[3], 1);
+    o[0] = h ? a : o[0];
+    o[1] = h ? o[1] : a;
+    o[2] = h ? b : o[2];
+    o[3] = h ? o[3] : b;
+  }
+}
+
+// A coordinate's net Pc ([i][j]) cut to [u0, u1] x [v0, v1] by four neighbouring lanes: lane c cuts
+// the theta1-curve c, then the theta2-curve c, and returns row S[c][0..3] (the operations of one
+// thread cutting all eight curves). All 32 lanes of the warp call it.
+__device__ __forceinline__ void cut_row(const double* __restrict__ Pc, int c, const double* R, double S[4]) {
+  const double in[4] = {__ldg(Pc + c), __ldg(Pc + 4 + c), __ldg(Pc + 8 + c), __ldg(Pc + 12 + c)};
+  double T[4];
+  curve_restrict(in, R[0], R[1], T);
+  transpose4(T, c);
+  curve_restrict(T, R[2], R[3], S);
+}
+
 // Cubic Bernstein polynomials and their derivatives at t.
 __device__ __forceinline__ void bernstein(double t, double B[4], double dB[4]) {
   const double s = 1.0 - t;
@@ -91,32 +125,56 @@ __device__ __forceinline__ void bernstein(double t, double B[4], double dB[4]) {
   dB[3] = 3.0 * t * t;
 }
 
-// x(u, v), x_u, x_v of the net P ([c][i][j]): sums over j first, then i.
+// x(u, v), x_u, x_v of one coordinate's net Pc ([i][j]) from the Bernstein values: sums over j first,
+// then i.
+__device__ __forceinline__ void bezier_eval_coord(const double* __restrict__ Pc, const double Bu[4], const double dBu[4],
+                                                  const double Bv[4], const double dBv[4], double& x, double& xu,
+                                                  double& xv) {
+  double Q[4], R[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const double* row = Pc + 4 * i;
+    const double p0 = __ldg(row), p1 = __ldg(row + 1), p2 = __ldg(row + 2), p3 = __ldg(row + 3);
+    Q[i] = ((Bv[0] * p0 + Bv[1] * p1) + Bv[2] * p2) + Bv[3] * p3;
+    R[i] = ((dBv[0] * p0 + dBv[1] * p1) + dBv[2] * p2) + dBv[3] * p3;
+  }
+  x = ((Bu[0] * Q[0] + Bu[1] * Q[1]) + Bu[2] * Q[2]) + Bu[3] * Q[3];
+  xu = ((dBu[0] * Q[0] + dBu[1] * Q[1]) + dBu[2] * Q[2]) + dBu[3] * Q[3];
+  xv = ((Bu[0] * R[0] + Bu[1] * R[1]) + Bu[2] * R[2]) + Bu[3] * R[3];
+}
+
+// x(u, v), x_u, x_v of the net P ([c][i][j]).
 static __device__ void bezier_eval(const double* __restrict__ P, double u, double v, double x[3], double xu[3],
                             double xv[3]) {
   double Bu[4], dBu[4], Bv[4], dBv[4];
   bernstein(u, Bu, dBu);
   bernstein(v, Bv, dBv);
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    double Q[4], R[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const double* row = P + 16 * c + 4 * i;
-      const double p0 = __ldg(row), p1 = __ldg(row + 1), p2 = __ldg(row + 2), p3 = __ldg(row + 3);
-      Q[i] = ((Bv[0] * p0 + Bv[1] * p1) + Bv[2] * p2) + Bv[3] * p3;
-      R[i] = ((dBv[0] * p0 + dBv[1] * p1) + dBv[2] * p2) + dBv[3] * p3;
-    }
-    x[c] = ((Bu[0] * Q[0] + Bu[1] * Q[1]) + Bu[2] * Q[2]) + Bu[3] * Q[3];
-    xu[c] = ((dBu[0] * Q[0] + dBu[1] * Q[1]) + dBu[2] * Q[2]) + dBu[3] * Q[3];
-    xv[c] = ((Bu[0] * R[0] + Bu[1] * R[1]) + Bu[2] * R[2]) + Bu[3] * R[3];
-  }
+  for (int c = 0; c < 3; ++c) bezier_eval_coord(P + 16 * c, Bu, dBu, Bv, dBv, x[c], xu[c], xv[c]);
 }
 
 __device__ __forceinline__ double det3(const double M[3][3]) {
   return (M[0][0] * (M[1][1] * M[2][2] - M[1][2] * M[2][1]) -
           M[0][1] * (M[1][0] * M[2][2] - M[1][2] * M[2][0])) +
          M[0][2] * (M[1][0] * M[2][1] - M[1][1] * M[2][0]);
+}
+
+// Component k of the Newton step -J^-1 F by Cramer's rule; *ok: |det J| is large enough.
+__device__ __forceinline__ double cramer_component(const double J[3][3], const double F[3], int k, bool* ok) {
+  const double det = det3(J);
+  *ok = fabs(det) > 1e-300;
+  double M[3][3];
+#pragma unroll
+  for (int r = 0; r < 3; ++r)
+#pragma unroll
+    for (int s = 0; s < 3; ++s) M[r][s] = s == k ? -F[r] : J[r][s];
+  return det3(M) / det;
+}
+
+// Lane of the n-th set bit of a warp mask (n from 0; 0 when there is none).
+__device__ __forceinline__ int nth_lane(unsigned mask, int n) {
+  const unsigned l = __fns(mask, 0, n + 1);
+  return l < 32 ? (int)l : 0;
 }
 
 // ------------------------------------------------------------------------------------------

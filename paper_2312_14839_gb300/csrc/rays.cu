@@ -23,11 +23,12 @@
 //                boxes are tested in FP32 first. FP64 issue bounds this kernel (one warp instruction per
 //                64 cycles and sub-partition), so an FP32 test costs a few percent of the box it saves,
 //                and its tilted lines prune where axis-aligned boxes overlap the ray at every level
-//                (near-tangent rays). Measured, 1024 x 768 rays: drape, Newton split 240 -> 17.4 ms
-//                (another drape, with more tangent rays, 373 -> 57 ms), midpoint split 217 -> 140 ms;
-//                512 x 384: cylinder, Newton split 61 -> 4.6 ms, plane 1.5 -> 0.37 ms. The midpoint
-//                split of the cylinder stays at 60 ms: its tail is rays that graze the surface within the
-//                test's margin, where the last levels' candidates are boxed as before.
+//                (near-tangent rays). Newton iterations run one at a time beside the other lanes' splits,
+//                few of them on four lanes each, and every box job on four lanes. Measured, 1024 x 768 rays:
+//                drape, Newton split 240 -> 12.8 ms (another drape, with more tangent rays, 373 -> 35 ms),
+//                midpoint split 217 -> 142 ms; 512 x 384: cylinder, Newton split 61 -> 3.3 ms, midpoint
+//                58 -> 51 ms, plane 1.5 -> 0.38 ms. What is left of the midpoint split are the levels
+//                below the test's margin, boxed as before.
 //   k_trace_rays_redo  the rays that found no free global heap, traced again from the start
 //                with one (the search is deterministic, so the result is the one an unbounded
 //                heap gives).
@@ -168,44 +169,77 @@ __global__ void __launch_bounds__(kNetBlock) k_ray_nets(int np, const int4* __re
 }
 
 // Newton's method on F(u, v, tau) = x(u, v) - o - tau d, Jacobian [x_u | x_v | -d] by Cramer's
-// rule. True with the root in (u, v, tau) on convergence; gives up when an iterate leaves the
-// window win (the candidate's rectangle widened by its extent on each side).
-__device__ bool newton_root(const double* __restrict__ P, const double o[3], const double d[3], double on,
-                            const double win[4], double& u, double& v, double& tau, int& iters) {
-  double uu = u, vv = v, tt = tau;
-  for (int it = 0; it < kNewtonIters; ++it) {
-    double x[3], xu[3], xv[3], F[3];
-    ++iters;
-    bezier_eval(P, uu, vv, x, xu, xv);
+// rule, at most kNewtonIters iterations; it gives up when an iterate leaves the window win (the
+// candidate's rectangle widened by its extent on each side). The lanes of a warp take one iteration
+// at a time, beside the splits of the lanes that need none: the number of iterations varies from one
+// to twelve, and a lane that ran them all at once would hold the others up.
+// One iteration from (u, v, tau) of every lane with `want`; state 1: converged (at the point given),
+// 2: it gives up, 0: the next point. Few lanes are served by four lanes each (a coordinate of the
+// surface point and a component of the step per lane: about 200 FP64 operations for eight iterations,
+// against 370 for one to 32), more by themselves. All 32 lanes of the warp call it.
+constexpr int kSharedNewton = 8;
+
+__device__ void newton_step(bool want, const double* __restrict__ nets, int patch, const double o[3], const double d[3],
+                            double on, const double win[4], double& u, double& v, double& tau, int& state) {
+  const unsigned mask = __ballot_sync(0xffffffffu, want);
+  const int count = __popc(mask), lane = threadIdx.x & 31;
+  if (count == 0) return;
+  double delta[3] = {0.0, 0.0, 0.0};
+  if (count <= kSharedNewton) {
+    const int own = nth_lane(mask, lane >> 2), c = min(lane & 3, 2), g = lane & 28;
+    const int p = __shfl_sync(0xffffffffu, patch, own);
+    const double uu = __shfl_sync(0xffffffffu, u, own), vv = __shfl_sync(0xffffffffu, v, own);
+    const double tt = __shfl_sync(0xffffffffu, tau, own), oon = __shfl_sync(0xffffffffu, on, own);
+    const double o0 = __shfl_sync(0xffffffffu, o[0], own), o1 = __shfl_sync(0xffffffffu, o[1], own),
+                 o2 = __shfl_sync(0xffffffffu, o[2], own);
+    const double d0 = __shfl_sync(0xffffffffu, d[0], own), d1 = __shfl_sync(0xffffffffu, d[1], own),
+                 d2 = __shfl_sync(0xffffffffu, d[2], own);
+    const double oc = c == 0 ? o0 : c == 1 ? o1 : o2, dc = c == 0 ? d0 : c == 1 ? d1 : d2;
+    double Bu[4], dBu[4], Bv[4], dBv[4], x, xu, xv;
+    bernstein(uu, Bu, dBu);
+    bernstein(vv, Bv, dBv);
+    bezier_eval_coord(nets + (size_t)p * 48 + 16 * c, Bu, dBu, Bv, dBv, x, xu, xv);
+    const double f = (x - oc) - tt * dc;
+    double F[3], J[3][3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) F[c] = (x[c] - o[c]) - tt * d[c];
+    for (int r = 0; r < 3; ++r) {
+      F[r] = __shfl_sync(0xffffffffu, f, g + r);
+      J[r][0] = __shfl_sync(0xffffffffu, xu, g + r);
+      J[r][1] = __shfl_sync(0xffffffffu, xv, g + r);
+      J[r][2] = -__shfl_sync(0xffffffffu, dc, g + r);
+    }
     const double fn = sqrt((F[0] * F[0] + F[1] * F[1]) + F[2] * F[2]);
-    if (fn <= 1e-12 * ((1.0 + on) + fabs(tt))) {
-      u = uu;
-      v = vv;
-      tau = tt;
-      return true;
-    }
+    bool regular;
+    const double step = cramer_component(J, F, c, &regular);
+    const int st = fn <= 1e-12 * ((1.0 + oon) + fabs(tt)) ? 1 : !regular ? 2 : 0;
+    const int src = 4 * __popc(mask & ((1u << lane) - 1u));   // the lanes that served this one
+    const int got = __shfl_sync(0xffffffffu, st, src & 31);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) delta[k] = __shfl_sync(0xffffffffu, step, (src + k) & 31);
+    if (!want) return;
+    state = got;
+  } else {
+    if (!want) return;
+    const double* P = nets + (size_t)patch * 48;
+    double x[3], xu[3], xv[3], F[3];
+    bezier_eval(P, u, v, x, xu, xv);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) F[c] = (x[c] - o[c]) - tau * d[c];
+    const double fn = sqrt((F[0] * F[0] + F[1] * F[1]) + F[2] * F[2]);
     const double J[3][3] = {{xu[0], xv[0], -d[0]}, {xu[1], xv[1], -d[1]}, {xu[2], xv[2], -d[2]}};
-    const double det = det3(J);
-    if (!(fabs(det) > 1e-300)) return false;
-    double delta[3];
+    bool regular = true;
+    state = fn <= 1e-12 * ((1.0 + on) + fabs(tau)) ? 1 : 0;
+    if (state == 0)
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      double M[3][3];
-#pragma unroll
-      for (int r = 0; r < 3; ++r)
-#pragma unroll
-        for (int s = 0; s < 3; ++s) M[r][s] = s == k ? -F[r] : J[r][s];
-      delta[k] = det3(M) / det;
-    }
-    uu += delta[0];
-    vv += delta[1];
-    tt += delta[2];
-    if (!isfinite(uu) || !isfinite(vv) || !isfinite(tt)) return false;
-    if (uu < win[0] || uu > win[1] || vv < win[2] || vv > win[3]) return false;   // left the window
+      for (int k = 0; k < 3; ++k) delta[k] = cramer_component(J, F, k, &regular);
+    if (!regular) state = 2;
   }
-  return false;
+  if (state) return;
+  u += delta[0];
+  v += delta[1];
+  tau += delta[2];
+  if (!isfinite(u) || !isfinite(v) || !isfinite(tau) || u < win[0] || u > win[1] || v < win[2] || v > win[3])
+    state = 2;   // left the window
 }
 
 struct Ray {
@@ -396,24 +430,28 @@ __device__ __forceinline__ int list_jobs(PlainSmem& sm, int lane, unsigned keep,
 // overflows.
 // kCull: children (and patch roots) that provably lead to no hit are left out; without it every child
 // is boxed, and the search statistics are those of the plain algorithm.
-template <bool kCull>
+template <bool kCull, bool kNewton>
 __device__ void search(Heap& h, const Ray& r, const double* __restrict__ nets, const CullNet* __restrict__ culls,
-                       int use_newton, Search& S, WarpSmem<kCull>& sm, int lane) {
+                       Search& S, WarpSmem<kCull>& sm, int lane) {
   S.on = sqrt((r.o[0] * r.o[0] + r.o[1] * r.o[1]) + r.o[2] * r.o[2]);
+  Cand c{};                // the candidate being split
+  int newton = -1;         // its Newton iterations so far; -1: none in progress
+  double u = 0.0, v = 0.0, t = 0.0;
+  bool cullable = false;
   while (__any_sync(0xffffffffu, S.live)) {
     int nch = 0;
-    bool cullable = false;
-    if (S.live) {
+    bool split = false, root = false;   // split c now; around the root (u, v, t)
+    if (S.live && newton < 0) {
       if (h.n == 0 || h.overflow) {
         S.live = false;
       } else {
-        const Cand c = h.pop();
+        c = h.pop();
         if (c.t0 >= S.best - kEpsTau) {                                    // nothing left can be closer
           S.live = false;
         } else if (c.ext <= kEpsTau || (c.u1 - c.u0 < 1e-13 && c.v1 - c.v0 < 1e-13)) {   // refined
-          const double t = 0.5 * (c.t0 + c.t1);
-          if (t < S.best - kEpsTau) {
-            S.best = t;
+          const double tm = 0.5 * (c.t0 + c.t1);
+          if (tm < S.best - kEpsTau) {
+            S.best = tm;
             S.bp = c.patch;
             S.bu = 0.5 * (c.u0 + c.u1);
             S.bv = 0.5 * (c.v0 + c.v1);
@@ -423,48 +461,63 @@ __device__ void search(Heap& h, const Ray& r, const double* __restrict__ nets, c
           S.live = false;
         } else if (!starts_culled<kCull>(sm, lane, c, r, culls, S.best, S.on, cullable)) {
           ++S.nexp;
-          const double* P = nets + (size_t)c.patch * 48;
-          const double um = 0.5 * (c.u0 + c.u1), vm = 0.5 * (c.v0 + c.v1);
-          bool pinwheel = false;
-          if (use_newton) {
+          u = 0.5 * (c.u0 + c.u1);
+          v = 0.5 * (c.v0 + c.v1);
+          if constexpr (kNewton) {
             double x[3], xu[3], xv[3];
-            bezier_eval(P, um, vm, x, xu, xv);
-            double u = um, v = vm;
-            double t = ((x[0] - r.o[0]) * r.d[0] + (x[1] - r.o[1]) * r.d[1]) + (x[2] - r.o[2]) * r.d[2];
-            const double wu = c.u1 - c.u0, wv = c.v1 - c.v0;
-            const double win[4] = {c.u0 - wu, c.u1 + wu, c.v0 - wv, c.v1 + wv};
-            if (newton_root(P, r.o, r.d, S.on, win, u, v, t, S.newton_iters) && u >= c.u0 && u <= c.u1 &&
-                v >= c.v0 && v <= c.v1 && t >= 0.0) {
-              if (t < S.best) {
-                S.best = t;
-                S.bp = c.patch;
-                S.bu = u;
-                S.bv = v;
-              }
-              // Fig. subany: drop [a1, a2] x [b1, b2] around the root, four rectangles remain
-              const double hu = kNbhd * (c.u1 - c.u0), hv = kNbhd * (c.v1 - c.v0);
-              const double a1 = fmax(c.u0, u - hu), a2 = fmin(c.u1, u + hu);
-              const double b1 = fmax(c.v0, v - hv), b2 = fmin(c.v1, v + hv);
-              put_rect(sm, lane, nch, c.u0, a1, b1, c.v1);
-              put_rect(sm, lane, nch, a1, c.u1, b2, c.v1);
-              put_rect(sm, lane, nch, c.u0, a2, c.v0, b1);
-              put_rect(sm, lane, nch, a2, c.u1, c.v0, b2);
-              pinwheel = true;
-            }
-          }
-          if (!pinwheel) {   // Fig. submid: four quarters at the parameter midpoint
-            put_rect(sm, lane, nch, c.u0, um, vm, c.v1);
-            put_rect(sm, lane, nch, um, c.u1, vm, c.v1);
-            put_rect(sm, lane, nch, c.u0, um, c.v0, vm);
-            put_rect(sm, lane, nch, um, c.u1, c.v0, vm);
-          }
-          sm.patch[lane] = c.patch;
-          h.boxes += nch;
-          if constexpr (kCull) {   // a root found above may have brought the best hit nearer
-            const float beyond = (float)(S.best - c.t0);
-            sm.path[lane][12] = beyond + 1e-6f * fabsf(beyond);
+            bezier_eval(nets + (size_t)c.patch * 48, u, v, x, xu, xv);
+            t = ((x[0] - r.o[0]) * r.d[0] + (x[1] - r.o[1]) * r.d[1]) + (x[2] - r.o[2]) * r.d[2];
+            newton = 0;
+          } else {
+            split = true;
           }
         }
+      }
+    }
+    if constexpr (kNewton) {
+      const bool want = newton >= 0;
+      const double wu = c.u1 - c.u0, wv = c.v1 - c.v0;
+      const double win[4] = {c.u0 - wu, c.u1 + wu, c.v0 - wv, c.v1 + wv};
+      int state = 0;
+      newton_step(want, nets, c.patch, r.o, r.d, S.on, win, u, v, t, state);
+      if (want) {
+        ++newton;
+        ++S.newton_iters;
+        if (state || newton == kNewtonIters) {
+          newton = -1;
+          split = true;
+          root = state == 1 && u >= c.u0 && u <= c.u1 && v >= c.v0 && v <= c.v1 && t >= 0.0;
+        }
+      }
+    }
+    if (split) {
+      if (root) {
+        if (t < S.best) {
+          S.best = t;
+          S.bp = c.patch;
+          S.bu = u;
+          S.bv = v;
+        }
+        // Fig. subany: drop [a1, a2] x [b1, b2] around the root, four rectangles remain
+        const double hu = kNbhd * (c.u1 - c.u0), hv = kNbhd * (c.v1 - c.v0);
+        const double a1 = fmax(c.u0, u - hu), a2 = fmin(c.u1, u + hu);
+        const double b1 = fmax(c.v0, v - hv), b2 = fmin(c.v1, v + hv);
+        put_rect(sm, lane, nch, c.u0, a1, b1, c.v1);
+        put_rect(sm, lane, nch, a1, c.u1, b2, c.v1);
+        put_rect(sm, lane, nch, c.u0, a2, c.v0, b1);
+        put_rect(sm, lane, nch, a2, c.u1, c.v0, b2);
+      } else {   // Fig. submid: four quarters at the parameter midpoint
+        const double um = 0.5 * (c.u0 + c.u1), vm = 0.5 * (c.v0 + c.v1);
+        put_rect(sm, lane, nch, c.u0, um, vm, c.v1);
+        put_rect(sm, lane, nch, um, c.u1, vm, c.v1);
+        put_rect(sm, lane, nch, c.u0, um, c.v0, vm);
+        put_rect(sm, lane, nch, um, c.u1, c.v0, vm);
+      }
+      sm.patch[lane] = c.patch;
+      h.boxes += nch;
+      if constexpr (kCull) {   // a root found above may have brought the best hit nearer
+        const float beyond = (float)(S.best - c.t0);
+        sm.path[lane][12] = beyond + 1e-6f * fabsf(beyond);
       }
     }
     unsigned keep = (1u << nch) - 1u;   // children to box
@@ -481,13 +534,27 @@ __device__ void search(Heap& h, const Ray& r, const double* __restrict__ nets, c
     }
     // the warp's pool of (lane, child, coordinate) range jobs
     const int total = list_jobs(sm, lane, keep, 3);
-    for (int j = lane; j < total; j += 32) {
-      const int code = sm.jobs[j], owner = code / 12, k = code - 12 * owner;
-      const double* R = sm.rect[owner][k / 3];
-      double mn, mx;
-      sub_range(nets + (size_t)sm.patch[owner] * 48, k % 3, R[0], R[1], R[2], R[3], mn, mx);
-      sm.range[owner][k][0] = mn;
-      sm.range[owner][k][1] = mx;
+    // four lanes per job: eight jobs a round, 110 FP64 operations long (one lane per job: 450)
+    for (int base = 0; base < total; base += 8) {
+      const int j = base + (lane >> 2), code = sm.jobs[min(j, total - 1)], owner = code / 12, k = code - 12 * owner;
+      double o[4];
+      cut_row(nets + (size_t)sm.patch[owner] * 48 + 16 * (k % 3), lane & 3, sm.rect[owner][k / 3], o);
+      double mn = o[0], mx = o[0];
+#pragma unroll
+      for (int i = 1; i < 4; ++i) {
+        if (o[i] < mn) mn = o[i];
+        if (o[i] > mx) mx = o[i];
+      }
+#pragma unroll
+      for (int off = 1; off < 4; off <<= 1) {
+        const double a = __shfl_xor_sync(0xffffffffu, mn, off), b = __shfl_xor_sync(0xffffffffu, mx, off);
+        if (a < mn) mn = a;
+        if (b > mx) mx = b;
+      }
+      if ((lane & 3) == 0 && j < total) {
+        sm.range[owner][k][0] = mn;
+        sm.range[owner][k][1] = mx;
+      }
     }
     __syncwarp();
     for (int ch = 0; ch < nch; ++ch) {
@@ -539,13 +606,13 @@ __device__ __forceinline__ void write_hit(const RayOut& out, long long k, const 
 // First pass: one ray per thread, a kHeapCap-entry heap in local memory, the search shared by the
 // warp. A ray whose heap overflows stops and is appended to redo_list for the second pass (or,
 // when the list is full, reported with SHELL_RAY_OVERFLOW).
-template <bool kCull>
+template <bool kCull, bool kNewton>
 __global__ void __launch_bounds__(kRayBlock, 4) k_trace_rays(long long n, const double* __restrict__ origins,
                                                           const double* __restrict__ dirs, int np,
                                                           const double* __restrict__ nets,
                                                           const double* __restrict__ boxes,
                                                           const double* __restrict__ gboxes,
-                                                          const CullNet* __restrict__ culls, int use_newton,
+                                                          const CullNet* __restrict__ culls,
                                                           RayOut out, int* __restrict__ redo_count,
                                                           int* __restrict__ redo_list, Cand* __restrict__ heaps) {
   using Box = std::conditional_t<kCull, float, double>;
@@ -594,7 +661,7 @@ __global__ void __launch_bounds__(kRayBlock, 4) k_trace_rays(long long n, const 
   h.boxes = np;
   Search S;
   S.live = active;
-  search<kCull>(h, r, nets, culls, use_newton, S, wsm[threadIdx.x >> 5], lane);
+  search<kCull, kNewton>(h, r, nets, culls, S, wsm[threadIdx.x >> 5], lane);
   if (!active) return;
   if (h.overflow) {
     const int slot = atomicAdd(redo_count, 1);
@@ -608,12 +675,12 @@ __global__ void __launch_bounds__(kRayBlock, 4) k_trace_rays(long long n, const 
 
 // Second pass over the rays whose first-pass heap overflowed: the same search from the start
 // with a kRedoHeap-entry heap per thread in global memory (heaps: kRedoThreads x kRedoHeap).
-template <bool kCull>
+template <bool kCull, bool kNewton>
 __global__ void __launch_bounds__(kRedoThreads) k_trace_rays_redo(const double* __restrict__ origins,
                                                                   const double* __restrict__ dirs, int np,
                                                                   const double* __restrict__ nets,
                                                                   const double* __restrict__ boxes,
-                                                                  const CullNet* __restrict__ culls, int use_newton,
+                                                                  const CullNet* __restrict__ culls,
                                                                   RayOut out, const int* __restrict__ redo_count,
                                                                   const int* __restrict__ redo_list,
                                                                   Cand* __restrict__ heaps) {
@@ -633,7 +700,7 @@ __global__ void __launch_bounds__(kRedoThreads) k_trace_rays_redo(const double* 
     h.boxes = np;
     Search S;
     S.live = active;
-    search<kCull>(h, r, nets, culls, use_newton, S, wsm[tid >> 5], lane);
+    search<kCull, kNewton>(h, r, nets, culls, S, wsm[tid >> 5], lane);
     if (active) write_hit(out, k, S, h);
   }
 }
@@ -696,19 +763,15 @@ extern "C" shell_status shell_trace_rays(shell_t* shell, const double* q, long l
   k_ray_nets<<<grid_for(np, kNetBlock), kNetBlock, 0, s.stream>>>(np, s.d_patch_nodes, q, s.grid.dxi1,
                                                                   s.grid.dxi2, nets, boxes, culls);
   k_ray_groups<<<grid_for(ngroups, kNetBlock), kNetBlock, 0, s.stream>>>(np, boxes, gboxes);
-  const int use_newton = variant == SHELL_RAY_NEWTON;
   const unsigned ctas = (unsigned)((n_rays + kRayBlock - 1) / kRayBlock);
-  if (culls) {
-    k_trace_rays<true><<<ctas, kRayBlock, 0, s.stream>>>(n_rays, origins, dirs, np, nets, boxes, gboxes, culls,
-                                                         use_newton, out, redo_count, redo_list, heaps);
-    k_trace_rays_redo<true><<<1, kRedoThreads, 0, s.stream>>>(origins, dirs, np, nets, boxes, culls, use_newton, out,
-                                                              redo_count, redo_list, heaps);
-  } else {
-    k_trace_rays<false><<<ctas, kRayBlock, 0, s.stream>>>(n_rays, origins, dirs, np, nets, boxes, gboxes, culls,
-                                                          use_newton, out, redo_count, redo_list, heaps);
-    k_trace_rays_redo<false><<<1, kRedoThreads, 0, s.stream>>>(origins, dirs, np, nets, boxes, culls, use_newton, out,
-                                                               redo_count, redo_list, heaps);
-  }
+  const bool newton = variant == SHELL_RAY_NEWTON;
+  auto trace = culls ? (newton ? k_trace_rays<true, true> : k_trace_rays<true, false>)
+                     : (newton ? k_trace_rays<false, true> : k_trace_rays<false, false>);
+  auto redo = culls ? (newton ? k_trace_rays_redo<true, true> : k_trace_rays_redo<true, false>)
+                    : (newton ? k_trace_rays_redo<false, true> : k_trace_rays_redo<false, false>);
+  trace<<<ctas, kRayBlock, 0, s.stream>>>(n_rays, origins, dirs, np, nets, boxes, gboxes, culls, out, redo_count,
+                                          redo_list, heaps);
+  redo<<<1, kRedoThreads, 0, s.stream>>>(origins, dirs, np, nets, boxes, culls, out, redo_count, redo_list, heaps);
   s.launches += 4;
   BHEM_CUDA(cudaGetLastError());
   return SHELL_OK;

@@ -100,3 +100,30 @@ def test_heap_spill_and_second_pass():
         assert 128 < int((ref[4][:, 1] > RAY_HEAP).sum()) < len(x0)
         gpu = _gpu_ccd(g, q, dq, x0, dx, variant)
         _assert_identical(gpu, ref, variant)
+
+
+@pytest.mark.parametrize("variant", ["newton", "midpoint"])
+@pytest.mark.parametrize("scale,shift", [(1.0, 0.0), (1e-3, 0.0), (1e3, 0.0), (1.0, 1e5)])
+def test_culled_search_gives_the_same_contacts(variant, scale, shift):
+    """The search without statistics, which culls sub-patches by an FP32 test, returns bit for bit the
+    contacts of the search with statistics, which tests every candidate: on the four scenes at sizes
+    from millimetres to kilometres, far from the origin, with points at rest and points that move along
+    the surface; few points (every job on several lanes) and many."""
+    from paper_2312_14839_gb300.bhem import Shell
+    for name in ("plane", "drape", "static", "cylinder"):
+        for n in (3, 2500):
+            g, q, dq, x0, dx = S.ccd_scene(name, n, 17)
+            dx[: n // 5] = 0.0
+            dx[n // 5: n // 4, 2] = 0.0
+            off = np.array([shift, -shift, 0.5 * shift])
+            q, dq, x0, dx = q * scale, dq * scale, x0 * scale + off, dx * scale
+            q[:, :3] += off
+            to = lambda a: torch.as_tensor(np.ascontiguousarray(a), dtype=torch.float64, device="cuda")  # noqa: E731
+            with Shell(g, S.SHEET_MATERIAL, to(q.reshape(-1)), precision="fp64") as sh:
+                args = (to(q.reshape(-1)), to(dq.reshape(-1)), to(x0), to(dx))
+                full = sh.ccd_points(*args, variant=variant, want_stats=True)
+                culled = sh.ccd_points(*args, variant=variant)
+                for k in culled:
+                    np.testing.assert_array_equal(culled[k].cpu().numpy(), full[k].cpu().numpy(), err_msg=f"{name} {k}")
+            if n > 100:
+                assert (full["flags"] & 1).sum() > 50, name
