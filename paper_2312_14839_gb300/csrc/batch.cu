@@ -49,6 +49,20 @@ struct ShellState {
 
 struct Counters { int n_active, n_running, n_restart, n_searching; };
 
+// Work lists over the shells that take part, rebuilt on the device whenever that set changes
+// (k_compact): groups of at most kRowNodes and of at most kGroupNodes consecutive nodes of one shell,
+// as (first node, nodes, shell, 0), and the shells themselves, all in shell order. The row kernels run
+// as many CTAs as are resident and go through their list, so a launch costs what its active shells
+// cost: with one CTA per 8 (16) rows of the whole batch, a PCG iteration of the last running shell of
+// 512 still started 62,000 CTAs that had nothing to do (512 sheets' step: 345 -> 236 ms with the
+// lists, the alpha and beta controllers in the last CTA of the kernels that sum for them, and all
+// blocks of a row in flight).
+struct WorkList {
+  int4 *g8, *g16;
+  int* shells;
+  int* counts;   // g8 entries, g16 entries, shells
+};
+
 // Device-side loop state of the captured Newton step (one CUDA graph per step: WHILE nodes for
 // the Newton iterations, the regulariser rounds, the PCG chunks and the line-search trials, each
 // condition set by a one-thread kernel from the counters), and the body executions of each loop
@@ -61,14 +75,14 @@ struct LoopState {
 struct StepInput { double tau_carry; };
 constexpr int kGraphPcgChunk = 4;   // PCG iterations per body of the PCG WHILE node
 
-constexpr int kRowNodes = 8;          // block rows per SpMV CTA (36 threads each)
+constexpr int kRowNodes = 8;          // block rows per SpMV group (36 threads each)
+constexpr int kGroupNodes = 16;       // nodes per group of the other row kernels (12 threads each)
 constexpr int kSpmvThreads = 288;
 constexpr int kNodeThreads = 192;     // 12 threads per node, 16 nodes per CTA
 
 // ------------------------------------------------------------------------------------------
-// Segmented CTA reductions: the rows of one CTA span at most two shells (every shell has at
-// least 4 nodes per patch row and the CTAs hold <= 16 nodes of consecutive shells... the
-// two-segment split is checked by the host at set-up: every shell has >= 16 nodes).
+// CTA reductions. A group's rows belong to one shell, so a CTA adds one FP64 atomic per value and
+// shell (or run of groups of a shell) into that shell's accumulators.
 // ------------------------------------------------------------------------------------------
 __device__ __forceinline__ double block_sum_d(double v, double* sbuf) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
@@ -81,31 +95,24 @@ __device__ __forceinline__ double block_sum_d(double v, double* sbuf) {
   return s;
 }
 
-// The rows of one CTA belong to at most two consecutive shells s0 <= s1 (every shell has at
-// least 16 nodes, checked at set-up). A thread's value v belongs to the shell of its row (v = 0
-// for rows without work); the CTA sums each segment and adds it with one FP64 atomic into acc
-// of that shell, when the CTA-uniform flag use0 / use1 says the shell takes part.
-__device__ __forceinline__ void seg_add_d(double v, int sh, int s0, int s1, bool use0, bool use1,
-                                          ShellState* st, int slot) {
-  __shared__ double sbuf[32];
-  const double a = block_sum_d(sh == s0 ? v : 0.0, sbuf);
-  const double b = block_sum_d(sh != s0 ? v : 0.0, sbuf);
-  if (threadIdx.x == 0) {
-    if (use0 && s0 >= 0) atomicAdd(&st[s0].acc[slot], a);
-    if (use1 && s1 >= 0 && s1 != s0) atomicAdd(&st[s1].acc[slot], b);
-  }
+__device__ __forceinline__ void add_f2(F2 v, ShellState* st, int s, int slot) {
+  __shared__ F2 sbuf2[1][32];
+  const F2 a = f2_block_sum(v, sbuf2, 0);
+  if (threadIdx.x == 0) atomicAdd(&st[s].acc[slot], (double)a.hi + (double)a.lo);
 }
 
-__device__ __forceinline__ void seg_add_f2(F2 v, int sh, int s0, int s1, bool use0, bool use1,
-                                           ShellState* st, int slot) {
-  __shared__ F2 sbuf2[1][32];
-  const F2 z{0.f, 0.f};
-  const F2 a = f2_block_sum(sh == s0 ? v : z, sbuf2, 0);
-  const F2 b = f2_block_sum(sh != s0 ? v : z, sbuf2, 0);
+// Whether this CTA is the last of the grid to get here (one thread takes a ticket; nothing waits).
+__device__ __forceinline__ bool last_cta(unsigned* ticket) {
+  __shared__ int last;
+  __syncthreads();
   if (threadIdx.x == 0) {
-    if (use0 && s0 >= 0) atomicAdd(&st[s0].acc[slot], (double)a.hi + (double)a.lo);
-    if (use1 && s1 >= 0 && s1 != s0) atomicAdd(&st[s1].acc[slot], (double)b.hi + (double)b.lo);
+    __threadfence();
+    last = atomicAdd(ticket, 1u) == gridDim.x - 1u;
+    if (last) *ticket = 0u;
   }
+  __syncthreads();
+  if (last) __threadfence();
+  return last != 0;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -304,32 +311,97 @@ k_eg64(int n_items, const int4* __restrict__ items, int P, const ShellPar* __res
 }
 
 // ------------------------------------------------------------------------------------------
-// Row kernels (12 threads per node, 16 nodes per CTA)
+// Work lists
 // ------------------------------------------------------------------------------------------
-__device__ __forceinline__ void cta_shells(int n, const int* __restrict__ nshell, int first_node,
-                                           int count, int* s0, int* s1) {
-  const int last = min(first_node + count, n) - 1;
-  *s0 = first_node < n ? nshell[first_node] : -1;
-  *s1 = last >= first_node ? nshell[last] : -1;
+__device__ __forceinline__ bool pcg_running(const ShellState& S) { return S.active && !S.pcg_done; }
+
+// Rebuilds a work list (one CTA): shells that are active (running = 0), or whose PCG runs. With cnt,
+// the number of running shells goes to cnt->n_running; with cond (1: first, 2: after a chunk) thread 0
+// sets the PCG WHILE node's condition, as k_cond_* do for the other loops.
+__global__ void __launch_bounds__(1024)
+k_compact(int S, const ShellState* st, const ShellPar* __restrict__ par, WorkList L, int running, Counters* cnt,
+          LoopState* loop, int limit, cudaGraphConditionalHandle h, int cond) {
+  __shared__ int3 wsum[32];
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  int3 base = make_int3(0, 0, 0);
+  for (int s0 = 0; s0 < S; s0 += 1024) {
+    const int s = s0 + t;
+    const bool in = s < S && st[s].active && !(running && st[s].pcg_done);
+    const int first = in ? par[s].node_off : 0, nodes = in ? par[s].node_end - first : 0;
+    const int3 own = make_int3((nodes + kRowNodes - 1) / kRowNodes, (nodes + kGroupNodes - 1) / kGroupNodes, in);
+    int3 v = own;   // inclusive sums over the warp, then over the warps
+    for (int o = 1; o < 32; o <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, v.x, o), y = __shfl_up_sync(0xffffffffu, v.y, o),
+                z = __shfl_up_sync(0xffffffffu, v.z, o);
+      if (lane >= o) v = make_int3(v.x + x, v.y + y, v.z + z);
+    }
+    __syncthreads();
+    if (lane == 31) wsum[wid] = v;
+    __syncthreads();
+    int3 all = make_int3(0, 0, 0);
+    for (int w = 0; w < 32; ++w) {
+      if (w == wid) v = make_int3(v.x + all.x, v.y + all.y, v.z + all.z);
+      all = make_int3(all.x + wsum[w].x, all.y + wsum[w].y, all.z + wsum[w].z);
+    }
+    const int o8 = base.x + v.x - own.x, o16 = base.y + v.y - own.y;
+    if (in) L.shells[base.z + v.z - 1] = s;
+    for (unsigned m = __ballot_sync(0xffffffffu, in); m; m &= m - 1) {   // the warp writes one shell's groups
+      const int l = __ffs(m) - 1;
+      const int f = __shfl_sync(0xffffffffu, first, l), n = __shfl_sync(0xffffffffu, nodes, l);
+      const int b8 = __shfl_sync(0xffffffffu, o8, l), b16 = __shfl_sync(0xffffffffu, o16, l);
+      const int sh = s0 + wid * 32 + l;
+      for (int k = lane; k * kRowNodes < n; k += 32)
+        L.g8[b8 + k] = make_int4(f + k * kRowNodes, min(kRowNodes, n - k * kRowNodes), sh, 0);
+      for (int k = lane; k * kGroupNodes < n; k += 32)
+        L.g16[b16 + k] = make_int4(f + k * kGroupNodes, min(kGroupNodes, n - k * kGroupNodes), sh, 0);
+    }
+    base = make_int3(base.x + all.x, base.y + all.y, base.z + all.z);
+  }
+  if (t == 0) {
+    L.counts[0] = base.x;
+    L.counts[1] = base.y;
+    L.counts[2] = base.z;
+    if (cnt) cnt->n_running = base.z;
+    if (cond) {
+      if (cond == 1) loop->pcg_iters = 0;
+      else loop->pcg_iters += kGraphPcgChunk;
+      const bool go = base.z > 0 && loop->pcg_iters < limit;
+      if (go) loop->n_pcg += 1;
+      cudaGraphSetConditional(h, go ? 1u : 0u);
+    }
+  }
 }
 
+// Zeroes the matrix rows of the listed shells.
+__global__ void __launch_bounds__(256)
+k_zero_rows(WorkList L, const int* __restrict__ rp, float* __restrict__ val) {
+  const int n = L.counts[1];
+  for (int w = blockIdx.x; w < n; w += gridDim.x) {
+    const int4 e = L.g16[w];
+    const size_t b0 = (size_t)rp[e.x] * 36, b1 = (size_t)rp[e.x + e.y] * 36;
+    for (size_t k = b0 + threadIdx.x; k < b1; k += blockDim.x)
+      reinterpret_cast<float4*>(val)[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+}
+
+// ------------------------------------------------------------------------------------------
+// Row kernels (12 threads per node, groups of 16 nodes of one shell)
+// ------------------------------------------------------------------------------------------
 // g = grad_el + M (q - y)/dt^2 - F (masked), gin; acc[0] += |g|^2 (shells with active != 0)
 __global__ void __launch_bounds__(kNodeThreads)
-k_grad_finish(int n, const int* __restrict__ nshell, ShellState* st, const int* __restrict__ rp,
+k_grad_finish(WorkList L, ShellState* st, const int* __restrict__ rp,
               const int* __restrict__ col, const double* __restrict__ mass,
               const double* __restrict__ fgrav, const double* __restrict__ q,
               const double* __restrict__ yv, double inv_dt2, double gx, double gy, double gz,
               const unsigned char* __restrict__ mask, double* __restrict__ g,
               double* __restrict__ gin, int* err) {
-  const int ln = threadIdx.x / 12, a = threadIdx.x % 12;
-  const int i = blockIdx.x * 16 + ln;
-  int s0, s1;
-  cta_shells(n, nshell, blockIdx.x * 16, 16, &s0, &s1);
-  double part = 0.0;
-  int sh = -1;
-  if (i < n) {
-    sh = nshell[i];
-    if (st[sh].active) {
+  __shared__ double sbuf[32];
+  const int ln = threadIdx.x / 12, a = threadIdx.x % 12, n = L.counts[1];
+  for (int w = blockIdx.x; w < n; w += gridDim.x) {
+    const int4 e = L.g16[w];
+    const int i = e.x + ln;
+    double part = 0.0;
+    if (ln < e.y && st[e.z].active) {
       const size_t gi = (size_t)i * 12 + a;
       const int r = a / 3, c = a % 3;
       const double grav = c == 0 ? gx : c == 1 ? gy : gz;
@@ -347,8 +419,9 @@ k_grad_finish(int n, const int* __restrict__ nshell, ShellState* st, const int* 
       gin[gi] = gi_in;
       part = gv * gv;
     }
+    const double tot = block_sum_d(part, sbuf);
+    if (threadIdx.x == 0) atomicAdd(&st[e.z].acc[0], tot);
   }
-  seg_add_d(part, sh, s0, s1, true, true, st, 0);
 }
 
 // Per shell and DOF kind over free DOFs: sum |A_ii| (acc2[3k]), count (acc2[3k+1]) and min A_ii
@@ -360,109 +433,104 @@ __device__ __forceinline__ int float_order(float f) {
 __device__ __forceinline__ float order_float(int i) { return __int_as_float(i >= 0 ? i : i ^ 0x7fffffff); }
 
 __global__ void __launch_bounds__(kNodeThreads)
-k_diag_stats(int n, const int* __restrict__ nshell, ShellState* st, const int* __restrict__ diag_block,
+k_diag_stats(WorkList L, ShellState* st, const int* __restrict__ diag_block,
              const float* __restrict__ val, const unsigned char* __restrict__ mask,
              int* __restrict__ dmin_bits) {
-  __shared__ double ssum[2][4], scnt[2][4];
-  __shared__ int smin[2][4];
-  const int ln = threadIdx.x / 12, a = threadIdx.x % 12, kind = a / 3;
-  const int i = blockIdx.x * 16 + ln;
-  int s0, s1;
-  cta_shells(n, nshell, blockIdx.x * 16, 16, &s0, &s1);
-  if (threadIdx.x < 8) {
-    ssum[threadIdx.x / 4][threadIdx.x % 4] = 0.0;
-    scnt[threadIdx.x / 4][threadIdx.x % 4] = 0.0;
-    smin[threadIdx.x / 4][threadIdx.x % 4] = 0x7fffffff;
-  }
-  __syncthreads();
-  if (i < n && !(mask && mask[(size_t)i * 12 + a])) {
-    const int sh = nshell[i];
-    if (st[sh].active) {
-      const float d = val[(size_t)diag_block[i] * 144 + a * 13];
-      const int seg = sh == s0 ? 0 : 1;
-      atomicAdd(&ssum[seg][kind], (double)fabsf(d));
-      atomicAdd(&scnt[seg][kind], 1.0);
-      atomicMin(&smin[seg][kind], float_order(d));
+  __shared__ double ssum[4], scnt[4];
+  __shared__ int smin[4];
+  const int ln = threadIdx.x / 12, a = threadIdx.x % 12, kind = a / 3, n = L.counts[1];
+  for (int w = blockIdx.x; w < n; w += gridDim.x) {
+    const int4 e = L.g16[w];
+    __syncthreads();
+    if (threadIdx.x < 4) {
+      ssum[threadIdx.x] = 0.0;
+      scnt[threadIdx.x] = 0.0;
+      smin[threadIdx.x] = 0x7fffffff;
     }
-  }
-  __syncthreads();
-  if (threadIdx.x < 8) {
-    const int seg = threadIdx.x / 4, k = threadIdx.x % 4;
-    const int sh = seg == 0 ? s0 : s1;
-    if (sh >= 0 && (seg == 0 || s1 != s0) && scnt[seg][k] > 0.0) {
-      atomicAdd(&st[sh].acc2[3 * k], ssum[seg][k]);
-      atomicAdd(&st[sh].acc2[3 * k + 1], scnt[seg][k]);
-      atomicMin(&dmin_bits[4 * sh + k], smin[seg][k]);
+    __syncthreads();
+    const int i = e.x + ln;
+    if (ln < e.y && !(mask && mask[(size_t)i * 12 + a])) {
+      const float d = val[(size_t)diag_block[i] * 144 + a * 13];
+      atomicAdd(&ssum[kind], (double)fabsf(d));
+      atomicAdd(&scnt[kind], 1.0);
+      atomicMin(&smin[kind], float_order(d));
+    }
+    __syncthreads();
+    if (threadIdx.x < 4 && scnt[threadIdx.x] > 0.0) {
+      const int k = threadIdx.x;
+      atomicAdd(&st[e.z].acc2[3 * k], ssum[k]);
+      atomicAdd(&st[e.z].acc2[3 * k + 1], scnt[k]);
+      atomicMin(&dmin_bits[4 * e.z + k], smin[k]);
     }
   }
 }
 
 __global__ void __launch_bounds__(192)
-k_precond(int n, const int* __restrict__ nshell, const ShellState* st,
+k_precond(WorkList L, const ShellState* st,
           const int* __restrict__ diag_block, const float* __restrict__ val,
           const unsigned char* __restrict__ mask, float* __restrict__ Dinv, int only_restart) {
   __shared__ float sL[16][12][13];
   __shared__ float sW[16][12][13];
   __shared__ float sdiag[16][12];
   __shared__ int sok[16];
-  const int ln = threadIdx.x / 12, a = threadIdx.x % 12;
-  const int i = blockIdx.x * 16 + ln;
-  bool active = i < n;
-  int s = 0;
-  if (active) {
-    s = nshell[i];
-    active = st[s].active && !st[s].pcg_done && (!only_restart || st[s].restart);
-  }
-  if (active) {
-    const float* Bv = val + (size_t)diag_block[i] * 144;
-    const bool fa = mask && mask[(size_t)i * 12 + a];
-    for (int b = 0; b < 12; ++b) {
-      const bool fb = mask && mask[(size_t)i * 12 + b];
-      float v = Bv[a * 12 + b];
-      if (fa || fb) v = (a == b) ? 1.f : 0.f;
-      else if (a == b) v += st[s].td[a / 3];
-      sL[ln][a][b] = v;
+  const int ln = threadIdx.x / 12, a = threadIdx.x % 12, n = L.counts[1];
+  for (int w = blockIdx.x; w < n; w += gridDim.x) {
+    const int4 e = L.g16[w];
+    const int s = e.z, i = e.x + ln;
+    if (!pcg_running(st[s]) || (only_restart && !st[s].restart)) continue;   // uniform over the CTA
+    const bool active = ln < e.y;
+    __syncthreads();
+    if (active) {
+      const float* Bv = val + (size_t)diag_block[i] * 144;
+      const bool fa = mask && mask[(size_t)i * 12 + a];
+      for (int b = 0; b < 12; ++b) {
+        const bool fb = mask && mask[(size_t)i * 12 + b];
+        float v = Bv[a * 12 + b];
+        if (fa || fb) v = (a == b) ? 1.f : 0.f;
+        else if (a == b) v += st[s].td[a / 3];
+        sL[ln][a][b] = v;
+      }
+      sdiag[ln][a] = sL[ln][a][a];
     }
-    sdiag[ln][a] = sL[ln][a][a];
-  }
-  if (a == 0) sok[ln] = 1;
-  __syncthreads();
-  for (int j = 0; j < 12; ++j) {
-    if (active && a == j && sok[ln]) {
-      float acc = sL[ln][j][j];
-      for (int k = 0; k < j; ++k) acc -= sL[ln][j][k] * sL[ln][j][k];
-      if (!(acc > 0.f)) sok[ln] = 0;
-      else sL[ln][j][j] = sqrtf(acc);
+    if (a == 0) sok[ln] = 1;
+    __syncthreads();
+    for (int j = 0; j < 12; ++j) {
+      if (active && a == j && sok[ln]) {
+        float acc = sL[ln][j][j];
+        for (int k = 0; k < j; ++k) acc -= sL[ln][j][k] * sL[ln][j][k];
+        if (!(acc > 0.f)) sok[ln] = 0;
+        else sL[ln][j][j] = sqrtf(acc);
+      }
+      __syncthreads();
+      if (active && a > j && sok[ln]) {
+        float u = sL[ln][a][j];
+        for (int k = 0; k < j; ++k) u -= sL[ln][a][k] * sL[ln][j][k];
+        sL[ln][a][j] = u / sL[ln][j][j];
+      }
+      __syncthreads();
+    }
+    const bool ok = active && sok[ln];
+    if (ok) {
+      for (int r = 0; r < 12; ++r) {
+        if (r < a) { sW[ln][r][a] = 0.f; continue; }
+        float u = (r == a) ? 1.f : 0.f;
+        for (int k = a; k < r; ++k) u -= sL[ln][r][k] * sW[ln][k][a];
+        sW[ln][r][a] = u / sL[ln][r][r];
+      }
     }
     __syncthreads();
-    if (active && a > j && sok[ln]) {
-      float u = sL[ln][a][j];
-      for (int k = 0; k < j; ++k) u -= sL[ln][a][k] * sL[ln][j][k];
-      sL[ln][a][j] = u / sL[ln][j][j];
+    if (!active) continue;
+    float* D = Dinv + (size_t)i * 144 + a * 12;
+    if (ok) {
+      for (int b = 0; b < 12; ++b) {
+        float acc = 0.f;
+        for (int k = (a > b ? a : b); k < 12; ++k) acc += sW[ln][k][a] * sW[ln][k][b];
+        D[b] = acc;
+      }
+    } else {
+      const float d = sdiag[ln][a];
+      for (int b = 0; b < 12; ++b) D[b] = (a == b) ? (d > 0.f ? 1.f / d : 1.f) : 0.f;
     }
-    __syncthreads();
-  }
-  const bool ok = active && sok[ln];
-  if (ok) {
-    for (int r = 0; r < 12; ++r) {
-      if (r < a) { sW[ln][r][a] = 0.f; continue; }
-      float u = (r == a) ? 1.f : 0.f;
-      for (int k = a; k < r; ++k) u -= sL[ln][r][k] * sW[ln][k][a];
-      sW[ln][r][a] = u / sL[ln][r][r];
-    }
-  }
-  __syncthreads();
-  if (!active) return;
-  float* D = Dinv + (size_t)i * 144 + a * 12;
-  if (ok) {
-    for (int b = 0; b < 12; ++b) {
-      float acc = 0.f;
-      for (int k = (a > b ? a : b); k < 12; ++k) acc += sW[ln][k][a] * sW[ln][k][b];
-      D[b] = acc;
-    }
-  } else {
-    const float d = sdiag[ln][a];
-    for (int b = 0; b < 12; ++b) D[b] = (a == b) ? (d > 0.f ? 1.f / d : 1.f) : 0.f;
   }
 }
 
@@ -473,143 +541,202 @@ __device__ __forceinline__ float apply_block(const float* __restrict__ D, const 
   return s;
 }
 
-// PCG init for shells that start (or restart) a solve: x = 0, r = rhs, z = D r, p = z;
-// acc[0] += r.z, acc[1] += r.r
+// PCG init for shells that start (or restart) a solve: x = 0, r = -g, z = D r; acc[0] += r.z,
+// acc[1] += r.r
 __global__ void __launch_bounds__(kNodeThreads)
-k_pcg_init(int n, const int* __restrict__ nshell, ShellState* st, const double* __restrict__ rhs,
+k_pcg_init(WorkList L, ShellState* st, const double* __restrict__ g,
            const float* __restrict__ Dinv, const unsigned char* __restrict__ mask,
-           float* __restrict__ x, float* __restrict__ r, float* __restrict__ z, float* __restrict__ p,
-           int only_restart) {
+           float* __restrict__ x, float* __restrict__ r, float* __restrict__ z, int only_restart) {
   __shared__ float sr[16][12];
-  const int ln = threadIdx.x / 12, a = threadIdx.x % 12;
-  const int i = blockIdx.x * 16 + ln;
-  int s0, s1;
-  cta_shells(n, nshell, blockIdx.x * 16, 16, &s0, &s1);
-  const size_t gi = (size_t)i * 12 + a;
-  bool act = false;
-  int sh = -1;
-  float ri = 0.f, zi = 0.f;
-  if (i < n) {
-    sh = nshell[i];
-    act = st[sh].active && !st[sh].pcg_done && (!only_restart || st[sh].restart);
-    if (act) {
-      ri = (mask && mask[gi]) ? 0.f : (float)rhs[gi];
+  const int ln = threadIdx.x / 12, a = threadIdx.x % 12, n = L.counts[1];
+  for (int w = blockIdx.x; w < n; w += gridDim.x) {
+    const int4 e = L.g16[w];
+    if (!pcg_running(st[e.z]) || (only_restart && !st[e.z].restart)) continue;   // uniform over the CTA
+    const int i = e.x + ln;
+    const size_t gi = (size_t)i * 12 + a;
+    float ri = 0.f, zi = 0.f;
+    if (ln < e.y) {
+      ri = (mask && mask[gi]) ? 0.f : (float)-g[gi];
       x[gi] = 0.f;
       r[gi] = ri;
       sr[ln][a] = ri;
     }
+    __syncthreads();
+    if (ln < e.y) {
+      zi = (mask && mask[gi]) ? 0.f : apply_block(Dinv + (size_t)i * 144, sr[ln], a);
+      z[gi] = zi;
+    }
+    add_f2(f2_prod(ri, zi), st, e.z, 0);   // ends with a barrier
+    add_f2(f2_prod(ri, ri), st, e.z, 1);
   }
-  __syncthreads();
-  if (act) {
-    zi = (mask && mask[gi]) ? 0.f : apply_block(Dinv + (size_t)i * 144, sr[ln], a);
-    z[gi] = zi;
-    p[gi] = zi;
-  }
-  auto starts = [&](int s) { return s >= 0 && st[s].active && !st[s].pcg_done && (!only_restart || st[s].restart); };
-  const bool use0 = starts(s0), use1 = starts(s1);
-  seg_add_f2(f2_prod(ri, zi), sh, s0, s1, use0, use1, st, 0);
-  seg_add_f2(f2_prod(ri, ri), sh, s0, s1, use0, use1, st, 1);
 }
 
-__device__ __forceinline__ bool pcg_running(const ShellState& S) { return S.active && !S.pcg_done; }
-
-// y = (A + tau D) p on rows of running shells; acc[0] += p.y
-// x is z: per running shell's own rows, p = z + beta p (the first iteration of a solve: p = z)
-// and y = Ap = (A + tau D) z + beta Ap, equal to (A + tau D) p by linearity, so no separate
-// p-update launch follows the update
-__global__ void __launch_bounds__(kSpmvThreads)
-k_spmv(int n, const int* __restrict__ nshell, ShellState* st, const int* __restrict__ rp,
+// One PCG iteration's product on the running shells: x is z; per own row p = z + beta p (the first
+// iteration of a solve: p = z) and y = Ap = (A + tau D) z + beta Ap, equal to (A + tau D) p by
+// linearity, so no separate p-update launch follows the update; p.y per shell, and in the last CTA
+// alpha = rz / p.y, or negative curvature. A CTA takes consecutive groups, so it sums p.y over a
+// shell's groups in registers and adds it once. Every block of a row is loaded before its use, as in
+// the single-shell product (4 CTAs per SM at 56 registers; 3 without the 180 bytes of spills: 12%
+// slower). Latency bounds it below about 100 shells, DRAM above.
+__global__ void __launch_bounds__(kSpmvThreads, 4)
+k_spmv(WorkList L, ShellState* st, const int* __restrict__ rp,
        const int* __restrict__ col, const float* __restrict__ val, const float* __restrict__ x,
-       const unsigned char* __restrict__ mask, float* __restrict__ p, float* __restrict__ y) {
-  __shared__ float sacc[kSpmvThreads];
-  const int t = threadIdx.x;
-  const int br = t / 36, w = t % 36, r = w / 3, cc = w % 3;
-  const int i = blockIdx.x * kRowNodes + br;
-  int s0, s1;
-  cta_shells(n, nshell, blockIdx.x * kRowNodes, kRowNodes, &s0, &s1);
-  const bool run0 = s0 >= 0 && pcg_running(st[s0]), run1 = s1 >= 0 && pcg_running(st[s1]);
-  if (!run0 && !run1) return;   // uniform over the CTA
-  int sh = -1;
-  bool run = false;
-  float acc = 0.f;
-  if (i < n) {
-    sh = nshell[i];
-    run = pcg_running(st[sh]);
-    if (run) {
-      const int k0 = rp[i], k1 = rp[i + 1];
-      for (int k = k0; k < k1; ++k) {
-        const float4 a = __ldcs(reinterpret_cast<const float4*>(val + (size_t)k * 144 + r * 12 + cc * 4));
-        const float4 xv = *reinterpret_cast<const float4*>(x + (size_t)col[k] * 12 + cc * 4);
-        acc += a.x * xv.x + a.y * xv.y + a.z * xv.z + a.w * xv.w;
-      }
-    }
-  }
-  sacc[t] = acc;
-  __syncthreads();
+       const unsigned char* __restrict__ mask, float* __restrict__ p, float* __restrict__ y, unsigned* ticket) {
+  __shared__ float sacc[2][kSpmvThreads];
+  const int t = threadIdx.x, n = L.counts[0];
+  const int br = t / 36, w36 = t % 36, r = w36 / 3, cc = w36 % 3;
+  const int per = (n + gridDim.x - 1) / gridDim.x, w0 = blockIdx.x * per, w1 = min(n, w0 + per);
   F2 part{0.f, 0.f};
-  if (run && cc == 0) {
-    const size_t gi = (size_t)i * 12 + r;
-    const float zi = x[gi];
-    float wi = (sacc[t] + sacc[t + 1]) + sacc[t + 2];
-    wi += st[sh].td[r / 3] * zi;
-    if (mask && mask[gi]) wi = 0.f;
-    float pi = zi, qi = wi;
-    if (st[sh].pcg_iters > 0) {
-      const float bf = (float)st[sh].beta;
-      pi = fmaf(bf, p[gi], zi);
-      qi = fmaf(bf, y[gi], wi);
+  int cur = -1;
+  for (int w = w0; w < w1; ++w) {
+    const int4 e = L.g8[w];
+    if (e.z != cur) {   // uniform over the CTA
+      if (cur >= 0) add_f2(part, st, cur, 0);
+      cur = e.z;
+      part = F2{0.f, 0.f};
     }
-    p[gi] = pi;
-    y[gi] = qi;
-    part = f2_prod(pi, qi);
+    const ShellState& T = st[cur];
+    if (!pcg_running(T)) continue;
+    const int i = e.x + br;
+    float acc = 0.f;
+    if (br < e.y) {
+      const int k0 = rp[i], k1 = rp[i + 1];
+      constexpr int U = 9;   // a node couples to at most 9 nodes
+      float4 v[U];
+      int j[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (k0 + u < k1) {
+          j[u] = col[k0 + u];
+          v[u] = __ldcs(reinterpret_cast<const float4*>(val + (size_t)(k0 + u) * 144 + r * 12 + cc * 4));
+        }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (k0 + u < k1) {
+          const float4 xv = *reinterpret_cast<const float4*>(x + (size_t)j[u] * 12 + cc * 4);
+          acc = __fmaf_rn(v[u].x, xv.x, acc);
+          acc = __fmaf_rn(v[u].y, xv.y, acc);
+          acc = __fmaf_rn(v[u].z, xv.z, acc);
+          acc = __fmaf_rn(v[u].w, xv.w, acc);
+        }
+    }
+    float* sa = sacc[w & 1];   // the other half may still be read
+    sa[t] = acc;
+    __syncthreads();
+    if (br < e.y && cc == 0) {
+      const size_t gi = (size_t)i * 12 + r;
+      const float zi = x[gi];
+      float wi = (sa[t] + sa[t + 1]) + sa[t + 2];
+      wi += T.td[r / 3] * zi;
+      if (mask && mask[gi]) wi = 0.f;
+      float pi = zi, qi = wi;
+      if (T.pcg_iters > 0) {
+        const float bf = (float)T.beta;
+        pi = fmaf(bf, p[gi], zi);
+        qi = fmaf(bf, y[gi], wi);
+      }
+      p[gi] = pi;
+      y[gi] = qi;
+      part = f2_add(part, f2_prod(pi, qi));
+    }
   }
-  seg_add_f2(part, sh, s0, s1, run0, run1, st, 0);
+  if (cur >= 0) add_f2(part, st, cur, 0);
+  if (!last_cta(ticket)) return;
+  for (int k = t; k < L.counts[2]; k += blockDim.x) {
+    ShellState& T = st[L.shells[k]];
+    const double pq = __ldcg(&T.acc[0]);
+    T.acc[0] = 0.0;
+    if (!pcg_running(T)) continue;
+    T.pq = pq;
+    if (!(pq > 0.0)) {
+      T.negcurv = 1;
+      T.pcg_done = 1;
+      T.alpha = 0.0;
+    } else {
+      T.alpha = T.rz / pq;
+    }
+  }
 }
 
-// x += alpha p, r -= alpha Ap, z = D r on running shells; acc[0] += r.z, acc[1] += r.r
+// x += alpha p, r -= alpha Ap, z = D r on the running shells; r.z and r.r per shell, and in the last
+// CTA beta, convergence and the iteration limit.
 __global__ void __launch_bounds__(kNodeThreads)
-k_pcg_update(int n, const int* __restrict__ nshell, ShellState* st, float* __restrict__ x,
+k_pcg_update(WorkList L, ShellState* st, float* __restrict__ x,
              float* __restrict__ r, float* __restrict__ z, const float* __restrict__ p,
              const float* __restrict__ Ap, const float* __restrict__ Dinv,
-             const unsigned char* __restrict__ mask) {
-  __shared__ float sr[16][12];
-  const int ln = threadIdx.x / 12, a = threadIdx.x % 12;
-  const int i = blockIdx.x * 16 + ln;
-  int s0, s1;
-  cta_shells(n, nshell, blockIdx.x * 16, 16, &s0, &s1);
-  const bool run0 = s0 >= 0 && pcg_running(st[s0]), run1 = s1 >= 0 && pcg_running(st[s1]);
-  if (!run0 && !run1) return;
-  const size_t gi = (size_t)i * 12 + a;
-  bool run = false;
-  int sh = -1;
-  float ri = 0.f, zi = 0.f;
-  if (i < n) {
-    sh = nshell[i];
-    run = pcg_running(st[sh]);
-    if (run) {
-      const float al = (float)st[sh].alpha;
+             const unsigned char* __restrict__ mask, unsigned* ticket) {
+  __shared__ float sr[2][16][12];
+  const int ln = threadIdx.x / 12, a = threadIdx.x % 12, n = L.counts[1];
+  const int per = (n + gridDim.x - 1) / gridDim.x, w0 = blockIdx.x * per, w1 = min(n, w0 + per);
+  F2 rz{0.f, 0.f}, rr{0.f, 0.f};
+  int cur = -1;
+  for (int w = w0; w < w1; ++w) {
+    const int4 e = L.g16[w];
+    if (e.z != cur) {   // uniform over the CTA
+      if (cur >= 0) {
+        add_f2(rz, st, cur, 0);
+        add_f2(rr, st, cur, 1);
+      }
+      cur = e.z;
+      rz = rr = F2{0.f, 0.f};
+    }
+    const ShellState& T = st[cur];
+    if (!pcg_running(T)) continue;
+    const int i = e.x + ln;
+    const size_t gi = (size_t)i * 12 + a;
+    const bool in = ln < e.y;
+    float4 d0, d1, d2;
+    float ri = 0.f, zi = 0.f;
+    if (in) {
+      const float4* drow = reinterpret_cast<const float4*>(Dinv + (size_t)i * 144 + a * 12);
+      d0 = __ldg(drow);
+      d1 = __ldg(drow + 1);
+      d2 = __ldg(drow + 2);
+      const float al = (float)T.alpha;
       x[gi] = fmaf(al, p[gi], x[gi]);
       ri = fmaf(-al, Ap[gi], r[gi]);
       r[gi] = ri;
-      sr[ln][a] = ri;
+      sr[w & 1][ln][a] = ri;
     }
+    __syncthreads();
+    if (in) {
+      if (!(mask && mask[gi])) {
+        const float* q = sr[w & 1][ln];   // the other half may still be read
+        zi = d0.x * q[0] + d0.y * q[1] + d0.z * q[2] + d0.w * q[3] + d1.x * q[4] + d1.y * q[5] + d1.z * q[6] +
+             d1.w * q[7] + d2.x * q[8] + d2.y * q[9] + d2.z * q[10] + d2.w * q[11];
+      }
+      z[gi] = zi;
+    }
+    rz = f2_add(rz, f2_prod(ri, zi));
+    rr = f2_add(rr, f2_prod(ri, ri));
   }
-  __syncthreads();
-  if (run) {
-    zi = (mask && mask[gi]) ? 0.f : apply_block(Dinv + (size_t)i * 144, sr[ln], a);
-    z[gi] = zi;
+  if (cur >= 0) {
+    add_f2(rz, st, cur, 0);
+    add_f2(rr, st, cur, 1);
   }
-  seg_add_f2(f2_prod(ri, zi), sh, s0, s1, run0, run1, st, 0);
-  seg_add_f2(f2_prod(ri, ri), sh, s0, s1, run0, run1, st, 1);
+  if (!last_cta(ticket)) return;
+  for (int k = threadIdx.x; k < L.counts[2]; k += blockDim.x) {
+    ShellState& T = st[L.shells[k]];
+    const double rz_new = __ldcg(&T.acc[0]), rr_new = __ldcg(&T.acc[1]);
+    T.acc[0] = 0.0;
+    T.acc[1] = 0.0;
+    if (!pcg_running(T)) continue;
+    T.rr = rr_new;
+    T.pcg_iters += 1;
+    T.pcg_iters_total += 1;
+    T.beta = rz_new / T.rz;
+    T.rz = rz_new;
+    if (T.rtol2 > 0.0 && T.rr <= T.rtol2 * T.bb) T.pcg_done = 1;
+    if (rz_new == 0.0) T.pcg_done = 1;
+    if (T.pcg_iters >= T.limit) T.pcg_done = 1;
+  }
 }
-
 
 // ------------------------------------------------------------------------------------------
 // Controllers: one thread per shell
 // ------------------------------------------------------------------------------------------
 // After k_pcg_init: rz, bb from acc[0..1]
-__global__ void k_ctrl_pcg_start(int S, ShellState* st, Counters* cnt, int only_restart,
-                                 double rtol, int pcg_max, int fixed) {
+__global__ void k_ctrl_pcg_start(int S, ShellState* st, int only_restart, double rtol, int pcg_max, int fixed) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= S) return;
   ShellState& T = st[s];
@@ -624,51 +751,6 @@ __global__ void k_ctrl_pcg_start(int S, ShellState* st, Counters* cnt, int only_
     T.negcurv = 0;
     T.restart = 0;
     if (T.bb == 0.0 || T.limit == 0) T.pcg_done = 1;
-  }
-  T.acc[0] = 0.0;
-  T.acc[1] = 0.0;
-  if (T.active && !T.pcg_done) atomicAdd(&cnt->n_running, 1);
-}
-
-__global__ void k_ctrl_count_running(int S, const ShellState* st, Counters* cnt) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s < S && st[s].active && !st[s].pcg_done) atomicAdd(&cnt->n_running, 1);
-}
-
-// After k_spmv: alpha = rz / p.Ap, or negative curvature
-__global__ void k_ctrl_alpha(int S, ShellState* st) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= S) return;
-  ShellState& T = st[s];
-  if (T.active && !T.pcg_done) {
-    const double pq = T.acc[0];
-    T.pq = pq;
-    if (!(pq > 0.0)) {
-      T.negcurv = 1;
-      T.pcg_done = 1;
-      T.alpha = 0.0;
-    } else {
-      T.alpha = T.rz / pq;
-    }
-  }
-  T.acc[0] = 0.0;
-}
-
-// After k_pcg_update: beta, convergence, iteration limit
-__global__ void k_ctrl_beta(int S, ShellState* st) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= S) return;
-  ShellState& T = st[s];
-  if (T.active && !T.pcg_done) {
-    const double rz_new = T.acc[0];
-    T.rr = T.acc[1];
-    T.pcg_iters += 1;
-    T.pcg_iters_total += 1;
-    T.beta = rz_new / T.rz;
-    T.rz = rz_new;
-    if (T.rtol2 > 0.0 && T.rr <= T.rtol2 * T.bb) T.pcg_done = 1;
-    if (rz_new == 0.0) T.pcg_done = 1;
-    if (T.pcg_iters >= T.limit) T.pcg_done = 1;
   }
   T.acc[0] = 0.0;
   T.acc[1] = 0.0;
@@ -830,7 +912,7 @@ __global__ void k_ctrl_ls_step(int S, ShellState* st, Counters* cnt) {
 // Conditions of the captured step's WHILE nodes (one thread). Each mirrors a loop bound of the
 // host-driven step: Newton while a shell is active and it <= newton_max; regulariser rounds while
 // a shell restarts, at most 16; PCG chunks while a shell runs and the iterations are below the
-// limit; line-search trials while a shell searches, at most 20.
+// limit (set by k_compact); line-search trials while a shell searches, at most 20.
 // ------------------------------------------------------------------------------------------
 __global__ void k_cond_newton(const Counters* cnt, LoopState* L, int newton_max, cudaGraphConditionalHandle h,
                               int first) {
@@ -856,14 +938,6 @@ __global__ void k_cond_reg(const Counters* cnt, LoopState* L, cudaGraphCondition
   cudaGraphSetConditional(h, go ? 1u : 0u);
 }
 
-__global__ void k_cond_pcg(const Counters* cnt, LoopState* L, int limit, cudaGraphConditionalHandle h, int first) {
-  if (first) L->pcg_iters = 0;
-  else L->pcg_iters += kGraphPcgChunk;
-  const bool go = cnt->n_running > 0 && L->pcg_iters < limit;
-  if (go) L->n_pcg += 1;
-  cudaGraphSetConditional(h, go ? 1u : 0u);
-}
-
 __global__ void k_cond_ls(const Counters* cnt, LoopState* L, cudaGraphConditionalHandle h, int first) {
   if (first) L->trial = 0;
   else L->trial += 1;
@@ -875,61 +949,41 @@ __global__ void k_cond_ls(const Counters* cnt, LoopState* L, cudaGraphConditiona
 // ------------------------------------------------------------------------------------------
 // Vector kernels over all DOFs (with per-shell coefficients)
 // ------------------------------------------------------------------------------------------
-__global__ void k_dots3(int n, const int* __restrict__ nshell, ShellState* st,
-                        const double* __restrict__ d, const double* __restrict__ Md,
-                        const double* __restrict__ gin, const double* __restrict__ g) {
-  const int ln = threadIdx.x / 12, a = threadIdx.x % 12;
-  const int i = blockIdx.x * 16 + ln;
-  int s0, s1;
-  cta_shells(n, nshell, blockIdx.x * 16, 16, &s0, &s1);
-  int sh = -1;
-  double v0 = 0.0, v1 = 0.0, v2 = 0.0;
-  if (i < n) {
-    sh = nshell[i];
-    if (st[sh].active) {
-      const size_t gi = (size_t)i * 12 + a;
-      v0 = d[gi] * Md[gi];
-      v1 = d[gi] * gin[gi];
-      v2 = g[gi] * d[gi];
-    }
-  }
-  // accumulate into acc2[0..2]
+// M d of the listed shells and, per shell, acc2[0..2] += d.Md, d.gin, g.d for the line search
+__global__ void __launch_bounds__(kNodeThreads)
+k_mass_dots(WorkList L, ShellState* st, const int* __restrict__ rp, const int* __restrict__ col,
+            const double* __restrict__ mass, const double* __restrict__ d, const double* __restrict__ gin,
+            const double* __restrict__ g) {
   __shared__ double sbuf[32];
-  const double a0 = block_sum_d(sh == s0 ? v0 : 0.0, sbuf), b0 = block_sum_d(sh >= 0 && sh != s0 ? v0 : 0.0, sbuf);
-  const double a1 = block_sum_d(sh == s0 ? v1 : 0.0, sbuf), b1 = block_sum_d(sh >= 0 && sh != s0 ? v1 : 0.0, sbuf);
-  const double a2 = block_sum_d(sh == s0 ? v2 : 0.0, sbuf), b2 = block_sum_d(sh >= 0 && sh != s0 ? v2 : 0.0, sbuf);
-  if (threadIdx.x == 0) {
-    if (s0 >= 0) {
-      atomicAdd(&st[s0].acc2[0], a0); atomicAdd(&st[s0].acc2[1], a1); atomicAdd(&st[s0].acc2[2], a2);
-    }
-    if (s1 >= 0 && s1 != s0) {
-      atomicAdd(&st[s1].acc2[0], b0); atomicAdd(&st[s1].acc2[1], b1); atomicAdd(&st[s1].acc2[2], b2);
-    }
-  }
-}
-
-__global__ void k_mass_mult(int n, const int* __restrict__ rp, const int* __restrict__ col,
-                            const double* __restrict__ mass, const double* __restrict__ x,
-                            double* __restrict__ y) {
-  const int ln = threadIdx.x / 12, a = threadIdx.x % 12;
-  const int i = blockIdx.x * 16 + ln;
-  if (i >= n) return;
+  const int ln = threadIdx.x / 12, a = threadIdx.x % 12, n = L.counts[1];
   const int r = a / 3, c = a % 3;
-  double sum = 0.0;
-  for (int k = rp[i]; k < rp[i + 1]; ++k) {
-    const int j = col[k];
-    for (int qq = 0; qq < 4; ++qq) sum += mass[(size_t)k * 16 + r * 4 + qq] * x[(size_t)j * 12 + qq * 3 + c];
+  for (int w = blockIdx.x; w < n; w += gridDim.x) {
+    const int4 e = L.g16[w];
+    double v[3] = {0.0, 0.0, 0.0};
+    if (ln < e.y && st[e.z].active) {
+      const int i = e.x + ln;
+      const size_t gi = (size_t)i * 12 + a;
+      double sum = 0.0;
+      for (int k = rp[i]; k < rp[i + 1]; ++k) {
+        const int j = col[k];
+        for (int qq = 0; qq < 4; ++qq) sum += mass[(size_t)k * 16 + r * 4 + qq] * d[(size_t)j * 12 + qq * 3 + c];
+      }
+      v[0] = d[gi] * sum;
+      v[1] = d[gi] * gin[gi];
+      v[2] = g[gi] * d[gi];
+    }
+    for (int q = 0; q < 3; ++q) {
+      const double tot = block_sum_d(v[q], sbuf);
+      if (threadIdx.x == 0) atomicAdd(&st[e.z].acc2[q], tot);
+    }
   }
-  y[(size_t)i * 12 + a] = sum;
 }
 
+// d = the solution of an active shell, 0 elsewhere
 __global__ void k_dir(int m, const int* __restrict__ nshell, const ShellState* st,
-                      const float* __restrict__ x32, const double* __restrict__ g,
-                      double* __restrict__ d, double* __restrict__ rhs, int mode) {
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < m; k += gridDim.x * blockDim.x) {
-    if (mode == 0) rhs[k] = -g[k];
-    else d[k] = st[nshell[k / 12]].active ? (double)x32[k] : 0.0;
-  }
+                      const float* __restrict__ x32, double* __restrict__ d) {
+  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < m; k += gridDim.x * blockDim.x)
+    d[k] = st[nshell[k / 12]].active ? (double)x32[k] : 0.0;
 }
 
 __global__ void k_update(int m, const int* __restrict__ nshell, const ShellState* st,
@@ -1011,9 +1065,15 @@ struct shell_batch_s {
   double *dxi = nullptr, *t64 = nullptr, *rest = nullptr, *restgp = nullptr, *mass = nullptr, *fgrav = nullptr;
   float *t32 = nullptr, *val = nullptr, *Dinv = nullptr;
   float *x32 = nullptr, *r32 = nullptr, *z32 = nullptr, *p32 = nullptr, *Ap32 = nullptr;
-  double *qn = nullptr, *y = nullptr, *g = nullptr, *gin = nullptr, *d = nullptr, *Md = nullptr;
-  double *rhs = nullptr, *Ep = nullptr, *qwork = nullptr, *vwork = nullptr, *qfix = nullptr, *warm = nullptr;
+  double *qn = nullptr, *y = nullptr, *g = nullptr, *gin = nullptr, *d = nullptr;
+  double *Ep = nullptr, *qwork = nullptr, *vwork = nullptr, *qfix = nullptr, *warm = nullptr;
   unsigned char* mask = nullptr;
+  // work lists of the active shells and of those whose PCG runs, the tickets of the PCG kernels (all
+  // in one allocation), and the resident CTAs of the row kernels
+  void* lists = nullptr;
+  WorkList active{}, running{};
+  unsigned* tickets = nullptr;
+  int grid_spmv = 0, grid_update = 0, grid_rows = 0;
   int* err = nullptr;
   int* h_err = nullptr;
   long long launches = 0;
@@ -1049,7 +1109,7 @@ void bfree_all(shell_batch_s* b) {
   void* ptrs[] = {b->par, b->st, b->cnt, b->nshell, b->pshell, b->row_ptr, b->col, b->diag, b->pblocks,
                   b->plist_color, b->dmin_bits, b->pnodes, b->items, b->eg_items, b->color_items, b->dxi,
                   b->t64, b->rest, b->restgp, b->mass, b->fgrav, b->t32, b->val, b->Dinv, b->x32, b->r32,
-                  b->z32, b->p32, b->Ap32, b->qn, b->y, b->g, b->gin, b->d, b->Md, b->rhs, b->Ep,
+                  b->z32, b->p32, b->Ap32, b->qn, b->y, b->g, b->gin, b->d, b->Ep, b->lists,
                   b->qwork, b->vwork, b->qfix, b->warm, b->mask, b->err, b->loop, b->input};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -1111,9 +1171,46 @@ shell_status element_attr(int device) {
   return SHELL_OK;
 }
 
+// Rebuilds the list of active shells.
+shell_status list_active(shell_batch_s& b) {
+  k_compact<<<1, 1024, 0, b.stream>>>(b.S, b.st, b.par, b.active, 0, nullptr, nullptr, 0, cudaGraphConditionalHandle{}, 0);
+  BHEM_CUDA(cudaGetLastError());
+  BL(b);
+  return SHELL_OK;
+}
+
+// The work lists' memory (groups are at most one per kRowNodes / kGroupNodes nodes plus one per shell)
+// and the grids of the kernels that go through them.
+shell_status setup_lists(shell_batch_s& b) {
+  const size_t n8 = b.N / kRowNodes + b.S, n16 = b.N / kGroupNodes + b.S;
+  const size_t one = sizeof(int4) * (n8 + n16) + sizeof(int) * (((size_t)b.S + 3 + 3) & ~(size_t)3);
+  char* m = nullptr;
+  BHEM_TRY(balloc(&m, 2 * one + 4 * sizeof(unsigned)));
+  b.lists = m;
+  for (WorkList* l : {&b.active, &b.running}) {
+    l->g8 = (int4*)m;
+    l->g16 = l->g8 + n8;
+    l->shells = (int*)(l->g16 + n16);
+    l->counts = l->shells + b.S;
+    m += one;
+  }
+  b.tickets = (unsigned*)m;
+  BHEM_CUDA(cudaMemsetAsync(b.tickets, 0, 4 * sizeof(unsigned), b.stream));
+  int nsm = 0, o = 0;
+  BHEM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, b.device));
+  BHEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_spmv, kSpmvThreads, 0));
+  b.grid_spmv = (int)std::min<size_t>(n8, (size_t)std::max(1, o) * nsm);
+  BHEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_pcg_update, kNodeThreads, 0));
+  b.grid_update = (int)std::min<size_t>(n16, (size_t)std::max(1, o) * nsm);
+  b.grid_rows = (int)std::min<size_t>(n16, (size_t)8 * nsm);
+  return SHELL_OK;
+}
+
 // FP32 element Hessians of active shells assembled into the BSR (+ mass_scale M)
 shell_status assemble(shell_batch_s& b, const double* q, double mass_scale) {
-  BHEM_CUDA(cudaMemsetAsync(b.val, 0, sizeof(float) * 144 * (size_t)b.NB, b.stream));
+  k_zero_rows<<<b.grid_rows, 256, 0, b.stream>>>(b.active, b.row_ptr, b.val);
+  BHEM_CUDA(cudaGetLastError());
+  BL(b);
   BHEM_TRY(element_attr(b.device));
   int nsm = 0;
   BHEM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, b.device));
@@ -1210,7 +1307,7 @@ shell_status residual(shell_batch_s& b, const double* q, const shell_step_params
       b.dxi, b.pnodes, q, nullptr, b.restgp, b.Ep, b.g, 0, b.err);
   BHEM_CUDA(cudaGetLastError());
   BL(b);
-  k_grad_finish<<<blocks_for(b.N, 16), kNodeThreads, 0, b.stream>>>(b.N, b.nshell, b.st, b.row_ptr, b.col,
+  k_grad_finish<<<b.grid_rows, kNodeThreads, 0, b.stream>>>(b.active, b.st, b.row_ptr, b.col,
       b.mass, b.fgrav, q, b.y, 1.0 / (P.dt * P.dt), P.gravity[0], P.gravity[1], P.gravity[2], mask, b.g,
       b.gin, b.err);
   BHEM_CUDA(cudaGetLastError());
@@ -1223,18 +1320,25 @@ shell_status residual(shell_batch_s& b, const double* q, const shell_step_params
   return read_counters(b);
 }
 
-constexpr int kPcgKernels = 4;   // per PCG iteration: SpMV (with the p-update), alpha, update, beta
+constexpr int kPcgKernels = 2;   // per PCG iteration: SpMV (with the p-update and alpha), update (with beta)
 
 shell_status pcg_chunk(shell_batch_s& b, const unsigned char* mask, int iters) {
   for (int k = 0; k < iters; ++k) {
-    k_spmv<<<blocks_for(b.N, kRowNodes), kSpmvThreads, 0, b.stream>>>(b.N, b.nshell, b.st, b.row_ptr, b.col,
-                                                                        b.val, b.z32, mask, b.p32, b.Ap32);
-    k_ctrl_alpha<<<blocks_for(b.S, 128), 128, 0, b.stream>>>(b.S, b.st);
-    k_pcg_update<<<blocks_for(b.N, 16), kNodeThreads, 0, b.stream>>>(b.N, b.nshell, b.st, b.x32, b.r32, b.z32,
-                                                                      b.p32, b.Ap32, b.Dinv, mask);
-    k_ctrl_beta<<<blocks_for(b.S, 128), 128, 0, b.stream>>>(b.S, b.st);
+    k_spmv<<<b.grid_spmv, kSpmvThreads, 0, b.stream>>>(b.running, b.st, b.row_ptr, b.col, b.val, b.z32, mask, b.p32,
+                                                       b.Ap32, b.tickets);
+    k_pcg_update<<<b.grid_update, kNodeThreads, 0, b.stream>>>(b.running, b.st, b.x32, b.r32, b.z32, b.p32, b.Ap32,
+                                                               b.Dinv, mask, b.tickets + 1);
   }
   BHEM_CUDA(cudaGetLastError());
+  return SHELL_OK;
+}
+
+// The shells whose PCG runs to the running list and cnt->n_running; cond, h: the PCG loop's condition
+// (captured form).
+shell_status list_running(shell_batch_s& b, int limit, cudaGraphConditionalHandle h, int cond) {
+  k_compact<<<1, 1024, 0, b.stream>>>(b.S, b.st, b.par, b.running, 1, b.cnt, b.loop, limit, h, cond);
+  BHEM_CUDA(cudaGetLastError());
+  BL(b);
   return SHELL_OK;
 }
 
@@ -1261,12 +1365,9 @@ shell_status pcg_chunk_graph(shell_batch_s& b, const unsigned char* mask, int it
 }
 
 shell_status solve_directions(shell_batch_s& b, const shell_step_params& P, const unsigned char* mask) {
-  // rhs = -g; regulariser scale and first admissible level per shell
-  k_dir<<<vblocks(b.M), 256, 0, b.stream>>>(b.M, b.nshell, b.st, b.x32, b.g, b.d, b.rhs, 0);
-  BL(b);
+  // regulariser scale and first admissible level per shell
   BHEM_CUDA(cudaMemsetAsync(b.dmin_bits, 0x7f, sizeof(int) * 4 * (size_t)b.S, b.stream));
-  k_diag_stats<<<blocks_for(b.N, 16), kNodeThreads, 0, b.stream>>>(b.N, b.nshell, b.st, b.diag, b.val, mask,
-                                                                     b.dmin_bits);
+  k_diag_stats<<<b.grid_rows, kNodeThreads, 0, b.stream>>>(b.active, b.st, b.diag, b.val, mask, b.dmin_bits);
   BL(b);
   k_ctrl_reg_init<<<blocks_for(b.S, 128), 128, 0, b.stream>>>(b.S, b.st, b.dmin_bits);
   BL(b);
@@ -1274,15 +1375,13 @@ shell_status solve_directions(shell_batch_s& b, const shell_step_params& P, cons
   BL(b);
   int only_restart = 0;
   for (int round = 0; round < 16; ++round) {
-    k_precond<<<blocks_for(b.N, 16), 192, 0, b.stream>>>(b.N, b.nshell, b.st, b.diag, b.val, mask, b.Dinv,
-                                                          only_restart);
-    k_pcg_init<<<blocks_for(b.N, 16), kNodeThreads, 0, b.stream>>>(b.N, b.nshell, b.st, b.rhs, b.Dinv, mask,
-                                                                    b.x32, b.r32, b.z32, b.p32, only_restart);
-    BHEM_TRY(zero_counters(b));
-    k_ctrl_pcg_start<<<blocks_for(b.S, 128), 128, 0, b.stream>>>(b.S, b.st, b.cnt, only_restart, P.pcg_rtol,
-                                                                 P.pcg_max, P.pcg_fixed_iters);
+    k_precond<<<b.grid_rows, 192, 0, b.stream>>>(b.active, b.st, b.diag, b.val, mask, b.Dinv, only_restart);
+    k_pcg_init<<<b.grid_rows, kNodeThreads, 0, b.stream>>>(b.active, b.st, b.g, b.Dinv, mask, b.x32, b.r32, b.z32,
+                                                           only_restart);
+    k_ctrl_pcg_start<<<blocks_for(b.S, 128), 128, 0, b.stream>>>(b.S, b.st, only_restart, P.pcg_rtol, P.pcg_max,
+                                                                 P.pcg_fixed_iters);
     b.launches += 3;
-    BHEM_CUDA(cudaGetLastError());
+    BHEM_TRY(list_running(b, 0, cudaGraphConditionalHandle{}, 0));
     BHEM_TRY(read_counters(b));
     int chunk = 4;
     const int limit = P.pcg_fixed_iters > 0 ? P.pcg_fixed_iters : P.pcg_max;
@@ -1292,9 +1391,7 @@ shell_status solve_directions(shell_batch_s& b, const shell_step_params& P, cons
       BHEM_TRY(pcg_chunk_graph(b, mask, c));
       done_iters += c;
       chunk = std::min(chunk * 2, 32);
-      BHEM_TRY(zero_counters(b));
-      k_ctrl_count_running<<<blocks_for(b.S, 128), 128, 0, b.stream>>>(b.S, b.st, b.cnt);
-      BL(b);
+      BHEM_TRY(list_running(b, 0, cudaGraphConditionalHandle{}, 0));
       BHEM_TRY(read_counters(b));
     }
     // negative curvature: move those shells up the regulariser ladder and restart them
@@ -1305,18 +1402,17 @@ shell_status solve_directions(shell_batch_s& b, const shell_step_params& P, cons
     if (b.h_cnt->n_restart == 0) break;
     only_restart = 1;
   }
-  k_dir<<<vblocks(b.M), 256, 0, b.stream>>>(b.M, b.nshell, b.st, b.x32, b.g, b.d, b.rhs, 1);
+  k_dir<<<vblocks(b.M), 256, 0, b.stream>>>(b.M, b.nshell, b.st, b.x32, b.d);
   BL(b);
   BHEM_CUDA(cudaGetLastError());
   return SHELL_OK;
 }
 
 shell_status line_search(shell_batch_s& b, const shell_step_params& P, const double* q) {
-  k_mass_mult<<<blocks_for(b.N, 16), kNodeThreads, 0, b.stream>>>(b.N, b.row_ptr, b.col, b.mass, b.d, b.Md);
-  k_dots3<<<blocks_for(b.N, 16), kNodeThreads, 0, b.stream>>>(b.N, b.nshell, b.st, b.d, b.Md, b.gin, b.g);
+  k_mass_dots<<<b.grid_rows, kNodeThreads, 0, b.stream>>>(b.active, b.st, b.row_ptr, b.col, b.mass, b.d, b.gin, b.g);
   BHEM_TRY(zero_counters(b));
   k_ctrl_ls_start<<<blocks_for(b.S, 128), 128, 0, b.stream>>>(b.S, b.st, b.cnt, 1.0 / (P.dt * P.dt));
-  b.launches += 3;
+  b.launches += 2;
   BHEM_CUDA(cudaGetLastError());
   BHEM_TRY(read_counters(b));
   int nsm = 0;
@@ -1392,7 +1488,7 @@ shell_status enqueue_residual(shell_batch_s& b, const double* q, const shell_ste
   BHEM_CUDA(cudaMemsetAsync(b.g, 0, sizeof(double) * b.M, b.stream));
   k_eg64<<<std::min(b.n_eg_items, nsm * 16), 128, 0, b.stream>>>(b.n_eg_items, b.eg_items, b.P, b.par, b.st,
       b.dxi, b.pnodes, q, nullptr, b.restgp, b.Ep, b.g, 0, b.err);
-  k_grad_finish<<<blocks_for(b.N, 16), kNodeThreads, 0, b.stream>>>(b.N, b.nshell, b.st, b.row_ptr, b.col,
+  k_grad_finish<<<b.grid_rows, kNodeThreads, 0, b.stream>>>(b.active, b.st, b.row_ptr, b.col,
       b.mass, b.fgrav, q, b.y, 1.0 / (P.dt * P.dt), P.gravity[0], P.gravity[1], P.gravity[2], mask, b.g,
       b.gin, b.err);
   BHEM_TRY(zero_counters(b));
@@ -1407,14 +1503,13 @@ shell_status enqueue_residual(shell_batch_s& b, const double* q, const shell_ste
 shell_status enqueue_newton_body(shell_batch_s& b, const shell_step_params& P, const unsigned char* mask,
                                  double* dq, int nsm, cudaGraphConditionalHandle h_newton) {
   const long long l0 = b.launches;
+  BHEM_TRY(list_active(b));
   BHEM_TRY(assemble(b, dq, 1.0 / (P.dt * P.dt)));
-  k_dir<<<vblocks(b.M), 256, 0, b.stream>>>(b.M, b.nshell, b.st, b.x32, b.g, b.d, b.rhs, 0);
   BHEM_CUDA(cudaMemsetAsync(b.dmin_bits, 0x7f, sizeof(int) * 4 * (size_t)b.S, b.stream));
-  k_diag_stats<<<blocks_for(b.N, 16), kNodeThreads, 0, b.stream>>>(b.N, b.nshell, b.st, b.diag, b.val, mask,
-                                                                     b.dmin_bits);
+  k_diag_stats<<<b.grid_rows, kNodeThreads, 0, b.stream>>>(b.active, b.st, b.diag, b.val, mask, b.dmin_bits);
   k_ctrl_reg_init<<<blocks_for(b.S, 128), 128, 0, b.stream>>>(b.S, b.st, b.dmin_bits);
   k_fix_diag<<<vblocks(b.M), 256, 0, b.stream>>>(b.M, b.nshell, b.st, b.diag, b.val, mask);
-  b.launches += 4;
+  b.launches += 3;
   cudaGraphConditionalHandle h_reg;
   BHEM_TRY(cap_handle(b.stream, &h_reg));
   k_cond_reg<<<1, 1, 0, b.stream>>>(b.cnt, b.loop, h_reg, 1);
@@ -1424,28 +1519,21 @@ shell_status enqueue_newton_body(shell_batch_s& b, const shell_step_params& P, c
   const int limit = P.pcg_fixed_iters > 0 ? P.pcg_fixed_iters : P.pcg_max;
   BHEM_TRY(cap_body(b, 2, reg_body, [&]() -> shell_status {
     const long long r0 = b.launches;
-    k_precond<<<blocks_for(b.N, 16), 192, 0, b.stream>>>(b.N, b.nshell, b.st, b.diag, b.val, mask, b.Dinv, 1);
-    k_pcg_init<<<blocks_for(b.N, 16), kNodeThreads, 0, b.stream>>>(b.N, b.nshell, b.st, b.rhs, b.Dinv, mask,
-                                                                    b.x32, b.r32, b.z32, b.p32, 1);
-    BHEM_TRY(zero_counters(b));
-    k_ctrl_pcg_start<<<blocks_for(b.S, 128), 128, 0, b.stream>>>(b.S, b.st, b.cnt, 1, P.pcg_rtol, P.pcg_max,
+    k_precond<<<b.grid_rows, 192, 0, b.stream>>>(b.active, b.st, b.diag, b.val, mask, b.Dinv, 1);
+    k_pcg_init<<<b.grid_rows, kNodeThreads, 0, b.stream>>>(b.active, b.st, b.g, b.Dinv, mask, b.x32, b.r32, b.z32, 1);
+    k_ctrl_pcg_start<<<blocks_for(b.S, 128), 128, 0, b.stream>>>(b.S, b.st, 1, P.pcg_rtol, P.pcg_max,
                                                                  P.pcg_fixed_iters);
     b.launches += 3;
     cudaGraphConditionalHandle h_pcg;
     BHEM_TRY(cap_handle(b.stream, &h_pcg));
-    k_cond_pcg<<<1, 1, 0, b.stream>>>(b.cnt, b.loop, limit, h_pcg, 1);
-    BL(b);
+    BHEM_TRY(list_running(b, limit, h_pcg, 1));
     cudaGraph_t pcg_body = nullptr;
     BHEM_TRY(cap_while(b.stream, h_pcg, &pcg_body));
     BHEM_TRY(cap_body(b, 3, pcg_body, [&]() -> shell_status {
       const long long p0 = b.launches;
       BHEM_TRY(pcg_chunk(b, mask, kGraphPcgChunk));
       b.launches += (long long)kPcgKernels * kGraphPcgChunk;
-      BHEM_TRY(zero_counters(b));
-      k_ctrl_count_running<<<blocks_for(b.S, 128), 128, 0, b.stream>>>(b.S, b.st, b.cnt);
-      k_cond_pcg<<<1, 1, 0, b.stream>>>(b.cnt, b.loop, limit, h_pcg, 0);
-      b.launches += 2;
-      BHEM_CUDA(cudaGetLastError());
+      BHEM_TRY(list_running(b, limit, h_pcg, 2));
       b.k_pcg = b.launches - p0;
       return SHELL_OK;
     }));
@@ -1457,13 +1545,12 @@ shell_status enqueue_newton_body(shell_batch_s& b, const shell_step_params& P, c
     b.k_reg = (b.launches - r0) - b.k_pcg;
     return SHELL_OK;
   }));
-  k_dir<<<vblocks(b.M), 256, 0, b.stream>>>(b.M, b.nshell, b.st, b.x32, b.g, b.d, b.rhs, 1);
+  k_dir<<<vblocks(b.M), 256, 0, b.stream>>>(b.M, b.nshell, b.st, b.x32, b.d);
   // line search
-  k_mass_mult<<<blocks_for(b.N, 16), kNodeThreads, 0, b.stream>>>(b.N, b.row_ptr, b.col, b.mass, b.d, b.Md);
-  k_dots3<<<blocks_for(b.N, 16), kNodeThreads, 0, b.stream>>>(b.N, b.nshell, b.st, b.d, b.Md, b.gin, b.g);
+  k_mass_dots<<<b.grid_rows, kNodeThreads, 0, b.stream>>>(b.active, b.st, b.row_ptr, b.col, b.mass, b.d, b.gin, b.g);
   BHEM_TRY(zero_counters(b));
   k_ctrl_ls_start<<<blocks_for(b.S, 128), 128, 0, b.stream>>>(b.S, b.st, b.cnt, 1.0 / (P.dt * P.dt));
-  b.launches += 4;
+  b.launches += 3;
   cudaGraphConditionalHandle h_ls;
   BHEM_TRY(cap_handle(b.stream, &h_ls));
   k_cond_ls<<<1, 1, 0, b.stream>>>(b.cnt, b.loop, h_ls, 1);
@@ -1526,6 +1613,7 @@ shell_status step_graph(shell_batch_s& b, const shell_step_params& P, const unsi
     k_predict<<<vblocks(b.M), 256, 0, b.stream>>>(b.M, dq, dv, P.dt, b.qn, b.y);
     k_fix<<<vblocks(b.M), 256, 0, b.stream>>>(b.M, dq, b.qn, mask, qfix);
     b.launches += 3;
+    BHEM_TRY(list_active(b));
     BHEM_TRY(enqueue_residual(b, dq, P, mask, 1, nsm));
     if (warm) {
       k_fix<<<vblocks(b.M), 256, 0, b.stream>>>(b.M, dq, warm, mask, qfix);
@@ -1701,7 +1789,7 @@ extern "C" shell_status shell_batch_create(int n_shells, const shell_grid* grids
   BA(b->t32, S * kPhiTable); BA(b->rest, M); BA(b->restgp, 13 * P * 16); BA(b->mass, NB * 16);
   BA(b->fgrav, N * 4); BA(b->val, NB * 144); BA(b->Dinv, N * 144); BA(b->x32, M); BA(b->r32, M);
   BA(b->z32, M); BA(b->p32, M); BA(b->Ap32, M); BA(b->qn, M); BA(b->y, M); BA(b->g, M); BA(b->gin, M);
-  BA(b->d, M); BA(b->Md, M); BA(b->rhs, M); BA(b->Ep, P); BA(b->qwork, M); BA(b->vwork, M);
+  BA(b->d, M); BA(b->Ep, P); BA(b->qwork, M); BA(b->vwork, M);
   BA(b->qfix, M); BA(b->warm, M); BA(b->mask, M); BA(b->err, 1);
 #undef BA
   if (st == SHELL_OK) {
@@ -1740,6 +1828,7 @@ extern "C" shell_status shell_batch_create(int n_shells, const shell_grid* grids
     return fail(SHELL_ERR_CUDA, std::string("batch upload: ") + cudaGetErrorString(e));
   }
   st = upload_items(*b, b->ppi);
+  if (st == SHELL_OK) st = setup_lists(*b);
   if (st == SHELL_OK) {
     k_tables<<<n_shells, 256, 0, b->stream>>>(n_shells, b->dxi, b->t64, b->t32);
     k_rest<<<blocks_for((long long)P * 16, 256), 256, 0, b->stream>>>(b->P, b->pshell, b->par, b->pnodes, b->rest,
@@ -1787,6 +1876,7 @@ extern "C" shell_status shell_batch_autotune(shell_batch_t* batch, const double*
   // every shell active for the trial assemblies
   k_begin_step<<<blocks_for(b.S, 128), 128, 0, b.stream>>>(b.S, b.st, nullptr);
   BL(b);
+  BHEM_TRY(list_active(b));
   const int ppis[4] = {4, 8, 16, 32};
   const int schemes[2] = {SHELL_ASM_ATOMIC, SHELL_ASM_COLOR};
   cudaEvent_t e0, e1;
@@ -1871,7 +1961,7 @@ extern "C" shell_status shell_batch_newton_step(shell_batch_t* batch, const shel
     k_predict<<<vblocks(b.M), 256, 0, b.stream>>>(b.M, dq, dv, P.dt, b.qn, b.y);
     k_fix<<<vblocks(b.M), 256, 0, b.stream>>>(b.M, dq, b.qn, mask, qfix);
     b.launches += 3;
-    BHEM_CUDA(cudaGetLastError());
+    BHEM_TRY(list_active(b));
     BHEM_TRY(residual(b, dq, P, mask, 1));
     if (warm) {
       k_fix<<<vblocks(b.M), 256, 0, b.stream>>>(b.M, dq, warm, mask, qfix);
@@ -1879,6 +1969,7 @@ extern "C" shell_status shell_batch_newton_step(shell_batch_t* batch, const shel
       BHEM_TRY(residual(b, dq, P, mask, 0));
     }
     for (int it = 0; it <= P.newton_max && b.h_cnt->n_active > 0; ++it) {
+      BHEM_TRY(list_active(b));
       BHEM_TRY(assemble(b, dq, 1.0 / (P.dt * P.dt)));
       BHEM_TRY(solve_directions(b, P, mask));
       BHEM_TRY(line_search(b, P, dq));
