@@ -251,15 +251,14 @@ SHELL_API shell_status shell_newton_step(shell_t* shell, const shell_step_params
    memory belongs entirely to their own pool allocator (cudaMalloc would fail or escape its
    accounting), latency-bound loops that cannot afford the device-wide synchronisation a
    cudaMalloc/cudaFree may cause, and plug-ins that receive a fixed memory budget from their
-   host. No shell object is needed: the patch topology comes from grid, the shape table and the
-   rest geometry are computed from rest_dofs on every call.
+   host. No shell object is needed: the patch topology comes from grid, the shape factors and the
+   rest geometry are computed from grid and rest_dofs on every call.
    Arguments: grid, material (host); rest_dofs, q: device [n_nodes * 12] FP64 (caller-owned,
    read only); energy: device, 1 double (overwritten); grad: device [n_nodes * 12] FP64 or NULL
    (overwritten); stream: cudaStream_t or NULL. Asynchronous: enqueues a memset of the ticket
-   (and of grad) and two kernels on stream, calls no cudaMalloc, cudaFree or allocating library
+   (and of grad) and one kernel on stream, calls no cudaMalloc, cudaFree or allocating library
    routine.
-   Scratch: one file-scope device array of about 141 KB (per-CTA energy sums, the shape table and
-   a counter), present on every GPU that loads the library until the process exits. Grids of
+   Scratch: one file-scope device array of about 131 KB (per-CTA energy sums and a counter), present on every GPU that loads the library until the process exits. Grids of
    more than 131072 patches are rejected with SHELL_ERR_ARG. The first call on a device looks up
    the array's device address (cudaGetSymbolAddress) with that device current; make that first
    call before any stream capture. The address is kept for the life of the process: after

@@ -67,3 +67,33 @@ def test_noalloc_rejects_grids_beyond_its_scratch():
     with pytest.raises(ShellError) as e:
         energy_grad_noalloc(g, S.SHEET_MATERIAL, x, x, x[:1], None)
     assert e.value.status == 1 and "131072" in str(e.value)
+
+
+# one warp per CTA up to 608 patches, four beyond, and a loop over patches from 65536 on
+FORMS = {
+    "1x1": lambda: S.sheet_noisy(1, 1e-3, 2),
+    "annulus2x3-periodic": lambda: (lambda g, r: (g, r, S.noisy(r, 1e-2, 4)))(*S.annulus(2, 3)),
+    "608": lambda: (lambda g, r: (g, r, S.noisy(r, 1e-3, 5)))(*S.flat_sheet(32, 19)),
+    "609": lambda: (lambda g, r: (g, r, S.noisy(r, 1e-3, 6)))(*S.annulus(29, 21)),
+    "66049-loop": lambda: S.sheet_sinusoid(257, 3),
+}
+
+
+@pytest.mark.parametrize("case", list(FORMS))
+def test_noalloc_launch_forms(case):
+    """Both CTA forms at the size where they meet, their remainders and the loop over patches, with and
+    without the gradient; same bound as above (FP64 on both entry points)."""
+    from paper_2312_14839_gb300.bhem import Shell, energy_grad_noalloc
+    g, rest, q = FORMS[case]()
+    mat = S.SHEET_MATERIAL
+    rest_d, q_d = _dev(rest), _dev(q)
+    with Shell(g, mat, rest_d, precision="fp64") as sh:
+        E_ref, G_ref = sh.energy_grad_hess(q_d, want_hessian=False)
+    E, E1 = (torch.full((1,), float("nan"), dtype=torch.float64, device="cuda") for _ in range(2))
+    G = torch.full_like(q_d, float("nan"))
+    energy_grad_noalloc(g, mat, rest_d, q_d, E, G)
+    energy_grad_noalloc(g, mat, rest_d, q_d, E1)
+    torch.cuda.synchronize()
+    assert float(E) == float(E1)
+    assert abs(float(E - E_ref)) <= TOL * abs(float(E_ref))
+    assert _rel(G, G_ref) <= TOL
