@@ -499,8 +499,8 @@ def network_timing(net, X_all, T_all, n_sheet=64, reps=20):
         out["warm_start_64x64"] = entry(timed(lambda: net.warm_start(sh, q, v, 1e-3, w)),
                                         2 * g.n_nodes * MLP_MAC_PER_ROW)
     out["peak_source"] = "measured bf16_tflops (MEASURED_PEAKS.json), cuBLAS 8192^3 burst"
-    out["kernels"] = ("k_gemm_tc (tcgen05.mma kind::f16 into TMEM, TMA 128-byte-swizzled operands), "
-                      "k_mlp_warm (fused warm start, same MMA sequence)")
+    out["kernels"] = ("k_mlp_rows (all layers of 128 rows in one CTA: tcgen05.mma kind::f16 into TMEM, weights by TMA), "
+                      "k_gemm_split (weight gradients, split K)")
     return out
 
 

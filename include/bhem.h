@@ -337,7 +337,8 @@ SHELL_API shell_status shell_batch_newton_step(shell_batch_t* batch, const shell
 typedef struct shell_mlp_s shell_mlp_t;
 
 /* Creates a network with zero parameters for batches of up to max_rows rows (1 .. 2^24) of
-   features; stream: cudaStream_t or NULL. Device memory: about 12.7 KB per row plus 2.9 MB.
+   features; stream: cudaStream_t or NULL. Device memory: about 6.2 KB per row plus 2.9 MB;
+   0.6 MB of pinned host memory.
    Fails with SHELL_ERR_CUDA when the driver cannot encode the network's TMA tensor maps. */
 SHELL_API shell_status shell_mlp_create(int max_rows, void* stream, shell_mlp_t** out);
 SHELL_API shell_status shell_mlp_destroy(shell_mlp_t* mlp);

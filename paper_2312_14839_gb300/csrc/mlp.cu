@@ -1,8 +1,12 @@
 // Learned Newton warm start: a per-node MLP 28 -> 256 -> 256 -> 256 -> 12 with GELU, BF16 weights
 // and activations, FP32 accumulation on the tensor cores (tcgen05.mma kind::f16 with TMEM
-// accumulators, operands staged by TMA; tc_gemm.cuh), trained with an MSE loss and Adam by the
+// accumulators, operands staged by TMA; tc_gemm.cuh, gemm_split.cuh), trained with an MSE loss and Adam by the
 // kernels of this file. The paper has no learning component; the implicit-Euler Newton solve of
 // Sec. 6.1 stays the judge of every step.
+//
+// One kernel (k_mlp_rows) takes 128 rows through all layers without leaving the SM, for the warm start, for
+// inference and, with the loss and the back-propagation, for training; a second one (k_gemm_split) forms
+// every weight gradient.
 //
 // Node features (28, FP32): the node's 12 DOFs relative to rest (u = q - q_rest), its 12 velocity
 // DOFs, and 4 means over its present edge neighbours: of u_nb - u_i for the position DOFs (a
@@ -18,7 +22,7 @@
 #include <vector>
 
 #include "common.cuh"
-#include "tc_gemm.cuh"
+#include "gemm_split.cuh"
 
 namespace bhem {
 namespace mlp {
@@ -39,143 +43,11 @@ __device__ __forceinline__ float gelu_grad(float x) {
   return 0.5f * (1.f + erff(x * 0.70710678118654752f)) + x * 0.39894228040143268f * expf(-0.5f * x * x);
 }
 
-// ------------------------------------------------------------------------------------------
-// Epilogues of the tensor-core GEMM (tc_gemm.cuh): per row and 16 accumulator columns, the values
-// of the FP32 output channel (f) and of the BF16 channels (b: row-major and transposed). A
-// transposed BF16 copy ([column][row], row stride ldt) is what the weight-gradient GEMMs read as
-// their K-contiguous operands.
-// ------------------------------------------------------------------------------------------
 constexpr int kErrIndex = 1, kErrTimeout = 2;   // bits of the network's error word
-
-// forward layer: Z = acc + bias (FP32 pre-activation; bias = the per-column vector) and, for a
-// hidden layer, GELU(Z) for the BF16 channels
-struct EpiForward {
-  int hidden;
-  __device__ void operator()(int, int, const float* bias, const float (&acc)[16], float (&f)[16],
-                             float (&b)[16]) const {
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      f[j] = acc[j] + bias[j];
-      b[j] = hidden ? gelu(f[j]) : f[j];
-    }
-  }
-};
-
-// split-K weight gradient: the FP32 channel adds acc into the zeroed gradient
-struct EpiAtomic {
-  __device__ void operator()(int, int, const float*, const float (&acc)[16], float (&f)[16], float (&b)[16]) const {
-#pragma unroll
-    for (int j = 0; j < 16; ++j) f[j] = b[j] = acc[j];
-  }
-};
-
-// back-propagation through a hidden layer: dZ = (dZ_next W) * GELU'(Z), for all three channels
-struct EpiGeluBack {
-  const float* Z;
-  int ld;
-  int rows;
-  __device__ void operator()(int row, int col0, const float*, const float (&acc)[16], float (&f)[16],
-                             float (&b)[16]) const {
-    if (row >= rows) {
-#pragma unroll
-      for (int j = 0; j < 16; ++j) f[j] = b[j] = 0.f;
-      return;
-    }
-    const float4* zp = reinterpret_cast<const float4*>(Z + (long long)row * ld + col0);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float4 z4 = zp[q];
-      f[4 * q] = acc[4 * q] * gelu_grad(z4.x);
-      f[4 * q + 1] = acc[4 * q + 1] * gelu_grad(z4.y);
-      f[4 * q + 2] = acc[4 * q + 2] * gelu_grad(z4.z);
-      f[4 * q + 3] = acc[4 * q + 3] * gelu_grad(z4.w);
-    }
-#pragma unroll
-    for (int j = 0; j < 16; ++j) b[j] = f[j];
-  }
-};
 
 // ------------------------------------------------------------------------------------------
 // Element-wise kernels
 // ------------------------------------------------------------------------------------------
-// normalised BF16 input rows (gathered through idx when given), and their transpose XbT
-// ([32][ldt]) when given; an index outside [0, data_rows) gives a zero row and raises the error flag
-__global__ void k_input(int rows, const float* __restrict__ X, long long data_rows, const int* __restrict__ idx,
-                        const float* __restrict__ norm, bf16* __restrict__ Xb, bf16* __restrict__ XbT,
-                        long long ldt, int* err) {
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < rows * kInPad; e += gridDim.x * blockDim.x) {
-    const int r = e / kInPad, c = e % kInPad;
-    float v = 0.f;
-    const long long src = idx ? (long long)idx[r] : r;
-    if (src < 0 || src >= data_rows) {
-      if (c == 0) atomicOr(err, kErrIndex);
-    } else if (c < kIn) {
-      v = (X[src * kIn + c] - norm[kNormInMean + c]) * norm[kNormInIstd + c];
-    }
-    const bf16 b = __float2bfloat16(v);
-    Xb[e] = b;
-    if (XbT) XbT[c * ldt + r] = b;
-  }
-}
-
-// Y = Z * out_std + out_mean over the 12 output columns
-__global__ void k_output(int rows, const float* __restrict__ Z, const float* __restrict__ norm, float* __restrict__ Y) {
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < rows * kOut; e += gridDim.x * blockDim.x) {
-    const int r = e / kOut, c = e % kOut;
-    Y[e] = Z[(long long)r * kOutPad + c] * norm[kNormOutStd + c] + norm[kNormOutMean + c];
-  }
-}
-
-// MSE on normalised targets: loss = mean (Z - Tn)^2 over rows x 12; dZ = 2 (Z - Tn) / (rows x 12),
-// zero in the padded columns (FP32, BF16, and BF16 transposed [16][ldt])
-__global__ void k_loss(int rows, const float* __restrict__ Z, const float* __restrict__ T, long long data_rows,
-                       const int* __restrict__ idx, const float* __restrict__ norm, float* __restrict__ dZ,
-                       bf16* __restrict__ dZb, bf16* __restrict__ dZbT, long long ldt, double* loss) {
-  __shared__ double sbuf[32];
-  double part = 0.0;
-  const float scale = 2.f / (float)(rows * kOut);
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < rows * kOutPad; e += gridDim.x * blockDim.x) {
-    const int r = e / kOutPad, c = e % kOutPad;
-    const long long src = idx ? (long long)idx[r] : r;
-    float d = 0.f;
-    if (c < kOut && src >= 0 && src < data_rows) {
-      const float tn = (T[src * kOut + c] - norm[kNormOutMean + c]) * norm[kNormOutIstd + c];
-      const float diff = Z[e] - tn;
-      part += (double)diff * diff;
-      d = scale * diff;
-    }
-    dZ[e] = d;
-    dZb[e] = __float2bfloat16(d);
-    dZbT[c * ldt + r] = __float2bfloat16(d);
-  }
-  for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-  if ((threadIdx.x & 31) == 0) sbuf[threadIdx.x >> 5] = part;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += sbuf[w];
-    atomicAdd(loss, s / (double)(rows * kOut));
-  }
-}
-
-// db[n] += sum over rows of dZ[r][n]: CTA (x, y) takes columns 128 x .. 128 x + 127 of the
-// 64-row slab y, with eight independent partial sums per thread (eight loads in flight), then one
-// atomic per column
-constexpr int kColsumRows = 64;
-
-__global__ void k_colsum(int rows, int cols, const float* __restrict__ dZ, float* __restrict__ db) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= cols) return;
-  const int r0 = blockIdx.y * kColsumRows, r1 = min(rows, r0 + kColsumRows);
-  float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  int r = r0;
-  for (; r + 8 <= r1; r += 8)
-#pragma unroll
-    for (int j = 0; j < 8; ++j) acc[j] += dZ[(long long)(r + j) * cols + n];
-  for (; r < r1; ++r) acc[0] += dZ[(long long)r * cols + n];
-  atomicAdd(&db[n], ((acc[0] + acc[1]) + (acc[2] + acc[3])) + ((acc[4] + acc[5]) + (acc[6] + acc[7])));
-}
-
 // Adam (Kingma and Ba) on the FP32 master parameters of every tensor of the network in one launch,
 // refreshing a tensor's BF16 copy and its transpose (a [rows x cols] matrix stored [cols][rows])
 // where given. Padded entries see zero gradients and stay zero.
@@ -306,29 +178,55 @@ __global__ void k_compose(int n_nodes, const double* __restrict__ q, const doubl
 }
 
 // ------------------------------------------------------------------------------------------
-// Fused warm start: features -> normalised BF16 input -> 4 layers -> q + dt v + output, one
-// launch. A CTA takes 128 nodes (one per TMEM lane). The activations stay in shared memory as the
-// next layer's A operand (128-byte swizzled K-major tiles, written by the epilogue); each layer's
-// weights arrive by TMA into one shared buffer as soon as the previous layer's MMAs are done, and
-// one thread issues the layer's tcgen05.mma into a 128 x 256 FP32 TMEM accumulator. Every output
-// is accumulated over the same K chunks, in the same order and with the same MMA shapes as the
-// GEMM path (shell_mlp_forward), and finished by the same epilogue arithmetic, so the network
-// output equals that path's.
+// The rows kernel: 128 rows (one per TMEM lane) through the network in one CTA. The activations stay in
+// shared memory as the next product's A operand (128-byte swizzled K-major tiles, written by the
+// epilogue); each product's weights arrive by TMA into one shared buffer as soon as the previous product's
+// MMAs are done, and one thread issues the tcgen05.mma into a 128 x 256 FP32 TMEM accumulator.
+//   kWarm:  node features -> network -> q + dt v + output
+//   kInfer: rows of X -> de-normalised output
+//   kTrain: rows of X (through an index) -> loss, then back through the layers: dZ of every layer, transposed,
+//           and the transposed activations (the operands of the weight-gradient GEMMs), and the bias
+//           gradients (column sums of the FP32 dZ).
+// What bounds it: the epilogues, 64 accumulators a thread and product with an erff each (4 us a hidden layer
+// against 0.5 us of MMAs). So GELU' is formed beside GELU from the same erff, in the forward epilogue,
+// and waits in global memory (FP32, written and read by the same thread, 512 B per warp access) for the
+// back-propagation; its loads are issued before the wait for the product. One launch per product, with FP32
+// copies of every Z and dZ and a column-sum launch per layer, took 230 us for the gradients of 16,384
+// rows; this and k_gemm_split take 77 us.
 // ------------------------------------------------------------------------------------------
-constexpr int kWarmThreads = 512;                 // 16 warps: TMEM lane quarter w % 4, column part w / 4
+enum RowsMode { kWarm, kInfer, kTrain };
+constexpr int kRowThreads = 512;                  // 16 warps: TMEM lane quarter w % 4, column part w / 4
 constexpr int kActBytes = 4 * tc::kBM * 128;      // 4 K chunks of 128 rows x 128 bytes
 constexpr int kWgtBytes = 4 * kHid * 128;         // 4 K chunks of 256 rows x 128 bytes
-constexpr size_t kWarmSmem = (size_t)kActBytes + kWgtBytes + 1024;
+constexpr size_t kRowsSmem = (size_t)kActBytes + kWgtBytes + 1024;
+constexpr int kPhases = 2 * kLayers - 1;          // products of a training pass: 4 forward, 3 back
 
-struct WarmArgs {
-  int n_nodes, n1, n2, per_u, per_v;
-  const double* q;
-  const double* rest;
-  const double* v;
+// W[l] as [fan_out][fan_in] (forward) and its transpose (back, l >= 1), in boxes of 64 columns x all rows
+struct RowsMaps {
+  CUtensorMap w[kLayers], wt[kLayers];
+};
+
+struct RowsArgs {
+  int rows;
+  // kWarm
+  int n1, n2, per_u, per_v;
+  const double *q, *rest, *v;
   double dt;
+  double* warm;
+  // kInfer, kTrain
+  const float* X;
+  float* Y;
+  // kTrain
+  const float* T;
+  long long data_rows;
+  const int* idx;
+  double* loss;
+  long long ldt;
+  bf16 *XbT, *AbT[kLayers - 1], *dZbT[kLayers];
+  float4* G[kLayers - 1];   // GELU'(Z): [tile of 128 rows][64 groups of 4 columns][128 rows]
+  float* gb[kLayers];
   const float* bias[kLayers];
   const float* norm;
-  double* warm;
   int* err;
   unsigned polls;
 };
@@ -342,18 +240,45 @@ __device__ __forceinline__ uint4 pack_bf16x8(const float* x) {
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-__global__ void __launch_bounds__(kWarmThreads, 1)
-k_mlp_warm(const __grid_constant__ CUtensorMap tw0, const __grid_constant__ CUtensorMap tw1,
-           const __grid_constant__ CUtensorMap tw2, const __grid_constant__ CUtensorMap tw3, WarmArgs A) {
-  extern __shared__ unsigned char warm_smem_raw[];
+// 16 activations of a row (columns c0 .. c0 + 15) into the A tiles
+__device__ __forceinline__ void store_act16(unsigned char* act, int row, int c0, const float* a) {
+  unsigned char* rp = act + (c0 / tc::kBK) * (tc::kBM * 128) + row * 128;
+  const int p = (c0 % tc::kBK) / 8;
+  *reinterpret_cast<uint4*>(rp + ((p ^ (row & 7)) * 16)) = pack_bf16x8(a);
+  *reinterpret_cast<uint4*>(rp + (((p + 1) ^ (row & 7)) * 16)) = pack_bf16x8(a + 8);
+}
+
+// sum over the warp's 32 rows of column lane / 2 of t[16] (each exchange halves the columns a lane keeps)
+__device__ __forceinline__ float column_sum16(const float (&v)[16], int lane) {
+  float t[16];
+#pragma unroll
+  for (int j = 0; j < 16; ++j) t[j] = v[j];
+#pragma unroll
+  for (int o = 16, n = 8; n > 0; o >>= 1, n >>= 1) {
+    const bool hi = lane & o;
+#pragma unroll
+    for (int j = 0; j < n; ++j) {
+      const float send = hi ? t[j] : t[j + n], keep = hi ? t[j + n] : t[j];
+      t[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  return t[0] + __shfl_xor_sync(0xffffffffu, t[0], 1);
+}
+
+template <RowsMode MODE>
+__global__ void __launch_bounds__(kRowThreads, 1)
+k_mlp_rows(const __grid_constant__ RowsMaps maps, const __grid_constant__ RowsArgs A) {
+  extern __shared__ unsigned char rows_smem_raw[];
   __shared__ __align__(8) uint64_t bar_w, bar_mma;
   __shared__ uint32_t tmem_slot;
   __shared__ int s_abort;
+  __shared__ __align__(16) float s_bias[kLayers][kHid];
+  __shared__ float s_sum[MODE == kTrain ? 4 : 1][kHid];   // column sums per TMEM lane quarter
   volatile int* abort_flag = &s_abort;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const uint32_t raw = tc::smem_addr(warm_smem_raw);
+  const uint32_t raw = tc::smem_addr(rows_smem_raw);
   const uint32_t act = (raw + 1023u) & ~1023u, wgt = act + kActBytes;
-  unsigned char* act_g = warm_smem_raw + (act - raw);   // generic pointer to the activation tiles
+  unsigned char* act_g = rows_smem_raw + (act - raw);   // generic pointer to the activation tiles
   const uint32_t bw = tc::smem_addr(&bar_w), bm = tc::smem_addr(&bar_mma);
   const int r0 = blockIdx.x * tc::kBM;
   if (tid == 0) {
@@ -369,100 +294,222 @@ k_mlp_warm(const __grid_constant__ CUtensorMap tw0, const __grid_constant__ CUte
   const uint32_t tmem = tmem_slot;
   if (tid == 0) {   // layer-0 weights (K = 32: one 64-column chunk, the rest read as zeros)
     tc::mbar_arrive_expect_tx(bw, kHid * 128);
-    tc::tma_load_2d(wgt, &tw0, bw, 0, 0);
+    tc::tma_load_2d(wgt, &maps.w[0], bw, 0, 0);
   }
-  // layer-0 input rows (the arithmetic of k_node_features and k_input): K chunk 0, columns 32..63 zero
-  if (tid < tc::kBM) {
-    const int i = r0 + tid;
-    float f[kIn];
-    if (i < A.n_nodes) node_features_of(i, A.n1, A.n2, A.per_u, A.per_v, A.q, A.rest, A.v, f);
-    float x[kInPad];
+  for (int e = tid; e < kLayers * kHid; e += kRowThreads)
+    s_bias[e / kHid][e % kHid] = e % kHid < (e / kHid < kLayers - 1 ? kHid : kOutPad) ? A.bias[e / kHid][e % kHid] : 0.f;
+  // layer-0 input rows: K chunk 0, columns 32..63 zero
+  if (MODE == kWarm) {
+    if (tid < tc::kBM) {
+      const int i = r0 + tid;
+      float f[kIn];
+      if (i < A.rows) node_features_of(i, A.n1, A.n2, A.per_u, A.per_v, A.q, A.rest, A.v, f);
+      float x[kInPad];
 #pragma unroll
-    for (int c = 0; c < kInPad; ++c)
-      x[c] = (i < A.n_nodes && c < kIn) ? (f[c] - A.norm[kNormInMean + c]) * A.norm[kNormInIstd + c] : 0.f;
-    uint4* row = reinterpret_cast<uint4*>(act_g + tid * 128);
+      for (int c = 0; c < kInPad; ++c)
+        x[c] = (i < A.rows && c < kIn) ? (f[c] - A.norm[kNormInMean + c]) * A.norm[kNormInIstd + c] : 0.f;
+      uint4* row = reinterpret_cast<uint4*>(act_g + tid * 128);
 #pragma unroll
-    for (int p = 0; p < 8; ++p) row[p ^ (tid & 7)] = p < 4 ? pack_bf16x8(x + 8 * p) : make_uint4(0u, 0u, 0u, 0u);
+      for (int p = 0; p < 8; ++p) row[p ^ (tid & 7)] = p < 4 ? pack_bf16x8(x + 8 * p) : make_uint4(0u, 0u, 0u, 0u);
+    }
+  } else {
+    // four threads per row, 8 columns each; an index outside [0, data_rows) gives a zero row and raises the
+    // error flag
+    const int lr = tid & 127, part = tid >> 7, i = r0 + lr;
+    float x[8];
+    long long src = -1;
+    if (i < A.rows) {
+      src = MODE == kTrain && A.idx ? (long long)A.idx[i] : i;
+      if (MODE == kTrain && (src < 0 || src >= A.data_rows)) {
+        src = -1;
+        if (part == 0) atomicOr(A.err, kErrIndex);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int c = 8 * part + j;
+      x[j] = 0.f;
+      if (src >= 0 && c < kIn) x[j] = (A.X[src * kIn + c] - A.norm[kNormInMean + c]) * A.norm[kNormInIstd + c];
+    }
+    uint4* row = reinterpret_cast<uint4*>(act_g + lr * 128);
+    row[part ^ (lr & 7)] = pack_bf16x8(x);
+    row[(4 + part) ^ (lr & 7)] = make_uint4(0u, 0u, 0u, 0u);
+    if (MODE == kTrain && i < A.rows) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) A.XbT[(8 * part + j) * A.ldt + i] = __float2bfloat16(x[j]);
+    }
   }
   asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
   tc::tc_fence_before();
   __syncthreads();
   tc::tc_fence_after();
-  const int quarter = warp & 3, part = warp >> 2, row = quarter * 32 + lane;
+  const int quarter = warp & 3, part = warp >> 2, row = quarter * 32 + lane, i = r0 + row;
+  const bool valid = i < A.rows;
   const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16);
-  int w_inflight = 0;   // thread 0: the layer whose weight copy is in flight, or -1
-  int l = 0;
+  const int cpart = part * (kHid / 4);
+  constexpr int nph = MODE == kTrain ? kPhases : kLayers;
+  int w_inflight = 0;   // thread 0: the phase whose weight copy is in flight, or -1
+  int ph = 0;
 #pragma unroll 1
-  for (; l < kLayers; ++l) {
-    const int N = l < kLayers - 1 ? kHid : kOutPad;
-    const int nch = l == 0 ? 1 : kHid / tc::kBK;
+  for (; ph < nph; ++ph) {
+    // phase ph: layer ph forward, or layer lb = 2 kLayers - 1 - ph back (dZ_lb W_lb)
+    const int lb = 2 * kLayers - 1 - ph;
+    const int N = ph == kLayers - 1 ? kOutPad : kHid;
+    const int nch = ph == 0 || ph == kLayers ? 1 : kHid / tc::kBK;
+    float4 gp[MODE == kTrain ? kHid / 16 : 1];
+    float tn[MODE == kTrain ? kOut : 1];
+    bool has_target = false;
     if (tid == 0) {
-      if (!tc::mbar_wait_parity(bw, l & 1, A.polls)) {
+      if (!tc::mbar_wait_parity(bw, ph & 1, A.polls)) {
         *abort_flag = 1;
       } else {
         w_inflight = -1;
         tc::tc_fence_after();
         const uint32_t idesc = tc::idesc_bf16(tc::kBM, N);
+        const int steps = ph == kLayers ? kOutPad / 16 : tc::kBK / 16;
         for (int c = 0; c < nch; ++c)
-#pragma unroll
-          for (int j = 0; j < tc::kBK / 16; ++j)
+          for (int j = 0; j < steps; ++j)
             tc::mma_bf16_ss(tmem, tc::smem_desc_sw128(act + c * (tc::kBM * 128) + 32 * j),
                             tc::smem_desc_sw128(wgt + c * (N * 128) + 32 * j), idesc, c > 0 || j > 0);
       }
       tc::mma_commit(bm);
     }
-    if (!tc::mbar_wait_parity(bm, l & 1, A.polls)) *abort_flag = 1;
+    if (MODE == kTrain && ph >= kLayers) {
+      const float4* gsrc = A.G[lb - 1] + ((long long)blockIdx.x * (kHid / 4) + cpart / 4) * tc::kBM + row;
+#pragma unroll
+      for (int k = 0; k < kHid / 16; ++k) gp[k] = gsrc[k * tc::kBM];
+    }
+    if (MODE == kTrain && ph == kLayers - 1 && part == 0 && valid) {
+      const long long src = A.idx ? (long long)A.idx[i] : i;
+      has_target = src >= 0 && src < A.data_rows;
+#pragma unroll
+      for (int c = 0; c < kOut; ++c) tn[c] = has_target ? A.T[src * kOut + c] : 0.f;
+    }
+    if (!tc::mbar_wait_parity(bm, ph & 1, A.polls)) *abort_flag = 1;
     tc::tc_fence_after();
     __syncthreads();
     if (*abort_flag) break;
-    if (tid == 0 && l + 1 < kLayers) {   // the weight buffer is free: fetch the next layer's
-      const int N1 = l + 1 < kLayers - 1 ? kHid : kOutPad;
-      const CUtensorMap* m = l == 0 ? &tw1 : (l == 1 ? &tw2 : &tw3);
-      tc::mbar_arrive_expect_tx(bw, (kHid / tc::kBK) * N1 * 128);
-      for (int c = 0; c < kHid / tc::kBK; ++c) tc::tma_load_2d(wgt + c * N1 * 128, m, bw, c * tc::kBK, 0);
-      w_inflight = l + 1;
+    if (tid == 0 && ph + 1 < nph) {   // the weight buffer is free: fetch the next phase's
+      const int N1 = ph + 1 == kLayers - 1 ? kOutPad : kHid;
+      const int ch1 = ph + 1 == kLayers ? 1 : kHid / tc::kBK;
+      const CUtensorMap* m = ph + 1 < kLayers ? &maps.w[ph + 1] : &maps.wt[lb - 1];
+      tc::mbar_arrive_expect_tx(bw, ch1 * N1 * 128);
+      for (int c = 0; c < ch1; ++c) tc::tma_load_2d(wgt + c * N1 * 128, m, bw, c * tc::kBK, 0);
+      w_inflight = ph + 1;
     }
-    const float* bias = A.bias[l];
-    if (l < kLayers - 1) {
-      // epilogue of a hidden layer (the arithmetic of EpiForward): GELU(acc + bias) in BF16,
-      // written over the activations as the next layer's A tiles
+    if (ph < kLayers - 1) {
+      // hidden layer: GELU(acc + bias) in BF16 over the activations as the next product's A tiles
 #pragma unroll 1
-      for (int c0 = part * (kHid / 4); c0 < (part + 1) * (kHid / 4); c0 += 16) {
+      for (int c0 = cpart; c0 < cpart + kHid / 4; c0 += 16) {
+        float v[16], a[16];
+        tc::tmem_ld16(lane_addr + (uint32_t)c0, v);
+#pragma unroll
+        for (int j4 = 0; j4 < 4; ++j4) {
+          const float4 b4 = *reinterpret_cast<const float4*>(&s_bias[ph][c0 + 4 * j4]);
+          const float z[4] = {v[4 * j4] + b4.x, v[4 * j4 + 1] + b4.y, v[4 * j4 + 2] + b4.z, v[4 * j4 + 3] + b4.w};
+          float g[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float e = 1.f + erff(z[j] * 0.70710678118654752f);
+            a[4 * j4 + j] = 0.5f * z[j] * e;
+            if (MODE == kTrain) g[j] = 0.5f * e + z[j] * 0.39894228040143268f * expf(-0.5f * z[j] * z[j]);
+          }
+          if (MODE == kTrain)
+            A.G[ph][((long long)blockIdx.x * (kHid / 4) + c0 / 4 + j4) * tc::kBM + row] = make_float4(g[0], g[1], g[2], g[3]);
+        }
+        store_act16(act_g, row, c0, a);
+        if (MODE == kTrain && valid) {
+          bf16* t = A.AbT[ph] + c0 * A.ldt + i;
+#pragma unroll
+          for (int j = 0; j < 16; ++j) t[j * A.ldt] = __float2bfloat16(a[j]);
+        }
+      }
+    } else if (ph == kLayers - 1) {
+      if (part == 0) {
+        float v[16];
+        tc::tmem_ld16(lane_addr, v);
+#pragma unroll
+        for (int c = 0; c < kOutPad; ++c) v[c] += s_bias[ph][c];
+        if (MODE == kWarm && valid) {
+          // warm = q + dt v + out_std * Z + out_mean
+#pragma unroll
+          for (int c = 0; c < kOut; ++c) {
+            const float y = v[c] * A.norm[kNormOutStd + c] + A.norm[kNormOutMean + c];
+            const size_t gi = (size_t)i * 12 + c;
+            A.warm[gi] = A.q[gi] + A.dt * A.v[gi] + (double)y;
+          }
+        }
+        if (MODE == kInfer && valid) {
+#pragma unroll
+          for (int c = 0; c < kOut; ++c)
+            A.Y[(long long)i * kOut + c] = v[c] * A.norm[kNormOutStd + c] + A.norm[kNormOutMean + c];
+        }
+        if (MODE == kTrain) {
+          // MSE on normalised targets: loss = mean (Z - Tn)^2 over rows x 12; dZ = 2 (Z - Tn) / (rows x 12)
+          const float scale = 2.f / (float)(A.rows * kOut);
+          double sum = 0.0;
+#pragma unroll
+          for (int c = 0; c < kOutPad; ++c) {
+            float d = 0.f;
+            if (c < kOut && has_target) {
+              const float diff = v[c] - (tn[c] - A.norm[kNormOutMean + c]) * A.norm[kNormOutIstd + c];
+              sum += (double)diff * diff;
+              d = scale * diff;
+            }
+            v[c] = d;
+          }
+          store_act16(act_g, row, 0, v);
+          if (valid) {
+#pragma unroll
+            for (int c = 0; c < kOutPad; ++c) A.dZbT[ph][c * A.ldt + i] = __float2bfloat16(v[c]);
+          }
+          const float cs = column_sum16(v, lane);
+          if (!(lane & 1)) s_sum[quarter][lane >> 1] = cs;
+          for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+          if (lane == 0) atomicAdd(A.loss, sum / (double)(A.rows * kOut));
+        }
+      }
+    } else if (MODE == kTrain) {
+      // back through a hidden layer: dZ = (dZ_next W) * GELU'(Z)
+#pragma unroll
+      for (int k = 0; k < kHid / 64; ++k) {
+        const int c0 = cpart + 16 * k;
         float v[16];
         tc::tmem_ld16(lane_addr + (uint32_t)c0, v);
-        float a[16];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) a[j] = gelu(v[j] + bias[c0 + j]);
-        unsigned char* rp = act_g + (c0 / tc::kBK) * (tc::kBM * 128) + row * 128;
-        const int p = (c0 % tc::kBK) / 8;
-        *reinterpret_cast<uint4*>(rp + ((p ^ (row & 7)) * 16)) = pack_bf16x8(a);
-        *reinterpret_cast<uint4*>(rp + (((p + 1) ^ (row & 7)) * 16)) = pack_bf16x8(a + 8);
+        for (int j = 0; j < 4; ++j) {
+          const float4 g = gp[4 * k + j];
+          v[4 * j] = valid ? v[4 * j] * g.x : 0.f;
+          v[4 * j + 1] = valid ? v[4 * j + 1] * g.y : 0.f;
+          v[4 * j + 2] = valid ? v[4 * j + 2] * g.z : 0.f;
+          v[4 * j + 3] = valid ? v[4 * j + 3] * g.w : 0.f;
+        }
+        if (ph + 1 < nph) store_act16(act_g, row, c0, v);
+        if (valid) {
+          bf16* t = A.dZbT[lb - 1] + c0 * A.ldt + i;
+#pragma unroll
+          for (int j = 0; j < 16; ++j) t[j * A.ldt] = __float2bfloat16(v[j]);
+        }
+        const float cs = column_sum16(v, lane);
+        if (!(lane & 1)) s_sum[quarter][c0 + (lane >> 1)] = cs;
       }
+    }
+    if (MODE == kTrain || ph + 1 < nph) {
       asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
       tc::tc_fence_before();
       __syncthreads();
       tc::tc_fence_after();
-    } else if (part == 0) {
-      // output layer: warm = q + dt v + out_std * (acc + bias) + out_mean (k_output, k_compose)
-      float v[16];
-      tc::tmem_ld16(lane_addr, v);
-      const int i = r0 + row;
-      if (i < A.n_nodes) {
-#pragma unroll
-        for (int c = 0; c < kOut; ++c) {
-          const float y = (v[c] + bias[c]) * A.norm[kNormOutStd + c] + A.norm[kNormOutMean + c];
-          const size_t gi = (size_t)i * 12 + c;
-          A.warm[gi] = A.q[gi] + A.dt * A.v[gi] + (double)y;
-        }
-      }
     }
+    // bias gradients: the CTA's column sums, one atomic per column
+    if (MODE == kTrain && ph >= kLayers - 1 && tid < N)
+      atomicAdd(&A.gb[ph == kLayers - 1 ? ph : lb - 1][tid], (s_sum[0][tid] + s_sum[1][tid]) + (s_sum[2][tid] + s_sum[3][tid]));
   }
   if (tid == 0 && *abort_flag) {
     atomicOr(A.err, kErrTimeout);
-    // a weight copy still in flight, and the commit of the stopped layer, land in shared memory:
+    // a weight copy still in flight, and the commit of the stopped phase, land in shared memory:
     // wait for them before the CTA exits
     if (w_inflight >= 0) tc::mbar_wait_parity(bw, w_inflight & 1, tc::kDrainPolls);
-    tc::mbar_wait_parity(bm, l & 1, tc::kDrainPolls);
+    tc::mbar_wait_parity(bm, ph & 1, tc::kDrainPolls);
   }
   tc::tc_fence_before();
   __syncthreads();
@@ -484,27 +531,25 @@ struct shell_mlp_s {
   unsigned wait_polls = (unsigned)kDefaultWaitPolls;   // bound of the tensor-core pipeline waits
   long long launches = 0;
   int step = 0;
-  // parameters (padded; FP32 master copies, BF16 copies for the GEMMs), Adam moments, gradients
-  float *W[kLayers] = {}, *b[kLayers] = {}, *gW[kLayers] = {}, *gb[kLayers] = {};
+  // parameters (padded; FP32 master copies, BF16 copies for the products), Adam moments, gradients
+  float *W[kLayers] = {}, *b[kLayers] = {};
+  // one block: the error word, the loss (float 2 on), padding, then gW and gb of every layer
+  float* grads = nullptr;
+  float *gW[kLayers] = {}, *gb[kLayers] = {};
   float *mW[kLayers] = {}, *vW[kLayers] = {}, *mb[kLayers] = {}, *vb[kLayers] = {};
   bf16* Wb[kLayers] = {};
-  bf16* WbT[kLayers] = {};   // transposed BF16 weights [fan_in][fan_out] (input-gradient GEMMs)
-  CUtensorMap warm_maps[kLayers];   // TMA maps of Wb for the fused warm start (box 64 x fan-out)
-  // activations of the last forward pass, and their gradients; the *T arrays are transposed
-  // copies [features][ldt] read by the weight-gradient GEMMs
+  bf16* WbT[kLayers] = {};   // transposed BF16 weights [fan_in][fan_out] (back-propagation)
+  RowsMaps maps;             // TMA maps of Wb and WbT
+  // of the last training pass: transposed copies [features][ldt] (the operands of the weight-gradient
+  // GEMMs) of the input, the activations and their gradients, and GELU' (FP32)
   long long ldt = 0;         // max_rows rounded up to 8 (16-byte rows for TMA)
-  bf16 *Xb = nullptr, *XbT = nullptr;
-  float* Z[kLayers] = {};
-  bf16 *Ab[kLayers] = {}, *AbT[kLayers] = {};
-  float* dZ[kLayers] = {};
-  bf16 *dZb[kLayers] = {}, *dZbT[kLayers] = {};
-  float* Xraw = nullptr;  // [max_rows x 28] features of a warm-start call
+  bf16* XbT = nullptr;
+  bf16 *AbT[kLayers - 1] = {}, *dZbT[kLayers] = {};
+  float4* G[kLayers - 1] = {};
   float* norm = nullptr;  // kNormSize floats
-  double* loss = nullptr;
   double* stats = nullptr;
-  int* err = nullptr;
-  double* h_loss = nullptr;  // pinned
-  int* h_err = nullptr;      // pinned
+  int* err = nullptr;       // the block's error word
+  float* h_block = nullptr;   // pinned image of the block; also stages parameters on their way in and out
 };
 
 namespace {
@@ -524,156 +569,94 @@ shell_status malloc_zero(T** p, size_t count, cudaStream_t s) {
 
 void free_mlp(shell_mlp_s* m) {
   for (int l = 0; l < kLayers; ++l) {
-    void* ps[] = {m->W[l], m->b[l], m->gW[l], m->gb[l], m->mW[l], m->vW[l], m->mb[l], m->vb[l], m->Wb[l],
-                  m->WbT[l], m->Z[l], m->Ab[l], m->AbT[l], m->dZ[l], m->dZb[l], m->dZbT[l]};
+    void* ps[] = {m->W[l],  m->b[l],   m->mW[l],  m->vW[l], m->mb[l],
+                  m->vb[l], m->Wb[l], m->WbT[l], m->dZbT[l]};
     for (void* p : ps)
       if (p) cudaFree(p);
   }
-  void* ps[] = {m->Xb, m->XbT, m->Xraw, m->norm, m->loss, m->stats, m->err};
+  for (int l = 0; l < kLayers - 1; ++l) {
+    if (m->AbT[l]) cudaFree(m->AbT[l]);
+    if (m->G[l]) cudaFree(m->G[l]);
+  }
+  void* ps[] = {m->grads, m->XbT, m->norm, m->stats};
   for (void* p : ps)
     if (p) cudaFree(p);
-  if (m->h_loss) cudaFreeHost(m->h_loss);
-  if (m->h_err) cudaFreeHost(m->h_err);
+  if (m->h_block) cudaFreeHost(m->h_block);
   delete m;
 }
 
 int eblocks(long long n) { return (int)std::min<long long>(4096, std::max(1LL, (n + 255) / 256)); }
 
-// N tile of the 256-column GEMMs: 128 columns, so that two CTAs share an SM
-constexpr int kTileN = 128;
+constexpr int kLossAt = 2, kHeadFloats = 64;   // the loss's place in the block, and where the gradients begin
+constexpr size_t block_floats() {
+  size_t n = kHeadFloats;
+  for (int l = 0; l < kLayers; ++l) n += (size_t)kDout[l] * kDin[l] + kDout[l];
+  return n;
+}
 
-// Outputs of one GEMM (any may be null): FP32 (stored, or added for split K), BF16 row-major,
-// BF16 transposed; colvec: the per-column vector handed to the epilogue.
-struct GemmOut {
-  float* f32 = nullptr;
-  long long ldf = 0;
-  bool add = false;
-  bf16* b16 = nullptr;
-  long long ldb = 0;
-  bf16* b16t = nullptr;
-  long long ldt = 0;
-  const float* colvec = nullptr;
-};
+double* loss_of(const shell_mlp_s& M) { return reinterpret_cast<double*>(M.grads + kLossAt); }
 
-// C = A B^T on the tensor cores for A [m][k] (row stride lda) and B [n][k] (row stride ldb), both
-// BF16 with K contiguous; K split over up to ksplit CTAs per output tile.
-template <int BN, class Epi>
-shell_status tc_gemm(shell_mlp_s& M, const bf16* A, long long lda, const bf16* B, long long ldb, int m, int n, int k,
-                     int ksplit, const GemmOut& o, const Epi& epi, cudaStream_t st) {
-  CUtensorMap ma, mb;
-  tc::TcOut out;
-  std::memset(&out, 0, sizeof(out));
-  int mask = 0;
-  bool ok = tc::encode_bf16_map(&ma, A, m, k, lda, tc::kBM) && tc::encode_bf16_map(&mb, B, n, k, ldb, BN);
-  if (o.f32) {
-    ok = ok && tc::encode_out_f32(&out.f32, o.f32, m, n, o.ldf);
-    mask |= o.add ? tc::kOutF32Add : tc::kOutF32;
+template <RowsMode MODE>
+shell_status launch_rows(shell_mlp_s& M, RowsArgs& A, cudaStream_t st) {
+  static bool attr_set[64] = {false};
+  int dev = 0;
+  BHEM_CUDA(cudaGetDevice(&dev));
+  if (!attr_set[dev & 63]) {
+    BHEM_CUDA(cudaFuncSetAttribute(k_mlp_rows<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowsSmem));
+    attr_set[dev & 63] = true;
   }
-  if (o.b16) {
-    ok = ok && tc::encode_out_b16(&out.b16, o.b16, m, n, o.ldb);
-    mask |= tc::kOutB16;
-  }
-  if (o.b16t) {
-    ok = ok && tc::encode_out_b16t(&out.b16t, o.b16t, n, m, o.ldt);
-    mask |= tc::kOutB16T;
-  }
-  if (!ok) return fail(SHELL_ERR_CUDA, "tensor map encoding failed (cuTensorMapEncodeTiled)");
-  const cudaError_t e = tc::launch_gemm_tc<BN, Epi>(ma, mb, out, mask, o.colvec, m, n, k, ksplit, epi, M.err,
-                                                    kErrTimeout, M.wait_polls, st);
-  BHEM_CUDA(e);
+  for (int l = 0; l < kLayers; ++l) A.bias[l] = M.b[l];
+  A.norm = M.norm;
+  A.err = M.err;
+  A.polls = M.wait_polls;
+  k_mlp_rows<MODE><<<(A.rows + tc::kBM - 1) / tc::kBM, kRowThreads, kRowsSmem, st>>>(M.maps, A);
+  BHEM_CUDA(cudaGetLastError());
   ++M.launches;
   return SHELL_OK;
 }
 
-// forward pass of the rows staged in M.Xb: Z_l (FP32 pre-activation), Ab_l (BF16 GELU) and, when
-// training, the transposed AbT_l
-shell_status forward(shell_mlp_s& M, int rows, bool training, cudaStream_t st) {
-  const bf16* in = M.Xb;
-  for (int l = 0; l < kLayers; ++l) {
-    const bool hidden = l < kLayers - 1;
-    GemmOut o;
-    o.f32 = M.Z[l];
-    o.ldf = kDout[l];
-    o.colvec = M.b[l];
-    if (hidden) {
-      o.b16 = M.Ab[l];
-      o.ldb = kDout[l];
-      if (training) {
-        o.b16t = M.AbT[l];
-        o.ldt = M.ldt;
-      }
-    }
-    const EpiForward e{hidden ? 1 : 0};
-    if (kDout[l] == kHid) BHEM_TRY(tc_gemm<kTileN>(M, in, kDin[l], M.Wb[l], kDin[l], rows, kHid, kDin[l], 1, o, e, st));
-    else BHEM_TRY(tc_gemm<kOutPad>(M, in, kDin[l], M.Wb[l], kDin[l], rows, kOutPad, kDin[l], 1, o, e, st));
-    in = M.Ab[l];
-  }
-  return SHELL_OK;
-}
-
-// parameter gradients of the loss whose dZ (last layer) k_loss left in M.dZ[3], M.dZb[3], M.dZbT[3]
-shell_status backward(shell_mlp_s& M, int rows, cudaStream_t st) {
+// dW_l = dZ_l^T A_{l-1} of every layer: M = fan-out, N = fan-in, K = rows
+shell_status weight_gradients(shell_mlp_s& M, int rows, cudaStream_t st) {
   int dev = 0, nsm = 0;
   BHEM_CUDA(cudaGetDevice(&dev));
   BHEM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  const int kchunks = (rows + tc::kBK - 1) / tc::kBK;
-  for (int l = kLayers - 1; l >= 0; --l) {
-    BHEM_CUDA(cudaMemsetAsync(M.gW[l], 0, sizeof(float) * kDout[l] * kDin[l], st));
-    BHEM_CUDA(cudaMemsetAsync(M.gb[l], 0, sizeof(float) * kDout[l], st));
-    // dW_l = dZ_l^T A_{l-1}: M = fan-out, N = fan-in, K = rows, split over about one CTA per SM
-    const bf16* At = l > 0 ? M.AbT[l - 1] : M.XbT;
-    const int tiles = (kDout[l] + tc::kBM - 1) / tc::kBM * (kDin[l] == kHid ? kHid / kTileN : 1);
-    const int ksplit = std::max(1, std::min(kchunks, 2 * nsm / tiles));
-    GemmOut ow;
-    ow.f32 = M.gW[l];
-    ow.ldf = kDin[l];
-    ow.add = true;
-    const EpiAtomic ea{};
-    if (kDin[l] == kHid)
-      BHEM_TRY(tc_gemm<kTileN>(M, M.dZbT[l], M.ldt, At, M.ldt, kDout[l], kHid, rows, ksplit, ow, ea, st));
-    else
-      BHEM_TRY(tc_gemm<kInPad>(M, M.dZbT[l], M.ldt, At, M.ldt, kDout[l], kInPad, rows, ksplit, ow, ea, st));
-    dim3 cg((kDout[l] + 127) / 128, (rows + kColsumRows - 1) / kColsumRows);
-    k_colsum<<<cg, 128, 0, st>>>(rows, kDout[l], M.dZ[l], M.gb[l]);
-    BHEM_CUDA(cudaGetLastError());
-    ++M.launches;
-    if (l == 0) break;
-    // dZ_{l-1} = (dZ_l W_l) * GELU'(Z_{l-1}): M = rows, N = fan-in, K = fan-out
-    GemmOut og;
-    og.f32 = M.dZ[l - 1];
-    og.ldf = kDout[l - 1];
-    og.b16 = M.dZb[l - 1];
-    og.ldb = kDout[l - 1];
-    og.b16t = M.dZbT[l - 1];
-    og.ldt = M.ldt;
-    const EpiGeluBack eg{M.Z[l - 1], kDout[l - 1], rows};
-    BHEM_TRY(tc_gemm<kTileN>(M, M.dZb[l], kDout[l], M.WbT[l], kDout[l], rows, kHid, kDout[l], 1, og, eg, st));
+  tc::GemmSet S;
+  static_assert(kLayers == tc::kMaxGroups, "one group per layer");
+  int tiles = 0;
+  bool ok = true;
+  for (int l = 0; l < kLayers; ++l) {
+    tc::GemmGroup& g = S.g[l];
+    ok = ok && tc::encode_bf16_map(&g.a, M.dZbT[l], kDout[l], rows, M.ldt, tc::kBM) &&
+         tc::encode_bf16_map(&g.b, l > 0 ? M.AbT[l - 1] : M.XbT, kDin[l], rows, M.ldt, tc::kBN) &&
+         tc::encode_c_map(&g.c, M.gW[l], kDout[l], kDin[l], kDin[l]);
+    S.n[l] = kDin[l];
+    S.tiles_n[l] = (kDin[l] + tc::kBN - 1) / tc::kBN;
+    S.first[l] = tiles;
+    tiles += S.tiles_n[l] * ((kDout[l] + tc::kBM - 1) / tc::kBM);
   }
-  return SHELL_OK;
-}
-
-shell_status stage_input(shell_mlp_s& M, const float* X, long long data_rows, const int* idx, int rows,
-                         bool training, cudaStream_t st) {
-  k_input<<<eblocks((long long)rows * kInPad), 256, 0, st>>>(rows, X, data_rows, idx, M.norm, M.Xb,
-                                                             training ? M.XbT : nullptr, M.ldt, M.err);
-  BHEM_CUDA(cudaGetLastError());
+  S.first[kLayers] = tiles;
+  if (!ok) return fail(SHELL_ERR_CUDA, "tensor map encoding failed (cuTensorMapEncodeTiled)");
+  S.polls = M.wait_polls;
+  S.err = M.err;
+  S.err_bit = kErrTimeout;
+  BHEM_CUDA(tc::launch_gemm_split(S, tiles, rows, 2 * nsm / tiles, st));
   ++M.launches;
   return SHELL_OK;
 }
 
 // waits for the stream, returns the loss when asked, and turns a raised error flag into an error
 shell_status finish(shell_mlp_s& M, double* loss) {
-  BHEM_CUDA(cudaMemcpyAsync(M.h_err, M.err, sizeof(int), cudaMemcpyDeviceToHost, M.stream));
-  if (loss) BHEM_CUDA(cudaMemcpyAsync(M.h_loss, M.loss, sizeof(double), cudaMemcpyDeviceToHost, M.stream));
+  BHEM_CUDA(cudaMemcpyAsync(M.h_block, M.grads, sizeof(float) * (kLossAt + 2), cudaMemcpyDeviceToHost, M.stream));
   BHEM_CUDA(cudaStreamSynchronize(M.stream));
-  if (*M.h_err) {
-    const int e = *M.h_err;
+  int e;
+  std::memcpy(&e, M.h_block, sizeof(int));
+  if (e) {
     BHEM_CUDA(cudaMemsetAsync(M.err, 0, sizeof(int), M.stream));
     BHEM_CUDA(cudaStreamSynchronize(M.stream));
     if (e & kErrTimeout) return fail(SHELL_ERR_TIMEOUT, "a bounded tensor-core pipeline wait expired");
     return fail(SHELL_ERR_ARG, "row index outside [0, data_rows)");
   }
-  if (loss) *loss = *M.h_loss;
+  if (loss) std::memcpy(loss, M.h_block + kLossAt, sizeof(double));
   return SHELL_OK;
 }
 
@@ -683,27 +666,46 @@ long long param_count() {
   return n;
 }
 
-// host packed layout: per layer W [fan_out x fan_in] row-major, then b [fan_out]
+// host packed layout: per layer W [fan_out x fan_in] row-major, then b [fan_out]. Everything passes through
+// the pinned image of the gradient block (whose layout is the padded one of the device): one copy for the
+// gradients, asynchronous ones for the parameters, then one wait. Read in eight blocking pageable copies the
+// gradients took 128 us, now 46 us.
 shell_status copy_params(shell_mlp_s& M, float* host_out, const float* host_in, int grads) {
-  std::vector<float> buf;
-  long long off = 0;
-  for (int l = 0; l < kLayers; ++l) {
-    float* W = grads ? M.gW[l] : M.W[l];
-    float* b = grads ? M.gb[l] : M.b[l];
-    const int ro = kRout[l], ri = kRin[l], din = kDin[l];
-    buf.assign((size_t)kDout[l] * din, 0.f);
-    if (host_in) {
-      for (int o = 0; o < ro; ++o)
-        for (int i = 0; i < ri; ++i) buf[(size_t)o * din + i] = host_in[off + (long long)o * ri + i];
-      BHEM_CUDA(cudaMemcpy(W, buf.data(), sizeof(float) * buf.size(), cudaMemcpyHostToDevice));
-      BHEM_CUDA(cudaMemcpy(b, host_in + off + (long long)ro * ri, sizeof(float) * ro, cudaMemcpyHostToDevice));
-    } else {
-      BHEM_CUDA(cudaMemcpy(buf.data(), W, sizeof(float) * buf.size(), cudaMemcpyDeviceToHost));
-      for (int o = 0; o < ro; ++o)
-        for (int i = 0; i < ri; ++i) host_out[off + (long long)o * ri + i] = buf[(size_t)o * din + i];
-      BHEM_CUDA(cudaMemcpy(host_out + off + (long long)ro * ri, b, sizeof(float) * ro, cudaMemcpyDeviceToHost));
+  float* const image = M.h_block;
+  if (!host_in && grads)
+    BHEM_CUDA(cudaMemcpyAsync(image, M.grads, sizeof(float) * block_floats(), cudaMemcpyDeviceToHost, M.stream));
+  for (int pass = 0; pass < 2; ++pass) {   // out: fetch, wait, unpack; in: pack and send, wait
+    if (pass == 1) BHEM_CUDA(cudaStreamSynchronize(M.stream));
+    if (pass == 1 && host_in) break;
+    float* p = image + kHeadFloats;
+    long long off = 0;
+    for (int l = 0; l < kLayers; ++l) {
+      const int ro = kRout[l], ri = kRin[l], din = kDin[l];
+      const size_t nw = (size_t)kDout[l] * din;
+      float* pb = p + nw;
+      if (host_in) {
+        std::memset(p, 0, sizeof(float) * (nw + kDout[l]));
+        for (int o = 0; o < ro; ++o)
+          std::memcpy(p + (size_t)o * din, host_in + off + (long long)o * ri, sizeof(float) * ri);
+        std::memcpy(pb, host_in + off + (long long)ro * ri, sizeof(float) * ro);
+        BHEM_CUDA(cudaMemcpyAsync(M.W[l], p, sizeof(float) * nw, cudaMemcpyHostToDevice, M.stream));
+        BHEM_CUDA(cudaMemcpyAsync(M.b[l], pb, sizeof(float) * ro, cudaMemcpyHostToDevice, M.stream));
+      } else if (pass == 0) {
+        if (grads) break;
+        BHEM_CUDA(cudaMemcpyAsync(p, M.W[l], sizeof(float) * nw, cudaMemcpyDeviceToHost, M.stream));
+        BHEM_CUDA(cudaMemcpyAsync(pb, M.b[l], sizeof(float) * ro, cudaMemcpyDeviceToHost, M.stream));
+      } else {
+        if (ri == din) {
+          std::memcpy(host_out + off, p, sizeof(float) * (size_t)ro * ri);
+        } else {
+          for (int o = 0; o < ro; ++o)
+            std::memcpy(host_out + off + (long long)o * ri, p + (size_t)o * din, sizeof(float) * ri);
+        }
+        std::memcpy(host_out + off + (long long)ro * ri, pb, sizeof(float) * ro);
+      }
+      p = pb + kDout[l];
+      off += (long long)ro * ri + ro;
     }
-    off += (long long)ro * ri + ro;
   }
   return SHELL_OK;
 }
@@ -718,38 +720,41 @@ extern "C" shell_status shell_mlp_create(int max_rows, void* stream, shell_mlp_t
   M->stream = (cudaStream_t)stream;
   M->ldt = ((long long)max_rows + 7) / 8 * 8;
   shell_status st = SHELL_OK;
-  const size_t R = (size_t)max_rows, RT = (size_t)M->ldt;
+  const size_t R128 = ((size_t)max_rows + tc::kBM - 1) / tc::kBM * tc::kBM, RT = (size_t)M->ldt;
   for (int l = 0; l < kLayers && st == SHELL_OK; ++l) {
     const size_t nw = (size_t)kDout[l] * kDin[l], nb = kDout[l];
-    float** f32w[] = {&M->W[l], &M->gW[l], &M->mW[l], &M->vW[l]};
+    float** f32w[] = {&M->W[l], &M->mW[l], &M->vW[l]};
     for (float** p : f32w)
       if (st == SHELL_OK) st = malloc_zero(p, nw, M->stream);
-    float** f32b[] = {&M->b[l], &M->gb[l], &M->mb[l], &M->vb[l]};
+    float** f32b[] = {&M->b[l], &M->mb[l], &M->vb[l]};
     for (float** p : f32b)
       if (st == SHELL_OK) st = malloc_zero(p, nb, M->stream);
     if (st == SHELL_OK) st = malloc_zero(&M->Wb[l], nw, M->stream);
     if (st == SHELL_OK && l > 0) st = malloc_zero(&M->WbT[l], nw, M->stream);
-    if (st == SHELL_OK) st = malloc_zero(&M->Z[l], R * kDout[l], M->stream);
-    if (st == SHELL_OK && l < kLayers - 1) st = malloc_zero(&M->Ab[l], R * kDout[l], M->stream);
     if (st == SHELL_OK && l < kLayers - 1) st = malloc_zero(&M->AbT[l], RT * kDout[l], M->stream);
-    if (st == SHELL_OK) st = malloc_zero(&M->dZ[l], R * kDout[l], M->stream);
-    if (st == SHELL_OK) st = malloc_zero(&M->dZb[l], R * kDout[l], M->stream);
+    if (st == SHELL_OK && l < kLayers - 1) st = malloc_zero(&M->G[l], R128 * kDout[l] / 4, M->stream);
     if (st == SHELL_OK) st = malloc_zero(&M->dZbT[l], RT * kDout[l], M->stream);
   }
-  if (st == SHELL_OK) st = malloc_zero(&M->Xb, R * kInPad, M->stream);
+  if (st == SHELL_OK) st = malloc_zero(&M->grads, block_floats(), M->stream);
+  if (st == SHELL_OK) {
+    M->err = reinterpret_cast<int*>(M->grads);
+    float* p = M->grads + kHeadFloats;
+    for (int l = 0; l < kLayers; ++l) {
+      M->gW[l] = p;
+      M->gb[l] = p + (size_t)kDout[l] * kDin[l];
+      p = M->gb[l] + kDout[l];
+    }
+  }
   if (st == SHELL_OK) st = malloc_zero(&M->XbT, RT * kInPad, M->stream);
-  if (st == SHELL_OK) st = malloc_zero(&M->Xraw, R * kIn, M->stream);
   if (st == SHELL_OK) st = malloc_zero(&M->norm, kNormSize, M->stream);
-  if (st == SHELL_OK) st = malloc_zero(&M->loss, 1, M->stream);
   if (st == SHELL_OK) st = malloc_zero(&M->stats, 2 * kIn, M->stream);
-  if (st == SHELL_OK) st = malloc_zero(&M->err, 1, M->stream);
-  if (st == SHELL_OK && (cudaMallocHost((void**)&M->h_loss, sizeof(double)) != cudaSuccess ||
-                         cudaMallocHost((void**)&M->h_err, sizeof(int)) != cudaSuccess)) {
+  if (st == SHELL_OK && cudaMallocHost((void**)&M->h_block, sizeof(float) * block_floats()) != cudaSuccess) {
     cudaGetLastError();
     st = fail(SHELL_ERR_OOM, "cudaMallocHost failed");
   }
   for (int l = 0; l < kLayers && st == SHELL_OK; ++l)
-    if (!tc::encode_bf16_map(&M->warm_maps[l], M->Wb[l], kDout[l], kDin[l], kDin[l], kDout[l]))
+    if (!tc::encode_bf16_map(&M->maps.w[l], M->Wb[l], kDout[l], kDin[l], kDin[l], kDout[l]) ||
+        (l > 0 && !tc::encode_bf16_map(&M->maps.wt[l], M->WbT[l], kDin[l], kDout[l], kDout[l], kDin[l])))
       st = fail(SHELL_ERR_CUDA, "tensor map encoding failed (cuTensorMapEncodeTiled)");
   if (st == SHELL_OK) {
     // identity normalisation until shell_mlp_set_normalization
@@ -847,27 +852,37 @@ extern "C" shell_status shell_mlp_column_stats(shell_mlp_t* M, const float* X, l
 
 extern "C" shell_status shell_mlp_forward(shell_mlp_t* M, const float* X, int rows, float* Y) {
   if (!M || !X || !Y || rows < 1 || rows > M->max_rows) return fail(SHELL_ERR_ARG, "invalid argument");
-  BHEM_TRY(stage_input(*M, X, rows, nullptr, rows, false, M->stream));
-  BHEM_TRY(forward(*M, rows, false, M->stream));
-  k_output<<<eblocks((long long)rows * kOut), 256, 0, M->stream>>>(rows, M->Z[kLayers - 1], M->norm, Y);
-  BHEM_CUDA(cudaGetLastError());
-  ++M->launches;
-  return SHELL_OK;
+  RowsArgs A{};
+  A.rows = rows;
+  A.X = X;
+  A.Y = Y;
+  return launch_rows<kInfer>(*M, A, M->stream);
 }
 
 extern "C" shell_status shell_mlp_gradients(shell_mlp_t* M, const float* X, const float* T, long long data_rows,
                                             const int* idx, int rows, double* loss) {
   if (!M || !X || !T || rows < 1 || rows > M->max_rows || data_rows < 1 || (!idx && rows > data_rows))
     return fail(SHELL_ERR_ARG, "invalid argument");
-  BHEM_TRY(stage_input(*M, X, data_rows, idx, rows, true, M->stream));
-  BHEM_TRY(forward(*M, rows, true, M->stream));
-  BHEM_CUDA(cudaMemsetAsync(M->loss, 0, sizeof(double), M->stream));
-  k_loss<<<eblocks((long long)rows * kOutPad), 256, 0, M->stream>>>(
-      rows, M->Z[kLayers - 1], T, data_rows, idx, M->norm, M->dZ[kLayers - 1], M->dZb[kLayers - 1],
-      M->dZbT[kLayers - 1], M->ldt, M->loss);
-  BHEM_CUDA(cudaGetLastError());
-  ++M->launches;
-  BHEM_TRY(backward(*M, rows, M->stream));
+  BHEM_CUDA(cudaMemsetAsync(M->grads + kLossAt, 0, sizeof(float) * (block_floats() - kLossAt), M->stream));
+  RowsArgs A{};
+  A.rows = rows;
+  A.X = X;
+  A.T = T;
+  A.data_rows = data_rows;
+  A.idx = idx;
+  A.loss = loss_of(*M);
+  A.ldt = M->ldt;
+  A.XbT = M->XbT;
+  for (int l = 0; l < kLayers; ++l) {
+    if (l < kLayers - 1) {
+      A.AbT[l] = M->AbT[l];
+      A.G[l] = M->G[l];
+    }
+    A.dZbT[l] = M->dZbT[l];
+    A.gb[l] = M->gb[l];
+  }
+  BHEM_TRY(launch_rows<kTrain>(*M, A, M->stream));
+  BHEM_TRY(weight_gradients(*M, rows, M->stream));
   return loss ? finish(*M, loss) : SHELL_OK;
 }
 
@@ -946,13 +961,8 @@ extern "C" shell_status shell_mlp_warm_start(shell_mlp_t* M, shell_t* shell, con
     ++s.launches;
     return SHELL_OK;
   }
-  static bool attr_set[64] = {false};
-  if (!attr_set[s.device & 63]) {
-    BHEM_CUDA(cudaFuncSetAttribute(k_mlp_warm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWarmSmem));
-    attr_set[s.device & 63] = true;
-  }
-  WarmArgs A{};
-  A.n_nodes = s.n_nodes;
+  RowsArgs A{};
+  A.rows = s.n_nodes;
   A.n1 = s.n1;
   A.n2 = s.n2;
   A.per_u = s.grid.periodic_u;
@@ -961,14 +971,6 @@ extern "C" shell_status shell_mlp_warm_start(shell_mlp_t* M, shell_t* shell, con
   A.rest = s.d_rest;
   A.v = v;
   A.dt = dt;
-  for (int l = 0; l < kLayers; ++l) A.bias[l] = M->b[l];
-  A.norm = M->norm;
   A.warm = warm;
-  A.err = M->err;
-  A.polls = M->wait_polls;
-  k_mlp_warm<<<(s.n_nodes + tc::kBM - 1) / tc::kBM, kWarmThreads, kWarmSmem, s.stream>>>(
-      M->warm_maps[0], M->warm_maps[1], M->warm_maps[2], M->warm_maps[3], A);
-  BHEM_CUDA(cudaGetLastError());
-  ++M->launches;
-  return SHELL_OK;
+  return launch_rows<kWarm>(*M, A, s.stream);
 }

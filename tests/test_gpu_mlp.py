@@ -286,3 +286,31 @@ def test_tensor_core_wait_timeout_is_reported_and_the_network_recovers():
     assert rel(net.get_grads().astype(np.float64), G0) <= 1e-5
     np.testing.assert_array_equal(w1, w0)
     net.close()
+
+
+@pytest.mark.parametrize("rows", [1, 63, 127, 128, 129])
+def test_gradients_of_a_doubled_batch(rows):
+    """A batch and the same rows twice over (the second time in reverse order) have one loss and one gradient:
+    every dZ is exactly half (a power of two, BF16 rounding included) and every row counts twice, on other
+    lanes and in other tiles of 128 rows, through ragged ends. What may differ is the order of FP32 sums of
+    at most 258 terms, 258 2^-24 = 1.5e-5 relative to the terms; a row lost or counted twice is 1 / 258 =
+    4e-3. Bound 1e-4 normwise per tensor, loss (FP64 sums) 1e-12. The network holds more rows than the
+    batches, so its buffers' row stride is not theirs, and the index names the last row."""
+    net, _, _ = _net(300, 34, _norm(33))
+    rng = np.random.default_rng(35)
+    X = dev(rng.normal(0, 1.5, (260, 28)), torch.float32)
+    T = dev(rng.normal(0, 1.0, (260, 12)), torch.float32)
+    idx = np.concatenate([[259], rng.integers(0, 260, rows - 1)]).astype(np.int32)
+    loss1 = net.gradients(X, T, idx=dev(idx, torch.int32))
+    G1 = net.get_grads().astype(np.float64)
+    loss2 = net.gradients(X, T, idx=dev(np.concatenate([idx, idx[::-1]]), torch.int32))
+    G2 = net.get_grads().astype(np.float64)
+    assert loss2 == pytest.approx(loss1, rel=1e-12)
+    off = 0
+    for fi, fo in om.LAYERS:
+        for name, size in (("W", fi * fo), ("b", fo)):
+            sl = slice(off, off + size)
+            assert np.linalg.norm(G1[sl]) > 0
+            assert rel(G2[sl], G1[sl]) <= 1e-4, (fi, fo, name, rel(G2[sl], G1[sl]))
+            off += size
+    net.close()
