@@ -128,7 +128,7 @@ __global__ void k_tables(int S, const double* __restrict__ dxi, double* __restri
   build_shape_table<double>(sphi, dxi[2 * s], dxi[2 * s + 1]);
   __syncthreads();
   for (int e = threadIdx.x; e < kPhiTable; e += blockDim.x) {
-    double v = e < kPhiSize ? sphi[e] : gauss_weight(e - kPhiSize, dxi[2 * s], dxi[2 * s + 1]);
+    const double v = shape_table_entry(sphi, dxi[2 * s], dxi[2 * s + 1], e);
     t64[(size_t)s * kPhiTable + e] = v;
     t32[(size_t)s * kPhiTable + e] = (float)v;
   }
@@ -213,7 +213,6 @@ struct ElemBatchArgs {
   const ShellPar* par;
   const ShellState* st;
   const float* t32;
-  const double* dxi;           // [2 * shells] parameter extents of one patch
   const int4* pnodes;
   const int* pblocks;
   const double* q;
@@ -229,7 +228,7 @@ k_element(ElemBatchArgs B) {
   constexpr int NW = ElemCfg<float>::kWarps;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float* sphi = reinterpret_cast<float*>(smem_raw);
-  float* w1d = sphi + ((kPhiTable + 3) & ~3);
+  float* const sphg = sphi + ((kPhiTable + 3) & ~3);
   WarpSmem<float>* Ws = reinterpret_cast<WarpSmem<float>*>(smem_raw + sizeof(float) * elem_table_elems<float>());
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   for (int it = blockIdx.x; it < B.n_items; it += gridDim.x) {
@@ -238,10 +237,8 @@ k_element(ElemBatchArgs B) {
     if (!B.st[s].active) continue;   // uniform over the CTA
     __syncthreads();
     load_shape_table<float>(sphi, B.t32 + (size_t)s * kPhiTable);
-    build_hermite_1d<float>(w1d, B.dxi[2 * s], threadIdx.x, blockDim.x);
-    build_hermite_1d<float>(w1d + kHerm1D, B.dxi[2 * s + 1], threadIdx.x, blockDim.x);
     __syncthreads();
-    build_phi_gauss(w1d + 2 * kHerm1D, sphi, threadIdx.x, blockDim.x);
+    build_phi_gauss(sphg, sphi, threadIdx.x, blockDim.x);
     __syncthreads();
     ElemArgs A{};
     A.pnodes = B.pnodes;
@@ -258,7 +255,7 @@ k_element(ElemBatchArgs B) {
     A.err = B.err;
     for (int k = item.y + wid; k < item.z; k += NW) {
       const int p = B.plist ? B.plist[k] : k;
-      element_patch<float>(sphi, w1d, w1d + 2 * kHerm1D, Ws[wid], p, A, lane);
+      element_patch<float>(sphi, sphi + kPhiHerm, sphg, Ws[wid], p, A, lane);
     }
   }
 }
@@ -268,11 +265,12 @@ k_element(ElemBatchArgs B) {
 // mode 1: acc[3] += E_p(q + alpha_s d) - Ep[p] (shells with searching != 0)
 __global__ void __launch_bounds__(128)
 k_eg64(int n_items, const int4* __restrict__ items, int P, const ShellPar* __restrict__ par,
-       ShellState* st, const double* __restrict__ dxi, const int4* __restrict__ pnodes,
+       ShellState* st, const double* __restrict__ t64, const int4* __restrict__ pnodes,
        const double* __restrict__ q, const double* __restrict__ dir,
        const double* __restrict__ restgp, double* __restrict__ Ep, double* __restrict__ grad,
        int mode, int* err) {
-  __shared__ double w1[kHerm1D], w2[kHerm1D];
+  __shared__ double w1[2 * kHerm1D];
+  const double* const w2 = w1 + kHerm1D;
   __shared__ double sq[kEgPatches][48];
   __shared__ double sT[kEgPatches][144];
   __shared__ double sG[kEgPatches][16][15];
@@ -284,8 +282,7 @@ k_eg64(int n_items, const int4* __restrict__ items, int P, const ShellPar* __res
     const bool run = mode == 0 ? st[s].active != 0 : st[s].searching != 0;
     if (!run) continue;   // uniform over the CTA
     __syncthreads();
-    build_hermite_1d(w1, dxi[2 * s], threadIdx.x, blockDim.x);
-    build_hermite_1d(w2, dxi[2 * s + 1], threadIdx.x, blockDim.x);
+    if (threadIdx.x < 2 * kHerm1D) w1[threadIdx.x] = t64[(size_t)s * kPhiTable + kPhiHerm + threadIdx.x];
     __syncthreads();
     const int p = item.y + hw;
     const bool active = p < item.z;
@@ -1218,7 +1215,6 @@ shell_status assemble(shell_batch_s& b, const double* q, double mass_scale) {
   A.par = b.par;
   A.st = b.st;
   A.t32 = b.t32;
-  A.dxi = b.dxi;
   A.pnodes = b.pnodes;
   A.pblocks = b.pblocks;
   A.q = q;
@@ -1304,7 +1300,7 @@ shell_status residual(shell_batch_s& b, const double* q, const shell_step_params
   int nsm = 0;
   BHEM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, b.device));
   k_eg64<<<std::min(b.n_eg_items, nsm * 16), 128, 0, b.stream>>>(b.n_eg_items, b.eg_items, b.P, b.par, b.st,
-      b.dxi, b.pnodes, q, nullptr, b.restgp, b.Ep, b.g, 0, b.err);
+      b.t64, b.pnodes, q, nullptr, b.restgp, b.Ep, b.g, 0, b.err);
   BHEM_CUDA(cudaGetLastError());
   BL(b);
   k_grad_finish<<<b.grid_rows, kNodeThreads, 0, b.stream>>>(b.active, b.st, b.row_ptr, b.col,
@@ -1419,7 +1415,7 @@ shell_status line_search(shell_batch_s& b, const shell_step_params& P, const dou
   BHEM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, b.device));
   for (int trial = 0; trial < 20 && b.h_cnt->n_searching > 0; ++trial) {
     k_eg64<<<std::min(b.n_eg_items, nsm * 16), 128, 0, b.stream>>>(b.n_eg_items, b.eg_items, b.P, b.par, b.st,
-        b.dxi, b.pnodes, q, b.d, b.restgp, b.Ep, nullptr, 1, b.err);
+        b.t64, b.pnodes, q, b.d, b.restgp, b.Ep, nullptr, 1, b.err);
     BHEM_TRY(zero_counters(b));
     k_ctrl_ls_step<<<blocks_for(b.S, 128), 128, 0, b.stream>>>(b.S, b.st, b.cnt);
     b.launches += 2;
@@ -1487,7 +1483,7 @@ shell_status enqueue_residual(shell_batch_s& b, const double* q, const shell_ste
                               const unsigned char* mask, int set_ref, int nsm) {
   BHEM_CUDA(cudaMemsetAsync(b.g, 0, sizeof(double) * b.M, b.stream));
   k_eg64<<<std::min(b.n_eg_items, nsm * 16), 128, 0, b.stream>>>(b.n_eg_items, b.eg_items, b.P, b.par, b.st,
-      b.dxi, b.pnodes, q, nullptr, b.restgp, b.Ep, b.g, 0, b.err);
+      b.t64, b.pnodes, q, nullptr, b.restgp, b.Ep, b.g, 0, b.err);
   k_grad_finish<<<b.grid_rows, kNodeThreads, 0, b.stream>>>(b.active, b.st, b.row_ptr, b.col,
       b.mass, b.fgrav, q, b.y, 1.0 / (P.dt * P.dt), P.gravity[0], P.gravity[1], P.gravity[2], mask, b.g,
       b.gin, b.err);
@@ -1560,7 +1556,7 @@ shell_status enqueue_newton_body(shell_batch_s& b, const shell_step_params& P, c
   BHEM_TRY(cap_body(b, 2, ls_body, [&]() -> shell_status {
     const long long s0 = b.launches;
     k_eg64<<<std::min(b.n_eg_items, nsm * 16), 128, 0, b.stream>>>(b.n_eg_items, b.eg_items, b.P, b.par, b.st,
-        b.dxi, b.pnodes, dq, b.d, b.restgp, b.Ep, nullptr, 1, b.err);
+        b.t64, b.pnodes, dq, b.d, b.restgp, b.Ep, nullptr, 1, b.err);
     BHEM_TRY(zero_counters(b));
     k_ctrl_ls_step<<<blocks_for(b.S, 128), 128, 0, b.stream>>>(b.S, b.st, b.cnt);
     k_cond_ls<<<1, 1, 0, b.stream>>>(b.cnt, b.loop, h_ls, 0);

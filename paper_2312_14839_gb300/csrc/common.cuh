@@ -92,6 +92,8 @@ struct DeviceScalars {
   int err;             // error bits
 };
 
+constexpr int kPhiTableCount = 1664;   // entries of a shell's shape table
+
 // ------------------------------------------------------------------------------------------
 // Shell: everything lives in device memory owned by the library.
 // ------------------------------------------------------------------------------------------
@@ -118,7 +120,7 @@ struct Shell {
   // reference configuration
   double* d_rest = nullptr;         // [n_dof]
   double* d_restgp = nullptr;       // [13 * np * 16] per-Gauss-point rest data (SoA)
-  double* d_phi64 = nullptr;        // shape table + Gauss weights (kPhiTable doubles)
+  double* d_phi64 = nullptr;        // shape table, Gauss weights, 1D factors (kPhiTableCount doubles)
   float* d_phi32 = nullptr;         // the same in FP32
   double* d_mass = nullptr;         // [n_blocks * 16] consistent mass, 4x4 scalar blocks
   double* d_qmy = nullptr;          // [n_dof] q - y of the residual's inertial term

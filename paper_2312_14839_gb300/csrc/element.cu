@@ -22,7 +22,7 @@ __global__ void k_shape_table(double d1, double d2, double* __restrict__ t64, fl
   build_shape_table<double>(sphi, d1, d2);
   __syncthreads();
   for (int e = threadIdx.x; e < kPhiTable; e += blockDim.x) {
-    double v = e < kPhiSize ? sphi[e] : gauss_weight(e - kPhiSize, d1, d2);
+    const double v = shape_table_entry(sphi, d1, d2, e);
     t64[e] = v;
     t32[e] = (float)v;
   }
@@ -128,33 +128,41 @@ shell_status launch_rest_setup(Shell& s) {
 }
 
 // ------------------------------------------------------------------------------------------
-// Light FP64 kernel: energy (and gradient) per patch, half a warp per patch, lane = Gauss point.
+// Light FP64 kernel: energy (and gradient) per patch, half a warp (or a warp) per patch, lane = Gauss point.
 // ------------------------------------------------------------------------------------------
+template <bool kWarpPatch>
 __global__ void __launch_bounds__(128)
 k_energy_grad64(int np, const int4* __restrict__ pnodes, const double* __restrict__ q,
                 const double* __restrict__ dir, double step, const double* __restrict__ restgp,
-                double dxi1, double dxi2, double h, double* __restrict__ energy_p,
+                const double* __restrict__ herm, double h, double* __restrict__ energy_p,
                 const double* __restrict__ energy_ref, double* __restrict__ grad, Reduce red,
                 double* scal_out, int* err) {
-  __shared__ double w1[kHerm1D], w2[kHerm1D];
-  __shared__ double sq[kEgPatches][48];
-  __shared__ double sT[kEgPatches][144];
-  __shared__ double sG[kEgPatches][16][15];
-  build_hermite_1d(w1, dxi1, threadIdx.x, blockDim.x);
-  build_hermite_1d(w2, dxi2, threadIdx.x, blockDim.x);
+  constexpr int kPer = kWarpPatch ? kEgPatches / 2 : kEgPatches;
+  __shared__ double w[2 * kHerm1D];
+  __shared__ double sq[kPer][48];
+  __shared__ double sT[kPer][144];
+  __shared__ double sG[kPer][16][15];
+  const double* const w1 = w;
+  const double* const w2 = w + kHerm1D;
+  if (threadIdx.x < 2 * kHerm1D) w[threadIdx.x] = herm[threadIdx.x];
   __syncthreads();
-  const int hw = threadIdx.x >> 4, g = threadIdx.x & 15;
-  const int p = blockIdx.x * kEgPatches + hw;
+  const int lane = threadIdx.x & 31, hw = kWarpPatch ? threadIdx.x >> 5 : threadIdx.x >> 4;
+  const int p = blockIdx.x * kPer + hw;
   const bool active = p < np;
   int nd[4] = {0, 0, 0, 0};
   if (active) {
     int4 pn = pnodes[p];
     nd[0] = pn.x; nd[1] = pn.y; nd[2] = pn.z; nd[3] = pn.w;
   }
-  const double ep = eg64_patch(w1, w2, sq[hw], sT[hw], sG[hw], p, active, g, nd, q, dir, step, restgp,
-                               (size_t)np * 16, h, grad, err);
+  double ep;
+  if constexpr (kWarpPatch)
+    ep = eg64_patch_warp(w1, w2, sq[hw], sT[hw], sG[hw], p, active, lane, nd, q, dir, step, restgp,
+                         (size_t)np * 16, h, grad, err);
+  else
+    ep = eg64_patch(w1, w2, sq[hw], sT[hw], sG[hw], p, active, lane & 15, nd, q, dir, step, restgp,
+                    (size_t)np * 16, h, grad, err);
   double contrib = 0.0;
-  if (active && g == 0) {
+  if (active && (lane & (kWarpPatch ? 31 : 15)) == 0) {
     if (!isfinite(ep)) atomicOr(err, ERRBIT_NONFINITE);
     if (energy_ref) contrib = ep - energy_ref[p];
     else contrib = ep;
@@ -169,12 +177,15 @@ k_energy_grad64(int np, const int4* __restrict__ pnodes, const double* __restric
 shell_status launch_energy_grad64(Shell& s, const double* q, const double* dir, double step,
                                   double* energy_p, const double* energy_ref, double* grad,
                                   double* scal_out) {
-  int blocks = (s.n_patches + kEgPatches - 1) / kEgPatches;
+  // A warp per patch while every SM sub-partition (four per SM) then has one patch at most: 215 FP64
+  // instructions one after another instead of 330; with more patches half a warp each does them in less.
+  const bool warp = s.n_patches <= 4 * s.num_sms;
+  const int per = warp ? kEgPatches / 2 : kEgPatches;
+  int blocks = (s.n_patches + per - 1) / per;
   if (blocks > s.red.stride) return fail(SHELL_ERR_ARG, "too many patches for one reduction");
-  k_energy_grad64<<<blocks, 128, 0, s.stream>>>(s.n_patches, s.d_patch_nodes, q, dir, step,
-                                                s.d_restgp, s.grid.dxi1, s.grid.dxi2,
-                                                s.mat.thickness, energy_p, energy_ref, grad, s.red,
-                                                scal_out, s.d_err);
+  auto k = warp ? k_energy_grad64<true> : k_energy_grad64<false>;
+  k<<<blocks, 128, 0, s.stream>>>(s.n_patches, s.d_patch_nodes, q, dir, step, s.d_restgp, s.d_phi64 + kPhiHerm,
+                                  s.mat.thickness, energy_p, energy_ref, grad, s.red, scal_out, s.d_err);
   BHEM_CUDA(cudaGetLastError());
   ++s.launches;
   return SHELL_OK;
@@ -189,12 +200,10 @@ k_element_full(ElemArgs A) {
   constexpr int NW = ElemCfg<R>::kWarps;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   R* sphi = reinterpret_cast<R*>(smem_raw);
-  R* w1d = sphi + ((kPhiTable + 3) & ~3);
+  R* w1d = sphi + kPhiHerm;
   WarpSmem<R>* Ws = reinterpret_cast<WarpSmem<R>*>(smem_raw + sizeof(R) * elem_table_elems<R>());
-  R* sphg = w1d + 2 * kHerm1D;
+  R* sphg = sphi + ((kPhiTable + 3) & ~3);
   load_shape_table<R>(sphi, reinterpret_cast<const R*>(A.phi));
-  build_hermite_1d<R>(w1d, A.d1, threadIdx.x, blockDim.x);
-  build_hermite_1d<R>(w1d + kHerm1D, A.d2, threadIdx.x, blockDim.x);
   __syncthreads();
   if constexpr (sizeof(R) == 4) {
     build_phi_gauss(sphg, sphi, threadIdx.x, blockDim.x);
@@ -210,9 +219,9 @@ k_element_full(ElemArgs A) {
       // the FP32 Hessian: the FP64 pipe works while other warps issue the FP32 pass. Every second
       // patch of a warp, its two half-warps evaluate that patch and the warp's next one, in the
       // warp's Gauss-point-matrix area (free between patches; 2 x 432 doubles).
-      __shared__ double w1_64[kHerm1D], w2_64[kHerm1D];
-      build_hermite_1d<double>(w1_64, A.d1, threadIdx.x, blockDim.x);
-      build_hermite_1d<double>(w2_64, A.d2, threadIdx.x, blockDim.x);
+      __shared__ double w1_64[2 * kHerm1D];
+      const double* const w2_64 = w1_64 + kHerm1D;
+      for (int e = threadIdx.x; e < 2 * kHerm1D; e += blockDim.x) w1_64[e] = A.herm64[e];
       __syncthreads();
       static_assert(sizeof(W.M) >= 2 * 432 * sizeof(double), "FP64 scratch fits the M_g area");
       const int hw = lane >> 4, g = lane & 15;
@@ -297,8 +306,6 @@ shell_status launch_element_full(Shell& s, const double* q, bool fp64, const Ele
   A.pblocks = s.d_patch_blocks;
   A.q = q;
   A.rest = s.d_rest;
-  A.d1 = s.grid.dxi1;
-  A.d2 = s.grid.dxi2;
   A.lam = s.lam;
   A.mu = s.mu;
   A.h = s.mat.thickness;
@@ -313,6 +320,7 @@ shell_status launch_element_full(Shell& s, const double* q, bool fp64, const Ele
   A.err = s.d_err;
   if (!fp64 && out.grad64) {
     A.restgp = s.d_restgp;
+    A.herm64 = s.d_phi64 + kPhiHerm;
     A.energy64 = out.energy64;
     A.grad64 = out.grad64;
   }

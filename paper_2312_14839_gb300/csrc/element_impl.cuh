@@ -35,7 +35,10 @@ __device__ __forceinline__ void gauss_unit(double th[4], double wt[4]) {
 // access patterns (lanes over g, lanes over I) free of bank conflicts.
 constexpr int kPhiStride = 97;
 constexpr int kPhiSize = 16 * kPhiStride;
-constexpr int kPhiTable = kPhiSize + 16;   // + the 16 Gauss weights W_g = dxi1 dxi2 w_g1 w_g2
+constexpr int kHerm1D = 48;
+constexpr int kPhiHerm = kPhiSize + 16;             // after the 16 Gauss weights W_g = dxi1 dxi2 w_g1 w_g2:
+constexpr int kPhiTable = kPhiHerm + 2 * kHerm1D;   // the 1D factors of theta^1 and theta^2 (hermite_1d)
+static_assert(kPhiTable == kPhiTableCount, "the shells' allocations");
 
 template <typename R>
 __device__ void build_shape_table(R* sphi, double d1, double d2) {
@@ -61,9 +64,10 @@ __device__ __forceinline__ double gauss_weight(int g, double d1, double d2) {
   return d1 * d2 * wt[g & 3] * wt[g >> 2];
 }
 
+// shape table, Gauss weights and (unless the caller has no use for them) 1D factors
 template <typename R>
-__device__ __forceinline__ void load_shape_table(R* sphi, const R* __restrict__ table) {
-  for (int e = threadIdx.x; e < kPhiTable; e += blockDim.x) sphi[e] = table[e];
+__device__ __forceinline__ void load_shape_table(R* sphi, const R* __restrict__ table, int count = kPhiTable) {
+  for (int e = threadIdx.x; e < count; e += blockDim.x) sphi[e] = table[e];
 }
 
 // ------------------------------------------------------------------------------------------
@@ -78,7 +82,17 @@ template <typename R> __device__ __forceinline__ R dot(V3<R> a, V3<R> b) { retur
 template <typename R> __device__ __forceinline__ V3<R> cross(V3<R> a, V3<R> b) {
   return {a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x};
 }
+// a . b - c and a x b + c as chains of fused multiply-adds
+template <typename R> __device__ __forceinline__ R dot_less(V3<R> a, V3<R> b, R c) { return a.x * b.x + (a.y * b.y + (a.z * b.z - c)); }
+template <typename R> __device__ __forceinline__ V3<R> cross_plus(V3<R> a, V3<R> b, V3<R> c) {
+  return {a.y * b.z + (c.x - a.z * b.y), a.z * b.x + (c.y - a.x * b.z), a.x * b.y + (c.z - a.y * b.x)};
+}
 template <typename R> __device__ __forceinline__ R comp(V3<R> a, int i) { return i == 0 ? a.x : i == 1 ? a.y : a.z; }
+
+__device__ __forceinline__ double from_lane(double v, int lane) { return __shfl_sync(0xffffffffu, v, lane); }
+__device__ __forceinline__ V3<double> from_lane(V3<double> v, int lane) {
+  return {from_lane(v.x, lane), from_lane(v.y, lane), from_lane(v.z, lane)};
+}
 
 // Interpolate the 5 derivative vectors a_1, a_2, a_{1,1}, a_{2,2}, a_{1,2} at Gauss point g from
 // 16 DOF triples (shared memory, [16][3]).
@@ -101,20 +115,25 @@ __device__ __forceinline__ void interp5(const R* sphi, const S* qv, int g, V3<R>
 // and d2-th derivatives of the factors. w[(d * 4 + g) * 4 + a] holds the d-th xi-derivative of
 // factor a at Gauss abscissa g (d = 0, 1, 2): herm(p, r, theta_g, d) dxi^r / dxi^d.
 // ------------------------------------------------------------------------------------------
-constexpr int kHerm1D = 48;
-
-template <typename R>
-__device__ __forceinline__ void build_hermite_1d(R* w, double dxi, int tid, int nthreads) {
+__device__ __forceinline__ double hermite_1d(double dxi, int e) {
   double th[4], wt[4];
   gauss_unit(th, wt);
-  for (int e = tid; e < kHerm1D; e += nthreads) {
-    const int d = e / 16, gi = (e / 4) % 4, a = e % 4;
-    const int p = a >> 1, r = a & 1;
-    double v = herm(p, r, th[gi], d);
-    if (r) v *= dxi;
-    for (int i = 0; i < d; ++i) v /= dxi;
-    w[e] = (R)v;
-  }
+  const int d = e / 16, gi = (e / 4) % 4, a = e % 4;
+  const int p = a >> 1, r = a & 1;
+  double v = herm(p, r, th[gi], d);
+  if (r) v *= dxi;
+  for (int i = 0; i < d; ++i) v /= dxi;
+  return v;
+}
+
+// Entry e of the table that the kernels read: shape functions (from sphi), Gauss weights, 1D factors. Formed
+// once per shell: with their FP64 divisions the factors cost a CTA of the energy kernel 6% of its
+// FP64 instructions, and 2 us before its first patch, when it built them itself.
+__device__ __forceinline__ double shape_table_entry(const double* sphi, double d1, double d2, int e) {
+  if (e < kPhiSize) return sphi[e];
+  if (e < kPhiHerm) return gauss_weight(e - kPhiSize, d1, d2);
+  const int h = e - kPhiHerm;
+  return h < kHerm1D ? hermite_1d(d1, h) : hermite_1d(d2, h - kHerm1D);
 }
 
 // FP32 Hessian stage: per Gauss point g and DOF triple J the five derivative values phi_,k and
@@ -122,11 +141,11 @@ __device__ __forceinline__ void build_hermite_1d(R* w, double dxi, int tid, int 
 // so that a lane reads them with two 16-byte loads.
 constexpr int kPhiGauss = 16 * 16 * 8;
 
-// Elements of the element kernels' shared memory before the per-warp areas: shape table, the two
-// 1D factor tables (theta^1, theta^2) and, for FP32, the per-Gauss-point table sphg
+// Elements of the element kernels' shared memory before the per-warp areas: shape table with its
+// 1D factors and, for FP32, the per-Gauss-point table sphg
 template <typename R>
 __host__ __device__ constexpr int elem_table_elems() {
-  return ((kPhiTable + 3) & ~3) + 2 * kHerm1D + (sizeof(R) == 4 ? kPhiGauss : 0);
+  return ((kPhiTable + 3) & ~3) + (sizeof(R) == 4 ? kPhiGauss : 0);
 }
 
 // Fills sphg from the shape table (FP32 kernels; all threads of the CTA, after sphi is complete).
@@ -148,7 +167,7 @@ constexpr int kRestFields = 13;
 // [16][15] gradient vectors (all shared). restgp is SoA over S = (total patches) * 16 entries.
 // Returns the patch energy in every lane.
 // ------------------------------------------------------------------------------------------
-constexpr int kEgPatches = 8;   // patches per CTA (128 threads)
+constexpr int kEgPatches = 8;   // patches per CTA (128 threads; 4 with a warp per patch)
 
 // DOF index (corner * 12 + kind * 3 + c) of the factor pair (a, b), component c
 __device__ __forceinline__ int dof_of(int a, int b, int c) {
@@ -214,29 +233,29 @@ __device__ __forceinline__ double eg64_patch(const double* w1, const double* w2,
     if (!(nn > 0.0)) atomicOr(err, ERRBIT_DEGENERATE);
     else isqa = rsqrt(nn);
     V3<double> a3 = isqa * n;
-    double b11 = dot(v[2], a3), b22 = dot(v[3], a3), b12 = dot(v[4], a3);
-    double al[3] = {0.5 * (dot(a1, a1) - ab11), 0.5 * (dot(a2, a2) - ab22), dot(a1, a2) - ab12};
-    double be[3] = {b11 - bb11, b22 - bb22, 2.0 * (b12 - bb12)};
+    // strains; the rest value opens each sum of products, so that subtracting it costs no instruction
+    const double al[3] = {0.5 * dot_less(a1, a1, ab11), 0.5 * dot_less(a2, a2, ab22), dot_less(a1, a2, ab12)};
+    const double be[3] = {dot_less(v[2], a3, bb11), dot_less(v[3], a3, bb22), 2.0 * dot_less(v[4], a3, bb12)};
     double sg[3] = {H00 * al[0] + H01 * al[1] + H02 * al[2], H01 * al[0] + H11 * al[1] + H12 * al[2],
                     H02 * al[0] + H12 * al[1] + H22 * al[2]};
     double mm[3] = {H00 * be[0] + H01 * be[1] + H02 * be[2], H01 * be[0] + H11 * be[1] + H12 * be[2],
                     H02 * be[0] + H12 * be[1] + H22 * be[2]};
-    const double h3 = h * h * h;
-    e = wgt * (0.5 * h * (al[0] * sg[0] + al[1] * sg[1] + al[2] * sg[2]) +
-               h3 * (1.0 / 24.0) * (be[0] * mm[0] + be[1] * mm[1] + be[2] * mm[2]));
+    const double wh = wgt * h, ws = wgt * (h * h * h * (1.0 / 12.0));
+    e = 0.5 * (wh * (al[0] * sg[0] + al[1] * sg[1] + al[2] * sg[2]) +
+               ws * (be[0] * mm[0] + be[1] * mm[1] + be[2] * mm[2]));
     if (grad) {
-      const double s = h3 * (1.0 / 12.0);
-      V3<double> ct = mm[0] * v[2] + mm[1] * v[3] + (2.0 * mm[2]) * v[4];
-      double bt = dot(ct, a3);
-      V3<double> t1 = cross(a2, a3), t2 = cross(a3, a1);
-      V3<double> e1 = isqa * (cross(a2, ct) - bt * t1);
-      V3<double> e2 = isqa * (cross(ct, a1) - bt * t2);
-      V3<double> G[5];
-      G[0] = wgt * (h * (sg[0] * a1 + sg[2] * a2) + s * e1);
-      G[1] = wgt * (h * (sg[1] * a2 + sg[2] * a1) + s * e2);
-      G[2] = (wgt * s * mm[0]) * a3;
-      G[3] = (wgt * s * mm[1]) * a3;
-      G[4] = (wgt * s * 2.0 * mm[2]) * a3;
+      // with the weights in sigma and m: K = (c~ - (c~ . a3) a3) / sqrt(a) carries both directions' normal
+      // derivative, a_2 x K and K x a_1
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        sg[k] *= wh;
+        mm[k] *= ws;
+      }
+      mm[2] += mm[2];
+      const V3<double> ct = mm[0] * v[2] + mm[1] * v[3] + mm[2] * v[4];
+      const V3<double> K = isqa * (ct - dot(ct, a3) * a3);
+      const V3<double> G[5] = {cross_plus(a2, K, sg[0] * a1 + sg[2] * a2), cross_plus(K, a1, sg[1] * a2 + sg[2] * a1),
+                               mm[0] * a3, mm[1] * a3, mm[2] * a3};
 #pragma unroll
       for (int k = 0; k < 5; ++k) {
         sG[g][k * 3 + 0] = G[k].x;
@@ -269,6 +288,137 @@ __device__ __forceinline__ double eg64_patch(const double* w1, const double* w2,
   if (active && grad) {
     // transpose of the theta^1 contraction: dE/dQ[a][b][c] = sum_{d1, gi} w1[d1][gi][a] U[d1][gi][b][c]
     for (int l = g; l < 48; l += 16) {
+      const int corner = l / 12, kind = (l / 3) % 4, c = l % 3;
+      const int a = 2 * (corner & 1) + (kind & 1), b = 2 * (corner >> 1) + (kind >> 1);
+      double s = 0.0;
+#pragma unroll
+      for (int dg = 0; dg < 12; ++dg) s = __fma_rn(w1[dg * 4 + a], sT[(dg * 4 + b) * 3 + c], s);
+      atomicAdd(&grad[(size_t)nd[corner] * 12 + kind * 3 + c], s);
+    }
+  }
+  __syncwarp();
+  return ep;
+}
+
+// The same for one patch by a whole warp (lane = 16 half + Gauss point), for launches that leave the FP64
+// pipes short of patches: what the two directions (or the membrane and the bending part) have alike is done
+// once per half. 215 FP64 instructions in a chain, where half a warp takes 330 for its patch and its
+// neighbour's: shorter for a warp that has one patch, longer for one that has many. sq, sT, sG as above,
+// one set per warp. All lanes call it; returns the patch energy in every lane.
+__device__ __forceinline__ double eg64_patch_warp(const double* w1, const double* w2, double* sq, double* sT,
+                                                  double (*sG)[15], int p, bool active, int lane, const int nd[4],
+                                                  const double* __restrict__ q,
+                                                  const double* __restrict__ dir, double step,
+                                                  const double* __restrict__ restgp, size_t S, double h,
+                                                  double* __restrict__ grad, int* err) {
+  const int half = lane >> 4, g = lane & 15, g1 = g & 3, g2 = g >> 2;
+  if (active) {
+    for (int l = lane; l < 48; l += 32) {
+      size_t a = (size_t)nd[l / 12] * 12 + (l % 12);
+      double v = q[a];
+      if (dir) v = __fma_rn(step, dir[a], v);
+      sq[l] = v;
+    }
+  }
+  __syncwarp();
+  if (active) {
+    for (int e = lane; e < 144; e += 32) {
+      const int c = e % 3, b = (e / 3) % 4, dg = e / 12;
+      double t = 0.0;
+#pragma unroll
+      for (int a = 0; a < 4; ++a) t = __fma_rn(w1[dg * 4 + a], sq[dof_of(a, b, c)], t);
+      sT[e] = t;
+    }
+  }
+  __syncwarp();
+  double e = 0.0;
+  {
+    // theta^2: half 0 the kinds (1,0), (0,1), half 1 (2,0), (0,2), both (1,1)
+    V3<double> m[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const int d1 = k == 2 ? 1 : k == 1 ? 0 : 1 + half, d2 = k == 2 ? 1 : k == 0 ? 0 : 1 + half;
+      double x = 0.0, y = 0.0, z = 0.0;
+      const double* T = sT + (d1 * 4 + g1) * 12;
+      const double* W = w2 + (d2 * 4 + g2) * 4;
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        x = __fma_rn(W[b], T[b * 3 + 0], x);
+        y = __fma_rn(W[b], T[b * 3 + 1], y);
+        z = __fma_rn(W[b], T[b * 3 + 2], z);
+      }
+      m[k] = mk<double>(x, y, z);
+    }
+    V3<double> a1 = from_lane(m[0], g), a2 = from_lane(m[1], g);
+    const V3<double> x11 = from_lane(m[0], 16 + g), x22 = from_lane(m[1], 16 + g), x12 = m[2];
+    const size_t o = (size_t)(active ? p : 0) * 16 + g;
+    // rest values of the half's strain: membrane a_bar (half 0), bending b_bar (half 1)
+    const double r11 = restgp[(half * 3 + 0) * S + o], r22 = restgp[(half * 3 + 1) * S + o];
+    const double r12 = restgp[(half * 3 + 2) * S + o];
+    const double H00 = restgp[6 * S + o], H01 = restgp[7 * S + o], H02 = restgp[8 * S + o];
+    const double H11 = restgp[9 * S + o], H12 = restgp[10 * S + o], H22 = restgp[11 * S + o];
+    const double wgt = restgp[12 * S + o];
+    V3<double> n = cross(a1, a2);
+    const double nn = dot(n, n);
+    double isqa = 1.0;
+    if (nn > 0.0) isqa = rsqrt(nn);
+    else if (active) atomicOr(err, ERRBIT_DEGENERATE);
+    V3<double> a3 = isqa * n;
+    const V3<double> y1 = half ? a3 : a1, y2 = half ? a3 : a2;
+    const V3<double> z1 = half ? x11 : a1, z2 = half ? x22 : a2, z3 = half ? x12 : a1;
+    const double f = half ? 1.0 : 0.5;
+    const double st[3] = {f * dot_less(z1, y1, r11), f * dot_less(z2, y2, r22), (f + f) * dot_less(z3, y2, r12)};
+    double t[3] = {H00 * st[0] + H01 * st[1] + H02 * st[2], H01 * st[0] + H11 * st[1] + H12 * st[2],
+                   H02 * st[0] + H12 * st[1] + H22 * st[2]};
+    const double w = wgt * (half ? h * h * h * (1.0 / 12.0) : h);
+    if (active) e = 0.5 * w * (st[0] * t[0] + st[1] * t[1] + st[2] * t[2]);
+    if (grad) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) t[k] *= w;
+      const double s1 = from_lane(t[0], g), s2 = from_lane(t[1], g), s12 = from_lane(t[2], g);
+      const double m0 = from_lane(t[0], 16 + g), m1 = from_lane(t[1], 16 + g);
+      double m2 = from_lane(t[2], 16 + g);
+      m2 += m2;
+      const V3<double> ct = m0 * x11 + m1 * x22 + m2 * x12;
+      V3<double> K = isqa * (ct - dot(ct, a3) * a3);
+      // half 0: sigma_1 a_1 + sigma_12 a_2 + a_2 x K, half 1: sigma_2 a_2 + sigma_12 a_1 - a_1 x K
+      const V3<double> P = half ? a1 : a2, own = half ? a2 : a1;
+      if (half) K = mk<double>(-K.x, -K.y, -K.z);
+      const V3<double> Gk = cross_plus(P, K, (half ? s2 : s1) * own + s12 * P);
+      const V3<double> Gb = (half ? m1 : m0) * a3, G4 = m2 * a3;
+      sG[g][half * 3 + 0] = Gk.x;
+      sG[g][half * 3 + 1] = Gk.y;
+      sG[g][half * 3 + 2] = Gk.z;
+      sG[g][6 + half * 3 + 0] = Gb.x;
+      sG[g][6 + half * 3 + 1] = Gb.y;
+      sG[g][6 + half * 3 + 2] = Gb.z;
+      if (!half) {
+        sG[g][12] = G4.x;
+        sG[g][13] = G4.y;
+        sG[g][14] = G4.z;
+      }
+    }
+  }
+  double ep = e;
+  for (int o = 16; o > 0; o >>= 1) ep += __shfl_xor_sync(0xffffffffu, ep, o);
+  __syncwarp();
+  if (active && grad) {
+    for (int e2 = lane; e2 < 144; e2 += 32) {
+      const int c = e2 % 3, b = (e2 / 3) % 4, gi = (e2 / 12) % 4, d1 = e2 / 48;
+      const int ka = d1 == 0 ? 1 : d1 == 1 ? 0 : 2, da = d1 == 0 ? 1 : 0;
+      const int kb = d1 == 0 ? 3 : 4, db = d1 == 0 ? 2 : 1;
+      double u = 0.0;
+#pragma unroll
+      for (int gj = 0; gj < 4; ++gj) {
+        u = __fma_rn(w2[(da * 4 + gj) * 4 + b], sG[gj * 4 + gi][ka * 3 + c], u);
+        if (d1 < 2) u = __fma_rn(w2[(db * 4 + gj) * 4 + b], sG[gj * 4 + gi][kb * 3 + c], u);
+      }
+      sT[e2] = u;
+    }
+  }
+  __syncwarp();
+  if (active && grad) {
+    for (int l = lane; l < 48; l += 32) {
       const int corner = l / 12, kind = (l / 3) % 4, c = l % 3;
       const int a = 2 * (corner & 1) + (kind & 1), b = 2 * (corner >> 1) + (kind >> 1);
       double s = 0.0;
@@ -340,7 +490,7 @@ struct ElemArgs {
   const int* pblocks;
   const double* q;
   const double* rest;
-  double d1, d2, lam, mu, h, rho_h, mass_scale;
+  double lam, mu, h, rho_h, mass_scale;
   int pseudo;
   double* energy_p;
   double* grad_p;
@@ -351,7 +501,9 @@ struct ElemArgs {
   int* err;
   // FP64 energy and gradient at the same q in the same warps (FP32 kernel only; grad64 null: off):
   // energy64[p] = E_p, grad64 += dE/dq (zeroed by the caller); restgp: rest Gauss-point data [13][np][16]
+  // and herm64 the shell's FP64 1D factors
   const double* restgp;
+  const double* herm64;
   double* energy64;
   double* grad64;
 };

@@ -66,7 +66,7 @@ static_assert(sizeof(WarpSmemTc::Mb) >= 2 * 432 * sizeof(double), "FP64 scratch"
 static_assert(sizeof(WarpSmemTc) % 16 == 0 && offsetof(WarpSmemTc, Mb) % 16 == 0, "16-byte block loads");
 
 constexpr size_t kSmemBytes =
-    1024 + 2 * kPsiBytes + sizeof(float) * ((kPhiTable + 3) & ~3) + sizeof(WarpSmemTc) * kWarps;
+    1024 + 2 * kPsiBytes + sizeof(float) * kPhiHerm + sizeof(WarpSmemTc) * kWarps;
 // the resident CTAs of an SM: their tensor memory (512 columns per SM), their shared memory
 // (228 KB per SM, 1 KB of it reserved per CTA, about 1 KB of static arrays each) and their
 // registers (64K per SM at the 168 the launch bounds allow)
@@ -109,23 +109,25 @@ __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.
 __device__ __forceinline__ int cd_c(int cd) { return cd < 3 ? 0 : (cd < 5 ? 1 : 2); }
 __device__ __forceinline__ int cd_d(int cd) { return cd < 3 ? cd : (cd < 5 ? cd - 2 : 2); }
 
+// kOneEach: no warp has a second patch, so the FP64 evaluation (A.grad64) takes a warp per patch; a form
+// of its own, because the two evaluations in one kernel cost it registers.
+template <bool kOneEach>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_element_tc(ElemArgs A, unsigned polls) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t bar_mma;
   __shared__ uint32_t tmem_slot;
-  __shared__ double w1_64[kHerm1D], w2_64[kHerm1D];
+  __shared__ double w1_64[2 * kHerm1D];
+  const double* const w2_64 = w1_64 + kHerm1D;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const uint32_t raw = tc::smem_addr(smem_raw);
   const uint32_t bbase = (raw + 1023u) & ~1023u;
   unsigned char* bptr = smem_raw + (bbase - raw);
   float* sphi = reinterpret_cast<float*>(bptr + 2 * kPsiBytes);
-  WarpSmemTc* Ws = reinterpret_cast<WarpSmemTc*>(sphi + ((kPhiTable + 3) & ~3));
+  WarpSmemTc* Ws = reinterpret_cast<WarpSmemTc*>(sphi + kPhiHerm);
 
-  load_shape_table<float>(sphi, reinterpret_cast<const float*>(A.phi));
-  if (A.grad64) {
-    build_hermite_1d<double>(w1_64, A.d1, tid, kThreads);
-    build_hermite_1d<double>(w2_64, A.d2, tid, kThreads);
-  }
+  load_shape_table<float>(sphi, reinterpret_cast<const float*>(A.phi), kPhiHerm);
+  if (A.grad64)
+    for (int e = tid; e < 2 * kHerm1D; e += kThreads) w1_64[e] = A.herm64[e];
   __syncthreads();
   // B operand: Psi[(g, k)][I] at K index 24 gq + 4 k + gi (g = 4 gq + gi; k = 5: the value phi)
   for (int e = tid; e < 16 * 96; e += kThreads) {
@@ -162,7 +164,26 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_element_tc(ElemArgs A,
     const int it = base + wid;
     const bool active = it < total;
     const int p = active ? (A.plist ? A.plist[it] : it) : 0;
-    if (A.grad64 && (k2 & 1) == 0) {
+    if (kOneEach && A.grad64) {
+      // FP64 energy and gradient at the same q, a warp per patch: each warp has this patch only
+      double* scratch = reinterpret_cast<double*>(&W.Mb[0][0]);
+      int nd[4] = {0, 0, 0, 0};
+      if (active) {
+        const int4 pn = A.pnodes[p];
+        nd[0] = pn.x;
+        nd[1] = pn.y;
+        nd[2] = pn.z;
+        nd[3] = pn.w;
+      }
+      const double ep = eg64_patch_warp(w1_64, w2_64, scratch, scratch + 48,
+                                        reinterpret_cast<double(*)[15]>(scratch + 192), p, active, lane, nd, A.q,
+                                        nullptr, 0.0, A.restgp, (size_t)A.np * 16, A.h, A.grad64, A.err);
+      if (active && lane == 0) {
+        if (!isfinite(ep)) atomicOr(A.err, ERRBIT_NONFINITE);
+        A.energy64[p] = ep;
+      }
+      __syncwarp();
+    } else if (!kOneEach && A.grad64 && (k2 & 1) == 0) {
       // FP64 energy and gradient at the same q (as in k_element_full): every second patch of a
       // warp, its two half-warps evaluate that patch and the warp's next one
       const int hw = lane >> 4, g = lane & 15;
@@ -331,8 +352,8 @@ shell_status launch_full_tc(Shell& s, const ElemArgs& A, int work) {
   static bool attr_done[64] = {false};
   const int dev = s.device < 64 ? s.device : 63;
   if (!attr_done[dev]) {
-    BHEM_CUDA(cudaFuncSetAttribute(etc::k_element_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)etc::kSmemBytes));
+    for (auto k : {etc::k_element_tc<false>, etc::k_element_tc<true>})
+      BHEM_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)etc::kSmemBytes));
     attr_done[dev] = true;
   }
   if (work <= 0) return SHELL_OK;
@@ -342,7 +363,8 @@ shell_status launch_full_tc(Shell& s, const ElemArgs& A, int work) {
   int blocks = (work + etc::kWarps - 1) / etc::kWarps;
   const int cap = s.num_sms * etc::kCtasPerSm;
   if (blocks > cap) blocks = cap;
-  etc::k_element_tc<<<blocks, etc::kThreads, etc::kSmemBytes, s.stream>>>(A, (unsigned)s.wait_polls);
+  auto k = A.grad64 && work <= blocks * etc::kWarps ? etc::k_element_tc<true> : etc::k_element_tc<false>;
+  k<<<blocks, etc::kThreads, etc::kSmemBytes, s.stream>>>(A, (unsigned)s.wait_polls);
   BHEM_CUDA(cudaGetLastError());
   ++s.launches;
   return SHELL_OK;

@@ -303,7 +303,7 @@ extern "C" shell_status shell_create(const shell_grid* grid, const shell_materia
   }
   A(s->d_x, m); A(s->d_r, m); A(s->d_z, m); A(s->d_p, m); A(s->d_Ap, m);
   A(s->d_scal, 1); A(s->d_p32, m); A(s->d_x32, m); A(s->d_r32, m); A(s->d_z32, m); A(s->d_Ap32, m);
-  A(s->d_phi64, 1568); A(s->d_phi32, 1568);
+  A(s->d_phi64, kPhiTableCount); A(s->d_phi32, kPhiTableCount);
   A(s->d_qn, m); A(s->d_y, m); A(s->d_g, m); A(s->d_gin, m); A(s->d_d, m); A(s->d_Md, m);
   A(s->d_rhs, m); A(s->d_Ep, np); A(s->d_qwork, m); A(s->d_vwork, m); A(s->d_qfix, m); A(s->d_qmy, m);
   A(s->d_warm, m); A(s->d_mask, m); A(s->d_energy_tmp, 1);

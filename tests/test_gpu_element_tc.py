@@ -199,3 +199,22 @@ def test_tensor_core_hessians_match_ffma_on_every_patch_at_full_size(monkeypatch
     worst = float((d / ref).max())
     print(f"full-size tensor-core against FFMA: worst patch {worst:.2e}")
     assert worst <= 5e-6, worst
+
+
+# one patch per warp (a warp's whole FP64 evaluation) up to 3 CTAs of 4 warps on each SM, pairs of patches
+# beyond; 608 and 609 patches are the same line of the energy kernel
+@pytest.mark.parametrize("grid", [(1, 1), (32, 19), (29, 21), (48, 38), (73, 25), (61, 60)])
+@pytest.mark.parametrize("assembly", ["atomic", "color"])
+def test_fp64_energy_and_gradient_beside_the_hessian(monkeypatch, grid, assembly):
+    """Energy and gradient are FP64 whether they are asked for with the Hessian or without (other kernels, other
+    orders of the same sums) and by the allocation-free entry point (its own arithmetic): 1e-11, as there."""
+    from paper_2312_14839_gb300.bhem import energy_grad_noalloc
+    g, rest = S.flat_sheet(*grid)
+    q = dev(S.noisy(rest, 1e-3, 7).reshape(-1))
+    E0, G0 = torch.empty(1, dtype=torch.float64, device="cuda"), torch.empty_like(q)
+    energy_grad_noalloc(g, THIN, dev(rest.reshape(-1)), q, E0, G0)
+    with shell(monkeypatch, "tc", g, THIN, rest, assembly=assembly) as sh:
+        for want in (True, False):
+            E, G = sh.energy_grad_hess(q, want_hessian=want)
+            assert abs(float(E) - float(E0)) <= 1e-11 * abs(float(E0)), want
+            assert rel(host(G), host(G0)) <= 1e-11, want
