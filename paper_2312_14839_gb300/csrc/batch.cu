@@ -223,13 +223,13 @@ struct ElemBatchArgs {
   int* err;
 };
 
-__global__ void __launch_bounds__(32 * ElemCfg<float>::kWarps)
+__global__ void __launch_bounds__(32 * kElemWarps)
 k_element(ElemBatchArgs B) {
-  constexpr int NW = ElemCfg<float>::kWarps;
+  constexpr int NW = kElemWarps;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float* sphi = reinterpret_cast<float*>(smem_raw);
-  float* const sphg = sphi + ((kPhiTable + 3) & ~3);
-  WarpSmem<float>* Ws = reinterpret_cast<WarpSmem<float>*>(smem_raw + sizeof(float) * elem_table_elems<float>());
+  float* const sphg = sphi + kElemTable;
+  WarpSmem* Ws = reinterpret_cast<WarpSmem*>(smem_raw + sizeof(float) * kElemTableFloats);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   for (int it = blockIdx.x; it < B.n_items; it += gridDim.x) {
     const int4 item = B.items[it];
@@ -255,7 +255,7 @@ k_element(ElemBatchArgs B) {
     A.err = B.err;
     for (int k = item.y + wid; k < item.z; k += NW) {
       const int p = B.plist ? B.plist[k] : k;
-      element_patch<float>(sphi, sphi + kPhiHerm, sphg, Ws[wid], p, A, lane);
+      element_patch(sphi, sphi + kPhiHerm, sphg, Ws[wid], p, A, lane);
     }
   }
 }
@@ -1156,7 +1156,7 @@ shell_status zero_counters(shell_batch_s& b) {
   return SHELL_OK;
 }
 
-size_t elem_smem() { return sizeof(float) * elem_table_elems<float>() + sizeof(WarpSmem<float>) * ElemCfg<float>::kWarps; }
+size_t elem_smem() { return sizeof(float) * kElemTableFloats + sizeof(WarpSmem) * kElemWarps; }
 
 // The element kernel's dynamic shared memory limit, set once per device (outside any capture)
 shell_status element_attr(int device) {
@@ -1230,7 +1230,7 @@ shell_status assemble(shell_batch_s& b, const double* q, double mass_scale) {
       if (i1 <= i0) continue;
       A.items = b.color_items + i0;
       A.n_items = i1 - i0;
-      k_element<<<std::min(A.n_items, nsm * 8), 32 * ElemCfg<float>::kWarps, elem_smem(), b.stream>>>(A);
+      k_element<<<std::min(A.n_items, nsm * 8), 32 * kElemWarps, elem_smem(), b.stream>>>(A);
       BHEM_CUDA(cudaGetLastError());
       BL(b);
     }
@@ -1240,7 +1240,7 @@ shell_status assemble(shell_batch_s& b, const double* q, double mass_scale) {
   A.items = b.items;
   A.n_items = b.n_items;
   A.plist = nullptr;
-  k_element<<<std::min(A.n_items, nsm * 8), 32 * ElemCfg<float>::kWarps, elem_smem(), b.stream>>>(A);
+  k_element<<<std::min(A.n_items, nsm * 8), 32 * kElemWarps, elem_smem(), b.stream>>>(A);
   BHEM_CUDA(cudaGetLastError());
   BL(b);
   return SHELL_OK;

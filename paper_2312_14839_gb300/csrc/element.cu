@@ -12,6 +12,8 @@
 // K += T phi per column J.
 #include "element_impl.cuh"
 
+#include <algorithm>
+
 namespace bhem {
 
 // Shape table and Gauss weights of one shell, built once (FP64 arithmetic) into global memory.
@@ -192,85 +194,186 @@ shell_status launch_energy_grad64(Shell& s, const double* q, const double* dir, 
 }
 
 // ------------------------------------------------------------------------------------------
-// Heavy kernel: one warp per patch computes E, gradient and the 48x48 Hessian.
+// Heavy kernels: E, gradient and the 48x48 Hessian of a patch, in FP32 (FFMA form) by a warp, in FP64 by a CTA.
 // ------------------------------------------------------------------------------------------
-template <typename R>
-__global__ void __launch_bounds__(32 * ElemCfg<R>::kWarps)
+__global__ void __launch_bounds__(32 * kElemWarps)
 k_element_full(ElemArgs A) {
-  constexpr int NW = ElemCfg<R>::kWarps;
+  constexpr int NW = kElemWarps;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  R* sphi = reinterpret_cast<R*>(smem_raw);
-  R* w1d = sphi + kPhiHerm;
-  WarpSmem<R>* Ws = reinterpret_cast<WarpSmem<R>*>(smem_raw + sizeof(R) * elem_table_elems<R>());
-  R* sphg = sphi + ((kPhiTable + 3) & ~3);
-  load_shape_table<R>(sphi, reinterpret_cast<const R*>(A.phi));
+  float* sphi = reinterpret_cast<float*>(smem_raw);
+  float* w1d = sphi + kPhiHerm;
+  float* sphg = sphi + kElemTable;
+  WarpSmem* Ws = reinterpret_cast<WarpSmem*>(sphi + kElemTableFloats);
+  load_shape_table<float>(sphi, reinterpret_cast<const float*>(A.phi));
   __syncthreads();
-  if constexpr (sizeof(R) == 4) {
-    build_phi_gauss(sphg, sphi, threadIdx.x, blockDim.x);
-    __syncthreads();
-  }
+  build_phi_gauss(sphg, sphi, threadIdx.x, blockDim.x);
+  __syncthreads();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  WarpSmem<R>& W = Ws[wid];
+  WarpSmem& W = Ws[wid];
   const int total = A.plist ? A.plist_n : A.np;
   const int stride = gridDim.x * NW;
-  if constexpr (sizeof(R) == 4) {
-    if (A.grad64) {
-      // FP64 energy and gradient at the same q (the arithmetic of k_energy_grad64) in the warps of
-      // the FP32 Hessian: the FP64 pipe works while other warps issue the FP32 pass. Every second
-      // patch of a warp, its two half-warps evaluate that patch and the warp's next one, in the
-      // warp's Gauss-point-matrix area (free between patches; 2 x 432 doubles).
-      __shared__ double w1_64[2 * kHerm1D];
-      const double* const w2_64 = w1_64 + kHerm1D;
-      for (int e = threadIdx.x; e < 2 * kHerm1D; e += blockDim.x) w1_64[e] = A.herm64[e];
-      __syncthreads();
-      static_assert(sizeof(W.M) >= 2 * 432 * sizeof(double), "FP64 scratch fits the M_g area");
-      const int hw = lane >> 4, g = lane & 15;
-      double* scratch = reinterpret_cast<double*>(&W.M[0][0]) + hw * 432;
-      int k = 0;
-      for (int it = blockIdx.x * NW + wid; it < total; it += stride, ++k) {
-        if ((k & 1) == 0) {
-          const int itp = it + hw * stride;
-          const bool active = itp < total;
-          const int pp = active ? (A.plist ? A.plist[itp] : itp) : 0;
-          int nd[4] = {0, 0, 0, 0};
-          if (active) {
-            const int4 pn = A.pnodes[pp];
-            nd[0] = pn.x;
-            nd[1] = pn.y;
-            nd[2] = pn.z;
-            nd[3] = pn.w;
-          }
-          const double ep = eg64_patch(w1_64, w2_64, scratch, scratch + 48,
-                                       reinterpret_cast<double(*)[15]>(scratch + 192), pp, active, g, nd, A.q,
-                                       nullptr, 0.0, A.restgp, (size_t)A.np * 16, A.h, A.grad64, A.err);
-          if (active && g == 0) {
-            if (!isfinite(ep)) atomicOr(A.err, ERRBIT_NONFINITE);
-            A.energy64[pp] = ep;
-          }
-          __syncwarp();
+  if (A.grad64) {
+    // FP64 energy and gradient at the same q (the arithmetic of k_energy_grad64) in the warps of
+    // the FP32 Hessian: the FP64 pipe works while other warps issue the FP32 pass. Every second
+    // patch of a warp, its two half-warps evaluate that patch and the warp's next one, in the
+    // warp's Gauss-point-matrix area (free between patches; 2 x 432 doubles).
+    __shared__ double w1_64[2 * kHerm1D];
+    const double* const w2_64 = w1_64 + kHerm1D;
+    for (int e = threadIdx.x; e < 2 * kHerm1D; e += blockDim.x) w1_64[e] = A.herm64[e];
+    __syncthreads();
+    static_assert(sizeof(W.M) >= 2 * 432 * sizeof(double), "FP64 scratch fits the M_g area");
+    const int hw = lane >> 4, g = lane & 15;
+    double* scratch = reinterpret_cast<double*>(&W.M[0][0]) + hw * 432;
+    int k = 0;
+    for (int it = blockIdx.x * NW + wid; it < total; it += stride, ++k) {
+      if ((k & 1) == 0) {
+        const int itp = it + hw * stride;
+        const bool active = itp < total;
+        const int pp = active ? (A.plist ? A.plist[itp] : itp) : 0;
+        int nd[4] = {0, 0, 0, 0};
+        if (active) {
+          const int4 pn = A.pnodes[pp];
+          nd[0] = pn.x;
+          nd[1] = pn.y;
+          nd[2] = pn.z;
+          nd[3] = pn.w;
         }
-        element_patch<R>(sphi, w1d, sphg, W, A.plist ? A.plist[it] : it, A, lane);
+        const double ep = eg64_patch(w1_64, w2_64, scratch, scratch + 48,
+                                     reinterpret_cast<double(*)[15]>(scratch + 192), pp, active, g, nd, A.q,
+                                     nullptr, 0.0, A.restgp, (size_t)A.np * 16, A.h, A.grad64, A.err);
+        if (active && g == 0) {
+          if (!isfinite(ep)) atomicOr(A.err, ERRBIT_NONFINITE);
+          A.energy64[pp] = ep;
+        }
+        __syncwarp();
       }
-      return;
+      element_patch(sphi, w1d, sphg, W, A.plist ? A.plist[it] : it, A, lane);
     }
+    return;
   }
   for (int it = blockIdx.x * NW + wid; it < total; it += stride)
-    element_patch<R>(sphi, w1d, sphg, W, A.plist ? A.plist[it] : it, A, lane);
+    element_patch(sphi, w1d, sphg, W, A.plist ? A.plist[it] : it, A, lane);
 }
 
-template <typename R>
-static size_t elem_smem_bytes() {
-  return sizeof(R) * elem_table_elems<R>() + sizeof(WarpSmem<R>) * ElemCfg<R>::kWarps;
+// FP64: one CTA per patch, so that its four warps keep the SM's four FP64 pipes busy on grids of fewer patches
+// than pipes (a warp instruction takes 64 cycles of one pipe; shared-memory reads and integer work are free
+// beside it). The Gauss-point matrices are shared out by blocks, T = Phi^T M is formed once, eight Gauss
+// points at a time, and only the entries (I, c), (J, c') with I <= J of the symmetric K are summed:
+// 136 pairs x 9, ten a thread. About 2,100 FP64 instructions a warp; with a warp per patch, T formed
+// twice and K in full it was 13,000: 10 x 10 patches 450 us a pass, now 80.
+struct Elem64Smem {
+  double table[kPhiTable];
+  double u[48], qb[48];
+  double F[288];             // the fields after the theta^1 contraction
+  double M[16][kSym15];
+  double G[16][15];
+  double ms[16], en[16];
+  double T[8][16 * 45];      // T[I][c * 15 + l * 3 + c'] of eight Gauss points; then K[48][48]
+};
+constexpr int kTasks64 = 136 * 9, kPerThread64 = (kTasks64 + 127) / 128;
+
+__global__ void __launch_bounds__(128)
+k_element64(ElemArgs A) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  Elem64Smem& W = *reinterpret_cast<Elem64Smem*>(smem_raw);
+  const double* const sphi = W.table;
+  const double* const w1d = W.table + kPhiHerm;
+  load_shape_table<double>(W.table, reinterpret_cast<const double*>(A.phi));
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  // this thread's entries: offset of (I, c, c') in T and of J in the shape table; the 408 with c = c', which
+  // take the mass term, come first
+  int task[kPerThread64];
+#pragma unroll
+  for (int k = 0; k < kPerThread64; ++k) {
+    const int t = tid + 128 * k, cls = t / 408, c = t % 3, cp = (c + cls) % 3;
+    int rest = (t % 408) / 3, I = 0;
+    while (rest >= 16 - I) rest -= 16 - I++;
+    const int J = I + rest;
+    // of a diagonal pair, (c, c') with c > c' is the mirror of another entry
+    task[k] = t < kTasks64 && !(I == J && c > cp) ? (I * 45 + c * 15 + cp) | (J * kPhiStride) << 16 : -1;
+  }
+  const int total = A.plist ? A.plist_n : A.np;
+  for (int it = blockIdx.x; it < total; it += gridDim.x) {
+    const int p = A.plist ? A.plist[it] : it;
+    __syncthreads();
+    gather_patch<double>(W, p, A, tid, 128);
+    __syncthreads();
+    theta1_fields(w1d, W.qb, W.u, W.F, tid, 128);
+    __syncthreads();
+    {
+      const int half = lane >> 4, g = lane & 15;
+      V3<double> mine[5];
+      theta2_field(w1d + kHerm1D, W.F + 144 * half, g, mine);
+      const double wg = sphi[kPhiSize + g];
+      if (wid == 0) gauss_point_matrix64<kPart00>(mine, wg, W, g, half, A);
+      else if (wid == 1) gauss_point_matrix64<kPart01>(mine, wg, W, g, half, A);
+      else if (wid == 2) gauss_point_matrix64<kPart0l>(mine, wg, W, g, half, A);
+      else gauss_point_matrix64<kPartkl | kPartBy>(mine, wg, W, g, half, A);
+    }
+    __syncthreads();
+    patch_byproducts<double>(sphi, W, p, A, tid, 128);
+    if (!A.hess_p && !A.bsr) continue;
+    double acc[kPerThread64];
+#pragma unroll
+    for (int k = 0; k < kPerThread64; ++k) acc[k] = 0.0;
+    for (int g0 = 0; g0 < 16; g0 += 8) {
+      for (int e = tid; e < 8 * 45; e += 128) {
+        const int gl = e / 45;
+        t_column<double>(w1d, W.M[g0 + gl], W.T[gl], 45, g0 + gl, e % 45);
+      }
+      __syncthreads();
+#pragma unroll 1
+      for (int gl = 0; gl < 8; ++gl) {
+        const int g = g0 + gl;
+        const double* T = W.T[gl];
+#pragma unroll
+        for (int k = 0; k < kPerThread64; ++k) {
+          if (task[k] < 0) continue;
+          const int to = task[k] & 0xffff;
+          const double* phi = sphi + (task[k] >> 16) + g;
+          double a = acc[k];
+#pragma unroll
+          for (int l = 0; l < 5; ++l) a = __fma_rn(T[to + 3 * l], phi[(l + 1) * 16], a);
+          if (tid + 128 * k < 408) a = __fma_rn(W.ms[g] * sphi[(to / 45) * kPhiStride + g], phi[0], a);
+          acc[k] = a;
+        }
+      }
+      __syncthreads();
+    }
+    double* K = &W.T[0][0];
+#pragma unroll
+    for (int k = 0; k < kPerThread64; ++k) {
+      if (task[k] < 0) continue;
+      const int to = task[k] & 0xffff, I = to / 45, J = (task[k] >> 16) / kPhiStride;
+      const int r = I * 3 + to % 45 / 15, q = J * 3 + to % 15;
+      K[r * 48 + q] = acc[k];
+      K[q * 48 + r] = acc[k];
+    }
+    __syncthreads();
+    if (A.hess_p) {
+      double* Hp = reinterpret_cast<double*>(A.hess_p) + (size_t)p * 2304;
+      for (int e = tid; e < 2304; e += 128) Hp[e] = K[e];
+    }
+    if (A.bsr) {
+      double* V = reinterpret_cast<double*>(A.bsr);
+      for (int e = tid; e < 2304; e += 128) {
+        const int ab = e / 144, w = e % 144;
+        double* dst = V + (size_t)A.pblocks[p * 16 + ab] * 144 + w;
+        const double v = K[((ab >> 2) * 12 + w / 12) * 48 + (ab & 3) * 12 + w % 12];
+        if (A.bsr_atomic) atomicAdd(dst, v);
+        else *dst += v;
+      }
+    }
+  }
 }
 
-template <typename R>
-static shell_status launch_full_t(Shell& s, const ElemArgs& A, int work) {
-  constexpr int NW = ElemCfg<R>::kWarps;
-  size_t smem = elem_smem_bytes<R>();
+static shell_status launch_full32(Shell& s, const ElemArgs& A, int work) {
+  constexpr int NW = kElemWarps;
+  const size_t smem = sizeof(float) * kElemTableFloats + sizeof(WarpSmem) * NW;
   static bool attr_done[64] = {false};
   int dev = s.device < 64 ? s.device : 63;
   if (!attr_done[dev]) {
-    BHEM_CUDA(cudaFuncSetAttribute(k_element_full<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    BHEM_CUDA(cudaFuncSetAttribute(k_element_full, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     attr_done[dev] = true;
   }
   if (work <= 0) return SHELL_OK;
@@ -278,10 +381,28 @@ static shell_status launch_full_t(Shell& s, const ElemArgs& A, int work) {
   int nsm = 0;
   BHEM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, s.device));
   int occ = 0;
-  BHEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_element_full<R>, 32 * NW, smem));
+  BHEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_element_full, 32 * NW, smem));
   int cap = nsm * (occ > 0 ? occ : 1) * 8;
   if (blocks > cap) blocks = cap;
-  k_element_full<R><<<blocks, 32 * NW, smem, s.stream>>>(A);
+  k_element_full<<<blocks, 32 * NW, smem, s.stream>>>(A);
+  BHEM_CUDA(cudaGetLastError());
+  ++s.launches;
+  return SHELL_OK;
+}
+
+static shell_status launch_full64(Shell& s, const ElemArgs& A, int work) {
+  constexpr size_t smem = sizeof(Elem64Smem);
+  static bool attr_done[64] = {false};
+  int dev = s.device < 64 ? s.device : 63;
+  if (!attr_done[dev]) {
+    BHEM_CUDA(cudaFuncSetAttribute(k_element64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    attr_done[dev] = true;
+  }
+  if (work <= 0) return SHELL_OK;
+  int nsm = 0, occ = 0;
+  BHEM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, s.device));
+  BHEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_element64, 128, smem));
+  k_element64<<<std::min(work, nsm * std::max(1, occ)), 128, smem, s.stream>>>(A);
   BHEM_CUDA(cudaGetLastError());
   ++s.launches;
   return SHELL_OK;
@@ -290,12 +411,9 @@ static shell_status launch_full_t(Shell& s, const ElemArgs& A, int work) {
 // element_tc.cu: the FP32 pass with the tensor-core contraction (same arguments and outputs)
 shell_status launch_full_tc(Shell& s, const ElemArgs& A, int work);
 
-template <typename R>
-static shell_status launch_full_pick(Shell& s, const ElemArgs& A, int work) {
-  if constexpr (sizeof(R) == 4) {
-    if (s.elem_tc) return launch_full_tc(s, A, work);
-  }
-  return launch_full_t<R>(s, A, work);
+static shell_status launch_full_pick(Shell& s, bool fp64, const ElemArgs& A, int work) {
+  if (fp64) return launch_full64(s, A, work);
+  return s.elem_tc ? launch_full_tc(s, A, work) : launch_full32(s, A, work);
 }
 
 shell_status launch_element_full(Shell& s, const double* q, bool fp64, const ElemOutputs& out) {
@@ -333,12 +451,12 @@ shell_status launch_element_full(Shell& s, const double* q, bool fp64, const Ele
       ElemArgs Ac = A;
       Ac.plist = s.d_color_list + b;
       Ac.plist_n = e - b;
-      BHEM_TRY(fp64 ? launch_full_t<double>(s, Ac, e - b) : launch_full_pick<float>(s, Ac, e - b));
+      BHEM_TRY(launch_full_pick(s, fp64, Ac, e - b));
     }
     return SHELL_OK;
   }
   A.bsr_atomic = 1;
-  return fp64 ? launch_full_t<double>(s, A, A.np) : launch_full_pick<float>(s, A, A.np);
+  return launch_full_pick(s, fp64, A, A.np);
 }
 
 }  // namespace bhem

@@ -141,12 +141,10 @@ __device__ __forceinline__ double shape_table_entry(const double* sphi, double d
 // so that a lane reads them with two 16-byte loads.
 constexpr int kPhiGauss = 16 * 16 * 8;
 
-// Elements of the element kernels' shared memory before the per-warp areas: shape table with its
-// 1D factors and, for FP32, the per-Gauss-point table sphg
-template <typename R>
-__host__ __device__ constexpr int elem_table_elems() {
-  return ((kPhiTable + 3) & ~3) + (sizeof(R) == 4 ? kPhiGauss : 0);
-}
+// Floats of the FP32 element kernels' shared memory before the per-warp areas: shape table with its
+// 1D factors, and the per-Gauss-point table sphg
+constexpr int kElemTable = (kPhiTable + 3) & ~3;
+constexpr int kElemTableFloats = kElemTable + kPhiGauss;
 
 // Fills sphg from the shape table (FP32 kernels; all threads of the CTA, after sphi is complete).
 __device__ __forceinline__ void build_phi_gauss(float* sphg, const float* sphi, int tid, int nthreads) {
@@ -432,11 +430,9 @@ __device__ __forceinline__ double eg64_patch_warp(const double* w1, const double
 }
 
 // ------------------------------------------------------------------------------------------
-// Heavy kernel: one warp per patch computes E, gradient and the 48x48 Hessian.
+// Heavy kernels: E, gradient and the 48x48 Hessian of a patch, in FP32 by a warp, in FP64 by a CTA.
 // ------------------------------------------------------------------------------------------
-template <typename R> struct ElemCfg;
-template <> struct ElemCfg<float> { static constexpr int kWarps = 4, kJP = 8; };
-template <> struct ElemCfg<double> { static constexpr int kWarps = 2, kJP = 4; };
+constexpr int kElemWarps = 4;   // patches in flight per CTA of the FP32 kernels
 
 // Packed upper triangle of a symmetric 15x15 matrix (120 entries), row-major.
 constexpr int kSym15 = 120;
@@ -465,20 +461,16 @@ __host__ __device__ constexpr BlkOff blk_off(int K1, int x, int L1, int y) {
                           K1 != L1 ? cd_index(x, x) * kBlk + L1 * kBlkRow + K1 : -1};
 }
 
-// Row stride of T: FP32 rows are padded to 52 (16-byte aligned, and the rows that 8 lanes read
-// together with 16-byte loads fall in distinct banks).
-template <typename R> struct TStride { static constexpr int v = 45; };
-template <> struct TStride<float> { static constexpr int v = 52; };
+constexpr int kTStride = 52;   // row stride of T: 16-byte aligned rows, and 8 lanes' 16-byte reads in distinct banks
 
-template <typename R>
 struct WarpSmem {
-  R u[48];        // displacement q - rest
-  R qb[48];       // rest DOFs
-  R M[16][kSym15];   // M_g per Gauss point (symmetric 15x15, packed upper triangle)
-  R T[16 * TStride<R>::v];   // T[I][c*15 + l*3 + c'] of the current Gauss point
-  R G[16][15];    // gradient vectors per Gauss point
-  R ms[16];       // mass_scale * rho h * W sqrt(a_bar) per Gauss point
-  R en[16];       // energy per Gauss point
+  float u[48];        // displacement q - rest
+  float qb[48];       // rest DOFs
+  float M[16][kSym15];     // M_g per Gauss point (symmetric 15x15, packed upper triangle)
+  float T[16 * kTStride];  // T[I][c*15 + l*3 + c'] of the current Gauss point
+  float G[16][15];    // gradient vectors per Gauss point
+  float ms[16];       // mass_scale * rho h * W sqrt(a_bar) per Gauss point
+  float en[16];       // energy per Gauss point
 };
 
 struct ElemArgs {
@@ -508,9 +500,39 @@ struct ElemArgs {
   double* grad64;
 };
 
+// Parameter derivatives a_1, a_2, x_,11, x_,22, x_,12 of one field (half 0: rest, half 1: displacement) at
+// the lane's Gauss point g, sum-factorised: T holds the field contracted along theta^1 (theta1_fields).
+__device__ __forceinline__ void theta2_field(const double* w2, const double* T, int g, V3<double> (&out)[5]) {
+  using R = double;
+  constexpr int kd1[5] = {1, 0, 2, 0, 1}, kd2[5] = {0, 1, 0, 2, 1};
+  const int g1 = g & 3, g2 = g >> 2;
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    const R* t = T + (kd1[k] * 4 + g1) * 12;
+    const R* w = w2 + (kd2[k] * 4 + g2) * 4;
+    V3<R> v = w[0] * mk<R>(t[0], t[1], t[2]);
+#pragma unroll
+    for (int b = 1; b < 4; ++b) v = v + w[b] * mk<R>(t[b * 3], t[b * 3 + 1], t[b * 3 + 2]);
+    out[k] = v;
+  }
+}
+
+// T[f * 144 + ((d1 * 4 + g1) * 4 + b) * 3 + c] = sum_a w1[d1][g1][a] field_f[a][b][c], f = 0: rest, 1: displacement
+__device__ __forceinline__ void theta1_fields(const double* w1, const double* qb, const double* u, double* T, int tid,
+                                              int nthreads) {
+  using R = double;
+  for (int e = tid; e < 288; e += nthreads) {
+    const int f = e / 144, k = e % 144, c = k % 3, b = (k / 3) % 4, dg = k / 12;
+    const R* x = f ? u : qb;
+    R t = w1[dg * 4] * x[dof_of(0, b, c)];
+#pragma unroll
+    for (int a = 1; a < 4; ++a) t += w1[dg * 4 + a] * x[dof_of(a, b, c)];
+    T[e] = t;
+  }
+}
+
 // Builds M_g (15x15) and the per-point energy, gradient vectors and mass weight for Gauss
-// point g of the warp's patch. kSplit = false (FP64 kernel): lanes 0..15, lane = g, every block.
-// kSplit = true (FP32 kernel): all 32 lanes, lane g and lane g + 16 share Gauss point g. The
+// point g of the warp's patch (FP32): lane g and lane g + 16 share Gauss point g. The
 // energy is unchanged when the two parameter directions are exchanged, so its Hessian
 // blocks of the exchanged frame are those of the original one with the derivative kinds relabeled
 // (xi^1 <-> xi^2: a_1 <-> a_2, x_,11 <-> x_,22, x_,12 fixed; sigma(k) = 1, 0, 3, 2, 4). Half 0 (the
@@ -518,11 +540,14 @@ struct ElemArgs {
 // instructions in the exchanged frame, which gives the blocks (sigma(k), sigma(l)) with k in
 // {1, 3}: together all 15 blocks. Half 1 discards the three blocks that map onto themselves
 // ((0, 1), (2, 3), (4, 4)) and the by-products (energy, gradient vectors, mass weight).
-template <typename R, bool kSplit, bool kBlocks = false, class WS = WarpSmem<R>>
-__device__ __forceinline__ void gauss_point_matrix(const R* sphi, WS& W, int g, int half,
-                                                   const ElemArgs& A) {
+// Every term is multiplied out entry by entry, zero rows of B included. Gathered as gauss_point_matrix64 does, or
+// with the zeros left out, a pass over 256 x 256 patches takes 778 or 813 us instead of 844, but roundings of
+// the FP32 Hessian move with it, and a solve of a set number of iterations shows them.
+template <bool kBlocks, class WS>
+__device__ __forceinline__ void gauss_point_matrix(const float* sphi, WS& W, int g, int half, const ElemArgs& A) {
+  using R = float;
   V3<R> ub[5], uu[5];   // rest a_bar_1, a_bar_2, x_bar_{,11}, x_bar_{,22}, x_bar_{,12}; displacement derivatives
-  if constexpr (kSplit) {
+  {
     // both halves need both fields at the same Gauss point: half 0 interpolates the rest DOFs,
     // half 1 the displacement, and they exchange (lane g <-> g + 16)
     V3<R> mine[5];
@@ -535,9 +560,6 @@ __device__ __forceinline__ void gauss_point_matrix(const R* sphi, WS& W, int g, 
       ub[k] = half ? other : mine[k];
       uu[k] = half ? mine[k] : other;
     }
-  } else {
-    interp5<R, R>(sphi, W.qb, g, ub);
-    interp5<R, R>(sphi, W.u, g, uu);
   }
   {
     // half 1: exchange the parameter directions (selects, no divergent branch)
@@ -658,7 +680,7 @@ __device__ __forceinline__ void gauss_point_matrix(const R* sphi, WS& W, int g, 
       for (int x = 0; x < 3; ++x)
 #pragma unroll
         for (int y = 0; y < 3; ++y) {
-          if (kSplit && (k == 1 || k == 3)) continue;   // half 1 produces these in the exchanged frame
+          if (k == 1 || k == 3) continue;   // half 1 produces these in the exchanged frame
           if (k == l && y < x) continue;
           R v = s * (comp(Bb[k][0], x) * comp(Qb[l][0], y) + comp(Bb[k][1], x) * comp(Qb[l][1], y) +
                      comp(Bb[k][2], x) * comp(Qb[l][2], y));
@@ -719,34 +741,219 @@ __device__ __forceinline__ void gauss_point_matrix(const R* sphi, WS& W, int g, 
         }
 }
 
-template <typename R>
-__device__ __forceinline__ void atomic_add_row12(R* dst, const R* v);
+// The same in FP64 (mine: the half's field, theta2_field), split between the halves of a warp in the same way.
+// The terms of App. B.2 are gathered before they are multiplied out: with a_3 the only vector of the second-
+// derivative rows, blocks (0, l >= 2) are one product per entry and (k >= 2, l) are scalings of
+// a_3 a_3^T; H B of the second direction follows from the first one's by symmetry; the exact Hessian's
+// terms in t_1, t_2, a_1, a_2 join vectors that the other terms multiply anyway. About 450 operations a
+// lane, where all B and H B multiplied out entry by entry, zeros included, took 1,150.
+//
+// PART: what this call computes (kPartBlocks: the blocks by bit, in the order below; kPartBy: by-products),
+// for warps that share a Gauss point.
+constexpr int kPart00 = 1, kPart01 = 2, kPart0l = 4, kPartkl = 8, kPartBy = 16;
 
-template <>
-__device__ __forceinline__ void atomic_add_row12<float>(float* dst, const float* v) {
+template <int PART, class WS>
+__device__ __forceinline__ void gauss_point_matrix64(const V3<double> (&mine)[5], double wg, WS& W, int g, int half,
+                                                     const ElemArgs& A) {
+  using R = double;
+  V3<R> ub[5], uu[5];   // rest a_bar_1, a_bar_2, x_bar_{,11}, x_bar_{,22}, x_bar_{,12}; displacement derivatives
+  // both halves need both fields, half 1 with the parameter directions exchanged
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    const V3<R> other = mk<R>(__shfl_xor_sync(0xffffffffu, mine[k].x, 16),
+                              __shfl_xor_sync(0xffffffffu, mine[k].y, 16),
+                              __shfl_xor_sync(0xffffffffu, mine[k].z, 16));
+    ub[k] = half ? other : mine[k];
+    uu[k] = half ? mine[k] : other;
+  }
+  {
+    const bool x = half != 0;
+    const V3<R> b0 = ub[0], b2 = ub[2], d0 = uu[0], d2 = uu[2];
+    ub[0] = x ? ub[1] : b0;
+    ub[1] = x ? b0 : ub[1];
+    ub[2] = x ? ub[3] : b2;
+    ub[3] = x ? b2 : ub[3];
+    uu[0] = x ? uu[1] : d0;
+    uu[1] = x ? d0 : uu[1];
+    uu[2] = x ? uu[3] : d2;
+    uu[3] = x ? d2 : uu[3];
+  }
+  const V3<R> ab1 = ub[0], ab2 = ub[1];
+  const V3<R> a1 = ab1 + uu[0], a2 = ab2 + uu[1];
+  V3<R> c[3] = {ub[2] + uu[2], ub[3] + uu[3], ub[4] + uu[4]};
+  // rest metric, contravariant metric, Voigt H (App. B.1)
+  R ab11 = dot(ab1, ab1), ab22 = dot(ab2, ab2), ab12 = dot(ab1, ab2);
+  R det = ab11 * ab22 - ab12 * ab12;
+  if (!(det > (R)0)) { atomicOr(A.err, ERRBIT_DEGENERATE); det = (R)1; }
+  R sqab = sqrt(det);
+  V3<R> ab3 = ((R)1 / sqab) * cross(ab1, ab2);
+  const R idet = (R)1 / det;
+  R ai11 = ab22 * idet, ai22 = ab11 * idet, ai12 = -ab12 * idet;
+  const R lam = (R)A.lam, mu = (R)A.mu, h = (R)A.h;
+  const R H00 = (lam + 2 * mu) * ai11 * ai11, H01 = lam * ai11 * ai22 + 2 * mu * ai12 * ai12;
+  const R H02 = (lam + 2 * mu) * ai11 * ai12, H11 = (lam + 2 * mu) * ai22 * ai22;
+  const R H12 = (lam + 2 * mu) * ai12 * ai22, H22 = (lam + mu) * ai12 * ai12 + mu * ai11 * ai22;
+  // deformed normal
+  V3<R> n = cross(a1, a2);
+  R sqa = sqrt(dot(n, n));
+  if (!(sqa > (R)0)) { atomicOr(A.err, ERRBIT_DEGENERATE); sqa = (R)1; }
+  const R isqa = (R)1 / sqa;
+  V3<R> a3 = isqa * n;
+  // strains from displacements (a_ab - a_bar_ab = a_bar_a.u_b + u_a.a_bar_b + u_a.u_b)
+  R al[3] = {dot(ab1, uu[0]) + (R)0.5 * dot(uu[0], uu[0]), dot(ab2, uu[1]) + (R)0.5 * dot(uu[1], uu[1]),
+             dot(ab1, uu[1]) + dot(uu[0], ab2) + dot(uu[0], uu[1])};
+  V3<R> da3 = a3 - ab3;
+  R br[3];
+#pragma unroll
+  for (int m = 0; m < 3; ++m) br[m] = dot(uu[2 + m], a3) + dot(ub[2 + m], da3);   // b - b_bar
+  R be[3] = {br[0], br[1], (R)2 * br[2]};
+  const R sg[3] = {H00 * al[0] + H01 * al[1] + H02 * al[2], H01 * al[0] + H11 * al[1] + H12 * al[2],
+                   H02 * al[0] + H12 * al[1] + H22 * al[2]};
+  const R mm[3] = {H00 * be[0] + H01 * be[1] + H02 * be[2], H01 * be[0] + H11 * be[1] + H12 * be[2],
+                   H02 * be[0] + H12 * be[1] + H22 * be[2]};
+  const R wgt = wg * sqab;
+  const R s = h * h * h * ((R)1 / (R)12);
+  const R hw = wgt * h, sw = wgt * s;
+  if ((PART & kPartBy) && !half) {
+    if (A.energy_p)
+      W.en[g] = (R)0.5 * (hw * (al[0] * sg[0] + al[1] * sg[1] + al[2] * sg[2]) +
+                          sw * (be[0] * mm[0] + be[1] * mm[1] + be[2] * mm[2]));
+    W.ms[g] = (R)(A.mass_scale * A.rho_h) * wgt;
+  }
+  // d b_m = (Phi_,1 up_m + Phi_,2 vp_m + its second derivative a_3) dq
+  V3<R> t1 = cross(a2, a3), t2 = cross(a3, a1);
+  V3<R> up[3], vp[3];
+#pragma unroll
+  for (int m = 0; m < 3; ++m) {
+    const R b = dot(c[m], a3);
+    up[m] = isqa * (cross(a2, c[m]) - b * t1);
+    vp[m] = isqa * (cross(c[m], a1) - b * t2);
+  }
+  up[2] = (R)2 * up[2];
+  vp[2] = (R)2 * vp[2];
+  const R coef[3] = {mm[0], mm[1], (R)2 * mm[2]};
+  if ((PART & kPartBy) && A.grad_p && !half) {
+    // gradient vectors G_k = W sqrt(a_bar) (h B_alpha,k^T sigma + s B_beta,k^T m)
+    const V3<R> G[5] = {sw * (mm[0] * up[0] + mm[1] * up[1] + mm[2] * up[2]) + hw * (sg[0] * a1 + sg[2] * a2),
+                        sw * (mm[0] * vp[0] + mm[1] * vp[1] + mm[2] * vp[2]) + hw * (sg[1] * a2 + sg[2] * a1),
+                        (sw * coef[0]) * a3, (sw * coef[1]) * a3, (sw * coef[2]) * a3};
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      W.G[g][k * 3 + 0] = G[k].x;
+      W.G[g][k * 3 + 1] = G[k].y;
+      W.G[g][k * 3 + 2] = G[k].z;
+    }
+  }
+  R* const M = W.M[g];
+  // entry (x, y) of block (k, l), k in {0, 2, 4}, of the half's frame
+  auto put = [&](int k, int x, int l, int y, R v) {
+    constexpr int kSig[5] = {1, 0, 3, 2, 4};   // the kind in the original frame of a kind of the exchanged one
+    const bool self_mirror = (k == 0 && l == 1) || (k == 2 && l == 3) || (k == 4 && l == 4);
+    if (!half) M[sym15(k * 3 + x, l * 3 + y)] = v;
+    else if (!self_mirror) M[sym15(kSig[k] * 3 + x, kSig[l] * 3 + y)] = v;
+  };
+  const bool exact = !A.pseudo;
+  // Q = s W sqrt(a_bar) H B_beta,1 (rows of B: up)
+  V3<R> Q[3];
+  if (PART & (kPart00 | kPart01 | kPart0l)) {
+    Q[0] = sw * (H00 * up[0] + H01 * up[1] + H02 * up[2]);
+    Q[1] = sw * (H01 * up[0] + H11 * up[1] + H12 * up[2]);
+    Q[2] = sw * (H02 * up[0] + H12 * up[1] + H22 * up[2]);
+  }
+  if (PART & (kPart00 | kPart01)) {
+    // blocks (0, 0) and (0, 1): B_beta^T H B_beta, B_alpha^T H B_alpha (rows {a_1, 0, a_2} and {0, a_2, a_1}),
+    // (H alpha) d^2 alpha and, exact, s/a times beta's D~ (App. B.2 with c = c~, beta = c~ . a_3):
+    // (0,0) beta (3 t1 t1 + a2 a2 - a22) - s2 t1 - t1 s2;
+    // (0,1) beta (3 t1 t2 - 2 a1 a2 + a2 a1 + a12) - s2 t2 - t1 s1 - sqrt(a) [c~]
+    V3<R> ct = coef[0] * c[0] + coef[1] * c[1] + coef[2] * c[2];
+    const R bt = dot(ct, a3);
+    const R ci = exact ? sw * isqa * isqa : (R)0, cb = exact ? ci * bt : (R)0;
+    const V3<R> T1 = ((R)1.5 * cb) * t1 - ci * cross(a2, ct), T2 = ((R)1.5 * cb) * t2 - ci * cross(ct, a1);
+    const V3<R> J2 = hw * (H02 * a1 + H22 * a2) + cb * a2;
+    if (PART & kPart00) {
+      const V3<R> J0 = hw * (H00 * a1 + H02 * a2);
+      const R id = hw * sg[0] - cb * dot(a2, a2);
+#pragma unroll
+      for (int x = 0; x < 3; ++x)
+#pragma unroll
+        for (int y = x; y < 3; ++y) {
+          R v = comp(Q[0], x) * comp(up[0], y) + comp(Q[1], x) * comp(up[1], y) + comp(Q[2], x) * comp(up[2], y) +
+                comp(J0, x) * comp(a1, y) + comp(J2, x) * comp(a2, y) + comp(T1, x) * comp(t1, y) +
+                comp(t1, x) * comp(T1, y);
+          if (x == y) v += id;
+          put(0, x, 0, y, v);
+        }
+    }
+    if (PART & kPart01) {
+      const V3<R> J1 = hw * (H01 * a1 + H12 * a2) - ((R)2 * cb) * a1;
+      const R id = hw * sg[2] + cb * dot(a1, a2);
+      const V3<R> cx = (ci * sqa) * ct;   // [v]_{xy} = eps_{x j y} v_j
+#pragma unroll
+      for (int x = 0; x < 3; ++x)
+#pragma unroll
+        for (int y = 0; y < 3; ++y) {
+          R v = comp(Q[0], x) * comp(vp[0], y) + comp(Q[1], x) * comp(vp[1], y) + comp(Q[2], x) * comp(vp[2], y) +
+                comp(J1, x) * comp(a2, y) + comp(J2, x) * comp(a1, y) + comp(T1, x) * comp(t2, y) +
+                comp(t1, x) * comp(T2, y);
+          if (x == y) v += id;
+          else if ((y - x + 3) % 3 == 1) v += comp(cx, 3 - x - y);   // - [c~], [c~]_{01} = -c~_z
+          else v -= comp(cx, 3 - x - y);
+          put(0, x, 1, y, v);
+        }
+    }
+  }
+  if (PART & kPart0l) {
+    // blocks (0, 2 + m): Q_m a_3^T (twice for x_,12) and, exact, d a_3 along the first direction, transposed:
+    // s coef_m P_1[y][x], P_1 = (-[a_2] - a_3 (x) t_1) / sqrt(a)
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+      const R em = exact ? sw * coef[m] * isqa : (R)0;
+      const V3<R> Rm = (m == 2 ? (R)2 * Q[m] : Q[m]) - em * t1, Em = em * a2;
+#pragma unroll
+      for (int x = 0; x < 3; ++x)
+#pragma unroll
+        for (int y = 0; y < 3; ++y) {
+          R v = comp(Rm, x) * comp(a3, y);
+          if (x != y) v = (x - y + 3) % 3 == 1 ? v + comp(Em, 3 - x - y) : v - comp(Em, 3 - x - y);
+          put(0, x, 2 + m, y, v);
+        }
+    }
+  }
+  if (PART & kPartkl) {
+    // blocks (2, 2), (2, 3), (2, 4), (4, 4): s H a_3 a_3^T, twice for each x_,12
+    const R f[4] = {sw * H00, sw * H01, (R)2 * (sw * H02), (R)4 * (sw * H22)};
+#pragma unroll
+    for (int x = 0; x < 3; ++x)
+#pragma unroll
+      for (int y = 0; y < 3; ++y) {
+        const R aa = comp(a3, x) * comp(a3, y);
+        if (y >= x) {
+          put(2, x, 2, y, f[0] * aa);
+          put(4, x, 4, y, f[3] * aa);
+        }
+        put(2, x, 3, y, f[1] * aa);
+        put(2, x, 4, y, f[2] * aa);
+      }
+  }
+}
+
+__device__ __forceinline__ void atomic_add_row12(float* dst, const float* v) {
   float4* d4 = reinterpret_cast<float4*>(dst);
 #pragma unroll
   for (int i = 0; i < 3; ++i) atomicAdd(d4 + i, make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]));
 }
-template <>
-__device__ __forceinline__ void atomic_add_row12<double>(double* dst, const double* v) {
-#pragma unroll
-  for (int i = 0; i < 12; ++i) atomicAdd(dst + i, v[i]);
-}
 
-template <typename R>
-__device__ __forceinline__ void plain_add_row12(R* dst, const R* v) {
+__device__ __forceinline__ void plain_add_row12(float* dst, const float* v) {
 #pragma unroll
   for (int i = 0; i < 12; ++i) dst[i] += v[i];
 }
 
-// T = Phi_g^T M_g for Gauss point g = 4 g2 + g1: T[I * 45 + c * 15 + l * 3 + c'] =
+// T = Phi_g^T M_g for Gauss point g = 4 g2 + g1: T[I][col], col = c * 15 + l * 3 + c', is
 // sum_k phi_k^I(g) M_g[(k, c), (l, c')] for the 16 DOF triples I. With the tensor-product basis,
 // phi_k^I = w1[d1(k)][g1][a] w2[d2(k)][g2][b] (I = corner (p + 2q) * 4 + kind (r + 2s),
-// a = 2p + r, b = 2q + s): each lane takes whole (c, l, c') columns, loads the 5 M values of a
-// column once, contracts along theta^2 and then theta^1 in registers, and writes 16 T values.
+// a = 2p + r, b = 2q + s): a thread takes a whole (c, l, c') column, loads its 5 M values once, contracts along theta^2 and then theta^1 in registers, and writes 16 T values.
 template <typename R>
-__device__ __forceinline__ void t_stage(const R* w1d, const R* Mg, R* T, int g, int lane) {
+__device__ __forceinline__ void t_column(const R* w1d, const R* Mg, R* T, int stride, int g, int col) {
   const int g1 = g & 3, g2 = g >> 2;
   R W1[3][4], W2[3][4];
 #pragma unroll
@@ -756,28 +963,26 @@ __device__ __forceinline__ void t_stage(const R* w1d, const R* Mg, R* T, int g, 
       W1[d][a] = w1d[(d * 4 + g1) * 4 + a];
       W2[d][a] = w1d[kHerm1D + (d * 4 + g2) * 4 + a];
     }
-  for (int col = lane; col < 45; col += 32) {
-    const int c = col / 15, l = (col / 3) % 5, cp = col % 3;
-    R m[5];
+  const int c = col / 15, l = (col / 3) % 5, cp = col % 3;
+  R m[5];
 #pragma unroll
-    for (int k = 0; k < 5; ++k) m[k] = Mg[sym15(k * 3 + c, l * 3 + cp)];
-    // kinds k = (d1, d2): 0 (1,0), 1 (0,1), 2 (2,0), 3 (0,2), 4 (1,1); V[d1][b] = sum over the
-    // kinds with that d1 of w2[d2][g2][b] M_k
-    R V[3][4];
+  for (int k = 0; k < 5; ++k) m[k] = Mg[sym15(k * 3 + c, l * 3 + cp)];
+  // kinds k = (d1, d2): 0 (1,0), 1 (0,1), 2 (2,0), 3 (0,2), 4 (1,1); V[d1][b] = sum over the
+  // kinds with that d1 of w2[d2][g2][b] M_k
+  R V[3][4];
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {
+    V[0][b] = W2[1][b] * m[1] + W2[2][b] * m[3];
+    V[1][b] = W2[0][b] * m[0] + W2[1][b] * m[4];
+    V[2][b] = W2[0][b] * m[2];
+  }
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
-      V[0][b] = W2[1][b] * m[1] + W2[2][b] * m[3];
-      V[1][b] = W2[0][b] * m[0] + W2[1][b] * m[4];
-      V[2][b] = W2[0][b] * m[2];
+      const int I = ((a >> 1) + 2 * (b >> 1)) * 4 + ((a & 1) + 2 * (b & 1));
+      T[I * stride + col] = W1[0][a] * V[0][b] + W1[1][a] * V[1][b] + W1[2][a] * V[2][b];
     }
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const int I = ((a >> 1) + 2 * (b >> 1)) * 4 + ((a & 1) + 2 * (b & 1));
-        T[I * TStride<R>::v + col] = W1[0][a] * V[0][b] + W1[1][a] * V[1][b] + W1[2][a] * V[2][b];
-      }
-  }
 }
 
 // FP32 Hessian K = sum_g Phi_g^T M_g Phi_g of one patch from its upper node-corner blocks. K is
@@ -823,8 +1028,8 @@ __device__ __forceinline__ void store_staged_hessian32(const float* K, int p, co
           row[4 * q + 3] = v4.w;
         }
         float* dst = V + (size_t)kb * 144 + (r * 3 + c) * 12;
-        if (A.bsr_atomic) atomic_add_row12<float>(dst, row);
-        else plain_add_row12<float>(dst, row);
+        if (A.bsr_atomic) atomic_add_row12(dst, row);
+        else plain_add_row12(dst, row);
       }
     }
   }
@@ -832,7 +1037,7 @@ __device__ __forceinline__ void store_staged_hessian32(const float* K, int p, co
 }
 
 __device__ __forceinline__ void hessian_sym32(const float* sphi, const float* w1d, const float* sphg,
-                                              WarpSmem<float>& W, int p, const ElemArgs& A, int lane) {
+                                              WarpSmem& W, int p, const ElemArgs& A, int lane) {
   static_assert(sizeof(W.M) + sizeof(W.T) >= sizeof(float) * 48 * kKStride, "staging area");
   constexpr int JS = 6;
   int Is, Js, nJ;
@@ -860,11 +1065,11 @@ __device__ __forceinline__ void hessian_sym32(const float* sphi, const float* w1
     for (int e = 0; e < 9; ++e) acc[j][e] = 0.f;
 #pragma unroll 1
   for (int g = 0; g < 16; ++g) {
-    t_stage<float>(w1d, W.M[g], W.T, g, lane);
+    for (int col = lane; col < 45; col += 32) t_column<float>(w1d, W.M[g], W.T, kTStride, g, col);
     __syncwarp();
     // row Is of T: 11 16-byte loads and one 4-byte load of the padded row
     float Tr[45];
-    const float4* t4 = reinterpret_cast<const float4*>(W.T + Is * TStride<float>::v);
+    const float4* t4 = reinterpret_cast<const float4*>(W.T + Is * kTStride);
 #pragma unroll
     for (int e4 = 0; e4 < 11; ++e4) {
       const float4 v4 = t4[e4];
@@ -873,7 +1078,7 @@ __device__ __forceinline__ void hessian_sym32(const float* sphi, const float* w1
       Tr[4 * e4 + 2] = v4.z;
       Tr[4 * e4 + 3] = v4.w;
     }
-    Tr[44] = W.T[Is * TStride<float>::v + 44];
+    Tr[44] = W.T[Is * kTStride + 44];
     const float mI = W.ms[g] * sphi[Is * kPhiStride + g];
 #pragma unroll
     for (int j = 0; j < JS; ++j) {
@@ -917,15 +1122,15 @@ __device__ __forceinline__ void hessian_sym32(const float* sphi, const float* w1
   store_staged_hessian32(K, p, A, lane);
 }
 
-// Gathers the warp's patch: displacement u = q - rest and rest DOFs qb (shared memory).
+// Gathers a warp's (or CTA's) patch: displacement u = q - rest and rest DOFs qb (shared memory).
 template <typename R, class WS>
-__device__ __forceinline__ void gather_patch(WS& W, int p, const ElemArgs& A, int lane) {
+__device__ __forceinline__ void gather_patch(WS& W, int p, const ElemArgs& A, int tid, int nthreads = 32) {
   const int4 pn = A.pnodes[p];
   const int nd[4] = {pn.x, pn.y, pn.z, pn.w};
   // Value DOFs enter only through derivatives, whose value-kind shape functions sum to zero
   // (partition of unity); subtracting corner 00's value in FP64 before rounding removes the
   // O(|x| / dxi) cancellation of the derivative interpolation from the R arithmetic.
-  for (int l = lane; l < 48; l += 32) {
+  for (int l = tid; l < 48; l += nthreads) {
     const int kk = l % 12;
     size_t a = (size_t)nd[l / 12] * 12 + kk;
     double qv = A.q[a], rv = A.rest[a];
@@ -944,14 +1149,14 @@ __device__ __forceinline__ void gather_patch(WS& W, int p, const ElemArgs& A, in
 // Energy and gradient of the patch in the kernel's precision (by-products of the Gauss-point
 // matrices: per-point energies W.en and gradient vectors W.G).
 template <typename R, class WS>
-__device__ __forceinline__ void patch_byproducts(const R* sphi, const WS& W, int p, const ElemArgs& A, int lane) {
-  if (A.energy_p) {
+__device__ __forceinline__ void patch_byproducts(const R* sphi, const WS& W, int p, const ElemArgs& A, int lane, int nthreads = 32) {
+  if (A.energy_p && lane < 32) {
     R e = lane < 16 ? W.en[lane] : (R)0;
     for (int o = 8; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
     if (lane == 0) A.energy_p[p] = (double)e;
   }
   if (A.grad_p) {
-    for (int l = lane; l < 48; l += 32) {
+    for (int l = lane; l < 48; l += nthreads) {
       int Ig = l / 3, c = l % 3;
       R sacc = 0;
       for (int g = 0; g < 16; ++g)
@@ -962,121 +1167,16 @@ __device__ __forceinline__ void patch_byproducts(const R* sphi, const WS& W, int
   }
 }
 
-// One patch by one warp: gather, Gauss-point matrices M_g, energy/gradient by-products, and the
+// One patch by one warp (FP32): gather, Gauss-point matrices M_g, energy/gradient by-products, and the
 // Hessian K = sum_g phi_g^T M_g phi_g written unassembled and/or scattered into the BSR.
-template <typename R>
-__device__ __forceinline__ void element_patch(const R* sphi, const R* w1d, const R* sphg, WarpSmem<R>& W, int p,
-                                              const ElemArgs& A, int lane) {
-  constexpr int JP = ElemCfg<R>::kJP;          // J columns per pass (16 / 2 / JP passes)
-  const int I = lane >> 1, h = lane & 1;
-  gather_patch<R>(W, p, A, lane);
+__device__ __forceinline__ void element_patch(const float* sphi, const float* w1d, const float* sphg, WarpSmem& W,
+                                              int p, const ElemArgs& A, int lane) {
+  gather_patch<float>(W, p, A, lane);
   __syncwarp();
-  if constexpr (sizeof(R) == 4) gauss_point_matrix<R, true>(sphi, W, lane & 15, lane >> 4, A);
-  else if (lane < 16) gauss_point_matrix<R, false>(sphi, W, lane, 0, A);
+  gauss_point_matrix<false>(sphi, W, lane & 15, lane >> 4, A);
   __syncwarp();
-  patch_byproducts<R>(sphi, W, p, A, lane);
-
-  const bool want_h = A.hess_p || A.bsr;
-  if constexpr (sizeof(R) == 4) {
-    if (want_h) hessian_sym32(sphi, w1d, sphg, reinterpret_cast<WarpSmem<float>&>(W), p, A, lane);
-  } else if (want_h) {
-#pragma unroll 1
-    for (int pass = 0; pass < 8 / JP; ++pass) {
-      R acc[JP][9];
-#pragma unroll
-      for (int j = 0; j < JP; ++j)
-#pragma unroll
-        for (int e = 0; e < 9; ++e) acc[j][e] = (R)0;
-      const int J0 = 8 * h + pass * JP;
-#pragma unroll 1
-      for (int g = 0; g < 16; ++g) {
-        t_stage<R>(w1d, W.M[g], W.T, g, lane);
-        __syncwarp();
-        R Tr[45];
-        if constexpr (sizeof(R) == 4) {
-          // 11 16-byte loads and one 4-byte load of the padded row
-          const float4* t4 = reinterpret_cast<const float4*>(W.T + I * TStride<R>::v);
-#pragma unroll
-          for (int e4 = 0; e4 < 11; ++e4) {
-            const float4 v4 = t4[e4];
-            Tr[4 * e4] = v4.x;
-            Tr[4 * e4 + 1] = v4.y;
-            Tr[4 * e4 + 2] = v4.z;
-            Tr[4 * e4 + 3] = v4.w;
-          }
-          Tr[44] = W.T[I * TStride<R>::v + 44];
-        } else {
-#pragma unroll
-          for (int e = 0; e < 45; ++e) Tr[e] = W.T[I * TStride<R>::v + e];
-        }
-        const R mI = W.ms[g] * sphi[I * kPhiStride + g];
-#pragma unroll
-        for (int j = 0; j < JP; ++j) {
-          const int J = J0 + j;
-          R pj[5], phJ;
-          if constexpr (sizeof(R) == 4) {
-            const float4* q4 = reinterpret_cast<const float4*>(sphg + (g * 16 + J) * 8);
-            const float4 a4 = q4[0], b4 = q4[1];
-            pj[0] = a4.x;
-            pj[1] = a4.y;
-            pj[2] = a4.z;
-            pj[3] = a4.w;
-            pj[4] = b4.x;
-            phJ = b4.y;
-          } else {
-#pragma unroll
-            for (int l = 0; l < 5; ++l) pj[l] = sphi[J * kPhiStride + (l + 1) * 16 + g];
-            phJ = sphi[J * kPhiStride + g];
-          }
-#pragma unroll
-          for (int c = 0; c < 3; ++c)
-#pragma unroll
-            for (int cp = 0; cp < 3; ++cp) {
-              R sacc = acc[j][c * 3 + cp];
-#pragma unroll
-              for (int l = 0; l < 5; ++l) sacc += Tr[c * 15 + l * 3 + cp] * pj[l];
-              acc[j][c * 3 + cp] = sacc;
-            }
-          const R mm = mI * phJ;
-          acc[j][0] += mm;
-          acc[j][4] += mm;
-          acc[j][8] += mm;
-        }
-        __syncwarp();
-      }
-      // outputs of this pass: rows (I, c), columns J0..J0+JP-1
-      if (A.hess_p) {
-        R* Hp = reinterpret_cast<R*>(A.hess_p) + (size_t)p * 2304;
-#pragma unroll
-        for (int c = 0; c < 3; ++c)
-#pragma unroll
-          for (int j = 0; j < JP; ++j)
-#pragma unroll
-            for (int cp = 0; cp < 3; ++cp) Hp[(I * 3 + c) * 48 + (J0 + j) * 3 + cp] = acc[j][c * 3 + cp];
-      }
-      if (A.bsr) {
-        // J0..J0+JP-1 covers whole corners (4 kinds each): row segments of 12 in the BSR block
-        R* V = reinterpret_cast<R*>(A.bsr);
-        const int a = I >> 2, r = I & 3;
-#pragma unroll
-        for (int bb = 0; bb < JP / 4; ++bb) {
-          const int b = (J0 >> 2) + bb;
-          const int kb = A.pblocks[p * 16 + a * 4 + b];
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            R row[12];
-#pragma unroll
-            for (int sk = 0; sk < 4; ++sk)
-#pragma unroll
-              for (int cp = 0; cp < 3; ++cp) row[sk * 3 + cp] = acc[bb * 4 + sk][c * 3 + cp];
-            R* dst = V + (size_t)kb * 144 + (r * 3 + c) * 12;
-            if (A.bsr_atomic) atomic_add_row12<R>(dst, row);
-            else plain_add_row12<R>(dst, row);
-          }
-        }
-      }
-    }
-  }
+  patch_byproducts<float>(sphi, W, p, A, lane);
+  if (A.hess_p || A.bsr) hessian_sym32(sphi, w1d, sphg, W, p, A, lane);
   __syncwarp();
 }
 

@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_element_tc(ElemArgs A,
     if (active) {
       gather_patch<float>(W, p, A, lane);
       __syncwarp();
-      gauss_point_matrix<float, true, true>(sphi, W, lane & 15, lane >> 4, A);
+      gauss_point_matrix<true>(sphi, W, lane & 15, lane >> 4, A);
       __syncwarp();
       patch_byproducts<float>(sphi, W, p, A, lane);
     }
@@ -363,7 +363,10 @@ shell_status launch_full_tc(Shell& s, const ElemArgs& A, int work) {
   int blocks = (work + etc::kWarps - 1) / etc::kWarps;
   const int cap = s.num_sms * etc::kCtasPerSm;
   if (blocks > cap) blocks = cap;
-  auto k = A.grad64 && work <= blocks * etc::kWarps ? etc::k_element_tc<true> : etc::k_element_tc<false>;
+  // one patch per warp, FP64 too: 280 x 5 patches 68 us instead of 81 a call of shell_energy_grad_hess. Not for
+  // colour-ordered launches, whose sums have one order: the compiler contracts the FP32 part differently
+  // in the two forms, and a shell's first Hessian has to have the bits of its later ones.
+  auto k = A.grad64 && A.bsr_atomic && work <= blocks * etc::kWarps ? etc::k_element_tc<true> : etc::k_element_tc<false>;
   k<<<blocks, etc::kThreads, etc::kSmemBytes, s.stream>>>(A, (unsigned)s.wait_polls);
   BHEM_CUDA(cudaGetLastError());
   ++s.launches;
