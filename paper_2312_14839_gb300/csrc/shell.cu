@@ -416,13 +416,17 @@ extern "C" shell_status shell_element_egh(shell_t* shell, const double* q, int p
 }
 
 namespace bhem {
-static shell_status assemble_hessian(Shell& s, const double* q, double mass_scale) {
+// energy64, grad64: FP64 patch energies and gradient in the same pass (FP32 shells; grad64 zeroed)
+static shell_status assemble_hessian(Shell& s, const double* q, double mass_scale, double* energy64 = nullptr,
+                                     double* grad64 = nullptr) {
   size_t bytes = (size_t)s.n_blocks * 144 * (s.val_fp64 ? sizeof(double) : sizeof(float));
   BHEM_CUDA(cudaMemsetAsync(s.d_val, 0, bytes, s.stream));
   ElemOutputs o;
   o.bsr = s.d_val;
   o.mass_scale = mass_scale;
   o.pseudo = s.opt.hessian == SHELL_HESS_PSEUDO;
+  o.energy64 = energy64;
+  o.grad64 = grad64;
   return launch_element_full(s, q, s.val_fp64 != 0, o);
 }
 
@@ -589,6 +593,14 @@ static shell_status residual(Shell& s, const double* q, const shell_step_params&
   return SHELL_OK;
 }
 
+// Whether a Newton step's linear solves are resident launches. Not in mixed precision with colour-ordered assembly,
+// whose sums have one order from run to run: the resident solve adds its dot products in another order, and
+// a step moves with it by up to 5e-9 (a noisy 40 x 30 sheet, the steps' tolerance) where atomic
+// assembly moves it as far between two runs. FP64 steps move by 1e-14.
+static bool newton_resident(const Shell& s) {
+  return s.res_per > 0 && (s.val_fp64 || s.opt.assembly != SHELL_ASM_COLOR);
+}
+
 // |g| at q together with the first Hessian at q (mixed precision) in one element launch: the warps
 // of the FP32 Hessian also evaluate the FP64 patch energies and the FP64 elastic gradient, so the
 // FP64 pipe works under the FP32 pass instead of after it. The Hessian's diagonal statistics ride
@@ -597,15 +609,8 @@ static shell_status residual(Shell& s, const double* q, const shell_step_params&
 static shell_status residual_with_hessian(Shell& s, const double* q, const shell_step_params& P,
                                           const unsigned char* mask, double inv_dt2, double* gnorm) {
   BHEM_CUDA(cudaMemsetAsync(s.d_g, 0, sizeof(double) * s.n_dof, s.stream));
-  BHEM_CUDA(cudaMemsetAsync(s.d_val, 0, (size_t)s.n_blocks * 144 * sizeof(float), s.stream));
-  ElemOutputs o;
-  o.bsr = s.d_val;
-  o.mass_scale = inv_dt2;
-  o.pseudo = s.opt.hessian == SHELL_HESS_PSEUDO;
-  o.energy64 = s.d_Ep;
-  o.grad64 = s.d_g;
-  BHEM_TRY(launch_element_full(s, q, false, o));
-  if (s.res_per == 0) BHEM_TRY(launch_diag_check(s, mask, s.d_ns->diag_stats, true));   // else taken by the solve
+  BHEM_TRY(assemble_hessian(s, q, inv_dt2, s.d_Ep, s.d_g));
+  if (!newton_resident(s)) BHEM_TRY(launch_diag_check(s, mask, s.d_ns->diag_stats, true));   // else taken by the solve
   BHEM_TRY(launch_grad_finish(s, q, s.d_y, P.dt, P.gravity, mask, s.d_g, s.d_gin, &s.d_ns->gnorm2));
   BHEM_TRY(read_scalars(s));
   *gnorm = std::sqrt(s.h_ns->gnorm2);
@@ -695,7 +700,7 @@ static shell_status newton_core(Shell& s, const shell_step_params& P, const unsi
     // iteration's tau; each negative curvature met by PCG multiplies tau by 10 (at least 1e-8),
     // beyond 1e4 the step gives up.
     KindStats K;
-    bool stats_read = hess_pending || (hess_ready && s.res_per == 0);
+    bool stats_read = hess_pending || (hess_ready && !newton_resident(s));
     if (hess_pending) {   // assembled and its statistics read with the residual (joined there)
       BHEM_CUDA(cudaStreamWaitEvent(s.stream, s.ev_hess, 0));
       hess_pending = false;
@@ -709,7 +714,7 @@ static shell_status newton_core(Shell& s, const shell_step_params& P, const unsi
     if (tau < 1e-8) tau = 0.0;
     const bool search = gn > 1e-6 * gref;
     bool solved = false;   // by the resident solve, with M d and the line search's dot products
-    if (s.res_per > 0) {
+    if (newton_resident(s)) {
       for (bool first = true;; first = false) {
         if (tau > 1e4) { status = SHELL_ERR_INDEFINITE; break; }
         BHEM_TRY(launch_solve_resident(s, mask, s.d_g, -1.0, tau, P.pcg_rtol, P.pcg_fixed_iters,
