@@ -273,6 +273,8 @@ shell_status launch_element_full(Shell& s, const double* q, bool fp64, const Ele
 // Light FP64 kernel: per-patch energy (and assembled gradient) at q + step * dir.
 //   mode 0: energy_p[p] = E_p, grad += dE/dq (grad may be null), total -> scal_out
 //   mode 1: total of (E_p(q + step dir) - energy_ref[p]) -> scal_out (no gradient)
+// *energy = sum of the n_patches patch energies
+shell_status launch_energy_sum(Shell& s, const double* energy_p, double* energy);
 shell_status launch_energy_grad64(Shell& s, const double* q, const double* dir, double step,
                                   double* energy_p, const double* energy_ref, double* grad,
                                   double* scal_out);

@@ -193,6 +193,19 @@ shell_status launch_energy_grad64(Shell& s, const double* q, const double* dir, 
   return SHELL_OK;
 }
 
+__global__ void __launch_bounds__(256) k_energy_sum(int np, const double* __restrict__ energy_p, Reduce red, double* out) {
+  double v[1] = {0.0};
+  for (int p = blockIdx.x * 256 + threadIdx.x; p < np; p += gridDim.x * 256) v[0] += energy_p[p];
+  grid_reduce<1>(v, red, out, gridDim.x);
+}
+
+shell_status launch_energy_sum(Shell& s, const double* energy_p, double* energy) {
+  k_energy_sum<<<std::min(128, (s.n_patches + 511) / 512), 256, 0, s.stream>>>(s.n_patches, energy_p, s.red, energy);
+  BHEM_CUDA(cudaGetLastError());
+  ++s.launches;
+  return SHELL_OK;
+}
+
 // ------------------------------------------------------------------------------------------
 // Heavy kernels: E, gradient and the 48x48 Hessian of a patch, in FP32 (FFMA form) by a warp, in FP64 by a CTA.
 // ------------------------------------------------------------------------------------------

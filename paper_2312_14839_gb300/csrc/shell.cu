@@ -439,8 +439,17 @@ static shell_status elastic_energy_grad(Shell& s, const double* q, double* energ
 extern "C" shell_status shell_energy_grad_hess(shell_t* shell, const double* q, double mass_scale,
                                                double* energy, double* grad, int want_hessian) {
   if (!shell || !q) return fail(SHELL_ERR_ARG, "NULL argument");
-  if (energy || grad) BHEM_TRY(elastic_energy_grad(*shell, q, energy, grad));
-  if (want_hessian) BHEM_TRY(assemble_hessian(*shell, q, mass_scale));
+  Shell& s = *shell;
+  if (want_hessian && grad && !s.val_fp64 && s.fuse_first_hessian) {
+    // all three in one pass over the elements, as a Newton step's first residual and Hessian: the FP64 pipe
+    // works beside the FP32 one, and a small shell pays one kernel's latency (280 x 5 patches: 36 us for the
+    // energy kernel alone)
+    BHEM_CUDA(cudaMemsetAsync(grad, 0, sizeof(double) * s.n_dof, s.stream));
+    BHEM_TRY(assemble_hessian(s, q, mass_scale, s.d_Ep, grad));
+    return launch_energy_sum(s, s.d_Ep, energy ? energy : s.d_energy_tmp);
+  }
+  if (energy || grad) BHEM_TRY(elastic_energy_grad(s, q, energy, grad));
+  if (want_hessian) BHEM_TRY(assemble_hessian(s, q, mass_scale));
   return SHELL_OK;
 }
 
