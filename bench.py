@@ -504,13 +504,13 @@ def network_timing(net, X_all, T_all, n_sheet=64, reps=20):
     return out
 
 
-# Algorithmic work per patch of the two arithmetic-bound kernels (the units are stated in DESIGN):
+# Algorithmic work per patch of the two arithmetic-bound kernels (the units are stated below):
 #  - element Hessian: the factored Phi^T M_g Phi contraction with symmetry, 16 x 15 x 48 x 5 (T)
 #    + 1,176 x 80 (K) = 151,680 FMA;
 #  - FP64 energy + gradient: sum-factorised interpolation 1,536 + gradient transpose 1,536 +
-#    about 190 FMA of nonlinear point work at each of the 16 Gauss points = 6,112 FMA.
+#    about 135 FP64 operations of nonlinear point work at each of the 16 Gauss points = 5,232.
 ELEMENT_FLOP_PER_PATCH = 2 * (16 * 15 * 48 * 5 + 1176 * 80)
-ENERGY64_FLOP_PER_PATCH = 2 * (1536 + 1536 + 16 * 190)
+ENERGY64_FLOP_PER_PATCH = 2 * (1536 + 1536 + 16 * 135)
 # The tensor-core form of the element pass (the default of a mixed-precision shell) issues per patch
 # 96 rows (6 component pairs x 16 J) x 16 columns x 96 K values (16 Gauss points x 6 kinds) TF32
 # multiply-adds, three times (head and tail products): 442,368 tensor MACs.
@@ -528,7 +528,7 @@ def element_kernel_name():
     if element_form() == "tc":
         return ("k_element_tc (FP32 exact Hessian: Gauss-point matrices and T rows on the FMA pipe, "
                 "the contraction K = Psi^T T on tcgen05 kind::tf32 from tensor memory")
-    return "k_element_full<float> (FP32 exact Hessian on the FMA pipe"
+    return "k_element_full (FP32 exact Hessian on the FMA pipe"
 
 
 def alu_rooflines(sh, q_d, P, n_patches, stream, reps=5):
@@ -659,6 +659,9 @@ def run_rays_bench(args):
         out = sh.trace_rays(dq, do, dd, variant=variant, want_stats=True)
         for _ in range(warmup):
             sh.trace_rays(dq, do, dd, variant=variant, out=out)
+        plain = {k: v for k, v in out.items() if k != "stats"}
+        for _ in range(warmup):
+            sh.trace_rays(dq, do, dd, variant=variant, out=plain)
         torch.cuda.synchronize()
         stats = out["stats"].cpu().numpy()
         flags = out["flags"].cpu().numpy()
@@ -677,12 +680,25 @@ def run_rays_bench(args):
                 torch.cuda.synchronize()
                 e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
                 e0.record(stream)
-                sh.trace_rays(dq, do, dd, variant=variant, out=out)
+                sh.trace_rays(dq, do, dd, variant=variant, out=plain)
                 e1.record(stream)
                 torch.cuda.synchronize()
                 ms.append(e0.elapsed_time(e1))
         clk = c.summary()
         res["gpu_launches_per_trace"] = (sh.kernel_launches() - l0) / max(steps, 1)
+        # with statistics the search executes every operation that they count (without, it leaves out
+        # sub-patches that an FP32 test rules out): the roofline's time
+        ms_all = []
+        for _ in range(min(steps, 3)):
+            flush.zero_()
+            torch.cuda.synchronize()
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record(stream)
+            sh.trace_rays(dq, do, dd, variant=variant, out=out)
+            e1.record(stream)
+            torch.cuda.synchronize()
+            ms_all.append(e0.elapsed_time(e1))
+        res["ms_per_trace_with_stats"] = float(np.mean(ms_all))
         res["ms_per_trace"] = float(np.mean(ms))
         res["rays_per_s"] = n / (res["ms_per_trace"] / 1e3)
         if want_e2e:
@@ -720,7 +736,7 @@ def run_rays_bench(args):
                                                              "splits_mean", "splits_max", "flagged")}
     peak64 = bhem.measure_fma_peak(True, 256, torch.cuda.current_stream())
     peak_ops = peak64 / 2.0     # one FP64 pipe instruction per add, multiply or compare
-    ach = main_res["fp64_ops_per_trace"] / (main_res["ms_per_trace"] / 1e3)
+    ach = main_res["fp64_ops_per_trace"] / (main_res["ms_per_trace_with_stats"] / 1e3)
     # the oracle on a seeded sample of the same frame, all host cores
     cpu = None
     if not args.no_cpu_baseline:
@@ -746,7 +762,9 @@ def run_rays_bench(args):
         "roofline": {"bound": "alu", "achieved": ach / 1e12, "peak": peak_ops / 1e12, "unit": "TFLOP/s",
                      "frac": ach / peak_ops, "traffic": None,
                      "kernel": "k_trace_rays (+ k_ray_nets, k_trace_rays_redo in the same events)",
-                     "work": "FP64 operations counted per ray from its splits, boxes and Newton iterations",
+                     "work": "FP64 operations counted per ray from its splits, boxes and Newton iterations, over the "
+                             "time of a trace with statistics, which executes them",
+                     "ms_per_trace_with_stats": main_res["ms_per_trace_with_stats"],
                      "peak_source": "measured FP64 FMA rate (shell_measure_fma_peak) as instructions/s"},
         "cpu_baseline": cpu, "search": {k: main_res[k] for k in ("hit_fraction", "flagged", "splits_mean",
                                                               "splits_max", "heap_peak_max", "newton_iters_mean",
@@ -792,6 +810,9 @@ def run_ccd_bench(args):
         out = sh.ccd_points(dq_, ddq, dx0, ddx, variant=variant, want_stats=True)
         for _ in range(warmup):
             sh.ccd_points(dq_, ddq, dx0, ddx, variant=variant, out=out)
+        plain = {k: v for k, v in out.items() if k != "stats"}
+        for _ in range(warmup):
+            sh.ccd_points(dq_, ddq, dx0, ddx, variant=variant, out=plain)
         torch.cuda.synchronize()
         stats, flags = out["stats"].cpu().numpy(), out["flags"].cpu().numpy()
         res = {"contact_fraction": float((flags & 1).mean()), "flagged": int((flags & 6).astype(bool).sum()),
@@ -806,12 +827,25 @@ def run_ccd_bench(args):
                 torch.cuda.synchronize()
                 e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
                 e0.record(stream)
-                sh.ccd_points(dq_, ddq, dx0, ddx, variant=variant, out=out)
+                sh.ccd_points(dq_, ddq, dx0, ddx, variant=variant, out=plain)
                 e1.record(stream)
                 torch.cuda.synchronize()
                 ms.append(e0.elapsed_time(e1))
         clk = c.summary()
         res["gpu_launches_per_call"] = (sh.kernel_launches() - l0) / max(steps, 1)
+        # with statistics the search executes every operation that they count (without, it leaves out
+        # sub-patches that an FP32 test rules out): the roofline's time
+        ms_all = []
+        for _ in range(min(steps, 3)):
+            flush.zero_()
+            torch.cuda.synchronize()
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record(stream)
+            sh.ccd_points(dq_, ddq, dx0, ddx, variant=variant, out=out)
+            e1.record(stream)
+            torch.cuda.synchronize()
+            ms_all.append(e0.elapsed_time(e1))
+        res["ms_per_call_with_stats"] = float(np.mean(ms_all))
         res["ms_per_call"] = float(np.mean(ms))
         res["queries_per_s"] = n / (res["ms_per_call"] / 1e3)
         if want_e2e:
@@ -844,7 +878,7 @@ def run_ccd_bench(args):
         others[f"{scene}_{variant}"] = {k: r[k] for k in ("queries_per_s", "ms_per_call", "contact_fraction",
                                                           "splits_mean", "splits_max", "flagged")}
     peak_ops = bhem.measure_fma_peak(True, 256, torch.cuda.current_stream()) / 2.0
-    ach = main_res["fp64_ops_per_call"] / (main_res["ms_per_call"] / 1e3)
+    ach = main_res["fp64_ops_per_call"] / (main_res["ms_per_call_with_stats"] / 1e3)
     cpu = None
     if not args.no_cpu_baseline:
         g, q, dq, x0, dx = S.ccd_scene("drape", n)
@@ -869,7 +903,9 @@ def run_ccd_bench(args):
         "roofline": {"bound": "alu", "achieved": ach / 1e12, "peak": peak_ops / 1e12, "unit": "TFLOP/s",
                      "frac": ach / peak_ops, "traffic": None,
                      "kernel": "k_ccd_points (+ k_ccd_nets, k_ccd_points_redo in the same events)",
-                     "work": "FP64 operations counted per point from its splits, feasibility tests and Newton iterations",
+                     "work": "FP64 operations counted per point from its splits, feasibility tests and Newton "
+                             "iterations, over the time of a call with statistics, which executes them",
+                     "ms_per_call_with_stats": main_res["ms_per_call_with_stats"],
                      "peak_source": "measured FP64 FMA rate (shell_measure_fma_peak) as instructions/s"},
         "cpu_baseline": cpu, "search": {k: main_res[k] for k in ("contact_fraction", "flagged", "splits_mean",
                                                               "splits_max", "heap_peak_max", "feasibility_tests_mean",

@@ -273,7 +273,7 @@ k_element_full(ElemArgs A) {
 // beside it). The Gauss-point matrices are shared out by blocks, T = Phi^T M is formed once, eight Gauss
 // points at a time, and only the entries (I, c), (J, c') with I <= J of the symmetric K are summed:
 // 136 pairs x 9, ten a thread. About 2,100 FP64 instructions a warp; with a warp per patch, T formed
-// twice and K in full it was 13,000: 10 x 10 patches 450 us a pass, now 80.
+// twice and K in full it was 13,000: 10 x 10 patches 446 us a pass, now 84.
 struct Elem64Smem {
   double table[kPhiTable];
   double u[48], qb[48];
