@@ -152,7 +152,7 @@ SHELL_API shell_status shell_info(const shell_t* shell, shell_info_t* info);
 
 /* Budget of the library's bounded device-side waits on this shell: the exchanges between the CTAs
    of the resident linear solve (the default on shells whose matrix fits the multiprocessors' shared
-   memory: up to 5,168 nodes in mixed precision, 2,584 in FP64, with 152 multiprocessors), the grid
+   memory: up to 4,864 nodes in mixed precision, 2,584 in FP64, with 152 multiprocessors), the grid
    barriers of the persistent mixed-precision PCG (one cooperative launch per solve; selected by the environment
    variable BHEM_PCG_LOOP=persistent when the shell is created), the mbarrier waits of
    the bulk-copy SpMV (SHELL_SPMV_TMA) and those of the tensor-core element pass (mixed

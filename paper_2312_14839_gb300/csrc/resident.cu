@@ -7,7 +7,7 @@
 // FP64), the statistics, the block inverses and the dot products are short latency-bound kernels with
 // a host round trip each, and the matrix (5 MB at 961 nodes) is read from L2 every time. Here every SM
 // keeps its rows' blocks, block-Jacobi inverses and vectors in shared memory and registers for the
-// whole solve (6.6 KB per FP32 row, so up to 34 rows per SM, 5,168 nodes; half of that in FP64), and
+// whole solve (6.6 KB per FP32 row; at most 32 rows per SM, 4,864 nodes on 152, or 17 in FP64), and
 // an iteration is two exchanges between the CTAs: the two-way latency of L2, about 3 us each with the
 // sums, and under 1.5 us of arithmetic. Measured per solve, statistics to dot products: 30 x 30
 // patches (27 iterations) 556 -> 245 us, 280 x 5 (88) 1,480 -> 890 us, 64 x 64 (26) 640 -> 345 us,
@@ -40,6 +40,8 @@ constexpr int kRowBlocks = 9;          // blocks of a node row (a node couples t
 constexpr int kResSlotCtas = 160;      // slots per reduced value (>= CTAs, a multiple of 32)
 constexpr int kResSlotWarps = kResSlotCtas / 32;
 constexpr int kResThreads = 512;       // 128 registers each: the matrix pieces of a few rows fit beside the rest
+constexpr int kRowsPerWarp = 2;        // rows whose DOFs a warp owns (12 lanes each)
+constexpr int kResMaxRows = kRowsPerWarp * (kResThreads / 32);   // rows per CTA that have an owner
 constexpr int kSlotPq = 0, kSlotRz = 1 /* r.z and r.r */, kSums = 3;   // values summed per PCG iteration
 
 struct alignas(16) Word2 { unsigned long long a, b; };
@@ -381,9 +383,9 @@ __global__ void __launch_bounds__(kResThreads, 1) k_solve_resident(ResidentArgs 
   __syncthreads();
   // a DOF of the CTA's rows per thread, two rows per warp (lanes 0-11, 12-23): a row's 12 values are
   // exchanged within the warp
-  const int myrow = 2 * wid + lane / 12, a = lane % 12;
-  const bool own = lane < 24 && myrow < rows;
-  const int own_warps = (rows + 1) / 2;
+  const int myrow = kRowsPerWarp * wid + lane / 12, a = lane % 12;
+  const bool own = lane < 12 * kRowsPerWarp && myrow < rows;
+  const int own_warps = (rows + kRowsPerWarp - 1) / kRowsPerWarp;
   const size_t gi = (size_t)(i0 + myrow) * 12 + a;
   const bool fixed_dof = own && P.mask && P.mask[gi];
   if (P.fix && s_flag) {
@@ -714,13 +716,13 @@ template <> ResidentKernel resident_kernel<float>(int per) {
   if (per <= 14) return k_solve_resident<float, 3, 1>;
   if (per <= 18) return k_solve_resident<float, 4, 2>;
   if (per <= 28) return k_solve_resident<float, 6, 2>;
-  return k_solve_resident<float, 0, 3>;
+  return k_solve_resident<float, 0, 2>;
 }
 template <> ResidentKernel resident_kernel<double>(int per) {
   if (per <= 9) return k_solve_resident<double, 2, 1>;
   return k_solve_resident<double, 0, 2>;
 }
-template <typename R> constexpr int kResMaxRows = sizeof(R) == 8 ? 33 : 49;   // 27 pieces per row in PIECES x 448
+static_assert(27 * kResMaxRows <= 2 * (kResThreads - 64), "the last forms' PIECES cover every row accepted");
 
 // Rows per CTA. An exchange grows with the CTAs (alone: 2,500 cycles for 64, 3,500 for 152), a CTA's
 // products with its rows, so FP32 takes at least 9 rows per CTA (30 x 30 nodes' solve of 27
@@ -746,7 +748,7 @@ shell_status resident_setup(Shell& s) {
   cudaFuncAttributes fa;
   BHEM_CUDA(cudaFuncGetAttributes(&fa, (const void*)k));
   const size_t smem = per * resident_row_bytes<R>();
-  if (smem + fa.sharedSizeBytes > (size_t)optin || per > kResMaxRows<R>) return SHELL_OK;
+  if (smem + fa.sharedSizeBytes > (size_t)optin || per > kResMaxRows) return SHELL_OK;
   BHEM_CUDA(cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  optin - (int)fa.sharedSizeBytes));
   BHEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void*)k, kResThreads, smem));
@@ -766,7 +768,7 @@ shell_status resident_setup(Shell& s) {
 
 }  // namespace
 
-// Mixed precision or FP64 shells whose rows fit one CTA per SM (FP32: 34 rows per SM);
+// Mixed precision or FP64 shells whose rows fit one CTA per SM (FP32: kResMaxRows per SM, FP64: 17);
 // only where the caller has not selected another form of the solve (shell_options.spmv,
 // BHEM_PCG_LOOP, BHEM_PCG_HOST_LOOP, BHEM_PCG_PUPDATE).
 shell_status setup_resident(Shell& s) {
