@@ -25,9 +25,15 @@
 // ERRBIT_TIMEOUT and leaves, and the others then expire too. The launch is cooperative, so all CTAs
 // are resident.
 //
-// Arithmetic: the p-update is applied by each CTA to its copies of the neighbours' p (p = z + beta p
-// on the same values everywhere), so A p is formed from p itself, as with separate kernels; sums
-// over a row's blocks and over CTAs are taken in another order than there.
+// Arithmetic. FP32: that of the separate kernels on shells of these sizes (k_precond32_thread,
+// k_spmv32_pcg, k_pcg32_update), operation by operation and in their order: Cholesky inverses, w =
+// (A + tau D) z along a row's blocks, p = z + beta p and q = w + beta q on the own rows, alpha and beta
+// as their FP64 quotients rounded to FP32. Only the double-float sums over the grid (48 bits) and the
+// statistics' FP64 sums are taken in another order, so a solve has the separate kernels' bits unless
+// one of its scalars lies that close to the middle of two FP32 numbers. (Sums over blocks in thirds,
+// A p formed from p itself and Gauss-Jordan inverses moved 50 iterations by 5e-7 and a step to 1e-8 by
+// 5e-9.) FP64: the p-update is applied by each CTA to its copies of the neighbours' p, a row is summed
+// in nine pieces and the inverses are by Gauss-Jordan elimination; a step moves by 1e-14 with it.
 #include <algorithm>
 
 #include "common.cuh"
@@ -73,15 +79,25 @@ template <> struct Acc<float> {
   static __device__ __forceinline__ double value(T a) { return (double)a.hi + (double)a.lo; }
   static __device__ __forceinline__ bool nonzero(T a) { return a.hi != 0.f || a.lo != 0.f; }
   static __device__ __forceinline__ bool positive(T a) { return a.hi > 0.f || (a.hi == 0.f && a.lo > 0.f); }
-  // a / b rounded to FP32: an FP32 quotient and one correction by the double-float remainder (the
-  // FP64 quotient of the separate kernels, which is rounded to FP32 there too, is a chain of
-  // dependent FP64 operations on this GPU: about 900 cycles against 200)
+  // a / b as the separate kernels form it, the FP64 quotient rounded to FP32: an FP32 quotient q and
+  // its correction d by the double-float remainder (the FP64 quotient is a chain of dependent FP64
+  // operations on this GPU, about 900 cycles against 200). q + d is within a few 2^-46 of a / b (the
+  // remainder is exact up to roundings of 2^-47 and d has 24 bits of at most 2^-23 q), so its rounding c
+  // is that of the quotient unless q + d lies within 2^-40 of the middle between c and a neighbour,
+  // or the operands leave the normal range: then the quotient is formed.
   static __device__ __forceinline__ float ratio(T a, T b) {
     const float q = __fdiv_rn(a.hi, b.hi);
     const F2 p = f2_prod(q, b.hi);
     const float rem = ((a.hi - p.hi) - p.lo) + __fmaf_rn(-q, b.lo, a.lo);
-    const float c = q + __fdiv_rn(rem, b.hi);
-    return isfinite(c) ? c : q;
+    const float d = __fdiv_rn(rem, b.hi);
+    const float c = q + d, off = fabsf((q - c) + d), m = fabsf(c);
+    const float below = 0.5f * (m - __int_as_float(__float_as_int(m) - 1));   // half the gaps to c's neighbours
+    const float above = 0.5f * (__int_as_float(__float_as_int(m) + 1) - m);
+    const float eps = 0x1p-40f * m;
+    const bool sure = m > 0x1p-60f && m < 0x1p60f && fabsf(a.hi) > 0x1p-60f && fabsf(a.hi) < 0x1p60f &&
+                      fabsf(b.hi) > 0x1p-60f && fabsf(b.hi) < 0x1p60f && fabsf(off - below) > eps &&
+                      fabsf(off - above) > eps;
+    return sure ? c : (float)(value(a) / value(b));
   }
   static __device__ __forceinline__ Word2 pack(T a, unsigned tag) {
     return Word2{tagged(__float_as_uint(a.hi), tag), tagged(__float_as_uint(a.lo), tag)};
@@ -311,15 +327,87 @@ __device__ bool all_stats(const ResidentArgs& P, const R* sA, const int* sdiag, 
   return true;
 }
 
-template <typename R>
-__host__ __device__ constexpr size_t resident_row_bytes() {
-  // matrix, block-Jacobi inverse, staged p of the row's columns, partial sums of the product
-  return sizeof(R) * (kRowBlocks * 144 + 144 + kRowBlocks * 12 + 108 + 12) + sizeof(int) * (kRowBlocks + 1);
+// Row l of a node's 12 x 12 block in m becomes row l of its inverse (lanes 0-11 of each half warp; all 32
+// lanes call it); false in every lane of the half when the block is not SPD (m is then void).
+// By Cholesky, A = L L^T, W = L^{-1}, A^{-1} = W^T W: the operations of k_precond32_thread on every entry, in
+// its order. Lane a holds row a of L, then column a of W.
+__device__ __forceinline__ bool cholesky_inverse_row(float (&m)[12], int l) {
+  bool spd = true;
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    const float piv = __shfl_sync(0xffffffffu, m[k], k, 16);
+    if (!(piv > 0.f)) spd = false;
+    const float r = sqrtf(piv);
+    m[k] = l == k ? r : m[k] / r;
+#pragma unroll
+    for (int j = k + 1; j < 12; ++j)   // entries above the diagonal are never read
+      m[j] = __fmaf_rn(-m[k], __shfl_sync(0xffffffffu, m[k], j, 16), m[j]);
+  }
+  float w[12];
+#pragma unroll
+  for (int r = 0; r < 12; ++r) {
+    float u = r == l ? 1.f : 0.f;
+#pragma unroll
+    for (int k = 0; k < r; ++k) u = __fmaf_rn(-__shfl_sync(0xffffffffu, m[k], r, 16), w[k], u);   // w[k] = 0 for k < l
+    w[r] = u / __shfl_sync(0xffffffffu, m[r], r, 16);
+  }
+#pragma unroll
+  for (int b = 0; b < 12; ++b) {
+    float s = 0.f;
+#pragma unroll
+    for (int k = b; k < 12; ++k) s = __fmaf_rn(w[k], __shfl_sync(0xffffffffu, w[k], b, 16), s);
+    m[b] = s;
+  }
+  return spd;
 }
 
-// A row's product is 108 pieces (3 blocks x 4 entries of one matrix row), of which a thread has up to
-// PASSES, in registers for the whole loop; PASSES 0: read from shared memory. Of the neighbours' p
-// (27 pieces of 4 DOFs per row) a thread of warps 2 and up has up to PIECES.
+// By Gauss-Jordan elimination without pivoting; its pivots are the squared pivots of a Cholesky
+// factorisation.
+__device__ __forceinline__ bool gauss_jordan_row(double (&m)[12], int l) {
+  bool spd = true;
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    const double piv = __shfl_sync(0xffffffffu, m[k], k, 16);
+    if (!(piv > 0.0)) spd = false;
+    const double inv = 1.0 / piv, f = m[k];
+    if (l == k) {   // the pivot row is scaled once, then broadcast
+      m[k] = 1.0;
+#pragma unroll
+      for (int b = 0; b < 12; ++b) m[b] *= inv;
+    }
+#pragma unroll
+    for (int b = 0; b < 12; ++b) {
+      const double rk = __shfl_sync(0xffffffffu, m[b], k, 16);
+      if (l != k) m[b] = b == k ? -f * rk : __fma_rn(-f, rk, m[b]);
+    }
+  }
+  return spd;
+}
+
+// How a row's product is shared out. A piece covers 4 entries of one matrix row in each of kBlocks blocks:
+// FP32 all nine, one chain of products as in k_spmv32_pcg (36 pieces per row); FP64 three (108 pieces).
+// Piece e of a CTA is piece e % kPieces of row e / kPieces; its matrix row's kSums sums lie side by side.
+template <typename R> struct Product {
+  static constexpr int kBlocks = sizeof(R) == 4 ? kRowBlocks : 3;
+  static constexpr int kEntries = 4 * kBlocks;
+  static constexpr int kSums = 3 * kRowBlocks / kBlocks;
+  static constexpr int kPieces = 12 * kSums;
+};
+// first block, matrix row and first column of piece w of a row
+template <typename R> __device__ __forceinline__ int3 piece_of(int w) {
+  using P = Product<R>;
+  return make_int3(w % P::kSums / 3 * P::kBlocks, w / P::kSums, w % 3 * 4);
+}
+
+template <typename R>
+__host__ __device__ constexpr size_t resident_row_bytes() {
+  // matrix, block-Jacobi inverse, staged vector of the row's columns, partial sums of the product
+  return sizeof(R) * (kRowBlocks * 144 + 144 + kRowBlocks * 12 + 12 * Product<R>::kSums + 12) + sizeof(int) * (kRowBlocks + 1);
+}
+
+// A row's product is Product<R>::kPieces pieces, of which a thread has up to PASSES, in registers for the
+// whole loop; PASSES 0: read from shared memory. Of the neighbours' exchanged values (27 pieces of 4
+// DOFs per row) a thread of warps 2 and up has up to PIECES.
 template <typename R, int PASSES, int PIECES>
 __global__ void __launch_bounds__(kResThreads, 1) k_solve_resident(ResidentArgs P) {
   using A = Acc<R>;
@@ -327,9 +415,9 @@ __global__ void __launch_bounds__(kResThreads, 1) k_solve_resident(ResidentArgs 
   extern __shared__ __align__(16) unsigned char sraw[];
   R* sA = reinterpret_cast<R*>(sraw);                      // [per][9][12][12]
   R* sD = sA + (size_t)P.per * kRowBlocks * 144;           // [per][12][12]
-  R* sx = sD + (size_t)P.per * 144;                        // [per][9][12] p of each block's column
-  R* sacc = sx + (size_t)P.per * kRowBlocks * 12;          // [per][12][9]
-  R* sr = sacc + (size_t)P.per * 108;                      // [per][12]
+  R* sx = sD + (size_t)P.per * 144;                        // [per][9][12] z (FP64: p) of each block's column
+  R* sacc = sx + (size_t)P.per * kRowBlocks * 12;          // [per][12][kSums]
+  R* sr = sacc + (size_t)P.per * 12 * Product<R>::kSums;   // [per][12]
   int* scol = reinterpret_cast<int*>(sr + (size_t)P.per * 12);   // [per][9]
   int* sdiag = scol + P.per * kRowBlocks;                  // [per] slot of the diagonal block
   __shared__ double swarp_d[96];                           // warp partials of up to three sums
@@ -402,9 +490,8 @@ __global__ void __launch_bounds__(kResThreads, 1) k_solve_resident(ResidentArgs 
     __syncthreads();
   }
 
-  // ---- block-Jacobi: (A_ii masked + tau D)^{-1} by Gauss-Jordan elimination without pivoting, one
-  // row per lane, two nodes per warp. Its pivots are the squared pivots of a Cholesky factorisation:
-  // a pivot that is not positive (block not SPD) falls back to the inverse of the diagonal.
+  // ---- block-Jacobi: (A_ii masked + tau D)^{-1}, one row per lane, two nodes per warp. A block that is
+  // not SPD falls back to the inverse of its diagonal.
   for (int base = wid * 2; base < rows; base += (nt >> 5) * 2) {
     const int l = lane & 15, row = base + (lane >> 4);
     const bool act = row < rows && l < 12;
@@ -422,22 +509,8 @@ __global__ void __launch_bounds__(kResThreads, 1) k_solve_resident(ResidentArgs 
       if (l == b) dg = v;
     }
     bool spd = true;
-#pragma unroll
-    for (int k = 0; k < 12; ++k) {
-      const R piv = __shfl_sync(0xffffffffu, m[k], k, 16);
-      if (!(piv > R(0))) spd = false;
-      const R inv = R(1) / piv, f = m[k];
-      if (l == k) {   // the pivot row is scaled once, then broadcast
-        m[k] = R(1);
-#pragma unroll
-        for (int b = 0; b < 12; ++b) m[b] *= inv;
-      }
-#pragma unroll
-      for (int b = 0; b < 12; ++b) {
-        const R rk = __shfl_sync(0xffffffffu, m[b], k, 16);
-        if (l != k) m[b] = b == k ? -f * rk : fma_r(-f, rk, m[b]);
-      }
-    }
+    if constexpr (sizeof(R) == 4) spd = cholesky_inverse_row(m, l);
+    else spd = gauss_jordan_row(m, l);
     if (act) {
       if (!spd) {
 #pragma unroll
@@ -447,32 +520,35 @@ __global__ void __launch_bounds__(kResThreads, 1) k_solve_resident(ResidentArgs 
       for (int b = 0; b < 12; ++b) sD[(size_t)row * 144 + l * 12 + b] = m[b];
     }
     __syncwarp();
-    // exactly symmetric: the mean of the two triangles
-    if (act) {
+    if constexpr (sizeof(R) == 8) {   // exactly symmetric: the mean of the two triangles
+      if (act) {
 #pragma unroll
-      for (int b = 0; b < 12; ++b) m[b] = R(0.5) * (m[b] + sD[(size_t)row * 144 + b * 12 + l]);
-    }
-    __syncwarp();
-    if (act) {
+        for (int b = 0; b < 12; ++b) m[b] = R(0.5) * (m[b] + sD[(size_t)row * 144 + b * 12 + l]);
+      }
+      __syncwarp();
+      if (act) {
 #pragma unroll
-      for (int b = 0; b < 12; ++b) sD[(size_t)row * 144 + l * 12 + b] = m[b];
+        for (int b = 0; b < 12; ++b) sD[(size_t)row * 144 + l * 12 + b] = m[b];
+      }
     }
   }
 
   // this thread's pieces of the products
-  R areg[PASSES > 0 ? PASSES : 1][12];
-  int xoff[PASSES > 0 ? PASSES : 1];   // the piece's entries of the staged p; its sum goes to sacc[t + s nt]
+  using PR = Product<R>;
+  R areg[PASSES > 0 ? PASSES : 1][PR::kEntries];
+  int xoff[PASSES > 0 ? PASSES : 1];   // the piece's entries of the staged vector; its sum goes to sacc[t + s nt]
   if (PASSES > 0) {
 #pragma unroll
     for (int s = 0; s < PASSES; ++s) {
-      const int e = t + s * nt, row = e / 108, w = e % 108, r = w / 9, bg = (w % 9) / 3, cc = w % 3;
-      xoff[s] = row < rows ? (row * kRowBlocks + bg * 3) * 12 + cc * 4 : 0;
+      const int e = t + s * nt, row = e / PR::kPieces;
+      const int3 w = piece_of<R>(e % PR::kPieces);
+      xoff[s] = row < rows ? (row * kRowBlocks + w.x) * 12 + w.z : 0;
 #pragma unroll
-      for (int k = 0; k < 12; ++k)
-        areg[s][k] = row < rows ? sA[(size_t)(row * kRowBlocks + bg * 3 + k / 4) * 144 + r * 12 + cc * 4 + k % 4] : R(0);
+      for (int k = 0; k < PR::kEntries; ++k)
+        areg[s][k] = row < rows ? sA[(size_t)(row * kRowBlocks + w.x + k / 4) * 144 + w.y * 12 + w.z + k % 4] : R(0);
     }
   }
-  // this thread's pieces of the neighbours' p: z as received, p, and the first DOF (-1: none)
+  // this thread's pieces of the neighbours' vectors: z as received, p (FP64), and the first DOF (-1: none)
   R zn[PIECES][4] = {}, pn[PIECES][4] = {};
   int piece_gi[PIECES];
 #pragma unroll
@@ -545,17 +621,19 @@ __global__ void __launch_bounds__(kResThreads, 1) k_solve_resident(ResidentArgs 
 
   // ---- PCG
   while (!done) {
-    // p = z + beta p of every block's column
+    // z (FP64: p = z + beta p) of every block's column
     const R beta = s_scal;
 #pragma unroll
     for (int s = 0; s < PIECES; ++s)
       if (piece_gi[s] >= 0) {
         R* x = sx + (t - 64 + s * (nt - 64)) * 4;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) x[k] = pn[s][k] = fma_r(beta, pn[s][k], zn[s][k]);
+        for (int k = 0; k < 4; ++k) {
+          if constexpr (sizeof(R) == 8) x[k] = pn[s][k] = fma_r(beta, pn[s][k], zn[s][k]);
+          else x[k] = zn[s][k];
+        }
       }
     __syncthreads();
-    // piece (row, r, bg, cc): 3 blocks x 4 entries of matrix row r, so that a row's 9 pieces are neighbours
     if (PASSES > 0) {
 #pragma unroll
       for (int s = 0; s < PASSES; ++s) {
@@ -563,17 +641,18 @@ __global__ void __launch_bounds__(kResThreads, 1) k_solve_resident(ResidentArgs 
         const R* x = sx + xoff[s];
         R acc = R(0);
 #pragma unroll
-        for (int k = 0; k < 12; ++k) acc = fma_r(areg[s][k], x[(k / 4) * 12 + k % 4], acc);
-        if (e < rows * 108) sacc[e] = acc;
+        for (int k = 0; k < PR::kEntries; ++k) acc = fma_r(areg[s][k], x[(k / 4) * 12 + k % 4], acc);
+        if (e < rows * PR::kPieces) sacc[e] = acc;
       }
     } else {
-      for (int e = t; e < rows * 108; e += nt) {
-        const int row = e / 108, w = e % 108, r = w / 9, bg = (w % 9) / 3, cc = w % 3;
-        const R* m = sA + (size_t)(row * kRowBlocks + bg * 3) * 144 + r * 12 + cc * 4;
-        const R* x = sx + (row * kRowBlocks + bg * 3) * 12 + cc * 4;
+      for (int e = t; e < rows * PR::kPieces; e += nt) {
+        const int row = e / PR::kPieces;
+        const int3 w = piece_of<R>(e % PR::kPieces);
+        const R* m = sA + (size_t)(row * kRowBlocks + w.x) * 144 + w.y * 12 + w.z;
+        const R* x = sx + (row * kRowBlocks + w.x) * 12 + w.z;
         R acc = R(0);
 #pragma unroll
-        for (int k = 0; k < 12; ++k) acc = fma_r(m[(k / 4) * 144 + k % 4], x[(k / 4) * 12 + k % 4], acc);
+        for (int k = 0; k < PR::kEntries; ++k) acc = fma_r(m[(k / 4) * 144 + k % 4], x[(k / 4) * 12 + k % 4], acc);
         sacc[e] = acc;
       }
     }
@@ -581,11 +660,19 @@ __global__ void __launch_bounds__(kResThreads, 1) k_solve_resident(ResidentArgs 
     if (wid < own_warps) {
       AT v[1] = {A::zero()};
       if (own) {
-        const R* s = sacc + (size_t)(myrow * 12 + a) * 9;
-        R y = (((s[0] + s[1]) + s[2]) + ((s[3] + s[4]) + s[5])) + ((s[6] + s[7]) + s[8]);
-        pv = sx[(myrow * kRowBlocks + sdiag[myrow]) * 12 + a];
-        y = fma_r(s_td[a / 3], pv, y);
-        qv = fixed_dof ? R(0) : y;
+        const R* s = sacc + (size_t)(myrow * 12 + a) * PR::kSums;
+        if constexpr (sizeof(R) == 8) {
+          R y = (((s[0] + s[1]) + s[2]) + ((s[3] + s[4]) + s[5])) + ((s[6] + s[7]) + s[8]);
+          pv = sx[(myrow * kRowBlocks + sdiag[myrow]) * 12 + a];
+          y = fma_r(s_td[a / 3], pv, y);
+          qv = fixed_dof ? R(0) : y;
+        } else {   // w = (A + tau D) z, p = z + beta p, q = w + beta q (= A p by linearity)
+          R w = (s[0] + s[1]) + s[2];
+          w = fma_r(s_td[a / 3], zv, w);
+          if (fixed_dof) w = R(0);
+          pv = fma_r(beta, pv, zv);
+          qv = fma_r(beta, qv, w);
+        }
         v[0] = A::prod(pv, qv);
       }
       warp_partials<R, 1>(v, swarp);
@@ -708,14 +795,13 @@ size_t resident_tail_bytes() {
 
 using ResidentKernel = void (*)(ResidentArgs);
 
-// The kernel for `per` rows per CTA: passes of 512 threads over 108 pieces per row, pieces of 448
-// threads over 27 per row. FP32 holds up to 6 passes of the matrix in registers (72), FP64 up to 2.
+// The kernel for `per` rows per CTA: passes of 512 threads over a row's pieces of the product (36 in FP32,
+// 108 in FP64), pieces of 448 threads over 27 per row. FP32 holds two passes of the matrix in registers
+// (72), FP64 two (24 FP64 values).
 template <typename R> ResidentKernel resident_kernel(int per);
 template <> ResidentKernel resident_kernel<float>(int per) {
-  if (per <= 9) return k_solve_resident<float, 2, 1>;
-  if (per <= 14) return k_solve_resident<float, 3, 1>;
-  if (per <= 18) return k_solve_resident<float, 4, 2>;
-  if (per <= 28) return k_solve_resident<float, 6, 2>;
+  if (per <= 14) return k_solve_resident<float, 1, 1>;
+  if (per <= 28) return k_solve_resident<float, 2, 2>;
   return k_solve_resident<float, 0, 2>;
 }
 template <> ResidentKernel resident_kernel<double>(int per) {

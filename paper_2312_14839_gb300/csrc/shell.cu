@@ -602,10 +602,11 @@ static shell_status residual(Shell& s, const double* q, const shell_step_params&
   return SHELL_OK;
 }
 
-// Whether a Newton step's linear solves are resident launches. Not in mixed precision with colour-ordered assembly,
-// whose sums have one order from run to run: the resident solve adds its dot products in another order, and
-// a step moves with it by up to 5e-9 (a noisy 40 x 30 sheet, the steps' tolerance) where atomic
-// assembly moves it as far between two runs. FP64 steps move by 1e-14.
+// Whether a Newton step's linear solves are resident launches. Mixed-precision shells with colour-ordered assembly,
+// chosen for steps with the same bits on every run, keep the separate kernels' bits too: both forms have one
+// order of sums from run to run, but not the same one, and a scalar that rounds the other way (a chance of
+// about 1e-5 each) would move a step by up to 5e-9, its tolerance, as far as atomic assembly moves it
+// between two runs. FP64 steps move by 1e-14.
 static bool newton_resident(const Shell& s) {
   return s.res_per > 0 && (s.val_fp64 || s.opt.assembly != SHELL_ASM_COLOR);
 }
