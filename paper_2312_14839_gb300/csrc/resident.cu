@@ -21,7 +21,9 @@
 // order, so all CTAs hold the same totals and take the same decisions. Tags grow
 // from exchange to exchange and from launch to launch (Shell::res_tag). A slot is rewritten only
 // after a later reduction to which every reader of its old value has contributed, so no reader can
-// miss a value. Each wait polls at most Shell::wait_polls times; on expiry the CTA raises
+// miss a value: z of an iteration after the next p.q, which a CTA joins when it has received its
+// neighbours' z. (Its part of r.z and r.r it sends before that, so when those sums end the loop z
+// may still be on its way to a late CTA: the solution travels in words of its own.) Each wait polls at most Shell::wait_polls times; on expiry the CTA raises
 // ERRBIT_TIMEOUT and leaves, and the others then expire too. The launch is cooperative, so all CTAs
 // are resident.
 //
@@ -185,6 +187,7 @@ struct ResidentArgs {
   const double *mass, *gin;          // dots only
   double* Md;
   unsigned long long* vec;           // exchanged vector, kDofWords words per DOF
+  unsigned long long* xvec;          // the same for the solution, written once per launch
   void* stat_records;                // [4][kResSlotCtas] KindStat of each CTA
   unsigned* stat_count;              // CTAs that have written theirs, over all launches
   unsigned stat_target;              // its value when those of this launch have
@@ -557,11 +560,11 @@ __global__ void __launch_bounds__(kResThreads, 1) k_solve_resident(ResidentArgs 
     const int j = t >= 64 && e < rows * 27 ? scol[e / 3] : -1;
     piece_gi[s] = j < 0 ? -1 : j * 12 + (e % 3) * 4;
   }
-  auto receive_pieces = [&](unsigned tag) -> bool {
+  auto receive_pieces = [&](const unsigned long long* vec, unsigned tag) -> bool {
     bool ok = true;
 #pragma unroll
     for (int s = 0; s < PIECES; ++s)
-      if (piece_gi[s] >= 0) ok = receive4(P.vec, piece_gi[s], tag, P.polls, zn[s]) && ok;
+      if (piece_gi[s] >= 0) ok = receive4(vec, piece_gi[s], tag, P.polls, zn[s]) && ok;
     return ok;
   };
 
@@ -606,7 +609,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_solve_resident(ResidentArgs 
         s_stop = first ? bb == 0.0 : (P.fixed == 0 && rr <= P.rtol2 * bb);
       }
     } else {
-      ok = receive_pieces(tag);
+      ok = receive_pieces(P.vec, tag);
     }
     if (!ok) s_fail = 1;
     __syncthreads();
@@ -722,9 +725,9 @@ __global__ void __launch_bounds__(kResThreads, 1) k_solve_resident(ResidentArgs 
   if (!P.dots || negcurv) return;
   // M d on the own rows and d.Md, d.gin, g.d (rhs = -g) for the line search, in FP64
   const unsigned tagx = P.tag + (unsigned)max(P.limit, 0) + 3u;
-  if (own) publish(P.vec, gi, xv, tagx);
+  if (own) publish(P.xvec, gi, xv, tagx);
   bool ok = true;
-  if (wid >= 2) ok = receive_pieces(tagx);
+  if (wid >= 2) ok = receive_pieces(P.xvec, tagx);
 #pragma unroll
   for (int s = 0; s < PIECES; ++s)
     if (piece_gi[s] >= 0) {
@@ -788,6 +791,11 @@ size_t resident_slot_bytes(int ctas) {
   return sizeof(Word2) * kResSlotCtas * kSums * ctas;
 }
 
+// the exchanged vectors: z and the solution
+size_t resident_vec_bytes(const Shell& s) {
+  return 2 * sizeof(unsigned long long) * (s.val_fp64 ? kDofWords<double> : kDofWords<float>) * (size_t)s.n_dof;
+}
+
 // the statistics' records, the dot products' partials, two counters
 size_t resident_tail_bytes() {
   return sizeof(KindStat<double>) * 4 * kResSlotCtas + sizeof(double) * 3 * kResSlotCtas + sizeof(unsigned) * 4;
@@ -840,9 +848,7 @@ shell_status resident_setup(Shell& s) {
   BHEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void*)k, kResThreads, smem));
   const int ctas = (s.n_nodes + per - 1) / per;
   if (occ < 1 || ctas > sms) return SHELL_OK;
-  const size_t vec_bytes = sizeof(unsigned long long) * kDofWords<R> * (size_t)s.n_dof;
-  const size_t slot_bytes = resident_slot_bytes(ctas);
-  const size_t bytes = slot_bytes + vec_bytes + resident_tail_bytes();
+  const size_t bytes = resident_slot_bytes(ctas) + resident_vec_bytes(s) + resident_tail_bytes();
   if (cudaMalloc(&s.d_resident, bytes) != cudaSuccess) {
     cudaGetLastError();
     s.d_resident = nullptr;
@@ -866,7 +872,7 @@ shell_status launch_solve_resident(Shell& s, const unsigned char* mask, const do
                                    bool* launched) {
   const int ctas = (s.n_nodes + s.res_per - 1) / s.res_per;
   const size_t slot_bytes = resident_slot_bytes(ctas);
-  const size_t vec_bytes = sizeof(unsigned long long) * (s.val_fp64 ? 2 : 1) * (size_t)s.n_dof;
+  const size_t vec_bytes = resident_vec_bytes(s);
   const unsigned used = (unsigned)std::max(limit, 0) + 8u;
   if (s.res_reset || s.res_tag > 0xffffffffu - used) {   // first use, after an error, or the tags wrap
     BHEM_CUDA(cudaMemsetAsync(s.d_resident, 0, slot_bytes + vec_bytes + resident_tail_bytes(), s.stream));
@@ -900,6 +906,7 @@ shell_status launch_solve_resident(Shell& s, const unsigned char* mask, const do
   char* base = (char*)s.d_resident;
   P.slots = (Word2*)base;
   P.vec = (unsigned long long*)(base + slot_bytes);
+  P.xvec = (unsigned long long*)(base + slot_bytes + vec_bytes / 2);
   P.stat_records = base + slot_bytes + vec_bytes;
   P.partials = (double*)(base + slot_bytes + vec_bytes + sizeof(KindStat<double>) * 4 * kResSlotCtas);
   P.ticket = (unsigned*)(P.partials + 3 * kResSlotCtas);
