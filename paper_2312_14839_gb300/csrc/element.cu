@@ -179,8 +179,9 @@ k_energy_grad64(int np, const int4* __restrict__ pnodes, const double* __restric
 shell_status launch_energy_grad64(Shell& s, const double* q, const double* dir, double step,
                                   double* energy_p, const double* energy_ref, double* grad,
                                   double* scal_out) {
-  // A warp per patch while every SM sub-partition (four per SM) then has one patch at most: 215 FP64
-  // instructions one after another instead of 330; with more patches half a warp each does them in less.
+  // A warp per patch while every SM sub-partition (four per SM) then has one patch at most: two thirds of the
+  // FP64 instructions one after another (24 x 24 patches 20.5 us a call, 30 x 30 by half a warp each 26.1); with
+  // more patches half a warp each does them in less.
   const bool warp = s.n_patches <= 4 * s.num_sms;
   const int per = warp ? kEgPatches / 2 : kEgPatches;
   int blocks = (s.n_patches + per - 1) / per;

@@ -82,10 +82,8 @@ template <typename R> __device__ __forceinline__ R dot(V3<R> a, V3<R> b) { retur
 template <typename R> __device__ __forceinline__ V3<R> cross(V3<R> a, V3<R> b) {
   return {a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x};
 }
-// a . b - c and a x b + c as chains of fused multiply-adds
-template <typename R> __device__ __forceinline__ R dot_less(V3<R> a, V3<R> b, R c) { return a.x * b.x + (a.y * b.y + (a.z * b.z - c)); }
-template <typename R> __device__ __forceinline__ V3<R> cross_plus(V3<R> a, V3<R> b, V3<R> c) {
-  return {a.y * b.z + (c.x - a.z * b.y), a.z * b.x + (c.y - a.x * b.z), a.x * b.y + (c.z - a.y * b.x)};
+template <typename R> __device__ __forceinline__ V3<R> pick(bool c, V3<R> a, V3<R> b) {
+  return {c ? a.x : b.x, c ? a.y : b.y, c ? a.z : b.z};
 }
 template <typename R> __device__ __forceinline__ R comp(V3<R> a, int i) { return i == 0 ? a.x : i == 1 ? a.y : a.z; }
 
@@ -231,29 +229,29 @@ __device__ __forceinline__ double eg64_patch(const double* w1, const double* w2,
     if (!(nn > 0.0)) atomicOr(err, ERRBIT_DEGENERATE);
     else isqa = rsqrt(nn);
     V3<double> a3 = isqa * n;
-    // strains; the rest value opens each sum of products, so that subtracting it costs no instruction
-    const double al[3] = {0.5 * dot_less(a1, a1, ab11), 0.5 * dot_less(a2, a2, ab22), dot_less(a1, a2, ab12)};
-    const double be[3] = {dot_less(v[2], a3, bb11), dot_less(v[3], a3, bb22), 2.0 * dot_less(v[4], a3, bb12)};
+    double b11 = dot(v[2], a3), b22 = dot(v[3], a3), b12 = dot(v[4], a3);
+    double al[3] = {0.5 * (dot(a1, a1) - ab11), 0.5 * (dot(a2, a2) - ab22), dot(a1, a2) - ab12};
+    double be[3] = {b11 - bb11, b22 - bb22, 2.0 * (b12 - bb12)};
     double sg[3] = {H00 * al[0] + H01 * al[1] + H02 * al[2], H01 * al[0] + H11 * al[1] + H12 * al[2],
                     H02 * al[0] + H12 * al[1] + H22 * al[2]};
     double mm[3] = {H00 * be[0] + H01 * be[1] + H02 * be[2], H01 * be[0] + H11 * be[1] + H12 * be[2],
                     H02 * be[0] + H12 * be[1] + H22 * be[2]};
-    const double wh = wgt * h, ws = wgt * (h * h * h * (1.0 / 12.0));
-    e = 0.5 * (wh * (al[0] * sg[0] + al[1] * sg[1] + al[2] * sg[2]) +
-               ws * (be[0] * mm[0] + be[1] * mm[1] + be[2] * mm[2]));
+    const double h3 = h * h * h;
+    e = wgt * (0.5 * h * (al[0] * sg[0] + al[1] * sg[1] + al[2] * sg[2]) +
+               h3 * (1.0 / 24.0) * (be[0] * mm[0] + be[1] * mm[1] + be[2] * mm[2]));
     if (grad) {
-      // with the weights in sigma and m: K = (c~ - (c~ . a3) a3) / sqrt(a) carries both directions' normal
-      // derivative, a_2 x K and K x a_1
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        sg[k] *= wh;
-        mm[k] *= ws;
-      }
-      mm[2] += mm[2];
-      const V3<double> ct = mm[0] * v[2] + mm[1] * v[3] + mm[2] * v[4];
-      const V3<double> K = isqa * (ct - dot(ct, a3) * a3);
-      const V3<double> G[5] = {cross_plus(a2, K, sg[0] * a1 + sg[2] * a2), cross_plus(K, a1, sg[1] * a2 + sg[2] * a1),
-                               mm[0] * a3, mm[1] * a3, mm[2] * a3};
+      const double s = h3 * (1.0 / 12.0);
+      V3<double> ct = mm[0] * v[2] + mm[1] * v[3] + (2.0 * mm[2]) * v[4];
+      double bt = dot(ct, a3);
+      V3<double> t1 = cross(a2, a3), t2 = cross(a3, a1);
+      V3<double> e1 = isqa * (cross(a2, ct) - bt * t1);
+      V3<double> e2 = isqa * (cross(ct, a1) - bt * t2);
+      V3<double> G[5];
+      G[0] = wgt * (h * (sg[0] * a1 + sg[2] * a2) + s * e1);
+      G[1] = wgt * (h * (sg[1] * a2 + sg[2] * a1) + s * e2);
+      G[2] = (wgt * s * mm[0]) * a3;
+      G[3] = (wgt * s * mm[1]) * a3;
+      G[4] = (wgt * s * 2.0 * mm[2]) * a3;
 #pragma unroll
       for (int k = 0; k < 5; ++k) {
         sG[g][k * 3 + 0] = G[k].x;
@@ -300,9 +298,10 @@ __device__ __forceinline__ double eg64_patch(const double* w1, const double* w2,
 
 // The same for one patch by a whole warp (lane = 16 half + Gauss point), for launches that leave the FP64
 // pipes short of patches: what the two directions (or the membrane and the bending part) have alike is done
-// once per half. 215 FP64 instructions in a chain, where half a warp takes 330 for its patch and its
-// neighbour's: shorter for a warp that has one patch, longer for one that has many. sq, sT, sG as above,
-// one set per warp. All lanes call it; returns the patch energy in every lane.
+// once per half. About two thirds of the FP64 instructions that half a warp takes in a chain for its patch and
+// its neighbour's (368): shorter for a warp that has one patch, longer for one that has many. sq, sT, sG as above,
+// one set per warp. All lanes call it; returns the patch energy in lanes 0-15. Every value is formed by the
+// operations of eg64_patch on it, so that a shell's results do not change with the form its size selects.
 __device__ __forceinline__ double eg64_patch_warp(const double* w1, const double* w2, double* sq, double* sT,
                                                   double (*sG)[15], int p, bool active, int lane, const int nd[4],
                                                   const double* __restrict__ q,
@@ -362,28 +361,29 @@ __device__ __forceinline__ double eg64_patch_warp(const double* w1, const double
     if (nn > 0.0) isqa = rsqrt(nn);
     else if (active) atomicOr(err, ERRBIT_DEGENERATE);
     V3<double> a3 = isqa * n;
-    const V3<double> y1 = half ? a3 : a1, y2 = half ? a3 : a2;
-    const V3<double> z1 = half ? x11 : a1, z2 = half ? x22 : a2, z3 = half ? x12 : a1;
-    const double f = half ? 1.0 : 0.5;
-    const double st[3] = {f * dot_less(z1, y1, r11), f * dot_less(z2, y2, r22), (f + f) * dot_less(z3, y2, r12)};
-    double t[3] = {H00 * st[0] + H01 * st[1] + H02 * st[2], H01 * st[0] + H11 * st[1] + H12 * st[2],
-                   H02 * st[0] + H12 * st[1] + H22 * st[2]};
-    const double w = wgt * (half ? h * h * h * (1.0 / 12.0) : h);
-    if (active) e = 0.5 * w * (st[0] * t[0] + st[1] * t[1] + st[2] * t[2]);
+    // strains of the half: 0.5 (a_1 . a_1 - a_bar_11), ... or x_,11 . a_3 - b_bar_11, ... (the factors are powers of
+    // two: no rounding)
+    const bool bend = half != 0;
+    const V3<double> y1 = pick(bend, a3, a1), y2 = pick(bend, a3, a2);
+    const V3<double> z1 = pick(bend, x11, a1), z2 = pick(bend, x22, a2), z3 = pick(bend, x12, a1);
+    const double f = bend ? 1.0 : 0.5;
+    const double st[3] = {f * (dot(z1, y1) - r11), f * (dot(z2, y2) - r22), (f + f) * (dot(z3, y2) - r12)};
+    const double t[3] = {H00 * st[0] + H01 * st[1] + H02 * st[2], H01 * st[0] + H11 * st[1] + H12 * st[2],
+                         H02 * st[0] + H12 * st[1] + H22 * st[2]};
+    const double part = st[0] * t[0] + st[1] * t[1] + st[2] * t[2], bending = from_lane(part, 16 + g);
+    const double h3 = h * h * h;
+    if (active && !half) e = wgt * (0.5 * h * part + h3 * (1.0 / 24.0) * bending);
     if (grad) {
-#pragma unroll
-      for (int k = 0; k < 3; ++k) t[k] *= w;
+      const double s = h3 * (1.0 / 12.0);
       const double s1 = from_lane(t[0], g), s2 = from_lane(t[1], g), s12 = from_lane(t[2], g);
-      const double m0 = from_lane(t[0], 16 + g), m1 = from_lane(t[1], 16 + g);
-      double m2 = from_lane(t[2], 16 + g);
-      m2 += m2;
-      const V3<double> ct = m0 * x11 + m1 * x22 + m2 * x12;
-      V3<double> K = isqa * (ct - dot(ct, a3) * a3);
-      // half 0: sigma_1 a_1 + sigma_12 a_2 + a_2 x K, half 1: sigma_2 a_2 + sigma_12 a_1 - a_1 x K
-      const V3<double> P = half ? a1 : a2, own = half ? a2 : a1;
-      if (half) K = mk<double>(-K.x, -K.y, -K.z);
-      const V3<double> Gk = cross_plus(P, K, (half ? s2 : s1) * own + s12 * P);
-      const V3<double> Gb = (half ? m1 : m0) * a3, G4 = m2 * a3;
+      const double m0 = from_lane(t[0], 16 + g), m1 = from_lane(t[1], 16 + g), m2 = from_lane(t[2], 16 + g);
+      const V3<double> ct = m0 * x11 + m1 * x22 + (2.0 * m2) * x12;
+      const double bt = dot(ct, a3);
+      // half 0: a_2 x c~ - (c~ . a_3) a_2 x a_3 and G_1, half 1: c~ x a_1 - (c~ . a_3) a_3 x a_1 and G_2
+      const V3<double> tn = cross(pick(bend, a3, a2), pick(bend, a1, a3));
+      const V3<double> en = isqa * (cross(pick(bend, ct, a2), pick(bend, a1, ct)) - bt * tn);
+      const V3<double> Gk = wgt * (h * ((bend ? s2 : s1) * pick(bend, a2, a1) + s12 * pick(bend, a1, a2)) + s * en);
+      const V3<double> Gb = (wgt * s * (bend ? m1 : m0)) * a3;
       sG[g][half * 3 + 0] = Gk.x;
       sG[g][half * 3 + 1] = Gk.y;
       sG[g][half * 3 + 2] = Gk.z;
@@ -391,14 +391,15 @@ __device__ __forceinline__ double eg64_patch_warp(const double* w1, const double
       sG[g][6 + half * 3 + 1] = Gb.y;
       sG[g][6 + half * 3 + 2] = Gb.z;
       if (!half) {
+        const V3<double> G4 = (wgt * s * 2.0 * m2) * a3;
         sG[g][12] = G4.x;
         sG[g][13] = G4.y;
         sG[g][14] = G4.z;
       }
     }
   }
-  double ep = e;
-  for (int o = 16; o > 0; o >>= 1) ep += __shfl_xor_sync(0xffffffffu, ep, o);
+  double ep = e;   // lanes 0-15 among themselves; 0 in the others
+  for (int o = 8; o > 0; o >>= 1) ep += __shfl_xor_sync(0xffffffffu, ep, o);
   __syncwarp();
   if (active && grad) {
     for (int e2 = lane; e2 < 144; e2 += 32) {
