@@ -267,6 +267,8 @@ struct ElemOutputs {
   // results of launch_energy_grad64 without its energy total), in the same launch; grad64 zeroed
   double* energy64 = nullptr;   // [np]
   double* grad64 = nullptr;     // [n_dof]
+  // those by a warp per patch where no warp has a second one; the FP32 Hessian may then round otherwise
+  bool warp64 = false;
 };
 shell_status launch_element_full(Shell& s, const double* q, bool fp64, const ElemOutputs& out);
 

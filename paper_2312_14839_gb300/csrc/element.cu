@@ -455,6 +455,7 @@ shell_status launch_element_full(Shell& s, const double* q, bool fp64, const Ele
     A.herm64 = s.d_phi64 + kPhiHerm;
     A.energy64 = out.energy64;
     A.grad64 = out.grad64;
+    A.warp64 = out.warp64;
   }
   if (out.bsr && s.opt.assembly == SHELL_ASM_COLOR) {
     // colour-ordered: patches of one colour share no node, plain read-modify-write

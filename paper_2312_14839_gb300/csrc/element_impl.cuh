@@ -499,6 +499,7 @@ struct ElemArgs {
   const double* herm64;
   double* energy64;
   double* grad64;
+  int warp64;              // ElemOutputs::warp64
 };
 
 // Parameter derivatives a_1, a_2, x_,11, x_,22, x_,12 of one field (half 0: rest, half 1: displacement) at

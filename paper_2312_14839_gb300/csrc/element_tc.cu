@@ -110,7 +110,8 @@ __device__ __forceinline__ int cd_c(int cd) { return cd < 3 ? 0 : (cd < 5 ? 1 : 
 __device__ __forceinline__ int cd_d(int cd) { return cd < 3 ? cd : (cd < 5 ? cd - 2 : 2); }
 
 // kOneEach: no warp has a second patch, so the FP64 evaluation (A.grad64) takes a warp per patch; a form
-// of its own, because the two evaluations in one kernel cost it registers.
+// of its own, because the two evaluations in one kernel cost it registers and change the compiler's
+// contraction of the FP32 part.
 template <bool kOneEach>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_element_tc(ElemArgs A, unsigned polls) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -363,10 +364,12 @@ shell_status launch_full_tc(Shell& s, const ElemArgs& A, int work) {
   int blocks = (work + etc::kWarps - 1) / etc::kWarps;
   const int cap = s.num_sms * etc::kCtasPerSm;
   if (blocks > cap) blocks = cap;
-  // one patch per warp, FP64 too: 280 x 5 patches 68 us instead of 81 a call of shell_energy_grad_hess. Not for
-  // colour-ordered launches, whose sums have one order: the compiler contracts the FP32 part differently
-  // in the two forms, and a shell's first Hessian has to have the bits of its later ones.
-  auto k = A.grad64 && A.bsr_atomic && work <= blocks * etc::kWarps ? etc::k_element_tc<true> : etc::k_element_tc<false>;
+  // one patch per warp, FP64 too: 280 x 5 patches 68 us instead of 81 a call of shell_energy_grad_hess. Only where
+  // the caller allows it: the FP32 part of that form rounds differently (1.6% of a strip's entries, by an
+  // ulp), and a step's first Hessian has to have the bits of its later ones: with it, steps of a strip one patch
+  // wide, whose atomic sums have no order, moved by 1e-6 after ten PCG iterations.
+  auto k = A.grad64 && A.warp64 && A.bsr_atomic && work <= blocks * etc::kWarps ? etc::k_element_tc<true>
+                                                                                : etc::k_element_tc<false>;
   k<<<blocks, etc::kThreads, etc::kSmemBytes, s.stream>>>(A, (unsigned)s.wait_polls);
   BHEM_CUDA(cudaGetLastError());
   ++s.launches;

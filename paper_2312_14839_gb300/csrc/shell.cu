@@ -416,9 +416,9 @@ extern "C" shell_status shell_element_egh(shell_t* shell, const double* q, int p
 }
 
 namespace bhem {
-// energy64, grad64: FP64 patch energies and gradient in the same pass (FP32 shells; grad64 zeroed)
+// energy64, grad64, warp64: FP64 patch energies and gradient in the same pass (ElemOutputs)
 static shell_status assemble_hessian(Shell& s, const double* q, double mass_scale, double* energy64 = nullptr,
-                                     double* grad64 = nullptr) {
+                                     double* grad64 = nullptr, bool warp64 = false) {
   size_t bytes = (size_t)s.n_blocks * 144 * (s.val_fp64 ? sizeof(double) : sizeof(float));
   BHEM_CUDA(cudaMemsetAsync(s.d_val, 0, bytes, s.stream));
   ElemOutputs o;
@@ -427,6 +427,7 @@ static shell_status assemble_hessian(Shell& s, const double* q, double mass_scal
   o.pseudo = s.opt.hessian == SHELL_HESS_PSEUDO;
   o.energy64 = energy64;
   o.grad64 = grad64;
+  o.warp64 = warp64;
   return launch_element_full(s, q, s.val_fp64 != 0, o);
 }
 
@@ -445,7 +446,7 @@ extern "C" shell_status shell_energy_grad_hess(shell_t* shell, const double* q, 
     // works beside the FP32 one, and a small shell pays one kernel's latency (280 x 5 patches: 36 us for the
     // energy kernel alone)
     BHEM_CUDA(cudaMemsetAsync(grad, 0, sizeof(double) * s.n_dof, s.stream));
-    BHEM_TRY(assemble_hessian(s, q, mass_scale, s.d_Ep, grad));
+    BHEM_TRY(assemble_hessian(s, q, mass_scale, s.d_Ep, grad, true));
     return launch_energy_sum(s, s.d_Ep, energy ? energy : s.d_energy_tmp);
   }
   if (energy || grad) BHEM_TRY(elastic_energy_grad(s, q, energy, grad));

@@ -44,3 +44,26 @@ def test_gradient_of_a_patch_is_the_same_by_a_warp_and_by_half_a_warp(noise):
             G.append(sh.energy_grad_hess(dev(q), want_hessian=False)[1].cpu().numpy())
     a, b = map(columns, G)
     assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("n", [1, 7, SHORT, LONG])
+@pytest.mark.parametrize("fixed", [10, 0])
+def test_steps_of_a_strip_do_not_depend_on_the_assembly(n, fixed):
+    """Colour-ordered and atomic assembly of a strip form the same sums, so a step has the same Hessians; its
+    linear solves are the separate kernels' and the resident one, whose solutions agree (1e-9, as in
+    test_gpu_resident_bits.py)."""
+    from paper_2312_14839_gb300 import bhem
+    g, rest = S.flat_sheet(n, 1, float(n) / SHORT, 1.0 / SHORT)
+    q0 = S.noisy(rest, 3e-5, 2)
+    mask = dev(S.pinned_mask(g, [0, g.n_nodes - 1]))
+    params = bhem.step_params(dt=1e-3, gravity=(0.0, 0.0, -9.81), newton_max=2 if fixed else 200, pcg_max=2000,
+                              pcg_fixed_iters=fixed)
+    out = []
+    for assembly in ("color", "atomic"):
+        with bhem.Shell(g, S.SHEET_MATERIAL, dev(rest), precision="mixed", assembly=assembly) as sh:
+            q, v = dev(q0).clone(), torch.zeros(g.n_dof, dtype=torch.float64, device="cuda")
+            st = sh.newton_step(q, v, params, mask=mask, q_fixed=dev(q0))
+            out.append((q.cpu().numpy(), v.cpu().numpy(), st["newton_iters"], st["status"]))
+    (qa, va, ia, sa), (qb, vb, ib, sb) = out
+    assert (ia, sa) == (ib, sb)
+    assert np.linalg.norm(qa - qb) <= 1e-9 * np.linalg.norm(qa) and np.linalg.norm(va - vb) <= 1e-9 * np.linalg.norm(va)
