@@ -271,6 +271,8 @@ struct ElemOutputs {
   bool warp64 = false;
 };
 shell_status launch_element_full(Shell& s, const double* q, bool fp64, const ElemOutputs& out);
+// patches that the tensor-core form of the FP32 element pass has in flight, one per warp
+int element_tc_warps(const Shell& s);
 
 // Light FP64 kernel: per-patch energy (and assembled gradient) at q + step * dir.
 //   mode 0: energy_p[p] = E_p, grad += dE/dq (grad may be null), total -> scal_out

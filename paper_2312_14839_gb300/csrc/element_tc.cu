@@ -348,6 +348,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_element_tc(ElemArgs A,
 
 }  // namespace etc
 
+int element_tc_warps(const Shell& s) { return s.num_sms * etc::kCtasPerSm * etc::kWarps; }
+
 // FP32 element pass with the tensor-core contraction; the arguments as for k_element_full<float>.
 shell_status launch_full_tc(Shell& s, const ElemArgs& A, int work) {
   static bool attr_done[64] = {false};

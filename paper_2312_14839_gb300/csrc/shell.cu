@@ -441,10 +441,15 @@ extern "C" shell_status shell_energy_grad_hess(shell_t* shell, const double* q, 
                                                double* energy, double* grad, int want_hessian) {
   if (!shell || !q) return fail(SHELL_ERR_ARG, "NULL argument");
   Shell& s = *shell;
-  if (want_hessian && grad && !s.val_fp64 && s.fuse_first_hessian) {
-    // all three in one pass over the elements, as a Newton step's first residual and Hessian: the FP64 pipe
-    // works beside the FP32 one, and a small shell pays one kernel's latency (280 x 5 patches: 36 us for the
-    // energy kernel alone)
+  // All three in one pass over the elements, as a Newton step's first residual and Hessian: the FP64 pipe works
+  // beside the FP32 one, and a small shell pays one kernel's latency (280 x 5 patches 69 us, in two passes 37 + 37).
+  // Two passes where that costs more. Colour-ordered: every colour's launch would pay the FP64 chain (6 x 6 patches
+  // 186 us against 20 + 111, 100 x 100 465 against 133 + 314, 181 x 181 1,167 against 377 + 800). Between one and
+  // two patches per warp: the FP64 chain of a warp is as long as with two (45 x 45 94 us against 37 + 49; 61 x 61,
+  // two per warp, 133 against 66 + 73).
+  const int warps = element_tc_warps(s);
+  if (want_hessian && grad && !s.val_fp64 && s.fuse_first_hessian && s.elem_tc && s.opt.assembly != SHELL_ASM_COLOR &&
+      (s.n_patches <= warps || s.n_patches >= 2 * warps)) {
     BHEM_CUDA(cudaMemsetAsync(grad, 0, sizeof(double) * s.n_dof, s.stream));
     BHEM_TRY(assemble_hessian(s, q, mass_scale, s.d_Ep, grad, true));
     return launch_energy_sum(s, s.d_Ep, energy ? energy : s.d_energy_tmp);
