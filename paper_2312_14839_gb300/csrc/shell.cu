@@ -644,17 +644,11 @@ static shell_status residual_reuse(Shell& s, const shell_step_params& P, const u
   return SHELL_OK;
 }
 
-static shell_status newton_core(Shell& s, const shell_step_params& P, const unsigned char* mask,
-                                const double* qfix, double* q, const double* v_in,
-                                const double* warm, double* v_out, shell_step_stats& st) {
+// The step from q (a copy of it in d_qn); on errors q holds whatever iterate it had come to.
+static shell_status newton_iterate(Shell& s, const shell_step_params& P, const unsigned char* mask,
+                                   const double* qfix, double* q, const double* v_in,
+                                   const double* warm, double* v_out, shell_step_stats& st) {
   const int m = s.n_dof;
-  if (s.aux_unjoined) {   // the previous step failed while its first Hessian was in flight
-    BHEM_CUDA(cudaStreamSynchronize(s.aux_stream));
-    s.aux_unjoined = false;
-  }
-  s.trace_n = 0;
-  mark(s, "start");
-  BHEM_CUDA(cudaMemcpyAsync(s.d_qn, q, sizeof(double) * m, cudaMemcpyDeviceToDevice, s.stream));
   BHEM_TRY(launch_predictor(s, s.d_qn, v_in, P.dt, s.d_y));
   if (mask) BHEM_TRY(launch_overwrite_fixed(s, q, s.d_qn, mask, qfix));
   double gref = 0.0, gn = 0.0, tau_carry = P.tau_carry;
@@ -837,12 +831,24 @@ static shell_status newton_core(Shell& s, const shell_step_params& P, const unsi
   BHEM_CUDA(cudaStreamSynchronize(s.stream));
   st.diag_fixes = s.h_ns->diag_fixes;
   st.tau_final = tau_carry;
-  if (status == SHELL_OK || status == SHELL_ERR_NOT_CONVERGED) {
-    BHEM_TRY(launch_velocity(s, q, s.d_qn, P.dt, v_out));
-  } else {
-    // leave q unchanged on failure
-    BHEM_CUDA(cudaMemcpyAsync(q, s.d_qn, sizeof(double) * m, cudaMemcpyDeviceToDevice, s.stream));
+  if (status == SHELL_OK || status == SHELL_ERR_NOT_CONVERGED) BHEM_TRY(launch_velocity(s, q, s.d_qn, P.dt, v_out));
+  return status;
+}
+
+static shell_status newton_core(Shell& s, const shell_step_params& P, const unsigned char* mask,
+                                const double* qfix, double* q, const double* v_in,
+                                const double* warm, double* v_out, shell_step_stats& st) {
+  s.trace_n = 0;
+  mark(s, "start");
+  const size_t bytes = sizeof(double) * s.n_dof;
+  BHEM_CUDA(cudaMemcpyAsync(s.d_qn, q, bytes, cudaMemcpyDeviceToDevice, s.stream));
+  const shell_status status = newton_iterate(s, P, mask, qfix, q, v_in, warm, v_out, st);
+  if (s.aux_unjoined) {   // it failed while its first Hessian, which reads q, was in flight
+    BHEM_CUDA(cudaStreamSynchronize(s.aux_stream));
+    s.aux_unjoined = false;
   }
+  if (status != SHELL_OK && status != SHELL_ERR_NOT_CONVERGED)   // whichever way it failed, q is left unchanged
+    BHEM_CUDA(cudaMemcpyAsync(q, s.d_qn, bytes, cudaMemcpyDeviceToDevice, s.stream));
   mark(s, "end");
   trace_report(s);
   return status;
