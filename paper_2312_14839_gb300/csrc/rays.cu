@@ -244,9 +244,10 @@ __device__ void newton_step(bool want, const double* __restrict__ nets, int patc
 
 struct Ray {
   double o[3], d[3], inv[3];
-  // culling: two directions about perpendicular to d and to each other; o and 1 / d in FP32 (infinite
-  // for a zero component, NaN for one too small for FP32: that axis then never rules a box out)
-  float e1[3], e2[3], o32[3], inv32[3];
+  // culling: |d| (0: nothing is culled), d / |d| and two unit directions about perpendicular to it and to each
+  // other; o and 1 / d in FP32 (infinite for a zero component, NaN for one too small or too large for
+  // FP32: that axis then never rules a box out)
+  float len, dir[3], e1[3], e2[3], o32[3], inv32[3];
 };
 
 __device__ __forceinline__ void load_ray(const double* __restrict__ origins, const double* __restrict__ dirs,
@@ -260,10 +261,16 @@ __device__ __forceinline__ void load_ray(const double* __restrict__ origins, con
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     r.o32[c] = (float)r.o[c];
-    r.inv32[c] = r.d[c] == 0.0 ? INFINITY : fabs(r.d[c]) < 1e-30 ? NAN : (float)r.inv[c];
+    r.inv32[c] = r.d[c] == 0.0 ? INFINITY : !(fabs(r.d[c]) >= 1e-30 && fabs(r.d[c]) <= 1e30) ? NAN : (float)r.inv[c];
   }
-  // e1 = d x (the axis d is least along), normalised; e2 = d x e1
-  const float dx = (float)r.d[0], dy = (float)r.d[1], dz = (float)r.d[2];
+  // directions are unit vectors by contract, but the search takes any: the culling works in distances along
+  // the ray, |d| times the differences of tau
+  const double len = sqrt((r.d[0] * r.d[0] + r.d[1] * r.d[1]) + r.d[2] * r.d[2]);
+  r.len = len >= 1e-15 && len <= 1e15 ? (float)len : 0.f;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) r.dir[c] = (float)(r.d[c] / len);
+  // e1 = dir x (the axis it is least along), normalised; e2 = dir x e1
+  const float dx = r.dir[0], dy = r.dir[1], dz = r.dir[2];
   const float ax = fabsf(dx), ay = fabsf(dy), az = fabsf(dz);
   float e[3] = {0.f, dz, -dy};
   if (ay < ax && ay <= az) { e[0] = -dz; e[1] = 0.f; e[2] = dx; }
@@ -321,7 +328,7 @@ struct PlainSmem {
   unsigned short jobs[32 * 12]; // lane * 12 + child * 3 + coordinate
 };
 struct CullSmem : PlainSmem {
-  float path[32][14];           // path point, e1, e2, d (from the patch's centre), best tau beyond it, margin
+  float path[32][14];           // path point from the patch's centre, e1, e2, dir, distance to the best hit, margin
   unsigned char cull[32][4];    // child proven not to lead to a hit
 };
 template <bool kCull> using WarpSmem = std::conditional_t<kCull, CullSmem, PlainSmem>;
@@ -358,7 +365,7 @@ __device__ __forceinline__ bool child_is_culled(const CullNet* __restrict__ N, c
   float mn = t[0];
 #pragma unroll
   for (int k = 1; k < 16; ++k) mn = fminf(mn, t[k]);
-  return mn > path[12] + eps;   // path[12]: best tau less the path point's, rounded up; +infinity without a hit
+  return mn > path[12] + eps;   // path[12]: distance_to_best; +infinity without a hit
 }
 
 __device__ __forceinline__ void put_rect(PlainSmem& sm, int lane, int& nch, double u0, double u1, double v0,
@@ -369,6 +376,12 @@ __device__ __forceinline__ void put_rect(PlainSmem& sm, int lane, int& nch, doub
   R[1] = u1;
   R[2] = v0;
   R[3] = v1;
+}
+
+// From the path point at t0 to the best hit, along the ray, rounded up.
+__device__ __forceinline__ float distance_to_best(const Ray& r, double best, double t0) {
+  const float beyond = (float)(best - t0) * r.len;
+  return beyond + 1e-6f * fabsf(beyond);
 }
 
 // Prepares the culling of candidate c's children: the ray from c's entry point on, relative to the
@@ -383,17 +396,16 @@ __device__ __forceinline__ bool starts_culled(WarpSmem<kCull>& sm, int lane, con
       path[k] = (float)((r.o[k] + c.t0 * r.d[k]) - culls[c.patch].c[k]);
       path[3 + k] = r.e1[k];
       path[6 + k] = r.e2[k];
-      path[9 + k] = (float)r.d[k];
+      path[9 + k] = r.dir[k];
     }
-    const float far = (float)on + fabsf((float)c.t0);
+    const float far = (float)on + fabsf((float)c.t0) * fmaxf(1.f, r.len);
     path[13] = fmaxf(kCullAbs, 4e-12f * (1.f + far));   // 4 x Newton's tolerance
     // nothing is culled among children of the margin's size: their tests are left out. Far from the
     // origin (FP64 distances above 1e4 are 1e-12 apart) equal keys are common and the order in which
     // the heap happens to hold them matters, so nothing is culled there either.
-    cullable = (float)c.ext > 8.f * cull_margin(culls + c.patch, path) && far < kCullFar;
+    cullable = r.len > 0.f && (float)c.ext > 8.f * cull_margin(culls + c.patch, path) && far < kCullFar;
     if (!cullable) return false;
-    const float beyond = (float)(best - c.t0);
-    path[12] = beyond + 1e-6f * fabsf(beyond);
+    path[12] = distance_to_best(r, best, c.t0);
     if (c.u1 - c.u0 == 1.0 && c.v1 - c.v0 == 1.0) {
       const double R[4] = {0.0, 1.0, 0.0, 1.0};
       return child_is_culled(culls + c.patch, path, R);
@@ -516,8 +528,7 @@ __device__ void search(Heap& h, const Ray& r, const double* __restrict__ nets, c
       sm.patch[lane] = c.patch;
       h.boxes += nch;
       if constexpr (kCull) {   // a root found above may have brought the best hit nearer
-        const float beyond = (float)(S.best - c.t0);
-        sm.path[lane][12] = beyond + 1e-6f * fabsf(beyond);
+        sm.path[lane][12] = distance_to_best(r, S.best, c.t0);
       }
     }
     unsigned keep = (1u << nch) - 1u;   // children to box
