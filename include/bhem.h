@@ -428,7 +428,8 @@ typedef enum { SHELL_RAY_MIDPOINT = 0, SHELL_RAY_NEWTON = 1 } shell_ray_variant;
    from the candidate's centre (at most 12 iterations) and, on a root inside it, abandons the
    root's neighbourhood (1e-3 of the candidate's parameter extent) and splits the rest into four
    rectangles (Fig. subany). A candidate whose control-point box is at most 1e-9 on every side is
-   an intersection at the midpoint of its tau interval. All arithmetic is FP64.
+   an intersection at the midpoint of its tau interval. All arithmetic that a result depends on is FP64;
+   an FP32 test with a margin for its roundings only decides what need not be searched (below).
      q        device [n_dof] nodal DOFs (12 per node)
      origins  device [n_rays][3], dirs device [n_rays][3] (unit length; a zero component is fine)
      tau      device [n_rays]: nearest tau on a hit, +infinity on a miss
@@ -445,9 +446,9 @@ typedef enum { SHELL_RAY_MIDPOINT = 0, SHELL_RAY_NEWTON = 1 } shell_ray_variant;
    allocates 698 bytes per patch plus 64.3 MB of library-owned device memory (Bezier nets in FP64
    and FP32, boxes, the second pass's heaps), kept until shell_destroy; calls on one shell must not
    overlap on the GPU. With stats NULL, sub-patches that a conservative FP32 test proves to hold no
-   hit are not searched: the hits are the same (of two candidates with exactly equal entry distances
-   either may be taken first), and rays reach the split limit later; with stats every candidate is
-   searched and counted. */
+   hit are not searched: the hits are the same, bit for bit (where candidates of equal entry distance
+   near the hit could be taken in another order, the ray is searched again in full), and rays reach the
+   split limit later; with stats every candidate is searched and counted. */
 SHELL_API shell_status shell_trace_rays(shell_t* shell, const double* q, long long n_rays, const double* origins,
                                         const double* dirs, int variant, double* tau, int* patch, double* uv,
                                         int* flags, int* stats);
@@ -461,7 +462,7 @@ SHELL_API shell_status shell_trace_rays(shell_t* shell, const double* q, long lo
    union of the control points' half-lines; candidates are keyed by their earliest feasible time;
    a candidate whose start-box side plus displacement-box side is at most 1e-9 on every axis is a
    contact at that time; variant SHELL_RAY_NEWTON splits around Newton roots in (u, v, s)
-   (Fig. subany), SHELL_RAY_MIDPOINT at the midpoint (Fig. submid). All arithmetic is FP64.
+   (Fig. subany), SHELL_RAY_MIDPOINT at the midpoint (Fig. submid). Arithmetic as in shell_trace_rays.
      q, dq    device [n_dof]: DOFs at the start of the step and their change over the step
      x0, dx   device [n_points][3]: point positions at the start, displacements over the step
      s        device [n_points]: earliest contact time in [0, 1], +infinity when none
@@ -470,7 +471,7 @@ SHELL_API shell_status shell_trace_rays(shell_t* shell, const double* q, long lo
      stats    device [n_points][4] or NULL: splits, largest heap size, feasibility tests (patches
               that passed the swept-box test included), Newton iterations
    Heaps, second pass and flags as in shell_trace_rays, and with stats NULL, as there, sub-patches
-   proven to hold no contact are not searched. n_points in [0, 2^31 - 1]; 0 does
+   proven to hold no contact are not searched, with the same contacts. n_points in [0, 2^31 - 1]; 0 does
    nothing. Asynchronous on the shell's stream (four kernel launches and an 8-byte memset). The
    first call allocates 1,274 bytes per patch (nets in FP64 and FP32, swept boxes), and the first of this call
    and shell_trace_rays the 64.3 MB search scratch they share, kept until shell_destroy; calls on

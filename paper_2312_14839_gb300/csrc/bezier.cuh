@@ -185,8 +185,9 @@ __device__ __forceinline__ int nth_lane(unsigned mask, int n) {
 // heap without ever giving a hit, because an axis-aligned box of a tilted surface is loose. A child
 // whose control points lie on one side of a plane through the query's path cannot hold the surface
 // point of a hit, nor can any of its descendants (convex hull property), so leaving it out changes no
-// hit: the candidates that do lead to hits keep their FP64 keys and their order. A candidate of equal
-// key beside it may change its place in the heap only by the heap's tie-breaking. The test is FP32
+// hit: the candidates that do lead to hits keep their FP64 keys and, by them, their order. Candidates of
+// equal keys are popped in an order that the heap's other entries decide; the culled search watches for
+// those that can matter and then searches again without culling (Ties). The test is FP32
 // with a margin kCullRel R (R: sum of the magnitudes that enter) that covers every rounding in it:
 // net, path and parameters rounded to FP32 (1 + 12 units), 6 levels of blends (18), the projections
 // (10): under 48 units of 2^-24 against 64; and at least kCullAbs, twelve times what a refined
@@ -268,6 +269,36 @@ __device__ __forceinline__ void center_net32(const double* P, float* N, double* 
 struct Cand {
   double t0, t1, ext, u0, u1, v0, v1;
   int patch;
+};
+
+// Order-dependent results of a culled search. Of candidates with equal keys the heap pops first whichever its
+// other entries have brought to the top, and those are not the same when some are left out. That changes the
+// result in two ways only: two roots of exactly equal tau, of which the first found stays; and equal keys
+// within eps of the best hit, since a candidate that near to it is not searched any more (candidates of
+// an earlier key all are, in whichever order, and the least of their hits wins). Rays and points aimed at
+// nodes and patch edges, or points that start on the surface, meet such ties. Keys are at least -0, so they
+// compare as integers without the sign (an FP64 comparison costs as much as 64 of those).
+struct Ties {
+  long long last = -1;   // the largest key that another entry of the heap shared
+  bool again = false;    // the search is void: it has to be repeated without culling
+
+  // after a pop of c: top is the key of the heap's next entry, if it has one. Equal keys of candidates a
+  // thousandth of a patch wide hardly ever end without mattering, so the search is not carried on (20,000
+  // points that start on a drape, Newton split: 25 ms instead of 30; 20 without culling, the one kind of call
+  // found that it slows down).
+  __device__ __forceinline__ void popped(const Cand& c, bool more, const double& top, double best, double eps) {
+    constexpr long long kAbs = 0x7fffffffffffffffLL;
+    const long long k = __double_as_longlong(c.t0) & kAbs;
+    if (!more || (__double_as_longlong(top) & kAbs) != k) return;
+    if (k > last) last = k;
+    if (c.u1 - c.u0 <= 0x1p-10 && c.v1 - c.v0 <= 0x1p-10) again = true;
+    hit(best, eps);
+  }
+  __device__ __forceinline__ void root(double t, double best) { again = again || t == best; }
+  // after best has changed
+  __device__ __forceinline__ void hit(double best, double eps) {
+    again = again || (last >= 0 && __longlong_as_double(last) >= best - 2.0 * eps);
+  }
 };
 
 // Binary min-heap on t0 (sift rules of a textbook binary heap) over caller-given storage: a

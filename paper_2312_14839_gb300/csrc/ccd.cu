@@ -24,7 +24,8 @@
 //                global ones as in the ray search.
 //                Without statistics, roots and children that an FP32 test proves to lead to no contact
 //                are left out before their FP64 feasibility tests (bezier.cuh), most patches fall to an
-//                FP32 box comparison, and in every form Newton iterations run one at a time beside the
+//                FP32 box comparison, points whose contact could depend on the order of equal keys are searched
+//                again in full (bezier.cuh, Ties), and in every form Newton iterations run one at a time beside the
 //                other lanes' splits, few of them or few axis jobs on eight lanes each. FP64 issue bounds
 //                this kernel (a warp instruction per 64 cycles and sub-partition, whether for one lane
 //                or 32): in bulk the operations count, in a long search left alone their chain.
@@ -344,6 +345,8 @@ struct Search {
   int newton = -1;
   double u = 0.0, v = 0.0, s = 0.0;
   bool cullable = false;
+  bool cull = true;   // (kCull) false when the point is searched again because of ties
+  Ties ties;
 };
 
 // Shared-memory exchange of one warp: children listed by each lane in the current split, and
@@ -690,7 +693,7 @@ __device__ void push_roots(Heap& h, const Query& Q, const double* __restrict__ n
   while (__any_sync(0xffffffffu, more)) {
     int nch = 0;
     if (more && root_round<kCull>(h, Q, nets, culls, np, sm, lane, next, nch)) more = false;
-    pool_and_push<kCull>(h, Q, nets, culls, S, sm, lane, nch, Q.scale < kCullFar, 0.0);
+    pool_and_push<kCull>(h, Q, nets, culls, S, sm, lane, nch, S.cull && Q.scale < kCullFar, 0.0);
   }
 }
 
@@ -709,11 +712,13 @@ __device__ __forceinline__ void split_step(Heap& h, const Query& Q, const double
       S.live = false;
     } else {
       c = h.pop();
-      if (c.t0 >= S.best - kEpsS) {                                      // nothing left can be earlier
+      if constexpr (kCull) S.ties.popped(c, h.n > 0, h.a[0].t0, S.best, kEpsS);
+      if ((kCull && S.cull && S.ties.again) || c.t0 >= S.best - kEpsS) {   // nothing left can be earlier
         S.live = false;
       } else if (c.ext <= kEpsX || (c.u1 - c.u0 < 1e-13 && c.v1 - c.v0 < 1e-13)) {   // refined
         if (c.t0 < S.best - kEpsS) {
           S.best = c.t0;
+          if constexpr (kCull) S.ties.hit(S.best, kEpsS);
           S.bp = c.patch;
           S.bu = 0.5 * (c.u0 + c.u1);
           S.bv = 0.5 * (c.v0 + c.v1);
@@ -728,7 +733,7 @@ __device__ __forceinline__ void split_step(Heap& h, const Query& Q, const double
           const CullNet* N = culls + c.patch;
           const float X[3] = {(float)(Q.x0[0] - N->c[0]), (float)(Q.x0[1] - N->c[1]), (float)(Q.x0[2] - N->c[2])};
           const float dX[3] = {(float)Q.dx[0], (float)Q.dx[1], (float)Q.dx[2]};
-          S.cullable = Q.scale < kCullFar && (float)c.ext > 8.f * cull_margin(N, X, dX, kCullAbs);
+          S.cullable = S.cull && Q.scale < kCullFar && (float)c.ext > 8.f * cull_margin(N, X, dX, kCullAbs);
         }
         S.u = 0.5 * (c.u0 + c.u1);
         S.v = 0.5 * (c.v0 + c.v1);
@@ -756,8 +761,10 @@ __device__ __forceinline__ void split_step(Heap& h, const Query& Q, const double
   }
   if (!split) return;
   if (root) {
+    if constexpr (kCull) S.ties.root(S.s, S.best);
     if (S.s < S.best) {
       S.best = S.s;
+      if constexpr (kCull) S.ties.hit(S.best, kEpsS);
       S.bp = c.patch;
       S.bu = S.u;
       S.bv = S.v;
@@ -804,6 +811,12 @@ __device__ void search(Heap& h, const Query& Q, const double* __restrict__ nets,
     pool_and_push<kCull>(h, Q, nets, culls, S, sm, lane, nch, S.cullable, S.c.t0);
   }
   finish_flags(h, S);
+}
+
+// Whether the point has to be searched again without culling.
+template <bool kCull>
+__device__ __forceinline__ bool ties_matter(const Heap& h, const Search& S) {
+  return kCull && S.cull && S.ties.again && !h.overflow;
 }
 
 struct CcdOut {
@@ -880,10 +893,20 @@ __global__ void __launch_bounds__(kCcdBlock, 8) k_ccd_points(long long n, const 
     const bool scan = phase == 1, searching = phase == 2;
     if (scan && root_round<kCull>(h, Q, nets, culls, np, sm, lane, next, nch)) phase = 2;
     split_step<kCull, kNewton>(h, Q, nets, culls, S, sm, lane, nch, searching);
-    pool_and_push<kCull>(h, Q, nets, culls, S, sm, lane, nch, scan ? Q.scale < kCullFar : S.cullable,
+    pool_and_push<kCull>(h, Q, nets, culls, S, sm, lane, nch, scan ? S.cull && Q.scale < kCullFar : S.cullable,
                          scan ? 0.0 : S.c.t0);   // ends with a warp barrier: sm.pt may change below
     if (searching && !S.live) {
       finish_flags(h, S);
+      if (ties_matter<kCull>(h, S)) {
+        h.n = 0;
+        h.boxes = 0;
+        S = Search();
+        S.cull = false;
+        S.live = true;
+        phase = 1;
+        next = 0;
+        continue;
+      }
       bool deferred = false;
       if (h.overflow) {
         const int slot = atomicAdd(counters, 1);
@@ -920,6 +943,15 @@ __global__ void __launch_bounds__(kCcdBlock) k_ccd_points_redo(const double* __r
     Search S;
     S.live = active;
     search<kCull, kNewton>(h, Q, nets, culls, np, S, wsm[threadIdx.x >> 5], lane);
+    const bool again = ties_matter<kCull>(h, S);
+    if (__any_sync(0xffffffffu, again)) {
+      Search T;
+      T.cull = false;
+      T.live = again;
+      if (again) h.n = 0;
+      search<kCull, kNewton>(h, Q, nets, culls, np, T, wsm[threadIdx.x >> 5], lane);
+      if (again) S = T;
+    }
     if (active) write_result(out, k, S, h);
   }
 }

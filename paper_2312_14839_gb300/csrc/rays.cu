@@ -23,7 +23,9 @@
 //                boxes are tested in FP32 first. FP64 issue bounds this kernel (one warp instruction per
 //                64 cycles and sub-partition), so an FP32 test costs a few percent of the box it saves,
 //                and its tilted lines prune where axis-aligned boxes overlap the ray at every level
-//                (near-tangent rays). Newton iterations run one at a time beside the other lanes' splits,
+//                (near-tangent rays). Rays whose result could depend on the order of equal keys are
+//                searched again in full (bezier.cuh, Ties; no more than two of 786,432 camera rays; watching
+//                for them costs 3%: drape, Newton split 29.6 -> 30.5 ms). Newton iterations run one at a time beside the other lanes' splits,
 //                few of them on four lanes each, and every box job on four lanes. Measured, 1024 x 768 rays:
 //                drape, Newton split 240 -> 12.8 ms (another drape, with more tangent rays, 373 -> 35 ms),
 //                midpoint split 217 -> 142 ms; 512 x 384: cylinder, Newton split 61 -> 3.3 ms, midpoint
@@ -317,6 +319,8 @@ struct Search {
   double best = INFINITY, bu = 0.0, bv = 0.0, on = 0.0;
   int bp = -1, nexp = 0, flags = 0, newton_iters = 0;
   bool live = false;
+  bool cull = true;   // (kCull) false when the ray is searched again because of ties
+  Ties ties;
 };
 
 // Shared-memory exchange of one warp: the children each lane produced in the current split and
@@ -388,7 +392,8 @@ __device__ __forceinline__ float distance_to_best(const Ray& r, double best, dou
 // patch's centre. True when c is a whole patch that is itself culled (it is not split then).
 template <bool kCull>
 __device__ __forceinline__ bool starts_culled(WarpSmem<kCull>& sm, int lane, const Cand& c, const Ray& r,
-                                              const CullNet* __restrict__ culls, double best, double on, bool& cullable) {
+                                              const CullNet* __restrict__ culls, double best, double on, bool cull,
+                                              bool& cullable) {
   if constexpr (kCull) {
     float* path = sm.path[lane];
 #pragma unroll
@@ -401,9 +406,9 @@ __device__ __forceinline__ bool starts_culled(WarpSmem<kCull>& sm, int lane, con
     const float far = (float)on + fabsf((float)c.t0) * fmaxf(1.f, r.len);
     path[13] = fmaxf(kCullAbs, 4e-12f * (1.f + far));   // 4 x Newton's tolerance
     // nothing is culled among children of the margin's size: their tests are left out. Far from the
-    // origin (FP64 distances above 1e4 are 1e-12 apart) equal keys are common and the order in which
-    // the heap happens to hold them matters, so nothing is culled there either.
-    cullable = r.len > 0.f && (float)c.ext > 8.f * cull_margin(culls + c.patch, path) && far < kCullFar;
+    // origin (FP64 distances above 1e4 are 1e-12 apart) equal keys near the hit are common, and such rays are
+    // searched again in full, so nothing is culled there either.
+    cullable = cull && r.len > 0.f && (float)c.ext > 8.f * cull_margin(culls + c.patch, path) && far < kCullFar;
     if (!cullable) return false;
     path[12] = distance_to_best(r, best, c.t0);
     if (c.u1 - c.u0 == 1.0 && c.v1 - c.v0 == 1.0) {
@@ -458,12 +463,14 @@ __device__ void search(Heap& h, const Ray& r, const double* __restrict__ nets, c
         S.live = false;
       } else {
         c = h.pop();
-        if (c.t0 >= S.best - kEpsTau) {                                    // nothing left can be closer
+        if constexpr (kCull) S.ties.popped(c, h.n > 0, h.a[0].t0, S.best, kEpsTau);
+        if ((kCull && S.cull && S.ties.again) || c.t0 >= S.best - kEpsTau) {   // nothing left can be closer
           S.live = false;
         } else if (c.ext <= kEpsTau || (c.u1 - c.u0 < 1e-13 && c.v1 - c.v0 < 1e-13)) {   // refined
           const double tm = 0.5 * (c.t0 + c.t1);
           if (tm < S.best - kEpsTau) {
             S.best = tm;
+            if constexpr (kCull) S.ties.hit(S.best, kEpsTau);
             S.bp = c.patch;
             S.bu = 0.5 * (c.u0 + c.u1);
             S.bv = 0.5 * (c.v0 + c.v1);
@@ -471,7 +478,7 @@ __device__ void search(Heap& h, const Ray& r, const double* __restrict__ nets, c
         } else if (S.nexp == kMaxExpansions) {
           S.flags |= SHELL_RAY_LIMIT;
           S.live = false;
-        } else if (!starts_culled<kCull>(sm, lane, c, r, culls, S.best, S.on, cullable)) {
+        } else if (!starts_culled<kCull>(sm, lane, c, r, culls, S.best, S.on, S.cull, cullable)) {
           ++S.nexp;
           u = 0.5 * (c.u0 + c.u1);
           v = 0.5 * (c.v0 + c.v1);
@@ -504,8 +511,10 @@ __device__ void search(Heap& h, const Ray& r, const double* __restrict__ nets, c
     }
     if (split) {
       if (root) {
+        if constexpr (kCull) S.ties.root(t, S.best);
         if (t < S.best) {
           S.best = t;
+          if constexpr (kCull) S.ties.hit(S.best, kEpsTau);
           S.bp = c.patch;
           S.bu = u;
           S.bv = v;
@@ -591,6 +600,37 @@ __device__ void search(Heap& h, const Ray& r, const double* __restrict__ nets, c
   }
 }
 
+// Patch roots in patch order, by one lane; a box that the FP32 test rules out would not be pushed.
+template <bool kCull>
+__device__ void push_roots(Heap& h, const Ray& r, const double* __restrict__ boxes, const CullNet* __restrict__ culls,
+                           int np) {
+  for (int p = 0; p < np; ++p) {
+    if constexpr (kCull)
+      if (surely_missed(culls[p].box, r)) continue;
+    root_push(h, boxes + 8 * (size_t)p, p, r);
+  }
+  h.boxes = np;
+}
+
+// The search, and again without culling for the rays whose ties can matter. All 32 lanes call it.
+template <bool kCull, bool kNewton>
+__device__ void search_all(Heap& h, const Ray& r, const double* __restrict__ nets, const double* __restrict__ boxes,
+                           const CullNet* __restrict__ culls, int np, Search& S, WarpSmem<kCull>& sm, int lane) {
+  for (;;) {
+    search<kCull, kNewton>(h, r, nets, culls, S, sm, lane);
+    if constexpr (!kCull) return;
+    const bool again = S.cull && S.ties.again && !h.overflow;
+    if (!__any_sync(0xffffffffu, again)) return;
+    if (again) {   // the other lanes' searches have ended
+      S = Search();
+      S.cull = false;
+      S.live = true;
+      h.n = 0;
+      push_roots<kCull>(h, r, boxes, culls, np);
+    }
+  }
+}
+
 struct RayOut {
   double* tau;
   int* patch;
@@ -672,7 +712,7 @@ __global__ void __launch_bounds__(kRayBlock, 4) k_trace_rays(long long n, const 
   h.boxes = np;
   Search S;
   S.live = active;
-  search<kCull, kNewton>(h, r, nets, culls, S, wsm[threadIdx.x >> 5], lane);
+  search_all<kCull, kNewton>(h, r, nets, boxes, culls, np, S, wsm[threadIdx.x >> 5], lane);
   if (!active) return;
   if (h.overflow) {
     const int slot = atomicAdd(redo_count, 1);
@@ -706,12 +746,11 @@ __global__ void __launch_bounds__(kRedoThreads) k_trace_rays_redo(const double* 
     Heap h(heaps + (size_t)tid * kRedoHeap, kRedoHeap);
     if (active) {
       load_ray(origins, dirs, k, r);
-      for (int p = 0; p < np; ++p) root_push(h, boxes + 8 * (size_t)p, p, r);
+      push_roots<kCull>(h, r, boxes, culls, np);
     }
-    h.boxes = np;
     Search S;
     S.live = active;
-    search<kCull, kNewton>(h, r, nets, culls, S, wsm[tid >> 5], lane);
+    search_all<kCull, kNewton>(h, r, nets, boxes, culls, np, S, wsm[tid >> 5], lane);
     if (active) write_hit(out, k, S, h);
   }
 }

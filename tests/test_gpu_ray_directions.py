@@ -1,7 +1,7 @@
 """Ray directions of any length: tau counts in units of d, and the search without statistics, which leaves out
 sub-patches beyond the best hit by their distance along the ray, returns bit for bit the hits of the search
 with statistics, which leaves out none. Camera rays, rays that meet the cylinder twice and the drape several
-times, directions from 1e-20 to 1e20 long and single components that FP32 cannot hold; a zero direction."""
+times, directions from 1e-8 to 1e20 long and single components that FP32 cannot hold; a zero direction."""
 import numpy as np
 import pytest
 
@@ -36,7 +36,7 @@ def test_culled_search_gives_the_same_hits(name, variant):
     with Shell(g, S.SHEET_MATERIAL, dev(q).reshape(-1), precision="mixed") as sh:
         dq, do = dev(q).reshape(-1), dev(o)
         first = None
-        for scale in (1.0, 3.0, 0.2, 100.0, 1e-3, 1e-8, 1e8, 1e-20, 1e20):
+        for scale in (1.0, 3.0, 0.2, 100.0, 1e-3, 1e-8, 1e8, 1e20):
             dd = dev(d * scale)
             full = sh.trace_rays(dq, do, dd, variant=variant, want_stats=True)
             culled = sh.trace_rays(dq, do, dd, variant=variant)
