@@ -573,7 +573,7 @@ k_pcg_init(WorkList L, ShellState* st, const double* __restrict__ g,
 // linearity, so no separate p-update launch follows the update; p.y per shell, and in the last CTA
 // alpha = rz / p.y, or negative curvature. A CTA takes consecutive groups, so it sums p.y over a
 // shell's groups in registers and adds it once. Every block of a row is loaded before its use, as in
-// the single-shell product (4 CTAs per SM at 56 registers; 3 without the 180 bytes of spills: 12%
+// the single-shell product; its four products are added up before the row's sum takes them (4 CTAs per SM at 56 registers; 3 without the 180 bytes of spills: 12%
 // slower). Latency bounds it below about 100 shells, DRAM above.
 __global__ void __launch_bounds__(kSpmvThreads, 4)
 k_spmv(WorkList L, ShellState* st, const int* __restrict__ rp,
@@ -611,10 +611,7 @@ k_spmv(WorkList L, ShellState* st, const int* __restrict__ rp,
       for (int u = 0; u < U; ++u)
         if (k0 + u < k1) {
           const float4 xv = *reinterpret_cast<const float4*>(x + (size_t)j[u] * 12 + cc * 4);
-          acc = __fmaf_rn(v[u].x, xv.x, acc);
-          acc = __fmaf_rn(v[u].y, xv.y, acc);
-          acc = __fmaf_rn(v[u].z, xv.z, acc);
-          acc = __fmaf_rn(v[u].w, xv.w, acc);
+          acc += v[u].x * xv.x + v[u].y * xv.y + v[u].z * xv.z + v[u].w * xv.w;
         }
     }
     float* sa = sacc[w & 1];   // the other half may still be read
@@ -699,8 +696,9 @@ k_pcg_update(WorkList L, ShellState* st, float* __restrict__ x,
     if (in) {
       if (!(mask && mask[gi])) {
         const float* q = sr[w & 1][ln];   // the other half may still be read
-        zi = d0.x * q[0] + d0.y * q[1] + d0.z * q[2] + d0.w * q[3] + d1.x * q[4] + d1.y * q[5] + d1.z * q[6] +
-             d1.w * q[7] + d2.x * q[8] + d2.y * q[9] + d2.z * q[10] + d2.w * q[11];
+        const float d[12] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w, d2.x, d2.y, d2.z, d2.w};
+#pragma unroll
+        for (int c = 0; c < 12; ++c) zi = __fmaf_rn(d[c], q[c], zi);   // as apply_block
       }
       z[gi] = zi;
     }
