@@ -573,8 +573,8 @@ k_pcg_init(WorkList L, ShellState* st, const double* __restrict__ g,
 // linearity, so no separate p-update launch follows the update; p.y per shell, and in the last CTA
 // alpha = rz / p.y, or negative curvature. A CTA takes consecutive groups, so it sums p.y over a
 // shell's groups in registers and adds it once. Every block of a row is loaded before its use, as in
-// the single-shell product; its four products are added up before the row's sum takes them (4 CTAs per SM at 56 registers; 3 without the 180 bytes of spills: 12%
-// slower). Latency bounds it below about 100 shells, DRAM above.
+// the single-shell product (4 CTAs per SM at 56 registers; 3 without the 180 bytes of spills: 12%
+// slower); its four products are added up before the row's sum takes them. Latency bounds it below about 100 shells, DRAM above.
 __global__ void __launch_bounds__(kSpmvThreads, 4)
 k_spmv(WorkList L, ShellState* st, const int* __restrict__ rp,
        const int* __restrict__ col, const float* __restrict__ val, const float* __restrict__ x,

@@ -38,11 +38,6 @@ constexpr int kNormSize = 96;
 
 using bf16 = __nv_bfloat16;
 
-__device__ __forceinline__ float gelu(float x) { return 0.5f * x * (1.f + erff(x * 0.70710678118654752f)); }
-__device__ __forceinline__ float gelu_grad(float x) {
-  return 0.5f * (1.f + erff(x * 0.70710678118654752f)) + x * 0.39894228040143268f * expf(-0.5f * x * x);
-}
-
 constexpr int kErrIndex = 1, kErrTimeout = 2;   // bits of the network's error word
 
 // ------------------------------------------------------------------------------------------
@@ -167,14 +162,10 @@ __global__ void k_targets(long long n_dof, const double* __restrict__ q_next, co
     T[e] = (float)(q_next[e] - q[e] - dt * v[e]);
 }
 
-// warm = q + dt v + out_std * Z + out_mean (the inertial predictor alone when Z is NULL)
-__global__ void k_compose(int n_nodes, const double* __restrict__ q, const double* __restrict__ v, double dt,
-                          const float* __restrict__ Z, const float* __restrict__ norm, double* __restrict__ warm) {
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n_nodes * kOut; e += gridDim.x * blockDim.x) {
-    const int r = e / kOut, c = e % kOut;
-    const float y = Z ? Z[(long long)r * kOutPad + c] * norm[kNormOutStd + c] + norm[kNormOutMean + c] : 0.f;
-    warm[e] = q[e] + dt * v[e] + (double)y;
-  }
+// warm = q + dt v, the inertial predictor alone
+__global__ void k_predict(int n_dof, const double* __restrict__ q, const double* __restrict__ v, double dt,
+                          double* __restrict__ warm) {
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n_dof; e += gridDim.x * blockDim.x) warm[e] = q[e] + dt * v[e];
 }
 
 // ------------------------------------------------------------------------------------------
@@ -955,8 +946,7 @@ extern "C" shell_status shell_mlp_warm_start(shell_mlp_t* M, shell_t* shell, con
   if (!shell || !q || !v || !warm) return fail(SHELL_ERR_ARG, "NULL argument");
   Shell& s = *shell;
   if (!M) {
-    k_compose<<<eblocks((long long)s.n_nodes * kOut), 256, 0, s.stream>>>(s.n_nodes, q, v, dt, nullptr, nullptr,
-                                                                          warm);
+    k_predict<<<eblocks(s.n_dof), 256, 0, s.stream>>>(s.n_dof, q, v, dt, warm);
     BHEM_CUDA(cudaGetLastError());
     ++s.launches;
     return SHELL_OK;
