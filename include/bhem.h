@@ -152,7 +152,8 @@ SHELL_API shell_status shell_info(const shell_t* shell, shell_info_t* info);
 
 /* Budget of the library's bounded device-side waits on this shell: the exchanges between the CTAs
    of the resident linear solve (the default on shells whose matrix fits the multiprocessors' shared
-   memory: up to 4,864 nodes in mixed precision, 2,584 in FP64, with 152 multiprocessors), the grid
+   memory and have a thread for every row: up to 4,864 nodes in mixed precision, 2,584 in FP64, with 152
+   multiprocessors), the grid
    barriers of the persistent mixed-precision PCG (one cooperative launch per solve; selected by the environment
    variable BHEM_PCG_LOOP=persistent when the shell is created), the mbarrier waits of
    the bulk-copy SpMV (SHELL_SPMV_TMA) and those of the tensor-core element pass (mixed
@@ -162,6 +163,9 @@ SHELL_API shell_status shell_info(const shell_t* shell, shell_info_t* info);
    bulk-copy SpMV and the tensor-core element pass still wait, with the default budget, for the
    copies or MMAs they have issued (then free their tensor memory), so that the device stays
    usable.
+   The resident solve starts when all its CTAs (up to one per multiprocessor) fit at once: beside a
+   kernel of another stream that holds multiprocessors it waits for that kernel, which the budget does
+   not count; BHEM_PCG_LOOP=graph at shell_create keeps separate kernels, which share the device.
    polls < 0 restores the default (2^20 polls); 0 makes every such wait expire at once (a test
    of the timeout path). Synchronises the shell's stream and drops its cached PCG graphs. No paper
    counterpart (a watchdog of this implementation). */
